@@ -262,6 +262,25 @@ def apply_group_sizes(k, factor_bits, tensor_cores=False):
     return out
 
 
+def front_group_sizes(k, factor_bits):
+    """Live right-hand sides of each pass of the apply with sparse factors: groups of up to 8 (FP32) or
+    2 (FP64)."""
+    out, r0 = [], 0
+    while r0 < k:
+        rem = k - r0
+        kr = min(rem, 2) if factor_bits == 64 else (8 if rem >= 5 else (4 if rem >= 3 else rem))
+        out.append(min(kr, rem))
+        r0 += out[-1]
+    return out
+
+
+def front_apply_bytes(arena_bytes, rows, nr):
+    """Algorithmic bytes of one pass of the apply with sparse factors: every stored factor entry once,
+    and per local unknown a 4 B index and, for each of the nr right-hand sides, a 16 B gather and a
+    16 B scatter."""
+    return float(arena_bytes) + rows * (4 + 32 * nr)
+
+
 TRAFFIC = os.path.join(ROOT, "profiles", "roofline_traffic.json")
 # the LU schedule and update kernel the committed counters must have been taken on
 UPDATE_VERSION = "tcgen05 update with 128x256 and 128x64 blocks, sub-panel schedule (left-looking sub-panels of 8 steps)"
@@ -307,7 +326,7 @@ def roofline(timings, upd_flops_per_factor, apply_bytes, factors, hbm, bf16_sus,
         cls["lu_update"] = (um + pm, un + pn)
     dom = max(cls, key=lambda c: cls[c][0])
     out = {}
-    if "lu_update" in cls:
+    if "lu_update" in cls and upd_flops_per_factor is not None:
         ms, _ = cls["lu_update"]
         achieved = upd_flops_per_factor * factors / (ms / 1e3) / 1e12
         if factor_bits == 64:
@@ -749,12 +768,11 @@ def run_ours(args, world, rank, local):
     # true residual of the last field, FP64, on the host with the library's own A (sanity)
     x_last = x_d.cpu().numpy()
     iters = max(i["iterations"] for i in infos[-1])
-    fb = 16 if w.factor_bits == 64 else 8
-    tc_apply = args.apply_engine == "auto" and w.factor_bits == 32 and krhs >= 8
-    groups = apply_group_sizes(krhs, w.factor_bits, tc_apply)
-    upd_flops, _ = work_model(O, h, w.nsub, 1, fb)
-    # bytes of one apply launch, averaged over the launches of a step (groups of right-hand sides)
-    apply_bytes = sum(work_model(O, h, w.nsub, g, fb)[1] for g in groups) / len(groups)
+    groups = front_group_sizes(krhs, w.factor_bits)
+    arena = O.oras_arena_bytes(h)
+    rows = sum(O.oras_subdomain_size(h, s)[0] for s in range(w.nsub))
+    # bytes of one apply pass, averaged over the passes of a step (groups of right-hand sides)
+    apply_bytes = sum(front_apply_bytes(arena, rows, g) for g in groups) / len(groups)
     nnz = O.oras_nnz(h)
     spmv_total = 0.0
     for info in infos:
@@ -762,23 +780,12 @@ def run_ours(args, world, rank, local):
         cyc = max(i["restarts"] for i in info)
         if w.factor_bits == 32:   # the Arnoldi SpMV (class "spmv"); true residuals are class "spmv64"
             spmv_total += it * sum(spmv_bytes(n, nnz, g, True) for g in rhs_groups(krhs, 8))
-    dom, roofs = roofline(timings, upd_flops, apply_bytes, args.steps, hbm, bf16_sus, w.factor_bits, spmv_total)
-    if "lu_update" in roofs and w.factor_bits == 32:
-        ru = roofs["lu_update"]
-        ru["traffic"] = measured_traffic("k_lu_update_tc", w.name, panel)
-        if ru["traffic"] is not None:
-            ru["traffic_note"] = ("DRAM read+write bytes per launch, averaged over every trailing-update launch of "
-                                  "a factorisation, from the ncu capture recorded in profiles/roofline_traffic.json")
-        else:
-            ru["traffic_note"] = ("null: the update's DRAM traffic is captured on the 8^3 profile workload at panel width "
-                                  "24 (profiles/k_lu_update_tc_head8.md, profiles/roofline_traffic.json); it does not "
-                                  "grow in proportion to the flops between workloads (the panel updates re-read the "
-                                  "panel's own rows and columns), so it is not scaled to this one")
-    if "apply" in roofs and tc_apply:
-        roofs["apply"]["kernel"] = ("k_apply_tc (ORAS preconditioner, tcgen05 kind::tf32 products, up to 32 "
-                                    "right-hand sides per arena pass)")
+    dom, roofs = roofline(timings, None, apply_bytes, args.steps, hbm, bf16_sus, w.factor_bits, spmv_total)
+    if "apply" in roofs:
+        roofs["apply"]["kernel"] = ("k_fr_fwd / k_fr_bwd (ORAS preconditioner with sparse local factors, one launch per tree "
+                                    "level and direction; the bytes count each stored entry once, the two "
+                                    "directions read the border entries twice)")
     roof = roofs[dom]
-    arena = O.oras_arena_bytes(h)
     O.oras_destroy(h)
     # ---------------- end to end through the public API with host buffers
     e2e_steps = args.e2e_steps if args.e2e_steps is not None else max(1, args.steps)
@@ -841,7 +848,7 @@ def run_ours(args, world, rank, local):
                        "nsub": w.nsub, "overlap_layers": w.overlap, "restart": w.restart, "tol": w.tol,
                        "rhs_per_step": krhs, "factor_arena_bytes": arena,
                        "l2": "512 MiB buffer written between timed steps; the step itself streams the "
-                             f"{arena / 1e9:.1f} GB factor arena",
+                             f"{arena / 1e9:.1f} GB of factors",
                        "step": "oras_factor (element matrices, A, A_s, batched LU) + oras_solve, device buffers",
                        "mesh_setup_s_untimed": t_mesh, "parallelism": f"replicas x{world}",
                        "lu_panel": panel, "lu_group": group,

@@ -66,11 +66,15 @@ enum {
 enum { ORAS_MEM_HOST = 0, ORAS_MEM_DEVICE = 1 };
 enum { ORAS_WEIGHTS_POU = 0 /* ORAS: R_s^T D_s */, ORAS_WEIGHTS_NONE = 1 /* OAS, Sec. 4 */ };
 enum { ORAS_OVERLAP_VERTEX = 0, ORAS_OVERLAP_FACE = 1 };
-enum { ORAS_LU_AUTO = 0 /* tensor cores for FP32 factors */, ORAS_LU_CUDA_CORES = 1 };
-/* Preconditioner apply with FP32 factors: AUTO streams the factor arena once per group of up to
- * 32 right-hand sides through tcgen05 tensor-core products (TF32 operands, FP32 accumulation)
- * when a call has 8 or more columns, and once per group of up to 4 on the CUDA cores (FP32)
- * otherwise; CUDA_CORES always takes the CUDA-core groups. */
+/* Local factorisations.  AUTO: sparse factors, block L D L^T of the complex symmetric A_s over a
+ * nested-dissection tree, pivots chosen inside a tree node (at most 128 unknowns, 64 in FP64).
+ * CUDA_CORES: dense LU, pivots chosen over whole columns. */
+enum { ORAS_LU_AUTO = 0, ORAS_LU_CUDA_CORES = 1 };
+/* Preconditioner apply with dense FP32 factors (ORAS_LU_CUDA_CORES): AUTO streams the factor arena
+ * once per group of up to 32 right-hand sides through tcgen05 tensor-core products (TF32 operands,
+ * FP32 accumulation) when a call has 8 or more columns, and once per group of up to 4 on the CUDA
+ * cores (FP32) otherwise; CUDA_CORES always takes the CUDA-core groups.  The sparse factors are
+ * applied in their own precision for every number of columns. */
 enum { ORAS_APPLY_AUTO = 0, ORAS_APPLY_CUDA_CORES = 1 };
 /* Transmission condition of the local problems (Sec. 4): impedance (ORAS: A_s = sum of the
  * element matrices of Omega_s^delta + i w~ S on its boundary faces) or Dirichlet (RAS:
@@ -119,13 +123,10 @@ typedef struct {
   int32_t factor_bits;        /* 32: complex FP32 local factors; 64: complex FP64 [32]  */
   int32_t weights;            /* ORAS_WEIGHTS_POU [default] or ORAS_WEIGHTS_NONE        */
   int32_t overlap_kind;       /* ORAS_OVERLAP_VERTEX [default] or ORAS_OVERLAP_FACE     */
-  int32_t lu_engine;          /* ORAS_LU_AUTO [default]: trailing updates of FP32 factors */
-                              /*   on tcgen05 tensor cores (TF32 inputs, FP32 accumulate);*/
-                              /*   ORAS_LU_CUDA_CORES: FP32 CUDA-core updates             */
-  int32_t lu_panel;           /* outer LU panel width in 64-column tiles [8]: the trailing */
+  int32_t lu_engine;          /* ORAS_LU_AUTO [default] (sparse) or ORAS_LU_CUDA_CORES (dense)   */
+  int32_t lu_panel;           /* dense LU: outer panel width in 64-column tiles [8]: the trailing */
                               /*   matrix is updated once per panel                        */
-  int32_t lu_group;           /* tensor-core update: 128-row output blocks per raster group  */
-                              /*   (operand reuse in L2) [8]                                 */
+  int32_t lu_group;           /* not used by the present factorisations (kept by oras_autotune)  */
   int32_t transmission;       /* ORAS_TRANSMISSION_IMPEDANCE [default] or _DIRICHLET (RAS) */
   int32_t graphs;             /* 1: run each Arnoldi step (apply, SpMV, orthogonalisation) as */
                               /*   a captured CUDA graph, captured on its second use and      */
@@ -190,9 +191,9 @@ int oras_create(const oras_problem* p, const oras_options* o, oras_handle** out)
 /* Numeric set-up on the GPU for one material set (Sec. 2-4): element matrices
  *   A_T = mu_r^{-1} int curl w_a . curl w_b - k0^2 eps_r int w_a . w_b      (FP64, exact)
  * plus i beta int (w_a x n).(w_b x n) on outer faces, beta from oras_problem.beta_face or else
- * k0 sqrt(Re mu_r Re eps_r) of the adjacent tetrahedron; global CSR matrix A; dense local matrices A_s with impedance
+ * k0 sqrt(Re mu_r Re eps_r) of the adjacent tetrahedron; global CSR matrix A; local matrices A_s with impedance
  * transmission i omega~ on interface faces (omega~ from the tetrahedron inside Omega_s);
- * batched LU with pivoting of every A_s in the factor precision.  eps_r, mu_r: [nt] arrays
+ * batched factorisation of every A_s in the factor precision (ORAS_LU_AUTO).  eps_r, mu_r: [nt] arrays
  * in `mem` (mu_r may be NULL -> 1).  May be called again with new materials (the mesh,
  * partition and device buffers are reused).  Errors: STATE, OUT_OF_MEMORY, CUDA,
  * SINGULAR_LOCAL, DEVICE_TIMEOUT. */
@@ -365,15 +366,16 @@ int oras_precond(oras_handle* h, const oras_complex* v, oras_complex* z, int32_t
  * synchronise the device and stall the other requests in flight.  The paper has no counterpart;
  * this is an interface convenience.  v, z: device pointers (current device = the handle's
  * device), N x k column-major, complex FP64, on the handle's stream; the call is asynchronous.
- * The local vectors live in one fixed 16 MiB device array compiled into the library (every GPU
- * that loads the library holds it until exit); sum over subdomains of the padded order times
- * the factor entry size (8 B FP32, 16 B FP64) must fit, else INVALID_ARG with the needed size.
- * The first call on a device resolves the array's device address (cudaGetSymbolAddress); make
+ * Sparse factors: the local vectors live in the handle's workspace that oras_factor allocated (calls
+ * on one handle that overlap on the GPU race on it).  Dense factors: in one fixed 16 MiB device array
+ * compiled into the library (every GPU that loads the library holds it until exit).  Either way
+ * the sum over subdomains of the padded order times the factor entry size (8 B FP32, 16 B FP64) must
+ * be at most 16 MiB, else INVALID_ARG with the needed size.  With the fixed array: the first call on a device resolves the array's device address (cudaGetSymbolAddress); make
  * that first call before any stream capture.  Every call shares the array and leaves its last
  * contents there; each call writes every entry before reading it.  Calls that overlap on the
  * GPU (other streams, other threads) race on the array.  Nothing is allocated or freed.  Cost:
  * the k columns go through the apply one after the other, so the factor arena is streamed k
- * times (oras_precond streams it once per group of up to 4 columns with FP32 factors).  The call
+ * times (oras_precond streams it once per group of columns).  The call
  * does not wait for the GPU, so a bounded device wait that gives up inside it is not reported
  * (the kernel stops the affected subdomain and returns; z is then not valid).
  * Errors: INVALID_ARG (NULL vector, k < 1 or > 64, or the scratch need above 16 MiB: checked
@@ -410,7 +412,7 @@ int oras_autotune(oras_handle* h, int32_t* panel, double* ms, int32_t nms);
 int32_t oras_lu_group(const oras_handle* h);
 
 /* Device bytes that oras_factor followed by an oras_solve of k right-hand sides allocate for
- * this handle (factor arena, inverted diagonal blocks, A, element matrices, Krylov basis of
+ * this handle (factors and their workspace, A, element matrices, Krylov basis of
  * restart+1 FP64 and restart FP32/FP64 vectors per right-hand side, staging), including the
  * allocator's rounding.  Host-only: valid right after oras_create.  No counterpart in the
  * paper (admission control of the serving runtime).  Errors: INVALID_ARG. */
@@ -503,11 +505,12 @@ void oras_server_destroy(oras_server* srv);
 /* Device time accumulated by kernel class since the last oras_reset_timings, measured with
  * CUDA event pairs on the handle's stream while timing is on: t[2c] = milliseconds and
  * t[2c+1] = kernel launches of class c, for c = 0 element and face matrices, 1 global CSR
- * values, 2 local matrices (incl. arena clear), 3 LU tournament pivoting, 4 LU row
- * interchanges and the final transposition of the U tiles, 5 LU triangular tile solves, 6 LU
- * trailing updates, 7 preconditioner apply, 8 SpMV of FP32-valued vectors (Arnoldi with FP32
+ * values, 2 local matrices (incl. the clear), 3 pivot blocks (sparse) or LU tournament pivoting
+ * (dense), 4 children's contributions added to the panels (sparse) or row interchanges and the final
+ * transposition of the U tiles (dense), 5 panels L = A21 S (sparse) or triangular tile solves
+ * (dense), 6 contribution blocks (sparse) or trailing updates (dense), 7 preconditioner apply, 8 SpMV of FP32-valued vectors (Arnoldi with FP32
  * factors), 9 orthogonalisation and Givens, 10 other, 11 SpMV of FP64 vectors (true residual;
- * Arnoldi with FP64 factors), 12 LU panel updates (the column a left-looking panel step brings
+ * Arnoldi with FP64 factors), 12 dense LU panel updates (the column a left-looking panel step brings
  * up to date and the step's pivot tile row; class 6 is then the trailing update after each
  * panel).  n: entries of t (26 covers all). */
 int oras_timings(const oras_handle* h, double* t, int32_t n);

@@ -29,6 +29,8 @@ int launch_port_dots(const oras_handle* h, int64_t nd, const int32_t* dofs, cons
 int launch_plane(const oras_handle* h, const double* dvec, const oras_complex* pvec, double k0,
                  const double* qs, const double* qw, int nq, cplx* bface, cplx* b);
 int launch_lu(oras_handle* h);
+int launch_front_rows(const oras_handle* h, double k0);
+int launch_front_factor(oras_handle* h);
 int lu_max_chunks(int64_t max_np, int factor_bits);
 int launch_apply_f64out(const oras_handle* h, const cplx* v, cplx* z, int k);
 int launch_apply_f32out(const oras_handle* h, const cplx* v, void* z, int k);
@@ -154,7 +156,9 @@ static void dfree_all(Device& d) {
                   d.sub_dofs, d.sub_pou, d.member, d.cm, d.ck, d.cs, d.fl, d.tc, d.ta, d.tm, d.eps, d.mu,
                   d.elem, d.fmat, d.vals, d.vals_df, d.arena, d.perm, d.gidx, d.sub_np_off, d.lu_cand, d.lu_cnt,
                   d.lu_ipiv, d.lu_diag, d.dinv, d.sub_inv_off, d.status, d.V, d.Zf, d.Zd, d.w, d.xk, d.bk, d.tmp, d.H, d.gcs, d.gsn,
-                  d.g, d.red, d.scal, d.ybuf, d.io, d.apply_subs};
+                  d.g, d.red, d.scal, d.ybuf, d.io, d.apply_subs,
+                  d.fr_nodes, d.fr_child, d.fr_border, d.fr_map, d.fr_pos, d.fr_row_node, d.fr_row_dof, d.fr_row_pou,
+                  d.fr_assemble, d.fr_lmul, d.fr_schur, d.fr_fwd, d.fr_bwd, d.fr_work, d.fr_c};
   for (void* p : ptrs)
     if (p) cudaFreeAsync(p, d.stream);
   cudaStreamSynchronize(d.stream);  // the frees have run: the memory is back in the pool
@@ -225,15 +229,31 @@ static int upload(oras_handle* h) {
   CK(dput(d.sub_dofs, m.sub_dofs, s));
   CK(dput(d.sub_pou, m.sub_pou, s));
   CK(dput(d.member, m.member, s));
-  std::vector<int64_t> npoff(m.nsub + 1, 0);
-  for (int q = 0; q < m.nsub; ++q) npoff[q + 1] = npoff[q] + m.sub_np[q];
-  CK(dput(d.sub_np_off, npoff, s));
-  {  // the apply's work split (which subdomains take four CTAs)
-    int nsm = 0;
-    CK(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, d.device));
-    d.num_sms = nsm;
+  CK(cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, d.device));
+  if (h->fronts.use) {
+    const Fronts& f = h->fronts;
+    CK(dput(d.fr_nodes, f.nodes, s));
+    CK(dput(d.fr_child, f.child, s));
+    CK(dput(d.fr_border, f.border, s));
+    CK(dput(d.fr_map, f.map, s));
+    CK(dput(d.fr_pos, f.pos, s));
+    CK(dput(d.fr_row_node, f.row_node, s));
+    CK(dput(d.fr_row_dof, f.row_dof, s));
+    CK(dput(d.fr_row_pou, f.row_pou, s));
+    CK(dput(d.fr_assemble, f.assemble.items, s));
+    CK(dput(d.fr_lmul, f.lmul.items, s));
+    CK(dput(d.fr_schur, f.schur.items, s));
+    CK(dput(d.fr_fwd, f.fwd.items, s));
+    CK(dput(d.fr_bwd, f.bwd.items, s));
+  } else {
+    std::vector<int64_t> npoff(m.nsub + 1, 0);
+    for (int q = 0; q < m.nsub; ++q) npoff[q + 1] = npoff[q] + m.sub_np[q];
+    CK(dput(d.sub_np_off, npoff, s));
+    CK(dalloc(d.perm, npoff[m.nsub]));
+    CK(dalloc(d.gidx, npoff[m.nsub]));
+    // the apply's work split (which subdomains take four CTAs)
     std::vector<int32_t> order;
-    d.apply_n4 = plan_apply_groups(h, nsm, order);
+    d.apply_n4 = plan_apply_groups(h, d.num_sms, order);
     // the split is an optimisation: without its side stream the apply keeps two CTAs each
     if (d.apply_n4 > 0 && !make_apply_side(h)) d.apply_n4 = 0;
     if (d.apply_n4 > 0) {
@@ -255,8 +275,6 @@ static int upload(oras_handle* h) {
   CK(dalloc(d.fmat, (size_t)std::max<int64_t>(1, m.nif) * m.nfl * m.nfl));
   CK(dalloc(d.vals, m.cols.size()));
   CK(dalloc(d.vals_df, m.cols.size()));
-  CK(dalloc(d.perm, npoff[m.nsub]));
-  CK(dalloc(d.gidx, npoff[m.nsub]));
   CK(dalloc(d.status, 8));
   d.host_pinned = pinned_scratch();
   if (!d.host_pinned) { h->err = "pinned host scratch allocation failed"; return ORAS_ERR_OUT_OF_MEMORY; }
@@ -280,8 +298,9 @@ static int alloc_factor_space(oras_handle* h, int bits) {
   auto& m = h->mesh;
   auto& d = h->dev;
   size_t el = bits == 64 ? 16 : 8;
-  // the factor tiles, then LU_SCRATCH scratch tiles per subdomain (inverted diagonal blocks)
-  size_t bytes = (size_t)(m.arena_tiles + (int64_t)LU_SCRATCH * m.nsub) * TB * TB * el;
+  // sparse factors: the panels; dense: the factor tiles
+  size_t bytes = h->fronts.use ? (size_t)std::max<int64_t>(1, h->fronts.panel_elems) * el
+                               : (size_t)m.arena_tiles * TB * TB * el;
   if (d.arena && d.factor_bits == bits && d.arena_bytes == bytes) return ORAS_OK;
   dfree_s(d.arena, d.stream);
   cudaError_t e = pool_malloc(&d.arena, bytes, d.stream);
@@ -292,6 +311,15 @@ static int alloc_factor_space(oras_handle* h, int bits) {
   }
   d.arena_bytes = bytes;
   d.factor_bits = bits;
+  if (h->fronts.use) {
+    dfree_s(d.fr_work, d.stream);
+    dfree_s(d.fr_c, d.stream);
+    CK(pool_malloc(&d.fr_work, bytes, d.stream));
+    CK(pool_malloc(&d.fr_c, (size_t)std::max<int64_t>(1, h->fronts.c_elems) * el, d.stream));
+    dfree_s(d.ybuf, d.stream);
+    d.ybuf_bytes = 0;
+    return ensure_ybuf(h, 1);
+  }
   d.lu_max_chunks = lu_max_chunks(m.max_np, bits);
   int slots = 2 * d.lu_max_chunks + 16;
   CK(dalloc(d.lu_cand, (size_t)m.nsub * slots * TB));
@@ -346,20 +374,31 @@ int64_t footprint_bytes(const oras_handle* h, int k) {
   add(std::max<int64_t>(1, m.nif) * m.nfl * m.nfl * 8);            // face matrices
   add((int64_t)m.cols.size() * 16);                                 // values of A
   add((int64_t)m.cols.size() * 16);                                 // values of A as FP32 pairs
-  add(total_np * 4);                                                // perm
-  add(total_np * 4);                                                // gidx
   add(8 * 4);                                                       // status
   // factor space
-  const int slots = 2 * lu_max_chunks(m.max_np, bits) + 16;
-  add((m.arena_tiles + (int64_t)LU_SCRATCH * m.nsub) * TB * TB * (int64_t)el);
-  add((int64_t)m.nsub * slots * TB * 4);
-  add((int64_t)m.nsub * slots * 4);
-  add((int64_t)m.nsub * (2 * TB * 2 + 1) * 4);
-  add((int64_t)m.nsub * TB * TB * (int64_t)el);
-  add((int64_t)(m.nsub + 1) * 8);
-  add(blocks * 2 * TB * TB * (int64_t)el);                          // inverted diagonal blocks
+  if (h->fronts.use) {
+    const Fronts& f = h->fronts;
+    for (int64_t x : {vb(f.nodes), vb(f.child), vb(f.border), vb(f.map), vb(f.pos), vb(f.row_node), vb(f.row_dof),
+                      vb(f.row_pou), vb(f.assemble.items), vb(f.lmul.items), vb(f.schur.items), vb(f.fwd.items),
+                      vb(f.bwd.items)})
+      add(x);
+    add(f.panel_elems * (int64_t)el);                               // panels
+    add(f.panel_elems * (int64_t)el);                               // assembly workspace
+    add(f.c_elems * (int64_t)el);                                   // contribution blocks
+  } else {
+    add(total_np * 4);                                                // perm
+    add(total_np * 4);                                                // gidx
+    const int slots = 2 * lu_max_chunks(m.max_np, bits) + 16;
+    add(m.arena_tiles * TB * TB * (int64_t)el);
+    add((int64_t)m.nsub * slots * TB * 4);
+    add((int64_t)m.nsub * slots * 4);
+    add((int64_t)m.nsub * (2 * TB * 2 + 1) * 4);
+    add((int64_t)m.nsub * TB * TB * (int64_t)el);
+    add((int64_t)(m.nsub + 1) * 8);
+    add(blocks * 2 * TB * TB * (int64_t)el);                          // inverted diagonal blocks
+    add((int64_t)m.nsub * 4);                                         // apply work split
+  }
   add((int64_t)apply_yglob_bytes_for(h, std::max(k, 1)));
-  add((int64_t)m.nsub * 4);                                         // apply work split
   // Krylov workspace and I/O staging
   const int64_t nk = N * std::max(k, 1), kk = std::max(k, 1);
   add(nk * (mm + 1) * 16);                                          // V
@@ -395,11 +434,15 @@ static int factor_device(oras_handle* h) {
   }
   {
     int b = prof_begin(h);
-    CK(cudaMemsetAsync(d.arena, 0, d.arena_bytes, d.stream));
-    if (launch_local_rows(h, k0)) CK(cudaGetLastError());
+    if (h->fronts.use) {
+      if (launch_front_rows(h, k0)) CK(cudaGetLastError());
+    } else {
+      CK(cudaMemsetAsync(d.arena, 0, d.arena_bytes, d.stream));
+      if (launch_local_rows(h, k0)) CK(cudaGetLastError());
+    }
     prof_end(h, KC_LOCAL_ROWS, b, 1);
   }
-  if (launch_lu(h)) CK(cudaGetLastError());
+  if (h->fronts.use ? launch_front_factor(h) : launch_lu(h)) CK(cudaGetLastError());
   prof_resolve(h);
   return sync_status(h);
 }
@@ -469,7 +512,15 @@ int oras_create(const oras_problem* p, const oras_options* o, oras_handle** out)
   int rc;
   try {
     rc = host_setup(p, h->opt.overlap_kind, h->mesh, g_err);
-    if (rc == ORAS_OK) h->tab = make_tables(p->r);
+    if (rc == ORAS_OK) {
+      h->tab = make_tables(p->r);
+      // sparse local factors, unless the caller asks for the dense CUDA-core LU with pivoting over
+      // whole columns
+      if (h->opt.lu_engine != ORAS_LU_CUDA_CORES) {
+        build_fronts(h->mesh, h->opt.factor_bits, h->opt.transmission == ORAS_TRANSMISSION_DIRICHLET, h->fronts);
+        h->fronts.use = true;
+      }
+    }
   } catch (const std::bad_alloc&) {
     g_err = "oras_create: host allocation failed";
     rc = ORAS_ERR_OUT_OF_MEMORY;

@@ -21,6 +21,11 @@ size_t apply_tc_ybytes(const oras_handle* h, int kt);
 int apply_tc_f64out(const oras_handle* h, const cplx* v, cplx* z, int k, int r0, int nr);
 int apply_tc_f32out(const oras_handle* h, const cplx* v, void* z, int k, int r0, int nr);
 int apply_tc_passes(int nr);
+// sparse local factors (fronts_apply.cu)
+int fronts_apply_f64out(const oras_handle* h, const cplx* v, cplx* z, int k, int64_t vs, int64_t rs);
+int fronts_apply_f32out(const oras_handle* h, const cplx* v, void* z, int k);
+size_t fronts_ybytes(const oras_handle* h, int k);
+int fronts_passes(const oras_handle* h, int k);
 
 // Columns from which a call takes the tensor-core passes (FP32 factors, ORAS_APPLY_AUTO).
 constexpr int APPLY_TC_MIN_K = 8;
@@ -181,16 +186,19 @@ static int apply_t(const oras_handle* h, const cplx* v, ZT* z, int k) {
 
 // z (FP64 complex [N][k]) = M^{-1} v
 int launch_apply_f64out(const oras_handle* h, const cplx* v, cplx* z, int k) {
+  if (h->fronts.use) return fronts_apply_f64out(h, v, z, k, k, 1);
   return h->dev.factor_bits == 64 ? apply_t<double, cplx>(h, v, z, k) : apply_t<float, cplx>(h, v, z, k);
 }
 // z (FP32 complex [N][k]) = M^{-1} v, FP32 factors only
 int launch_apply_f32out(const oras_handle* h, const cplx* v, void* z, int k) {
+  if (h->fronts.use) return fronts_apply_f32out(h, v, z, k);
   return apply_t<float, CT<float>>(h, v, (CT<float>*)z, k);
 }
 
 // Number of arena passes for k right-hand sides (each pass is one launch, or two when the largest
 // subdomains take four CTAs).
 int apply_passes(const oras_handle* h, int k) {
+  if (h->fronts.use) return fronts_passes(h, k);
   if (use_tc(h, k) && apply_tc_available(h)) return apply_tc_passes(k);
   const int maxkr = h->dev.factor_bits == 64 ? APPLY_MAX_KR_F64 : APPLY_MAX_KR_F32;
   int n = 0;
@@ -223,6 +231,7 @@ size_t apply_yglob_bytes(const oras_handle* h, int kr) {
 // Largest scratch any group of a k-vector apply needs (the tensor-core passes keep their y strips
 // in global memory: at most 32 columns per pass, complex FP32).
 size_t apply_yglob_bytes_for(const oras_handle* h, int k) {
+  if (h->fronts.use) return fronts_ybytes(h, k);
   const int maxkr = h->opt.factor_bits == 64 ? APPLY_MAX_KR_F64 : APPLY_MAX_KR_F32;
   size_t b = 0;
   if (use_tc(h, k)) b = apply_tc_ybytes(h, k > 16 ? 32 : (k > 8 ? 16 : 8));

@@ -1,0 +1,64 @@
+// Sparse local factorisations (block L D L^T over a nested-dissection tree): the plan shared by
+// the host set-up (fronts_plan.cpp), the numeric kernels (fronts.cu) and the apply (fronts_apply.cu).
+#pragma once
+
+#include <cstdint>
+#include <vector>
+
+namespace oras {
+
+// One node of a subdomain's elimination tree: n1 unknowns eliminated together (its own rows) and the
+// n2 later-eliminated unknowns they couple to (its border, ascending).  The factor panel holds
+// S = A11^{-1} (n1 rows) over L = A21 S (n2 rows), row-major with ld entries a row.
+struct FrontNode {
+  int64_t panel;    // first entry of the panel in the factor arena (and in the assembly workspace)
+  int64_t cblk;     // first entry of the contribution block C = A22 - L A21^T (n2 x ldc, lower tiles)
+  int64_t bord;     // first entry in the border list, and in the apply's border vectors
+  int64_t map;      // children's maps, nch x (n1 + n2): position in the child's border or -1;
+                    //   map = -1: one child whose border is exactly this front (identity)
+  int32_t row0;     // first own row (elimination positions of all subdomains, one after the other)
+  int32_t sub;
+  int32_t n1, n2, ld, ldc;
+  int32_t child0, nch;   // children: entries [child0, child0 + nch) of the child list
+};
+
+// A block's share of a level's work: tile `t` of node `node`.
+struct FrontItem { int32_t node, t; };
+
+constexpr int FR_TILE = 64;     // tile of the panel and contribution products
+constexpr int FR_ASM_ROWS = 32; // panel rows per assembly block
+constexpr int FR_FWD_ROWS = 64; // border rows per block of the forward pass
+constexpr int FR_BWD_COLS = 32; // own columns per block of the backward pass
+
+// Largest number of unknowns eliminated together: the pivot block is inverted by one thread block
+// in registers.
+inline int front_nb(int factor_bits) { return factor_bits == 64 ? 64 : 128; }
+
+struct FrontLevels {  // per level: [ptr[l], ptr[l + 1]) of the item list
+  std::vector<FrontItem> items;
+  std::vector<int64_t> ptr;
+};
+
+struct Fronts {
+  bool use = false;
+  std::vector<FrontNode> nodes;       // by level, wide pivot blocks first within a level
+  std::vector<int32_t> level_ptr;     // [nlev + 1] first node of each level
+  std::vector<int32_t> level_wide;    // [nlev] nodes of the level with more than front_nb / 2 own rows
+  std::vector<int32_t> child;         // child lists
+  std::vector<int32_t> border;        // positions
+  std::vector<int32_t> map;
+  std::vector<int32_t> pos;           // [sum ns] position (within its subdomain) of the local unknown i
+  std::vector<int32_t> row_node;      // [sum ns] node that eliminates the unknown at a position
+  std::vector<int32_t> row_dof;       // [sum ns] global unknown at a position
+  std::vector<uint8_t> row_pou;       // [sum ns] its partition-of-unity weight
+  FrontLevels assemble, lmul, schur, fwd, bwd;
+  int64_t panel_elems = 0, c_elems = 0, border_elems = 0;
+  int nlev() const { return (int)level_wide.size(); }
+};
+
+struct HostMesh;
+// Elimination trees of every subdomain of m for factors of the given precision (dirichlet: of the
+// matrices R_s A R_s^T).
+void build_fronts(const HostMesh& m, int factor_bits, bool dirichlet, Fronts& f);
+
+}  // namespace oras

@@ -11,14 +11,12 @@
 #include <cuda_runtime.h>
 
 #include "../../include/oras.h"
+#include "fronts.h"
 
 namespace oras {
 
 constexpr int TB = 64;            // tile order of the local-factor arena (TB x TB complex)
 constexpr int LU_SUB = 8;         // sub-panel width (tile columns) of the LU's left-looking steps
-// scratch tiles per subdomain after the factor tiles: the inverted unit-lower diagonal blocks
-// L_kk^{-1} of a sub-panel's steps (slots 0 .. LU_SUB-1) and U_kk^{-1} of the current step
-constexpr int LU_SCRATCH = LU_SUB + 1;
 constexpr int MAX_NFL = 15;       // face-local DOFs r(r+2) for r <= 3
 constexpr int MAX_NL = 45;        // tet-local DOFs for r <= 3
 constexpr int MAX_RHS = 64;
@@ -174,6 +172,15 @@ struct Device {
   int apply_n4 = 0;
   int num_sms = 0;                              // SMs of the handle's device
   int64_t apply_np4 = 0, apply_np2 = 0;
+  // sparse local factors (oras_handle::fronts): the plan, the assembly workspace and the contribution
+  // blocks; the panels are the arena
+  FrontNode* fr_nodes = nullptr;
+  int32_t* fr_child = nullptr; int32_t* fr_border = nullptr; int32_t* fr_map = nullptr;
+  int32_t* fr_pos = nullptr; int32_t* fr_row_node = nullptr; int32_t* fr_row_dof = nullptr;
+  uint8_t* fr_row_pou = nullptr;
+  FrontItem* fr_assemble = nullptr; FrontItem* fr_lmul = nullptr; FrontItem* fr_schur = nullptr;
+  FrontItem* fr_fwd = nullptr; FrontItem* fr_bwd = nullptr;
+  void* fr_work = nullptr; void* fr_c = nullptr;
   cplx* io = nullptr;                           // staging for host I/O [N][k] col-major
   size_t io_elems = 0;
   double* host_pinned = nullptr;                // small pinned host scalars (per host thread)
@@ -245,6 +252,7 @@ inline void allow_max_smem(const void* fn) {
 struct oras_handle {
   oras::HostMesh mesh;
   oras::Tables tab;
+  oras::Fronts fronts;   // use: sparse local factors (every engine but ORAS_LU_CUDA_CORES)
   oras::Device dev;
   oras_options opt{};
   std::string err;
@@ -257,12 +265,6 @@ struct oras_handle {
   mutable std::vector<int> marks;                    // (class, begin event, end event, launches)*
   double cls_ms[oras::KC_COUNT] = {0};
   double cls_n[oras::KC_COUNT] = {0};
-  // tcgen05 operand tensor map over this handle's factor arena (a CUtensorMap, 128 bytes),
-  // rebuilt when the arena moves; per handle, so concurrent handles never share one
-  alignas(64) unsigned char tc_map[128] = {0};
-  const void* tc_map_base = nullptr;
-  int64_t tc_map_tiles = 0;
-  bool tc_map_ok = false;
   // captured Arnoldi steps (oras_options.graphs): one executable graph per inner index j, valid
   // for the stream, k, restart length and workspace it was captured with
   std::vector<cudaGraphExec_t> step_graph;

@@ -19,19 +19,12 @@
 //  3. the pivot tile row, right of column k, receives the updates it still lacks
 //     (C_kJ -= sum_j L_kj U_jJ over the steps listed below);
 //  4. L21 = A21 U11^{-1} below and U12 = L11^{-1} A12 along (part of) the tile row.
-// Tensor-core path (FP32 factors).  At a sub-panel's start its LU_SUB columns, for every row from
-// k1 down, receive the updates of the panel's earlier sub-panels in one contraction (the
-// sub-panel level is left-looking too); steps 3-4 cover the pivot row inside the sub-panel
-// only; after the sub-panel's last step its rows are completed right of it by a blocked
-// triangular solve with the panel's L: one product brings in the panel's earlier sub-panels,
-// then row by row the sub-panel's earlier rows and U_kJ = L_kk^{-1} C_kJ (the sub-panel's
-// L_kk^{-1} wait in scratch tiles for this).  A pivot row thus re-reads at most LU_SUB - 1
-// earlier U rows one at a time instead of up to W - 1, and the left-looking steps at most
-// LU_SUB - 1 earlier L columns.
-// CUDA-core path (FP64 factors, or the CUDA-core engine).  After a sub-panel's last step a mid
-// update brings the panel's later columns, for every row below, up to date with the sub-panel;
-// step 3 covers the pivot row inside the panel from the sub-panel's earlier steps and beyond it
-// from all the panel's earlier steps; step 4 the whole row.
+// After a sub-panel's last step a mid update brings the panel's later columns, for every row below,
+// up to date with the sub-panel; step 3 covers the pivot row inside the panel from the sub-panel's
+// earlier steps and beyond it from all the panel's earlier steps; step 4 the whole row.
+//
+// This is the LU of ORAS_LU_CUDA_CORES: it pivots over whole columns, at the cost of dense factors.  Every
+// other handle takes the sparse factors of fronts.cu.
 // After the W columns of a panel, the trailing matrix gets one update with a W-tile-deep
 // contraction, C_IJ -= sum_k L_Ik U_kJ, which reads and writes every trailing tile once per
 // panel instead of once per column.  Right of column k, every row not yet a pivot row is in
@@ -823,24 +816,16 @@ __device__ void invert_block(const CT<R>* D, const CT<R>* rd, CT<R>* X, int task
   }
 }
 
-// Stores L^{-1} with row-major planes at Li and U^{-1} at Ui, with row-major planes when
-// u_rowmajor (the preconditioner apply) or column-major planes (the B operand of the tensor-core
-// tile solves, K-major along the row index).  A null pointer skips that factor.
+// Stores L^{-1} at Li and U^{-1} at Ui, both with row-major planes.
 template <typename R>
-__device__ void store_inverses(const CT<R>* X, R* Li, R* Ui, bool u_rowmajor) {
+__device__ void store_inverses(const CT<R>* X, R* Li, R* Ui) {
   for (int e = threadIdx.x; e < TB * TB; e += blockDim.x) {
     const int hi = e / TB, lo = e % TB;
-    if (Li) {
-      const CT<R> l = X[lo * PS + hi];                // Linv(i = hi, j = lo): row-major storage
-      Li[e] = l.re;
-      Li[TILE_PLANE + e] = l.im;
-    }
-    if (Ui) {
-      const CT<R> u = u_rowmajor ? X[TB * PS + lo * PS + hi]   // Uinv(i = hi, j = lo)
-                                 : X[TB * PS + hi * PS + lo];  // Uinv(i = lo, j = hi)
-      Ui[e] = u.re;
-      Ui[TILE_PLANE + e] = u.im;
-    }
+    const CT<R> l = X[lo * PS + hi], u = X[TB * PS + lo * PS + hi];  // entry (i = hi, j = lo)
+    Li[e] = l.re;
+    Li[TILE_PLANE + e] = l.im;
+    Ui[e] = u.re;
+    Ui[TILE_PLANE + e] = u.im;
   }
 }
 
@@ -875,7 +860,7 @@ __global__ void __launch_bounds__(INV_THREADS) k_lu_diag_inv(LuArgs a, void* are
   invert_block<R>(D, rd, X, 0, 2 * TB);
   __syncthreads();
   R* Li = (R*)inv + (inv_off[s] + I) * 4 * TILE_PLANE;
-  store_inverses<R>(X, Li, Li + 2 * TILE_PLANE, true);
+  store_inverses<R>(X, Li, Li + 2 * TILE_PLANE);
 }
 
 // After the factorisation: the tiles above the block diagonal (U), stored with column-major planes
@@ -905,38 +890,6 @@ __global__ void __launch_bounds__(256) k_lu_upper_rowmajor(LuArgs a, void* arena
     const int p = e / (TB * TB), q = e % (TB * TB);   // row-major index i * TB + j
     T[e] = buf[p * TB * (TB + 1) + (q % TB) * (TB + 1) + (q / TB)];
   }
-}
-
-// The step's factored diagonal block (from the tournament root): written to tile (k, k) and
-// inverted into the subdomain's scratch tiles for the tensor-core triangular solves: L_kk^{-1}
-// into slot `slot` (kept until the sub-panel's rows are solved beyond the panel), U_kk^{-1}
-// into slot LU_SUB.  Two blocks per subdomain (blockIdx.x): 0 inverts L and writes the tile,
-// 1 inverts U.
-template <typename R>
-__global__ void __launch_bounds__(INV_THREADS) k_lu_step_inv(LuArgs a, void* arena, int64_t scratch_base, int slot) {
-  extern __shared__ unsigned char smem_raw[];
-  CT<R>* D = (CT<R>*)smem_raw;  // [TB][PS]
-  CT<R>* X = D + TB * PS;       // [2][TB][PS]
-  CT<R>* rd = X + 2 * TB * PS;  // [TB]
-  const int s = blockIdx.y, half = blockIdx.x;
-  const int64_t nts = a.np[s] / TB;
-  const int k = a.k;
-  if (k >= nts) return;
-  const CT<R>* dg = (const CT<R>*)a.diag + (int64_t)s * TB * TB;  // element (e % TB, e / TB)
-  R* dst = tile_base<R>(arena, a, s, k, k);
-  for (int e = threadIdx.x; e < TB * TB; e += blockDim.x) {
-    const CT<R> v = dg[e];
-    D[(e / TB) * PS + (e % TB)] = v;
-    if (half == 0) tstore<R>(dst, true, e % TB, e / TB, v);
-  }
-  __syncthreads();
-  if (half == 1) diag_reciprocals<R>(D, rd);
-  __syncthreads();
-  invert_block<R>(D, rd, X, half * TB, (half + 1) * TB);
-  __syncthreads();
-  R* Li = (R*)arena + (scratch_base + (int64_t)LU_SCRATCH * s + slot) * 2 * TILE_PLANE;
-  R* Ui = (R*)arena + (scratch_base + (int64_t)LU_SCRATCH * s + LU_SUB) * 2 * TILE_PLANE;
-  store_inverses<R>(X, half == 0 ? Li : nullptr, half == 1 ? Ui : nullptr, false);
 }
 
 // number of output tiles of the update regions for the largest subdomain
@@ -983,13 +936,7 @@ static int lu_run(oras_handle* h) {
   allow_max_smem((const void*)k_lu_trsm<R>);
   allow_max_smem((const void*)k_lu_update<R>);
   const size_t smem_i = ((size_t)3 * TB * PS + TB) * sizeof(CT<R>);
-  allow_max_smem((const void*)k_lu_step_inv<R>);
-  const bool tc = sizeof(R) == 4 && h->opt.lu_engine == ORAS_LU_AUTO && tc_update_available(h);
   auto update = [&](const UpdArgs& u, int cls) {
-    if (tc) {
-      launch_update_tc(h, u, max_nts, cls);
-      return;
-    }
     int64_t blocks = region_blocks(u, max_nts);
     if (blocks <= 0) return;
     int pb = prof_begin(h);
@@ -1015,11 +962,6 @@ static int lu_run(oras_handle* h) {
       int64_t nrem = max_nts - k - 1;
       const int k1 = k0 + (k - k0) / LU_SUB * LU_SUB;                    // first step of the sub-panel
       const int ks = std::min(std::min(k1 + LU_SUB, kend), max_nts);     // first step after it
-      if (tc && k == k1 && k1 > k0) {
-        // sub-panel start (tensor-core path): its columns, for every row from k1 down, receive
-        // the updates of the panel's earlier sub-panels in one contraction
-        panel_update(k0, k1, {k1, INT_MAX, k1, ks});
-      }
       if (k > k1) {
         // left-looking sub-panel step: column k, on and below the diagonal, receives the updates
         // of the sub-panel's earlier steps just before its pivot search (every row there is in
@@ -1036,14 +978,10 @@ static int lu_run(oras_handle* h) {
       k_lu_swap<R><<<dim3(max_nts + 1, m.nsub), 256, smem_s, d.stream>>>(a, d.arena);
       prof_end(h, KC_LU_SWAP, pb, 1);
       // the pivot tile row right of column k: the rows below keep updates deferred, so a pivot
-      // row swapped up from there receives them now.  Tensor-core path: inside the sub-panel from
-      // its earlier steps (the rest of the row is solved with the sub-panel's other rows after
-      // its last step).  CUDA-core path: inside the panel from the sub-panel's earlier steps
-      // (earlier sub-panels reached it through their mid updates), beyond the panel from all the
-      // panel's earlier steps.
-      if (tc) {
-        if (k > k1 && k + 1 < ks) panel_update(k1, k, {k, k + 1, k + 1, ks});
-      } else if (k > k0) {
+      // row swapped up from there receives them now: inside the panel from the sub-panel's earlier
+      // steps (earlier sub-panels reached it through their mid updates), beyond the panel from
+      // all the panel's earlier steps.
+      if (k > k0) {
         if (k1 == k0) {
           panel_update(k0, k, {k, k + 1, k + 1, INT_MAX});
         } else {
@@ -1052,34 +990,14 @@ static int lu_run(oras_handle* h) {
         }
       }
       pb = prof_begin(h);
-      if (tc) {
-        k_lu_step_inv<R><<<dim3(2, m.nsub), INV_THREADS, smem_i, d.stream>>>(a, d.arena, m.arena_tiles, k - k1);
-        launch_trsm_tc(h, k, max_nts, true, k + 1, ks, k - k1);
-        prof_end(h, KC_LU_TRSM, pb, 2);
-      } else {
-        k_lu_trsm<R><<<dim3((unsigned)(2 * nrem + 1), m.nsub), TB, smem_r, d.stream>>>(a, d.arena);
-        prof_end(h, KC_LU_TRSM, pb, 1);
-      }
+      k_lu_trsm<R><<<dim3((unsigned)(2 * nrem + 1), m.nsub), TB, smem_r, d.stream>>>(a, d.arena);
+      prof_end(h, KC_LU_TRSM, pb, 1);
       count_launches(3);
       const int kb = k + 1;
-      if (kb == ks) {  // the sub-panel's last step
-        if (tc && kb < max_nts) {
-          // the sub-panel's rows right of it (a blocked triangular solve with the panel's L):
-          // first the contributions of the panel's earlier sub-panels in one product, then row by
-          // row those of the sub-panel's earlier rows and the solve with L_rr^{-1}
-          if (k1 > k0) panel_update(k0, k1, {k1, kb, kb, INT_MAX});
-          for (int r = k1; r < kb; ++r) {
-            if (r > k1) panel_update(k1, r, {r, r + 1, kb, INT_MAX});
-            pb = prof_begin(h);
-            launch_trsm_tc(h, r, max_nts, false, kb, INT_MAX, r - k1);
-            prof_end(h, KC_LU_TRSM, pb, 1);
-          }
-        }
-        if (!tc && kb < kend && kb < max_nts) {
-          // mid update (CUDA-core path): the panel's later columns, for every row below the
-          // sub-panel, from the sub-panel's steps
-          panel_update(k1, kb, {kb, INT_MAX, kb, kend});
-        }
+      if (kb == ks && kb < kend && kb < max_nts) {
+        // the sub-panel's last step, mid update: the panel's later columns, for every row below the
+        // sub-panel, from the sub-panel's steps
+        panel_update(k1, kb, {kb, INT_MAX, kb, kend});
       }
     }
     UpdArgs u;  // outer update of the trailing matrix

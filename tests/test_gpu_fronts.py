@@ -1,0 +1,119 @@
+"""The sparse local factors (block L D L^T over an elimination tree, pivots inside a tree node) against
+the dense LU with pivoting over whole columns (lu_engine CUDA_CORES) of the same matrices, and against
+the oracle's ORAS (Sec. 4), over the forms oras_create accepts.
+
+FP32 bars: the factors round at 2^-24, amplified by the condition number of the local matrices (1e3 to
+4e3 at degrees 1 and 2 in the lossy medium, up to 3e4 at degree 3 and 7e4 without losses): 2^-24 cond,
+3e-4 at degrees 1 and 2, 5e-3 else.  FP64: 1e-9, as for every FP64 apply.
+"""
+import numpy as np
+import pytest
+
+import synth
+from oracle import dd, problem
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def O():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1605_04521_gb300 import build
+    build.build()
+    from paper_1605_04521_gb300 import oras
+    return oras
+
+
+def rel(a, b):
+    return np.linalg.norm(np.ravel(a) - np.ravel(b)) / max(np.linalg.norm(np.ravel(b)), 1e-300)
+
+
+def shuffled(xyz, tets, seed):
+    """The same mesh with its vertices renumbered, its tetrahedra reordered and their vertices permuted."""
+    rng = np.random.default_rng(seed)
+    p = rng.permutation(len(xyz))
+    t = p[tets][rng.permutation(len(tets))]
+    x = np.empty_like(xyz)
+    x[p] = xyz
+    return x, np.ascontiguousarray(rng.permuted(t, axis=1)).astype(np.int32)
+
+
+CASES = {
+    # one node a subdomain (19-dof tetrahedra groups); odd and single subdomains; chains of pivot blocks
+    "one_node": dict(n=3, r=1, nsub=54, ov=0),
+    "one_subdomain": dict(n=4, r=2, nsub=1, ov=0),
+    "odd_subdomains": dict(n=4, r=1, nsub=7, ov=2),
+    "degree3": dict(n=3, r=3, nsub=5, ov=1),
+    # unstructured numbering, a random partition (disconnected subdomains), face overlap
+    "shuffled": dict(n=4, r=2, nsub=6, ov=1, shuffle=3),
+    "random_partition": dict(n=3, r=2, nsub=6, ov=0, shuffle=4, random_part=True),
+    "face_overlap": dict(n=4, r=2, nsub=5, ov=1, opts=dict(overlap_kind=1)),
+    # R_s A R_s^T couples unknowns through tetrahedra outside the subdomain
+    "dirichlet": dict(n=4, r=2, nsub=6, ov=1, opts=dict(transmission=1)),
+    "dirichlet_random_partition": dict(n=3, r=1, nsub=5, ov=0, shuffle=5, random_part=True, opts=dict(transmission=1)),
+    "oas": dict(n=4, r=2, nsub=6, ov=1, opts=dict(weights=1)),
+    "metallic": dict(n=4, r=2, nsub=6, ov=1, metal=True),
+    "lossless": dict(n=4, r=2, nsub=4, ov=1, eps=4.0, k0=2.5),
+}
+
+
+@pytest.mark.parametrize("bits", [32, 64])
+@pytest.mark.parametrize("name", sorted(CASES))
+def test_sparse_factors_match_dense_lu_and_oracle(O, name, bits):
+    c = CASES[name]
+    xyz, tets = synth.kuhn_cube(c["n"])
+    if "shuffle" in c:
+        xyz, tets = shuffled(xyz, tets, c["shuffle"])
+    nt, r, nsub, ov = len(tets), c["r"], c["nsub"], c["ov"]
+    eps, mu = synth.head_materials(xyz, tets) if "eps" not in c else (np.full(nt, c["eps"] + 0j), np.ones(nt, complex))
+    k0, opts = c.get("k0", synth.K0), c.get("opts", {})
+    part = None
+    if c.get("random_part"):
+        part = np.random.default_rng(9).permutation(np.arange(nt) % nsub).astype(np.int32)
+    kind = None
+    if c.get("metal"):
+        faces = np.stack([xyz[np.delete(tets, q, axis=1)] for q in range(4)], axis=1)
+        kind = np.all(faces[:, :, :, 2] == 0.0, axis=2).astype(np.uint8)
+    hs = [O.oras_setup(xyz, tets, eps, mu, k0, r, nsub, ov, part=part, face_kind=kind, factor_bits=bits, lu_engine=e, **opts)
+          for e in (O.ORAS_LU_AUTO, O.ORAS_LU_CUDA_CORES)]
+    try:
+        n = O.oras_ndof(hs[0])
+        rng = np.random.default_rng(7)
+        bar = 1e-9 if bits == 64 else (5e-3 if r == 3 or name == "lossless" else 3e-4)
+        prob = problem.build(xyz, tets, eps, mu, k0, r, [], nsub=nsub, delta=ov, part=part, face_kind=kind,
+                             with_oras=not opts)
+        orac = prob.oras
+        if "overlap_kind" not in opts and opts:
+            dec = dd.decompose(prob.topo, xyz, nsub, ov, part)
+            orac = dd.ORAS(prob.topo, xyz, eps, mu, k0, dec, weights="none" if "weights" in opts else "pou",
+                           transmission="dirichlet" if "transmission" in opts else "impedance", A_global=prob.A.tocsr())
+        for k in (1, 2, 3, 5, 8, 11):  # every group size, full and partly used
+            V = rng.normal(size=(n, k)) + 1j * rng.normal(size=(n, k))
+            Z, D = (np.asarray(O.oras_precond(h, V, k=k)).reshape(n, k) for h in hs)
+            for j in range(k):
+                # many columns on the dense FP32 factors go through TF32 products: against the oracle only
+                if bits == 64 or k < 8:
+                    assert rel(Z[:, j], D[:, j]) <= bar
+                if orac is not None:
+                    assert rel(Z[:, j], orac.apply(V[:, j])) <= bar
+    finally:
+        for h in hs:
+            O.oras_destroy(h)
+
+
+@pytest.mark.parametrize("nsub", [1, 2])
+def test_half_dead_medium_stays_singular(O, nsub):
+    """eps_r = 0 and 1/mu_r = 0 in half of the tetrahedra make local matrices with exactly zero rows: refused
+    with one subdomain over both halves and with one each, as by the dense LU."""
+    xyz, tets = synth.kuhn_cube(3)
+    nt = len(tets)
+    dead = xyz[tets].mean(axis=1)[:, 0] < 0.5
+    eps = np.where(dead, 0.0, 44.0 - 20.0j)
+    mu = np.where(dead, 1e300, 1.0).astype(complex)
+    part = (dead.astype(np.int32) if nsub == 2 else np.zeros(nt, dtype=np.int32))
+    for engine in (O.ORAS_LU_AUTO, O.ORAS_LU_CUDA_CORES):
+        with pytest.raises(O.OrasError) as e:
+            O.oras_setup(xyz, tets, eps, mu, synth.K0, 2, nsub, 0, part=part, lu_engine=engine)
+        assert e.value.code == O.ORAS_ERR_SINGULAR_LOCAL
