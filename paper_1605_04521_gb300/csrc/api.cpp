@@ -41,11 +41,11 @@ void launch_spmv_f64(const oras_handle* h, const cplx* x, cplx* y, int k);
 void launch_spmv_f32(const oras_handle* h, const void* x, cplx* y, int k);
 void launch_split_vals(const oras_handle* h);
 void launch_to_internal_c64(const oras_handle* h, int k, const void* src, void* dst);
-void launch_dot(const oras_handle* h, const cplx* a, const cplx* b, cplx* partials, int k);
-void launch_mgs_step(const oras_handle* h, int k, int m, int i, int j, const cplx* Vi, const cplx* Vn, cplx* w,
-                     const cplx* pin, cplx* pout, cplx* H);
-void launch_mgs_finish(const oras_handle* h, int k, int m, int j, const cplx* w, cplx* Vn, const cplx* pin,
-                       cplx* H, double* cs, cplx* sn, cplx* g, double* res);
+void launch_mgs(const oras_handle* h, int k, int m, int j, const cplx* V, cplx* w, cplx* red, cplx* H);
+void launch_mgs_finish(const oras_handle* h, int k, int m, int j, const cplx* w, cplx* Vn, const cplx* red,
+                       cplx* H, double* cs, cplx* sn, cplx* g, double* host_res, int32_t* host_status);
+int mgs_launches(int j);
+size_t red_elems(int k);
 void launch_hsolve(const oras_handle* h, int k, int m, int kk, const cplx* H, const cplx* g, const int32_t* active,
                    cplx* y);
 void launch_xupdate_f64(const oras_handle* h, int k, int m, int kk, const cplx* Z, const cplx* y, cplx* x);
@@ -56,7 +56,6 @@ void launch_restart(const oras_handle* h, int k, int m, const cplx* rv, const do
                     cplx* V0, cplx* g);
 void launch_to_internal(const oras_handle* h, int k, const cplx* src, cplx* dst);
 void launch_to_external(const oras_handle* h, int k, const cplx* src, cplx* dst);
-int red_blocks();
 int launch_wait_selftest(const oras_handle* h);
 // shared with the block FGMRES driver (block_fgmres.cpp)
 int ensure_ws(oras_handle* h, int k, int m);
@@ -408,7 +407,7 @@ int64_t footprint_bytes(const oras_handle* h, int k) {
   add(kk * mm * 8);
   add(kk * mm * 16);
   add(kk * (mm + 1) * 16);
-  add((int64_t)2 * red_blocks() * kk * 2 * 8);
+  add((int64_t)red_elems((int)kk) * 16);
   add((kk * 8 + kk * mm * 2 + 64) * 8);
   add(nk * 16);                                                     // io
   return b + (int64_t)nalloc * (2 << 20);
@@ -814,7 +813,7 @@ int oras::ensure_ws(oras_handle* h, int k, int m) {
   CK(dalloc(d.gcs, (size_t)kk * mm));
   CK(dalloc(d.gsn, (size_t)kk * mm));
   CK(dalloc(d.g, (size_t)kk * (mm + 1)));
-  CK(dalloc(d.red, (size_t)2 * red_blocks() * kk * 2));
+  CK(dalloc(d.red, red_elems(kk) * 2));
   CK(dalloc(d.scal, (size_t)kk * 8 + (size_t)kk * mm * 2 + 64));
   d.ws_k = kk;
   d.ws_m = mm;
@@ -937,9 +936,7 @@ static int fgmres(oras_handle* h, int k, double tol, oras_info* info) {
   if (rc) return rc;
   const size_t nk = (size_t)N * k;
   cplx* pA = (cplx*)d.red;
-  cplx* pB = pA + (size_t)red_blocks() * k;
   double* beta_d = d.scal;                     // [k]
-  double* res_d = d.scal + k;                  // [k]
   int32_t* active_d = (int32_t*)(d.scal + 2 * k);
   cplx* y_d = (cplx*)(d.scal + 3 * k + 8);     // [k][m]
   double* hp = d.host_pinned;                  // [0,k): norms; [k,2k): res
@@ -964,7 +961,7 @@ static int fgmres(oras_handle* h, int k, double tol, oras_info* info) {
       // true residual r = b - A x
       int pb = prof_begin(h);
       launch_spmv_f64(h, d.xk, d.tmp, k);
-      prof_end(h, KC_SPMV64, pb, (k + 7) / 8);
+      prof_end(h, KC_SPMV64, pb, 1);
       launch_residual(h, k, d.bk, d.tmp, pA);
       launch_norms(h, k, pA, beta_d);
       CK(cudaMemcpyAsync(hp, beta_d, k * sizeof(double), cudaMemcpyDeviceToHost, d.stream));
@@ -995,26 +992,18 @@ static int fgmres(oras_handle* h, int k, double tol, oras_info* info) {
         prof_end(h, KC_APPLY, pb, apply_passes(h, k));
         pb = prof_begin(h);
         spmv_z(h, k, j, d.w);
-        prof_end(h, d.factor_bits == 64 ? KC_SPMV64 : KC_SPMV, pb, (k + 7) / 8);
+        prof_end(h, d.factor_bits == 64 ? KC_SPMV64 : KC_SPMV, pb, 1);
         pb = prof_begin(h);
-        launch_dot(h, d.V, d.w, pA, k);
-        cplx* pin = pA;
-        cplx* pout = pB;
-        for (int i = 0; i <= j; ++i) {
-          launch_mgs_step(h, k, m, i, j, d.V + nk * i, i < j ? d.V + nk * (i + 1) : nullptr, d.w, pin, pout, d.H);
-          std::swap(pin, pout);
-        }
-        launch_mgs_finish(h, k, m, j, d.w, Vn, pin, d.H, d.gcs, d.gsn, d.g, res_d);
-        prof_end(h, KC_ORTH, pb, j + 3);
+        launch_mgs(h, k, m, j, d.V, d.w, pA, d.H);
+        launch_mgs_finish(h, k, m, j, d.w, Vn, pA, d.H, d.gcs, d.gsn, d.g, hp + k, st_h);
+        prof_end(h, KC_ORTH, pb, mgs_launches(j));
         return ORAS_OK;
       };
       if ((graphs ? run_step(h, j, k, m, step) : step()) != ORAS_OK) return ORAS_ERR_CUDA;
       kk = j + 1;
       for (int r = 0; r < k; ++r)
         if (active[r]) ++iters[r];
-      CK(cudaMemcpyAsync(hp + k, res_d, k * sizeof(double), cudaMemcpyDeviceToHost, d.stream));
-      CK(cudaMemcpyAsync(st_h, d.status, 8 * sizeof(int32_t), cudaMemcpyDeviceToHost, d.stream));
-      CK(cudaStreamSynchronize(d.stream));
+      CK(cudaStreamSynchronize(d.stream));  // the step wrote its residuals and the status to hp + k and st_h
       // a bounded wait that gave up in this step's apply: the step's vectors are not valid
       if (int sc = status_code(h, st_h)) return sc;
       bool more = false;

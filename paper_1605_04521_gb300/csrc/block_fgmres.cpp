@@ -230,7 +230,7 @@ int fgmres_block(oras_handle* h, int p, double tol, oras_info* info) {
       prof_end(h, KC_APPLY, pb, 1);
       pb = prof_begin(h);
       spmv_z(h, p, j, d.w);
-      prof_end(h, d.factor_bits == 64 ? KC_SPMV64 : KC_SPMV, pb, (p + 7) / 8);
+      prof_end(h, d.factor_bits == 64 ? KC_SPMV64 : KC_SPMV, pb, 1);
       pb = prof_begin(h);
       std::vector<zc> col((size_t)p * (j + 2) * p, zc(0.0));  // [c][row], rows (j+2)p
       const int64_t cr = (int64_t)(j + 2) * p;

@@ -1,6 +1,6 @@
 // FP64 Krylov kernels of the right-preconditioned FGMRES(m) (Sec. 5): complex CSR SpMV,
-// modified Gram-Schmidt Arnoldi with fused (axpy + next dot) passes, complex Givens rotations
-// on the device, the small triangular solve and the solution update.  Multi-vectors are
+// modified Gram-Schmidt Arnoldi in blocks of basis vectors with fused (update + next dots) passes,
+// complex Givens rotations on the device, the small triangular solve and the solution update.  Multi-vectors are
 // stored [N][k] (the k right-hand sides of a pseudo-block solve adjacent in memory).
 // Every reduction is a fixed two-stage sum (block partials, then a fixed-order sum), so the
 // results do not depend on scheduling.
@@ -18,33 +18,67 @@ template <> __device__ __forceinline__ cplx ld_c<CT<float>>(const CT<float>* p, 
   return {(double)v.re, (double)v.im};
 }
 
-// y = A x  (x: [N][k] in XT, y: [N][k] FP64).  One warp per row, up to 8 RHS per pass.
-template <typename XT>
-__global__ void k_spmv(int64_t n, const int64_t* __restrict__ rowptr, const int32_t* __restrict__ cols,
-                       const cplx* __restrict__ vals, const XT* __restrict__ x, cplx* __restrict__ y,
-                       int k, int r0, int kc) {
-  int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (row >= n) return;
-  cplx acc[8];
-#pragma unroll
-  for (int q = 0; q < 8; ++q) acc[q] = {0.0, 0.0};
-  for (int64_t p = rowptr[row] + lane; p < rowptr[row + 1]; p += 32) {
-    cplx a = vals[p];
-    int64_t c = cols[p];
-#pragma unroll
-    for (int q = 0; q < 8; ++q)
-      if (q < kc) acc[q] = cadd(acc[q], cmul(a, ld_c<XT>(x, c * k + r0 + q)));
+// Both products with A give a row SPMV_LPR lanes: KL of them take one right-hand side each (x and y rows are
+// adjacent in memory over the right-hand sides, a value of A is broadcast), the EL = SPMV_LPR / KL groups
+// share the row's entries.  Each lane issues the (value, column) loads of SPMV_UNR entries at once, then their x
+// gathers, then the arithmetic.  With more than KL right-hand sides the blocks of the same rows are
+// neighbours in the grid, so the rows of A come from L2 after the first.
+constexpr int SPMV_LPR = 8;
+constexpr int SPMV_UNR = 4;
+
+template <int KL> struct SpmvLane {
+  static constexpr int EL = SPMV_LPR / KL;
+  int64_t row;
+  int r, el;
+  bool on;
+  __device__ SpmvLane(int64_t n, int k, int chunks) {
+    const int sl = threadIdx.x % SPMV_LPR;
+    row = ((int64_t)(blockIdx.x / chunks) * blockDim.x + threadIdx.x) / SPMV_LPR;
+    r = (int)(blockIdx.x % chunks) * KL + sl % KL;
+    el = sl / KL;
+    on = row < n && r < k;
   }
+};
+
+// y = A x  (x: [N][k] in XT, y: [N][k] FP64), four fused multiply-adds an entry: bound by the FP64 pipe
+// (2 lanes a clock an SM), so no lane idles for a whole row and the sums over lanes are few.  8 fields of the
+// 20^3 degree-2 problem: a warp a row, unfused, 2.99 ms.
+template <typename XT, int KL>
+__global__ void __launch_bounds__(256) k_spmv(int64_t n, const int64_t* __restrict__ rowptr,
+                                              const int32_t* __restrict__ cols, const cplx* __restrict__ vals,
+                                              const XT* __restrict__ x, cplx* __restrict__ y, int k, int chunks) {
+  const SpmvLane<KL> L(n, k, chunks);
+  constexpr int EL = SpmvLane<KL>::EL;
+  cplx acc = {0.0, 0.0};
+  if (L.on) {
+    const int64_t p1 = rowptr[L.row + 1];
+    for (int64_t p = rowptr[L.row] + L.el; p < p1; p += EL * SPMV_UNR) {
+      cplx a[SPMV_UNR], v[SPMV_UNR];
+      int64_t c[SPMV_UNR];
 #pragma unroll
-  for (int q = 0; q < 8; ++q) {
-    if (q >= kc) break;
-    for (int o = 16; o > 0; o >>= 1) {
-      acc[q].re += __shfl_down_sync(0xffffffffu, acc[q].re, o);
-      acc[q].im += __shfl_down_sync(0xffffffffu, acc[q].im, o);
+      for (int u = 0; u < SPMV_UNR; ++u) {
+        const bool in = p + u * EL < p1;
+        a[u] = in ? vals[p + u * EL] : cplx{0.0, 0.0};
+        c[u] = in ? (int64_t)cols[p + u * EL] : -1;
+      }
+#pragma unroll
+      for (int u = 0; u < SPMV_UNR; ++u) v[u] = c[u] >= 0 ? ld_c<XT>(x, c[u] * k + L.r) : cplx{0.0, 0.0};
+#pragma unroll
+      for (int u = 0; u < SPMV_UNR; ++u)
+        if (c[u] >= 0) {
+          acc.re = fma(a[u].re, v[u].re, acc.re);
+          acc.im = fma(a[u].re, v[u].im, acc.im);
+          acc.re = fma(-a[u].im, v[u].im, acc.re);
+          acc.im = fma(a[u].im, v[u].re, acc.im);
+        }
     }
-    if (lane == 0) y[row * k + r0 + q] = acc[q];
   }
+#pragma unroll
+  for (int o = SPMV_LPR / 2; o >= KL; o >>= 1) {
+    acc.re += __shfl_down_sync(0xffffffffu, acc.re, o, SPMV_LPR);
+    acc.im += __shfl_down_sync(0xffffffffu, acc.im, o, SPMV_LPR);
+  }
+  if (L.on && L.el == 0) y[L.row * k + L.r] = acc;
 }
 
 // ------------------------------------------------------------------ FP32-pipe SpMV, FP64 accuracy
@@ -96,124 +130,110 @@ __global__ void k_split_vals(int64_t nnz, const cplx* __restrict__ vals, float4*
   out[p] = make_float4(rh, ih, (float)(v.re - (double)rh), (float)(v.im - (double)ih));
 }
 
-// y = A x with x complex FP32 ([N][k]), y FP64 ([N][k]).  SPMV_LPR lanes per row (32 / SPMV_LPR
-// rows per warp); KC right-hand sides per pass (kc <= KC of them live).  The kernel is bound by the
-// latency of its dependent loads (column index, then the gathered x), so each lane issues the
-// (value, column) loads of SPMV_UNR of its entries at once, then their x gathers, then the
-// arithmetic: SPMV_UNR entries in flight per lane.
-constexpr int SPMV_LPR = 8;
-constexpr int SPMV_UNR = 4;
-
-template <int KC>
+// y = A x with x complex FP32 ([N][k]), y FP64 ([N][k]).
+template <int KL>
 __global__ void __launch_bounds__(256) k_spmv_df(int64_t n, const int64_t* __restrict__ rowptr,
                                                  const int32_t* __restrict__ cols, const float4* __restrict__ vals,
                                                  const CT<float>* __restrict__ x, cplx* __restrict__ y, int k,
-                                                 int r0, int kc) {
-  const int64_t row = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / SPMV_LPR;
-  const int sl = threadIdx.x % SPMV_LPR;
-  const bool live = row < n;
-  float rh[KC], rl[KC], ih[KC], il[KC];
-#pragma unroll
-  for (int q = 0; q < KC; ++q) rh[q] = rl[q] = ih[q] = il[q] = 0.0f;
-  if (live) {
-    const int64_t p1 = rowptr[row + 1];
-    for (int64_t p = rowptr[row] + sl; p < p1; p += SPMV_LPR * SPMV_UNR) {
+                                                 int chunks) {
+  const SpmvLane<KL> L(n, k, chunks);
+  constexpr int EL = SpmvLane<KL>::EL;
+  float rh = 0.0f, rl = 0.0f, ih = 0.0f, il = 0.0f;
+  if (L.on) {
+    const int64_t p1 = rowptr[L.row + 1];
+    for (int64_t p = rowptr[L.row] + L.el; p < p1; p += EL * SPMV_UNR) {
       float4 a[SPMV_UNR];
       int64_t c[SPMV_UNR];
 #pragma unroll
       for (int u = 0; u < SPMV_UNR; ++u) {
-        const int64_t pu = p + (int64_t)u * SPMV_LPR;
-        const bool in = pu < p1;
-        a[u] = in ? vals[pu] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        c[u] = in ? (int64_t)cols[pu] : -1;
+        const bool in = p + u * EL < p1;
+        a[u] = in ? vals[p + u * EL] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        c[u] = in ? (int64_t)cols[p + u * EL] : -1;
       }
-      CT<float> xv[SPMV_UNR][KC];
+      CT<float> xv[SPMV_UNR];
 #pragma unroll
-      for (int u = 0; u < SPMV_UNR; ++u)
+      for (int u = 0; u < SPMV_UNR; ++u) xv[u] = c[u] >= 0 ? x[c[u] * k + L.r] : CT<float>{0.0f, 0.0f};
 #pragma unroll
-        for (int q = 0; q < KC; ++q)
-          xv[u][q] = (c[u] >= 0 && q < kc) ? x[c[u] * k + r0 + q] : CT<float>{0.0f, 0.0f};
-#pragma unroll
-      for (int u = 0; u < SPMV_UNR; ++u)
-#pragma unroll
-        for (int q = 0; q < KC; ++q)
-          if (q < kc) {
-            df_mac(rh[q], rl[q], a[u].x, a[u].z, xv[u][q].re);    // + a_re x_re
-            df_mac(rh[q], rl[q], -a[u].y, -a[u].w, xv[u][q].im);  // - a_im x_im
-            df_mac(ih[q], il[q], a[u].x, a[u].z, xv[u][q].im);    // + a_re x_im
-            df_mac(ih[q], il[q], a[u].y, a[u].w, xv[u][q].re);    // + a_im x_re
-          }
+      for (int u = 0; u < SPMV_UNR; ++u) {
+        df_mac(rh, rl, a[u].x, a[u].z, xv[u].re);    // + a_re x_re
+        df_mac(rh, rl, -a[u].y, -a[u].w, xv[u].im);  // - a_im x_im
+        df_mac(ih, il, a[u].x, a[u].z, xv[u].im);    // + a_re x_im
+        df_mac(ih, il, a[u].y, a[u].w, xv[u].re);    // + a_im x_re
+      }
     }
   }
 #pragma unroll
-  for (int q = 0; q < KC; ++q) {
-    if (q >= kc) break;
-#pragma unroll
-    for (int o = SPMV_LPR / 2; o > 0; o >>= 1) {
-      const float h2 = __shfl_down_sync(0xffffffffu, rh[q], o, SPMV_LPR), l2 = __shfl_down_sync(0xffffffffu, rl[q], o, SPMV_LPR);
-      const float h3 = __shfl_down_sync(0xffffffffu, ih[q], o, SPMV_LPR), l3 = __shfl_down_sync(0xffffffffu, il[q], o, SPMV_LPR);
-      df_add(rh[q], rl[q], h2, l2);
-      df_add(ih[q], il[q], h3, l3);
-    }
-    if (live && sl == 0) y[row * k + r0 + q] = {f2d_bits(rh[q]) + f2d_bits(rl[q]), f2d_bits(ih[q]) + f2d_bits(il[q])};
+  for (int o = SPMV_LPR / 2; o >= KL; o >>= 1) {
+    const float h2 = __shfl_down_sync(0xffffffffu, rh, o, SPMV_LPR), l2 = __shfl_down_sync(0xffffffffu, rl, o, SPMV_LPR);
+    const float h3 = __shfl_down_sync(0xffffffffu, ih, o, SPMV_LPR), l3 = __shfl_down_sync(0xffffffffu, il, o, SPMV_LPR);
+    df_add(rh, rl, h2, l2);
+    df_add(ih, il, h3, l3);
   }
+  if (L.on && L.el == 0) y[L.row * k + L.r] = {f2d_bits(rh) + f2d_bits(rl), f2d_bits(ih) + f2d_bits(il)};
 }
 
 // Reductions over [N][k] multi-vectors (element e belongs to right-hand side e % k).  The grid's
 // threads are cut to a multiple of k, teff = floor(T / k) k, and thread t < teff visits the
 // elements t, t + teff, t + 2 teff, ...: all of one right-hand side r = t % k, so each thread
-// keeps a single accumulator.  Block partial sums per right-hand side are formed in a fixed order
-// (warp shuffles over the lanes of the same r when k divides 32, else a sequential sum of the
-// block's per-thread values), then the fixed-order sum over blocks (sum_partials_warp): the results do
-// not depend on scheduling.
+// keeps one accumulator per reduced value.  Block partial sums per value and right-hand side, then a
+// sum over the blocks by one warp each (k_sum_partials), all in a fixed order that depends on the
+// sizes only: the results do not depend on scheduling.
 __device__ __forceinline__ int64_t red_teff(int k) {
   const int64_t T = (int64_t)gridDim.x * blockDim.x;
   return T / k * k;
 }
 
-// partials[blockIdx.x][r] = sum of the per-thread values v of the block's threads with RHS r
-__device__ void block_reduce_store(cplx v, int k, cplx* partials) {
-  __shared__ cplx sh[RED_THREADS];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int64_t base = (int64_t)blockIdx.x * blockDim.x;
-  if (32 % k == 0) {  // lane l holds RHS l % k (blockDim and 32 are multiples of k)
-    for (int o = 16; o >= k; o >>= 1) {
-      v.re += __shfl_xor_sync(0xffffffffu, v.re, o);
-      v.im += __shfl_xor_sync(0xffffffffu, v.im, o);
-    }
-    if (lane < k) sh[warp * k + lane] = v;
-    __syncthreads();
-    if (threadIdx.x < k) {
-      cplx t = {0.0, 0.0};
-      for (int w = 0; w < RED_THREADS / 32; ++w) t = cadd(t, sh[w * k + threadIdx.x]);
-      partials[(int64_t)blockIdx.x * k + threadIdx.x] = t;
-    }
-    return;
-  }
-  sh[threadIdx.x] = v;
-  __syncthreads();
-  for (int r = threadIdx.x; r < k; r += blockDim.x) {
-    cplx t = {0.0, 0.0};
-    for (int q = (int)(((int64_t)r - base % k + k) % k); q < RED_THREADS; q += k) t = cadd(t, sh[q]);
-    partials[(int64_t)blockIdx.x * k + r] = t;
-  }
+__device__ __forceinline__ cplx shfl_down_c(cplx v, int d) {
+  return {__shfl_down_sync(0xffffffffu, v.re, d), __shfl_down_sync(0xffffffffu, v.im, d)};
 }
 
-// Fixed-order sum of the block partials of the previous pass, by one warp: lane l loads the
-// partials of blocks l, l + 32, ... at once (their loads overlap instead of each waiting for the
-// previous add), adds them in that order, and a fixed xor-shuffle tree combines the lanes.  Every
-// lane returns the total.
-__device__ __forceinline__ cplx sum_partials_warp(const cplx* partials, int k, int r, int lane) {
+// partials[(q k + r) gridDim.x + blockIdx.x] = sum of v[q] over the block's threads of right-hand side r,
+// q < nv.  Through shared memory, one warp a value: lane r + k p adds the threads of r numbered p, p + P, ...
+// (P = 32 / k lanes a right-hand side), then a tree over p.  FP64 adds cost 64 cycles a warp on a
+// quarter of an SM, so every sum is formed once (a butterfly of all values over all lanes took 5x as many).
+template <int NV>
+__device__ void block_reduce_store(const cplx (&v)[NV], int nv, int k, cplx* __restrict__ partials) {
+  __shared__ cplx sh[NV][RED_THREADS];
+#pragma unroll
+  for (int q = 0; q < NV; ++q)
+    if (q < nv) sh[q][threadIdx.x] = v[q];
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int base = (int)((int64_t)blockIdx.x * blockDim.x % k);  // right-hand side of thread 0
+  const int P = k < 32 ? 32 / k : 1;
+  for (int q = warp; q < nv; q += RED_THREADS / 32)
+    for (int r0 = 0; r0 < k; r0 += 32) {
+      const int r = r0 + lane % (k < 32 ? k : 32), p = k < 32 ? lane / k : 0;
+      const bool on = r < k && p < P;
+      cplx t = {0.0, 0.0};
+      if (on) {
+        const int first = r >= base ? r - base : r - base + k;  // first thread of right-hand side r
+        for (int i = first + k * p; i < RED_THREADS; i += k * P) t = cadd(t, sh[q][i]);
+      }
+      for (int left = P; left > 1;) {
+        const int half = (left + 1) / 2;
+        const cplx o = shfl_down_c(t, half * k & 31);
+        if (on && p + half < left) t = cadd(t, o);
+        left = half;
+      }
+      if (on && p == 0) partials[((int64_t)q * k + r) * gridDim.x + blockIdx.x] = t;
+    }
+}
+
+// Fixed-order sum of nb block partials by one warp: lane l adds those of blocks l, l + 32, ... (their loads
+// overlap), a fixed xor-shuffle tree combines the lanes.  Every lane returns the total.
+__device__ __forceinline__ cplx sum_partials_warp(const cplx* __restrict__ partials, int nb, int lane) {
   constexpr int PER = (RED_BLOCKS + 31) / 32;
   cplx v[PER];
 #pragma unroll
   for (int q = 0; q < PER; ++q) {
     const int b = lane + 32 * q;
-    v[q] = b < RED_BLOCKS ? partials[(int64_t)b * k + r] : cplx{0.0, 0.0};
+    v[q] = b < nb ? partials[b] : cplx{0.0, 0.0};
   }
   cplx t = v[0];
 #pragma unroll
-  for (int q = 1; q < PER; ++q) t = cadd(t, v[q]);
+  for (int q = 1; q < PER; ++q)
+    if (32 * q < nb) t = cadd(t, v[q]);
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     t.re += __shfl_xor_sync(0xffffffffu, t.re, o);
@@ -222,91 +242,111 @@ __device__ __forceinline__ cplx sum_partials_warp(const cplx* partials, int k, i
   return t;
 }
 
-// first dot of step j: partial <V_0, w>
-__global__ void __launch_bounds__(RED_THREADS) k_dot(int64_t nk, int k, const cplx* __restrict__ a,
-                                                     const cplx* __restrict__ b, cplx* __restrict__ partials) {
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, teff = red_teff(k);
-  cplx acc = {0.0, 0.0};
-  if (t < teff)
-    for (int64_t e = t; e < nk; e += teff) {
-      const cplx x = a[e], y = b[e];
-      acc.re += x.re * y.re + x.im * y.im;
-      acc.im += x.re * y.im - x.im * y.re;
-    }
-  block_reduce_store(acc, k, partials);
+// hs[q k + r] = sum of the block partials; with H, also stored as H[r][i0 + q][j].  One warp a sum.
+__global__ void __launch_bounds__(256) k_sum_partials(int n, int k, int nb, const cplx* __restrict__ partials,
+                                                      cplx* __restrict__ hs, int m, int i0, int j,
+                                                      cplx* __restrict__ H) {
+  const int w = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (w >= n * k) return;
+  const cplx t = sum_partials_warp(partials + (int64_t)w * nb, nb, lane);
+  if (lane != 0) return;
+  hs[w] = t;
+  if (H) H[((int64_t)(w % k) * (m + 1) + i0 + w / k) * m + j] = t;
 }
 
-// h = sum(partials_in) (H[r][i][j] stored by block 0); w -= h V_i; then partial <V_next, w> or |w|^2.
-__global__ void __launch_bounds__(RED_THREADS) k_mgs_step(int64_t nk, int k, int m, int i, int j,
-                                                          const cplx* __restrict__ Vi, const cplx* __restrict__ Vn,
-                                                          cplx* __restrict__ w, const cplx* __restrict__ pin,
-                                                          cplx* __restrict__ pout, cplx* __restrict__ H) {
-  __shared__ cplx hs[MAX_RHS];
-  for (int r = threadIdx.x >> 5; r < k; r += blockDim.x >> 5) {  // one warp per right-hand side
-    const cplx t = sum_partials_warp(pin, k, r, threadIdx.x & 31);
-    if ((threadIdx.x & 31) == 0) {
-      hs[r] = t;
-      if (blockIdx.x == 0) H[((int64_t)r * (m + 1) + i) * m + j] = t;
-    }
-  }
-  __syncthreads();
+// One pass of the blocked modified Gram-Schmidt: w -= sum_q h_q V_q over the nv basis vectors from V (h
+// from hs), then the block partials of <Vn_q, w> over the nn vectors from Vn (nn = 0: of |w|^2 instead).
+// Vectors are nk apart.  A block's coefficients are taken together (its vectors are orthonormal to the
+// basis's own accuracy), blocks one after the other.  Bound: the FP64 pipe, 8 fused multiply-adds an entry
+// and basis vector; one vector a pass (a launch, a reduction and w through memory each) ran at a third of
+// that: 21 us a vector of 542,736 entries, now 7.6.
+constexpr int MGS_BLOCK = 8;
+__global__ void __launch_bounds__(RED_THREADS) k_mgs_block(int64_t nk, int k, int nv, const cplx* __restrict__ V,
+                                                           int nn, const cplx* __restrict__ Vn,
+                                                           cplx* __restrict__ w, const cplx* __restrict__ hs,
+                                                           cplx* __restrict__ partials) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, teff = red_teff(k);
-  cplx acc = {0.0, 0.0};
+  cplx acc[MGS_BLOCK];
+#pragma unroll
+  for (int q = 0; q < MGS_BLOCK; ++q) acc[q] = {0.0, 0.0};
   if (t < teff) {
-    const cplx h = hs[t % k];
+    cplx h[MGS_BLOCK];
+#pragma unroll
+    for (int q = 0; q < MGS_BLOCK; ++q) h[q] = q < nv ? hs[q * k + t % k] : cplx{0.0, 0.0};
     for (int64_t e = t; e < nk; e += teff) {
-      const cplx v = Vi[e];
       cplx x = w[e];
-      x.re -= h.re * v.re - h.im * v.im;
-      x.im -= h.re * v.im + h.im * v.re;
-      w[e] = x;
-      if (Vn) {
-        const cplx u = Vn[e];
-        acc.re += u.re * x.re + u.im * x.im;
-        acc.im += u.re * x.im - u.im * x.re;
+      cplx u[MGS_BLOCK];
+      if (nv > 0) {
+#pragma unroll
+        for (int q = 0; q < MGS_BLOCK; ++q)
+          if (q < nv) u[q] = V[q * nk + e];
+#pragma unroll
+        for (int q = 0; q < MGS_BLOCK; ++q)
+          if (q < nv) {
+            x.re = fma(-h[q].re, u[q].re, x.re);
+            x.im = fma(-h[q].re, u[q].im, x.im);
+            x.re = fma(h[q].im, u[q].im, x.re);
+            x.im = fma(-h[q].im, u[q].re, x.im);
+          }
+        w[e] = x;
+      }
+      if (nn > 0) {
+#pragma unroll
+        for (int q = 0; q < MGS_BLOCK; ++q)
+          if (q < nn) u[q] = Vn[q * nk + e];
+#pragma unroll
+        for (int q = 0; q < MGS_BLOCK; ++q)
+          if (q < nn) {
+            acc[q].re = fma(u[q].re, x.re, acc[q].re);
+            acc[q].im = fma(u[q].re, x.im, acc[q].im);
+            acc[q].re = fma(u[q].im, x.im, acc[q].re);
+            acc[q].im = fma(-u[q].im, x.re, acc[q].im);
+          }
       } else {
-        acc.re += x.re * x.re + x.im * x.im;
+        acc[0].re = fma(x.re, x.re, acc[0].re);
+        acc[0].re = fma(x.im, x.im, acc[0].re);
       }
     }
   }
-  block_reduce_store(acc, k, pout);
+  block_reduce_store<MGS_BLOCK>(acc, nn > 0 ? nn : 1, k, partials);
 }
 
-// h_{j+1,j} = ||w||; V_{j+1} = w / h (0 if h == 0); block 0 then runs the Givens update of
-// every RHS: apply rotations 0..j-1 to column j of H, build rotation j, update g, res = |g_{j+1}|.
+// h_{j+1,j} = ||w|| (hs[r] = |w|^2); V_{j+1} = w / h (0 if h == 0).  The last block instead runs the
+// Givens update of every RHS beside them: apply rotations 0..j-1 to column j of H, build rotation j, update
+// g, res = |g_{j+1}|; res and the device status go straight to the host's pinned words.
 __global__ void __launch_bounds__(RED_THREADS) k_mgs_finish(int64_t nk, int k, int m, int j,
                                                             const cplx* __restrict__ w, cplx* __restrict__ Vn,
-                                                            const cplx* __restrict__ pin, cplx* __restrict__ H,
+                                                            const cplx* __restrict__ hs, cplx* __restrict__ H,
                                                             double* __restrict__ cs, cplx* __restrict__ sn,
-                                                            cplx* __restrict__ g, double* __restrict__ res) {
-  __shared__ double hn[MAX_RHS];
-  for (int r = threadIdx.x >> 5; r < k; r += blockDim.x >> 5) {  // one warp per right-hand side
-    const cplx t = sum_partials_warp(pin, k, r, threadIdx.x & 31);
-    if ((threadIdx.x & 31) == 0) hn[r] = sqrt(t.re);
+                                                            cplx* __restrict__ g, double* __restrict__ host_res,
+                                                            const int32_t* __restrict__ status,
+                                                            int32_t* __restrict__ host_status) {
+  if (blockIdx.x + 1 < gridDim.x) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t T = (int64_t)(gridDim.x - 1) * blockDim.x, teff = T / k * k;
+    if (t >= teff) return;
+    const double h = sqrt(hs[t % k].re), inv = h > 0.0 ? 1.0 / h : 0.0;
+    for (int64_t e = t; e < nk; e += teff) {
+      const cplx x = w[e];
+      Vn[e] = h > 0.0 ? cplx{x.re * inv, x.im * inv} : cplx{0.0, 0.0};
+    }
+    return;
   }
-  __syncthreads();
-  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nk; e += (int64_t)gridDim.x * blockDim.x) {
-    int r = (int)(e % k);
-    double h = hn[r];
-    cplx x = w[e];
-    Vn[e] = h > 0.0 ? cplx{x.re / h, x.im / h} : cplx{0.0, 0.0};
-  }
-  if (blockIdx.x != 0) return;
+  if (threadIdx.x < 8) host_status[threadIdx.x] = status[threadIdx.x];
   for (int r = threadIdx.x; r < k; r += blockDim.x) {
     cplx* Hr = H + (int64_t)r * (m + 1) * m;
     double* c = cs + (int64_t)r * m;
     cplx* s = sn + (int64_t)r * m;
     cplx* gr = g + (int64_t)r * (m + 1);
-    Hr[(int64_t)(j + 1) * m + j] = {hn[r], 0.0};
+    const double bb = sqrt(hs[r].re);
+    cplx a = Hr[j];                       // the running entry of column j
     for (int q = 0; q < j; ++q) {
-      cplx a = Hr[(int64_t)q * m + j], b = Hr[(int64_t)(q + 1) * m + j];
-      cplx t = cadd(cscale(a, c[q]), cmul(s[q], b));
-      cplx u = csub(cscale(b, c[q]), cmul(cconj(s[q]), a));
-      Hr[(int64_t)q * m + j] = t;
-      Hr[(int64_t)(q + 1) * m + j] = u;
+      const cplx b = Hr[(int64_t)(q + 1) * m + j];
+      const double cq = c[q];
+      const cplx sq = s[q];
+      Hr[(int64_t)q * m + j] = cadd(cscale(a, cq), cmul(sq, b));
+      a = csub(cscale(b, cq), cmul(cconj(sq), a));
     }
-    cplx a = Hr[(int64_t)j * m + j];
-    double bb = hn[r];
     double aa = hypot(a.re, a.im);
     double cj;
     cplx sj;
@@ -324,7 +364,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_mgs_finish(int64_t nk, int k, i
     cplx gj = gr[j];
     gr[j + 1] = cscale(cmul(cconj(sj), gj), -1.0);
     gr[j] = cscale(gj, cj);
-    res[r] = hypot(gr[j + 1].re, gr[j + 1].im);
+    host_res[r] = hypot(gr[j + 1].re, gr[j + 1].im);
   }
 }
 
@@ -356,7 +396,13 @@ __global__ void k_xupdate(int64_t nk, int k, int m, int kk, const ZT* __restrict
   if (e >= nk) return;
   int r = (int)(e % k);
   cplx acc = x[e];
-  for (int q = 0; q < kk; ++q) acc = cadd(acc, cmul(y[(int64_t)r * m + q], ld_c<ZT>(Z, (int64_t)q * nk + e)));
+  for (int q = 0; q < kk; ++q) {
+    const cplx c = y[(int64_t)r * m + q], v = ld_c<ZT>(Z, (int64_t)q * nk + e);
+    acc.re = fma(c.re, v.re, acc.re);
+    acc.im = fma(c.re, v.im, acc.im);
+    acc.re = fma(-c.im, v.im, acc.re);
+    acc.im = fma(c.im, v.re, acc.im);
+  }
   x[e] = acc;
 }
 
@@ -364,20 +410,21 @@ __global__ void k_xupdate(int64_t nk, int k, int m, int kk, const ZT* __restrict
 __global__ void __launch_bounds__(RED_THREADS) k_residual(int64_t nk, int k, const cplx* __restrict__ b,
                                                           cplx* __restrict__ r, cplx* __restrict__ partials) {
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, teff = red_teff(k);
-  cplx acc = {0.0, 0.0};
+  cplx acc[1] = {{0.0, 0.0}};
   if (t < teff)
     for (int64_t e = t; e < nk; e += teff) {
       const cplx v = csub(b[e], r[e]);
       r[e] = v;
-      acc.re += v.re * v.re + v.im * v.im;
+      acc[0].re = fma(v.re, v.re, acc[0].re);
+      acc[0].re = fma(v.im, v.im, acc[0].re);
     }
-  block_reduce_store(acc, k, partials);
+  block_reduce_store<1>(acc, 1, k, partials);
 }
 
-// norms[r] = sqrt(sum partials) (single block)
-__global__ void k_norms(int k, const cplx* __restrict__ partials, double* __restrict__ out) {
+// norms[r] = sqrt(sum of the nb block partials) (single block)
+__global__ void k_norms(int k, int nb, const cplx* __restrict__ partials, double* __restrict__ out) {
   for (int r = threadIdx.x >> 5; r < k; r += blockDim.x >> 5) {  // one warp per right-hand side
-    const cplx t = sum_partials_warp(partials, k, r, threadIdx.x & 31);
+    const cplx t = sum_partials_warp(partials + (int64_t)r * nb, nb, threadIdx.x & 31);
     if ((threadIdx.x & 31) == 0) out[r] = sqrt(t.re);
   }
 }
@@ -389,7 +436,8 @@ __global__ void k_restart(int64_t nk, int k, int m, const cplx* __restrict__ rv,
   if (e < nk) {
     int q = (int)(e % k);
     double b = beta[q];
-    V0[e] = (active[q] && b > 0.0) ? cplx{rv[e].re / b, rv[e].im / b} : cplx{0.0, 0.0};
+    const double inv = 1.0 / b;
+    V0[e] = (active[q] && b > 0.0) ? cplx{rv[e].re * inv, rv[e].im * inv} : cplx{0.0, 0.0};
   }
   if (e < k) {
     for (int l = 0; l <= m; ++l) g[(int64_t)e * (m + 1) + l] = {0.0, 0.0};
@@ -419,32 +467,28 @@ __global__ void k_to_external(int64_t n, int k, const cplx* __restrict__ src, cp
 }
 
 // ------------------------------------------------------------------ launchers
-template <typename XT>
-static void spmv_t(const oras_handle* h, const XT* x, cplx* y, int k) {
-  const auto& m = h->mesh;
-  const auto& d = h->dev;
-  int64_t blocks = (m.ndof * 32 + 255) / 256;
-  for (int r0 = 0; r0 < k; r0 += 8) {
-    int kc = k - r0 < 8 ? k - r0 : 8;
-    k_spmv<XT><<<(unsigned)blocks, 256, 0, d.stream>>>(m.ndof, d.rowptr, d.cols, d.vals, x, y, k, r0, kc);
-    count_launches(1);
-  }
+// Lanes on right-hand sides for k columns, and the launch of f(KL, blocks, chunks).
+template <typename F>
+static void spmv_launch(const oras_handle* h, int k, F&& f) {
+  const int kl = k >= 5 ? 8 : (k >= 3 ? 4 : k), chunks = (k + kl - 1) / kl;
+  const int64_t blocks = (h->mesh.ndof * SPMV_LPR + 255) / 256 * chunks;
+  f(kl, (unsigned)blocks, chunks);
+  count_launches(1);
 }
-void launch_spmv_f64(const oras_handle* h, const cplx* x, cplx* y, int k) { spmv_t<cplx>(h, x, y, k); }
+void launch_spmv_f64(const oras_handle* h, const cplx* x, cplx* y, int k) {
+  const auto& d = h->dev;
+  spmv_launch(h, k, [&](int kl, unsigned blocks, int chunks) {
+    auto* fn = kl == 8 ? k_spmv<cplx, 8> : kl == 4 ? k_spmv<cplx, 4> : kl == 2 ? k_spmv<cplx, 2> : k_spmv<cplx, 1>;
+    fn<<<blocks, 256, 0, d.stream>>>(h->mesh.ndof, d.rowptr, d.cols, d.vals, x, y, k, chunks);
+  });
+}
 // complex FP32 x: FP32-pipe kernel with FP64-class accuracy (k_spmv_df)
 void launch_spmv_f32(const oras_handle* h, const void* x, cplx* y, int k) {
-  const auto& m = h->mesh;
   const auto& d = h->dev;
-  const int64_t blocks = (m.ndof * SPMV_LPR + 255) / 256;
-  for (int r0 = 0; r0 < k; r0 += 8) {
-    const int kc = k - r0 < 8 ? k - r0 : 8;
-    const CT<float>* xx = (const CT<float>*)x;
-    if (kc == 1) k_spmv_df<1><<<(unsigned)blocks, 256, 0, d.stream>>>(m.ndof, d.rowptr, d.cols, d.vals_df, xx, y, k, r0, kc);
-    else if (kc == 2) k_spmv_df<2><<<(unsigned)blocks, 256, 0, d.stream>>>(m.ndof, d.rowptr, d.cols, d.vals_df, xx, y, k, r0, kc);
-    else if (kc <= 4) k_spmv_df<4><<<(unsigned)blocks, 256, 0, d.stream>>>(m.ndof, d.rowptr, d.cols, d.vals_df, xx, y, k, r0, kc);
-    else k_spmv_df<8><<<(unsigned)blocks, 256, 0, d.stream>>>(m.ndof, d.rowptr, d.cols, d.vals_df, xx, y, k, r0, kc);
-    count_launches(1);
-  }
+  spmv_launch(h, k, [&](int kl, unsigned blocks, int chunks) {
+    auto* fn = kl == 8 ? k_spmv_df<8> : kl == 4 ? k_spmv_df<4> : kl == 2 ? k_spmv_df<2> : k_spmv_df<1>;
+    fn<<<blocks, 256, 0, d.stream>>>(h->mesh.ndof, d.rowptr, d.cols, d.vals_df, (const CT<float>*)x, y, k, chunks);
+  });
 }
 void launch_split_vals(const oras_handle* h) {
   const int64_t nnz = (int64_t)h->mesh.cols.size();
@@ -452,18 +496,39 @@ void launch_split_vals(const oras_handle* h) {
   count_launches(1);
 }
 
-void launch_dot(const oras_handle* h, const cplx* a, const cplx* b, cplx* partials, int k) {
-  k_dot<<<RED_BLOCKS, RED_THREADS, 0, h->dev.stream>>>(h->mesh.ndof * k, k, a, b, partials);
-  count_launches(1);
+// Blocks of the reductions over nk entries: two per SM, fewer for short vectors (at least 512 entries each).
+static int red_grid(int64_t nk) {
+  const int64_t b = (nk + 2 * RED_THREADS - 1) / (2 * RED_THREADS);
+  return (int)(b < 1 ? 1 : (b < RED_BLOCKS ? b : RED_BLOCKS));
 }
-void launch_mgs_step(const oras_handle* h, int k, int m, int i, int j, const cplx* Vi, const cplx* Vn, cplx* w,
-                     const cplx* pin, cplx* pout, cplx* H) {
-  k_mgs_step<<<RED_BLOCKS, RED_THREADS, 0, h->dev.stream>>>(h->mesh.ndof * k, k, m, i, j, Vi, Vn, w, pin, pout, H);
-  count_launches(1);
+// Orthogonalisation of w against V_0..V_j ([j + 1][N][k]): column j of H, |w|^2 in hs; partials and hs:
+// red_elems(k) entries from `red`.
+void launch_mgs(const oras_handle* h, int k, int m, int j, const cplx* V, cplx* w, cplx* red, cplx* H) {
+  const int64_t nk = h->mesh.ndof * k;
+  const int grid = red_grid(nk);
+  cplx* hs = red;
+  cplx* partials = red + (int64_t)MGS_BLOCK * k;
+  cudaStream_t st = h->dev.stream;
+  for (int i0 = -MGS_BLOCK; i0 <= j; i0 += MGS_BLOCK) {  // the first pass has nothing to subtract
+    const int i1 = i0 + MGS_BLOCK;
+    const int nv = i0 < 0 ? 0 : (j + 1 - i0 < MGS_BLOCK ? j + 1 - i0 : MGS_BLOCK);
+    const int nn = i1 > j ? 0 : (j + 1 - i1 < MGS_BLOCK ? j + 1 - i1 : MGS_BLOCK);
+    k_mgs_block<<<grid, RED_THREADS, 0, st>>>(nk, k, nv, V + (i0 < 0 ? 0 : i0) * nk, nn, V + i1 * nk, w, hs, partials);
+    const int sums = (nn > 0 ? nn : 1) * k;
+    k_sum_partials<<<(sums + 7) / 8, 256, 0, st>>>(nn > 0 ? nn : 1, k, grid, partials, hs, m, i1, j,
+                                                   nn > 0 ? H : nullptr);
+    count_launches(2);
+  }
 }
-void launch_mgs_finish(const oras_handle* h, int k, int m, int j, const cplx* w, cplx* Vn, const cplx* pin,
-                       cplx* H, double* cs, cplx* sn, cplx* g, double* res) {
-  k_mgs_finish<<<RED_BLOCKS, RED_THREADS, 0, h->dev.stream>>>(h->mesh.ndof * k, k, m, j, w, Vn, pin, H, cs, sn, g, res);
+int mgs_launches(int j) { return 2 * (j / MGS_BLOCK + 2) + 1; }
+size_t red_elems(int k) { return (size_t)(RED_BLOCKS + 1) * MGS_BLOCK * k; }
+void launch_mgs_finish(const oras_handle* h, int k, int m, int j, const cplx* w, cplx* Vn, const cplx* red,
+                       cplx* H, double* cs, cplx* sn, cplx* g, double* host_res, int32_t* host_status) {
+  const int64_t nk = h->mesh.ndof * k;
+  int64_t blocks = (nk + RED_THREADS - 1) / RED_THREADS;
+  if (blocks > 4 * RED_BLOCKS) blocks = 4 * RED_BLOCKS;
+  k_mgs_finish<<<(unsigned)blocks + 1, RED_THREADS, 0, h->dev.stream>>>(nk, k, m, j, w, Vn, red, H, cs, sn, g, host_res,
+                                                                       h->dev.status, host_status);
   count_launches(1);
 }
 void launch_hsolve(const oras_handle* h, int k, int m, int kk, const cplx* H, const cplx* g, const int32_t* active,
@@ -482,11 +547,11 @@ void launch_xupdate_f32(const oras_handle* h, int k, int m, int kk, const void* 
   count_launches(1);
 }
 void launch_residual(const oras_handle* h, int k, const cplx* b, cplx* r, cplx* partials) {
-  k_residual<<<RED_BLOCKS, RED_THREADS, 0, h->dev.stream>>>(h->mesh.ndof * k, k, b, r, partials);
+  k_residual<<<red_grid(h->mesh.ndof * k), RED_THREADS, 0, h->dev.stream>>>(h->mesh.ndof * k, k, b, r, partials);
   count_launches(1);
 }
 void launch_norms(const oras_handle* h, int k, const cplx* partials, double* out) {
-  k_norms<<<1, 256, 0, h->dev.stream>>>(k, partials, out);
+  k_norms<<<1, 256, 0, h->dev.stream>>>(k, red_grid(h->mesh.ndof * k), partials, out);
   count_launches(1);
 }
 void launch_restart(const oras_handle* h, int k, int m, const cplx* rv, const double* beta, const int32_t* active,
@@ -511,6 +576,5 @@ void launch_to_external(const oras_handle* h, int k, const cplx* src, cplx* dst)
   k_to_external<<<(unsigned)((nk + 255) / 256), 256, 0, h->dev.stream>>>(h->mesh.ndof, k, src, dst);
   count_launches(1);
 }
-int red_blocks() { return RED_BLOCKS; }
 
 }  // namespace oras

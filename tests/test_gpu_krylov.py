@@ -1,0 +1,70 @@
+"""Krylov kernels over the column counts where their lane and block layouts change: 1, 2, 3-4 and 5-8 right-hand
+sides a group, several groups, counts that do not divide a warp, more than 32.
+
+Bars: products with A 1e-13 relative per column, as in test_gpu_parity.py; solves 1e-8 in the true residual
+against the oracle's A.
+"""
+import numpy as np
+import pytest
+
+import synth
+from oracle import problem
+
+pytestmark = pytest.mark.gpu
+
+COLUMNS = [1, 2, 3, 4, 5, 7, 8, 9, 12, 17, 31, 32, 33, 64]
+
+
+@pytest.fixture(scope="module")
+def setup():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1605_04521_gb300 import build
+    build.build()
+    from paper_1605_04521_gb300 import oras as O
+    w = synth.small(n=5, r=2, nsub=8, overlap=0, restart=30)
+    p = problem.from_workload(w, with_oras=False)
+    xyz, tets = w.mesh()
+    eps, mu = w.materials(xyz, tets)
+    h = O.oras_setup(xyz, tets, eps, mu, w.k0, w.r, w.nsub, w.overlap, restart=w.restart)
+    yield O, h, p
+    O.oras_destroy(h)
+
+
+def rel(a, b):
+    return np.linalg.norm(np.ravel(a) - np.ravel(b)) / max(np.linalg.norm(np.ravel(b)), 1e-300)
+
+
+@pytest.mark.parametrize("k", COLUMNS)
+def test_products_with_a(setup, k):
+    O, h, p = setup
+    rng = np.random.default_rng(k)
+    X = rng.normal(size=(p.A.shape[0], k)) + 1j * rng.normal(size=(p.A.shape[0], k))
+    Y = np.asarray(O.oras_matvec(h, X, k=k)).reshape(-1, k)
+    Z = X.astype(np.complex64)
+    Y32 = np.asarray(O.oras_matvec_c64(h, Z, k=k)).reshape(-1, k)
+    R, R32 = p.A @ X, p.A @ Z.astype(np.complex128)
+    for j in range(k):
+        assert rel(Y[:, j], R[:, j]) <= 1e-13
+        assert rel(Y32[:, j], R32[:, j]) <= 1e-13
+
+
+@pytest.mark.parametrize("k", COLUMNS)
+def test_blocked_orthogonalisation_in_the_solve(setup, k):
+    """Random right-hand sides, one of them zero; without overlap the solve takes several blocks of 8 basis
+    vectors and restarts."""
+    O, h, p = setup
+    rng = np.random.default_rng(100 + k)
+    B = rng.normal(size=(p.A.shape[0], k)) + 1j * rng.normal(size=(p.A.shape[0], k))
+    if k > 2:
+        B[:, k // 2] = 0.0
+    X, info, rc = O.oras_solve(h, B, 1e-8, k=k)
+    X = np.asarray(X).reshape(-1, k)
+    assert rc == O.ORAS_OK
+    for j in range(k):
+        if not B[:, j].any():
+            assert not X[:, j].any()
+            continue
+        assert np.linalg.norm(B[:, j] - p.A @ X[:, j]) <= 1e-8 * np.linalg.norm(B[:, j])
+    assert max(i["iterations"] for i in info) > 16
