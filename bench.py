@@ -263,13 +263,11 @@ def apply_group_sizes(k, factor_bits, tensor_cores=False):
 
 
 def front_group_sizes(k, factor_bits):
-    """Live right-hand sides of each pass of the apply with sparse factors: groups of up to 8 (FP32) or
-    2 (FP64)."""
+    """Live right-hand sides of each pass of the apply with sparse factors: up to 32 (FP32) or 2 (FP64)."""
     out, r0 = [], 0
     while r0 < k:
         rem = k - r0
-        kr = min(rem, 2) if factor_bits == 64 else (8 if rem >= 5 else (4 if rem >= 3 else rem))
-        out.append(min(kr, rem))
+        out.append(min(rem, 2 if factor_bits == 64 else 32))
         r0 += out[-1]
     return out
 

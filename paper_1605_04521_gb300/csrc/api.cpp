@@ -156,8 +156,8 @@ static void dfree_all(Device& d) {
                   d.elem, d.fmat, d.vals, d.vals_df, d.arena, d.perm, d.gidx, d.sub_np_off, d.lu_cand, d.lu_cnt,
                   d.lu_ipiv, d.lu_diag, d.dinv, d.sub_inv_off, d.status, d.V, d.Zf, d.Zd, d.w, d.xk, d.bk, d.tmp, d.H, d.gcs, d.gsn,
                   d.g, d.red, d.scal, d.ybuf, d.io, d.apply_subs,
-                  d.fr_nodes, d.fr_child, d.fr_border, d.fr_map, d.fr_pos, d.fr_row_node, d.fr_row_dof, d.fr_row_pou,
-                  d.fr_assemble, d.fr_lmul, d.fr_schur, d.fr_fwd, d.fr_bwd, d.fr_work, d.fr_c};
+                  d.fr_nodes, d.fr_border, d.fr_own_src, d.fr_border_src, d.fr_pos, d.fr_row_node, d.fr_row_dof, d.fr_row_pou,
+                  d.fr_assemble, d.fr_lmul, d.fr_schur, d.fr_fwd, d.fr_bwd, d.fr_bwd_multi, d.fr_work, d.fr_c};
   for (void* p : ptrs)
     if (p) cudaFreeAsync(p, d.stream);
   cudaStreamSynchronize(d.stream);  // the frees have run: the memory is back in the pool
@@ -232,9 +232,9 @@ static int upload(oras_handle* h) {
   if (h->fronts.use) {
     const Fronts& f = h->fronts;
     CK(dput(d.fr_nodes, f.nodes, s));
-    CK(dput(d.fr_child, f.child, s));
     CK(dput(d.fr_border, f.border, s));
-    CK(dput(d.fr_map, f.map, s));
+    CK(dput(d.fr_own_src, f.own_src, s));
+    CK(dput(d.fr_border_src, f.border_src, s));
     CK(dput(d.fr_pos, f.pos, s));
     CK(dput(d.fr_row_node, f.row_node, s));
     CK(dput(d.fr_row_dof, f.row_dof, s));
@@ -244,6 +244,7 @@ static int upload(oras_handle* h) {
     CK(dput(d.fr_schur, f.schur.items, s));
     CK(dput(d.fr_fwd, f.fwd.items, s));
     CK(dput(d.fr_bwd, f.bwd.items, s));
+    CK(dput(d.fr_bwd_multi, f.bwd_multi.items, s));
   } else {
     std::vector<int64_t> npoff(m.nsub + 1, 0);
     for (int q = 0; q < m.nsub; ++q) npoff[q + 1] = npoff[q] + m.sub_np[q];
@@ -377,9 +378,9 @@ int64_t footprint_bytes(const oras_handle* h, int k) {
   // factor space
   if (h->fronts.use) {
     const Fronts& f = h->fronts;
-    for (int64_t x : {vb(f.nodes), vb(f.child), vb(f.border), vb(f.map), vb(f.pos), vb(f.row_node), vb(f.row_dof),
+    for (int64_t x : {vb(f.nodes), vb(f.border), vb(f.own_src), vb(f.border_src), vb(f.pos), vb(f.row_node), vb(f.row_dof),
                       vb(f.row_pou), vb(f.assemble.items), vb(f.lmul.items), vb(f.schur.items), vb(f.fwd.items),
-                      vb(f.bwd.items)})
+                      vb(f.bwd.items), vb(f.bwd_multi.items)})
       add(x);
     add(f.panel_elems * (int64_t)el);                               // panels
     add(f.panel_elems * (int64_t)el);                               // assembly workspace

@@ -25,14 +25,14 @@ namespace oras {
 // device copies of the plan (fronts.h)
 struct FrDev {
   const FrontNode* nodes;
-  const int32_t* child;
   const int32_t* border;
-  const int32_t* map;
+  const FrontSrc* own_src;
+  const FrontSrc* border_src;
 };
 
 static FrDev fr_dev(const oras_handle* h) {
   const auto& d = h->dev;
-  return {d.fr_nodes, d.fr_child, d.fr_border, d.fr_map};
+  return {d.fr_nodes, d.fr_border, d.fr_own_src, d.fr_border_src};
 }
 
 // ------------------------------------------------------------------ original entries
@@ -86,25 +86,29 @@ __global__ void k_fr_rows(RowArgs A, FrDev f, int nsub, int64_t total_rows, cons
 }
 
 // ------------------------------------------------------------------ children's contributions
-// Entry (i, j) of the front of node n, i, j numbering its own unknowns then its border, summed over
-// the children's contribution blocks (lower entries stored).
+__device__ __forceinline__ FrontSrc front_src(const FrDev& f, const FrontNode& n, int i) {
+  return i < n.n1 ? f.own_src[n.row0 + i] : f.border_src[n.bord + i - n.n1];
+}
+
+// The children's contributions to an entry of the front of node n whose rows have the sources s and t
+// (lower entries of their blocks are stored).
 template <typename R>
-__device__ __forceinline__ CT<R> pull(const FrDev& f, const FrontNode& n, const CT<R>* __restrict__ C, int i, int j) {
-  CT<R> t = {R(0), R(0)};
-  for (int c = 0; c < n.nch; ++c) {
-    const FrontNode& ch = f.nodes[f.child[n.child0 + c]];
-    int ci = i, cj = j;
-    if (n.map >= 0) {
-      const int32_t* mp = f.map + n.map + (int64_t)c * (n.n1 + n.n2);
-      ci = mp[i];
-      cj = mp[j];
-      if (ci < 0 || cj < 0) continue;
-    }
-    const CT<R> v = C[ch.cblk + (int64_t)(ci > cj ? ci : cj) * ch.ldc + (ci > cj ? cj : ci)];
-    t.re += v.re;
-    t.im += v.im;
+__device__ __forceinline__ CT<R> pull(const FrDev& f, const FrontNode& n, const CT<R>* __restrict__ C, FrontSrc s,
+                                      FrontSrc t) {
+  CT<R> r = {R(0), R(0)};
+  if (s.a >= 0 && t.a >= 0) {
+    const FrontNode& c = f.nodes[n.child[0]];
+    const int64_t lo = min(s.a, t.a) - c.bord, hi = max(s.a, t.a) - c.bord;
+    r = C[c.cblk + hi * c.ldc + lo];
   }
-  return t;
+  if (s.b >= 0 && t.b >= 0) {
+    const FrontNode& c = f.nodes[n.child[1]];
+    const int64_t lo = min(s.b, t.b) - c.bord, hi = max(s.b, t.b) - c.bord;
+    const CT<R> v = C[c.cblk + hi * c.ldc + lo];
+    r.re += v.re;
+    r.im += v.im;
+  }
+  return r;
 }
 
 // Panel rows of the nodes with children: 32 rows a block, lanes along the own columns.
@@ -117,7 +121,7 @@ __global__ void __launch_bounds__(256) k_fr_assemble(FrDev f, const FrontItem* _
   const int rows = n.n1 + n.n2 - r0 < FR_ASM_ROWS ? n.n1 + n.n2 - r0 : FR_ASM_ROWS;
   for (int e = threadIdx.x; e < rows * n.n1; e += 256) {
     const int i = r0 + e / n.n1, j = e % n.n1;
-    const CT<R> t = pull<R>(f, n, C, i, j);
+    const CT<R> t = pull<R>(f, n, C, front_src(f, n, i), f.own_src[n.row0 + j]);
     CT<R>& w = work[n.panel + (int64_t)i * n.ld + j];
     w.re += t.re;
     w.im += t.im;
@@ -308,7 +312,7 @@ __global__ void __launch_bounds__(256) k_fr_mul(FrDev f, const FrontItem* __rest
     while (ti * (ti + 1) / 2 > it.t) --ti;
     tj = it.t - ti * (ti + 1) / 2;
   } else {
-    const int nj = (n1 + FR_TILE - 1) / FR_TILE;
+    const int nj = (n1 + FR_TILE - 1) / FR_TILE;  // > 0: nodes that eliminate nothing have no such tiles
     ti = it.t / nj;
     tj = it.t % nj;
   }
@@ -349,16 +353,23 @@ __global__ void __launch_bounds__(256) k_fr_mul(FrDev f, const FrontItem* __rest
         }
     }
   }
+  FrontSrc sj[4];
+  if (SCHUR) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) sj[q] = j0 + tx + 16 * q < n2 ? f.border_src[n.bord + j0 + tx + 16 * q] : FrontSrc{-1, -1};
+  }
 #pragma unroll
   for (int p = 0; p < 4; ++p) {
     const int i = i0 + ty * 4 + p;
     if (i >= n2) continue;
+    FrontSrc si = {-1, -1};
+    if (SCHUR) si = f.border_src[n.bord + i];
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int j = j0 + tx + 16 * q;
       if (SCHUR) {
         if (j >= n2) continue;
-        const CT<R> v = pull<R>(f, n, C, n1 + i, n1 + j);
+        const CT<R> v = pull<R>(f, n, C, si, sj[q]);
         C[n.cblk + (int64_t)i * n.ldc + j] = {v.re - acc[p][q].re, v.im - acc[p][q].im};
       } else if (j < ld) {  // columns n1 .. ld-1 are written as zeros
         fac[n.panel + (int64_t)(n1 + i) * ld + j] = acc[p][q];
@@ -415,9 +426,9 @@ static int factor_t(oras_handle* h) {
     }
     count_launches((wide ? 1 : 0) + (all > wide ? 1 : 0));
     prof_end(h, KC_LU_TOURNAMENT, pb, 1);
-    if (!count(f.lmul)) continue;
+    if (!count(f.schur)) continue;
     pb = prof_begin(h);
-    k_fr_mul<R, false><<<count(f.lmul), 256, 0, st>>>(fd, d.fr_lmul + f.lmul.ptr[l], work, fac, C);
+    if (count(f.lmul)) k_fr_mul<R, false><<<count(f.lmul), 256, 0, st>>>(fd, d.fr_lmul + f.lmul.ptr[l], work, fac, C);
     prof_end(h, KC_LU_TRSM, pb, 1);
     pb = prof_begin(h);
     k_fr_mul<R, true><<<count(f.schur), 256, 0, st>>>(fd, d.fr_schur + f.schur.ptr[l], work, fac, C);

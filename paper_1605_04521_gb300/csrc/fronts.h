@@ -14,13 +14,14 @@ struct FrontNode {
   int64_t panel;    // first entry of the panel in the factor arena (and in the assembly workspace)
   int64_t cblk;     // first entry of the contribution block C = A22 - L A21^T (n2 x ldc, lower tiles)
   int64_t bord;     // first entry in the border list, and in the apply's border vectors
-  int64_t map;      // children's maps, nch x (n1 + n2): position in the child's border or -1;
-                    //   map = -1: one child whose border is exactly this front (identity)
   int32_t row0;     // first own row (elimination positions of all subdomains, one after the other)
   int32_t sub;
   int32_t n1, n2, ld, ldc;
-  int32_t child0, nch;   // children: entries [child0, child0 + nch) of the child list
+  int32_t child[2]; // nodes, -1: none
 };
+// Where a row of a front is in the borders of its node's two children: entries of the border list, -1: not
+// there.  Own rows: own_src[row0 + i]; border rows: border_src[bord + i].
+struct alignas(8) FrontSrc { int32_t a, b; };
 
 // A block's share of a level's work: tile `t` of node `node`.
 struct FrontItem { int32_t node, t; };
@@ -28,7 +29,8 @@ struct FrontItem { int32_t node, t; };
 constexpr int FR_TILE = 64;     // tile of the panel and contribution products
 constexpr int FR_ASM_ROWS = 32; // panel rows per assembly block
 constexpr int FR_FWD_ROWS = 64; // border rows per block of the forward pass
-constexpr int FR_BWD_COLS = 32; // own columns per block of the backward pass
+constexpr int FR_BWD_COLS = 32; // own columns per block of the backward pass at the widest
+constexpr int FR_BWD_BLOCKS = 1216;  // levels with fewer blocks than this (8 an SM) take narrower ones
 
 // Largest number of unknowns eliminated together: the pivot block is inverted by one thread block
 // in registers.
@@ -44,14 +46,15 @@ struct Fronts {
   std::vector<FrontNode> nodes;       // by level, wide pivot blocks first within a level
   std::vector<int32_t> level_ptr;     // [nlev + 1] first node of each level
   std::vector<int32_t> level_wide;    // [nlev] nodes of the level with more than front_nb / 2 own rows
-  std::vector<int32_t> child;         // child lists
   std::vector<int32_t> border;        // positions
-  std::vector<int32_t> map;
+  std::vector<FrontSrc> own_src, border_src;
   std::vector<int32_t> pos;           // [sum ns] position (within its subdomain) of the local unknown i
   std::vector<int32_t> row_node;      // [sum ns] node that eliminates the unknown at a position
   std::vector<int32_t> row_dof;       // [sum ns] global unknown at a position
   std::vector<uint8_t> row_pou;       // [sum ns] its partition-of-unity weight
-  FrontLevels assemble, lmul, schur, fwd, bwd;
+  FrontLevels assemble, lmul, schur, fwd, bwd, bwd_multi;
+  std::vector<int32_t> bwd_cols;      // [nlev] own columns per block of bwd: 8, 16 or 32
+  std::vector<int32_t> multi_cols;    // [nlev] and of bwd_multi: 16 or 64
   int64_t panel_elems = 0, c_elems = 0, border_elems = 0;
   int nlev() const { return (int)level_wide.size(); }
 };

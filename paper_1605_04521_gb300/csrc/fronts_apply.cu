@@ -4,13 +4,19 @@
 // hand up, y = b + sum of theirs; it hands up u = (the children's on its border) - L y.  Backward, from
 // the roots: x = S y - L^T x(border), the panel [S; L] times [y; -x(border)] column by column (S is
 // symmetric).  Every panel is read once a direction.  All nodes of a tree level run in one launch; a
-// border row is formed by one block and children are added in a fixed order, so results do not depend on
-// scheduling (OAS adds overlapping contributions into z with atomics).
+// row of a result is formed by one block and children are added in a fixed order, so results do not depend
+// on scheduling (OAS adds overlapping contributions into z with atomics).
 //
-// Bound: HBM, (S + 2 L) entries of 8 B (FP32): 3.5 GB a pass on the 16^3 degree-2 64-subdomain problem,
-// where dense factors of the same matrices were 87 GB.
-#include "fronts.h"
-
+// Up to 4 right-hand sides a pass (k_fr_fwd, k_fr_bwd): bound by HBM, (S + 2 L) entries of 8 B (FP32):
+// 3.2 GB a pass on the 16^3 degree-2 64-subdomain problem.  What costs beside it is the latency of a level
+// (index, gather, panel, reduction, 30-odd levels a pass), so a block issues its panel loads and indices,
+// which do not depend on the level before, first and only then waits for that level (programmatic dependent
+// launch: the next level's blocks load while the last ones of this level finish), panels are read past L2
+// (they are used once a direction, the vectors and indices stay), and the backward blocks get narrower
+// where a level has few nodes.  ms an apply, before -> with these: 16^3 1.29 -> 0.81 (3.2 GB: 58% of the copy
+// rate), 24^3 with 512 subdomains 0.54 -> 0.38, 8^3 0.24 -> 0.086.
+// 5 and more right-hand sides (k_fr_fwd_multi, k_fr_bwd_multi): up to 32 a pass as small matrix products, bound
+// by the FP32 pipes: 32 columns of the 16^3 128-subdomain problem 5.2 -> 2.2 ms (four passes of 8 before).
 #include <algorithm>
 
 #include "apply.cuh"
@@ -19,9 +25,9 @@ namespace oras {
 
 struct FrApply {
   const FrontNode* nodes;
-  const int32_t* child;
   const int32_t* border;
-  const int32_t* map;
+  const FrontSrc* own_src;
+  const FrontSrc* border_src;
   const int32_t* row_dof;
   const uint8_t* row_pou;
   int weights;
@@ -32,69 +38,116 @@ struct FrApply {
 constexpr int FR_THREADS = 256;
 constexpr int FR_MAX_NB = 128;
 
-// Handed up by the children at front index i (own unknowns, then border).
+// Programmatic dependent launch: lets the next kernel of the stream start its independent loads / waits until
+// the kernels before this one have finished and their results are visible.
+// The vectors that a kernel reads after the wait are plain pointers: through a restrict-qualified pointer to
+// const the compiler may load them before it.
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Two adjacent complex entries, read once: past L1, first out of L2.
+__device__ __forceinline__ void ld_stream(const CT<float>* p, CT<float>& a, CT<float>& b) {
+  const float4 t = __ldcs(reinterpret_cast<const float4*>(p));
+  a = {t.x, t.y}; b = {t.z, t.w};
+}
+__device__ __forceinline__ void ld_stream(const CT<double>* p, CT<double>& a, CT<double>& b) {
+  const double2 t0 = __ldcs(reinterpret_cast<const double2*>(p)), t1 = __ldcs(reinterpret_cast<const double2*>(p) + 1);
+  a = {t0.x, t0.y}; b = {t1.x, t1.y};
+}
+
+template <typename R> __device__ __forceinline__ void cfma(CT<R>& t, CT<R> m, CT<R> y) {
+  t.re = fma(m.re, y.re, t.re); t.re = fma(-m.im, y.im, t.re);
+  t.im = fma(m.re, y.im, t.im); t.im = fma(m.im, y.re, t.im);
+}
+
+// Handed up by the children for a front row with sources s.
 template <typename R, int KR>
-__device__ __forceinline__ CT<R> pull_vec(const FrApply& a, const FrontNode& n, const CT<R>* __restrict__ u, int i,
-                                          int r) {
+__device__ __forceinline__ CT<R> pull_vec(const CT<R>* u, FrontSrc s, int r) {
   CT<R> t = {R(0), R(0)};
-  for (int c = 0; c < n.nch; ++c) {
-    const FrontNode& ch = a.nodes[a.child[n.child0 + c]];
-    const int ci = n.map >= 0 ? a.map[n.map + (int64_t)c * (n.n1 + n.n2) + i] : i;
-    if (ci < 0) continue;
-    const CT<R> v = u[(ch.bord + ci) * KR + r];
+  if (s.a >= 0) t = u[(int64_t)s.a * KR + r];
+  if (s.b >= 0) {
+    const CT<R> v = u[(int64_t)s.b * KR + r];
     t.re += v.re;
     t.im += v.im;
   }
   return t;
 }
 
-// One block: 64 border rows of a node, 8 lanes a row.
+// One block: 64 border rows of a node, 8 lanes a row, 32 rows at a time.
 template <typename R, int KR>
 __global__ void __launch_bounds__(FR_THREADS) k_fr_fwd(FrApply a, const FrontItem* __restrict__ items,
-                                                       const CT<R>* __restrict__ fac, const cplx* __restrict__ v,
-                                                       CT<R>* __restrict__ y, CT<R>* __restrict__ u) {
-  __shared__ __align__(16) CT<R> own[KR][FR_MAX_NB];
+                                                       const CT<R>* __restrict__ fac, const cplx* v,
+                                                       CT<R>* y, CT<R>* u) {
+  constexpr int NB = sizeof(R) == 4 ? FR_MAX_NB : FR_MAX_NB / 2, NQ = NB / 16;
+  constexpr int ROUND = FR_THREADS / 8;
+  __shared__ __align__(16) CT<R> own[KR][NB];
+  pdl_release();
   const FrontItem it = items[blockIdx.x];
   const FrontNode n = a.nodes[it.node];
-  const int n1 = n.n1, ld = n.ld;
-  for (int e = threadIdx.x; e < ld * KR; e += FR_THREADS) {
-    const int c = e / KR, r = e % KR;
+  const int n1 = n.n1, ld = n.ld, sub = threadIdx.x & 7;
+  const CT<R>* rows = fac + n.panel + (int64_t)n1 * ld;
+  CT<R> m0[NQ], m1[NQ];
+  auto load = [&](int i) {  // the lane's entries of border row i
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      const int c = 2 * sub + 16 * q;
+      if (i < n.n2 && c < ld) ld_stream(rows + (int64_t)i * ld + c, m0[q], m1[q]);
+    }
+  };
+  int i = it.t * FR_FWD_ROWS + (threadIdx.x >> 3);
+  load(i);
+  FrontSrc src = {-1, -1};
+  if (i < n.n2) src = a.border_src[n.bord + i];
+  // own unknown of this thread in the gather (one right-hand side after the other)
+  const int c0 = threadIdx.x / KR, r0 = threadIdx.x % KR;
+  FrontSrc osrc = {-1, -1};
+  int32_t dof = 0;
+  if (c0 < n1) {
+    osrc = a.own_src[n.row0 + c0];
+    dof = a.row_dof[n.row0 + c0];
+  }
+  pdl_wait();
+  for (int c = c0; c < ld; c += FR_THREADS / KR) {
     CT<R> t = {R(0), R(0)};
     if (c < n1) {
-      if (r < a.nr) {
-        const cplx b = v[(int64_t)a.row_dof[n.row0 + c] * a.vs + a.off + r];
+      if (c != c0) {
+        osrc = a.own_src[n.row0 + c];
+        dof = a.row_dof[n.row0 + c];
+      }
+      if (r0 < a.nr) {
+        const cplx b = v[(int64_t)dof * a.vs + a.off + r0];
         t = {R(b.re), R(b.im)};
       }
-      const CT<R> up = pull_vec<R, KR>(a, n, u, c, r);
+      const CT<R> up = pull_vec<R, KR>(u, osrc, r0);
       t.re += up.re;
       t.im += up.im;
-      if (it.t == 0) y[(int64_t)(n.row0 + c) * KR + r] = t;
+      if (it.t == 0) y[(int64_t)(n.row0 + c) * KR + r0] = t;
     }
-    own[r][c] = t;
+    own[r0][c] = t;
   }
   __syncthreads();
-  const int sub = threadIdx.x & 7;
 #pragma unroll
-  for (int rr = 0; rr < FR_FWD_ROWS; rr += FR_THREADS / 8) {
-    const int i = it.t * FR_FWD_ROWS + rr + (threadIdx.x >> 3);
+  for (int h = 0; h < FR_FWD_ROWS / ROUND; ++h) {
+    if (h > 0) {
+      i += ROUND;
+      load(i);
+      if (i < n.n2) src = a.border_src[n.bord + i];
+    }
     CT<R> acc[KR];
 #pragma unroll
     for (int r = 0; r < KR; ++r) acc[r] = {R(0), R(0)};
     if (i < n.n2) {
-      const CT<R>* row = fac + n.panel + (int64_t)(n1 + i) * ld;
-#pragma unroll 4
-      for (int c = 2 * sub; c < ld; c += 16) {
-        CT<R> m0, m1;
-        ld_cpair(row + c, m0, m1);
 #pragma unroll
-        for (int r = 0; r < KR; ++r) {
-          CT<R> y0, y1;
-          ld_cpair(&own[r][c], y0, y1);
-          CT<R>& t = acc[r];
-          t.re = fma(m0.re, y0.re, t.re); t.re = fma(-m0.im, y0.im, t.re);
-          t.re = fma(m1.re, y1.re, t.re); t.re = fma(-m1.im, y1.im, t.re);
-          t.im = fma(m0.re, y0.im, t.im); t.im = fma(m0.im, y0.re, t.im);
-          t.im = fma(m1.re, y1.im, t.im); t.im = fma(m1.im, y1.re, t.im);
+      for (int q = 0; q < NQ; ++q) {
+        const int c = 2 * sub + 16 * q;
+        if (c < ld) {
+#pragma unroll
+          for (int r = 0; r < KR; ++r) {
+            CT<R> y0, y1;
+            ld_cpair(&own[r][c], y0, y1);
+            cfma(acc[r], m0[q], y0);
+            cfma(acc[r], m1[q], y1);
+          }
         }
       }
     }
@@ -106,61 +159,103 @@ __global__ void __launch_bounds__(FR_THREADS) k_fr_fwd(FrApply a, const FrontIte
         acc[r].im += __shfl_xor_sync(0xffffffffu, acc[r].im, o);
       }
       if (i < n.n2 && sub == r) {  // KR <= 8 lanes: one right-hand side each
-        const CT<R> up = pull_vec<R, KR>(a, n, u, n1 + i, r);
+        const CT<R> up = pull_vec<R, KR>(u, src, r);
         u[(n.bord + i) * KR + r] = {up.re - acc[r].re, up.im - acc[r].im};
       }
     }
   }
 }
 
-// One block: 32 own unknowns of a node, lane = unknown, the warps share the panel's rows.
-template <typename R, typename ZT, int KR>
+// One block: CW own unknowns of a node, a lane two of them; the CW / 2-lane groups share the panel's rows.
+template <typename R, typename ZT, int KR, int CW>
 __global__ void __launch_bounds__(FR_THREADS) k_fr_bwd(FrApply a, const FrontItem* __restrict__ items,
-                                                       const CT<R>* __restrict__ fac, const CT<R>* __restrict__ y,
-                                                       CT<R>* __restrict__ x, ZT* __restrict__ z) {
-  constexpr int ROWS = 256, NW = FR_THREADS / 32;
+                                                       const CT<R>* __restrict__ fac, const CT<R>* y,
+                                                       CT<R>* x, ZT* z) {
+  constexpr int LW = CW / 2, NG = FR_THREADS / LW;      // lanes a row, row groups
+  constexpr int NQ = sizeof(R) == 4 ? 8 : 4;            // rows a group loads at once
+  constexpr int ROWS = 512;                             // rows of [y; -x] staged at once
+  constexpr int NW = FR_THREADS / 32;
   __shared__ CT<R> w[ROWS][KR];
-  __shared__ CT<R> red[NW][32][KR];
+  __shared__ CT<R> red[NW][CW][KR];
+  pdl_release();
   const FrontItem it = items[blockIdx.x];
   const FrontNode n = a.nodes[it.node];
   const int n1 = n.n1, m = n.n1 + n.n2, ld = n.ld;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int j = it.t * FR_BWD_COLS + lane;
-  const CT<R>* panel = fac + n.panel;
-  CT<R> acc[KR];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, grp = threadIdx.x / LW;
+  const int j = it.t * CW + 2 * (threadIdx.x % LW);
+  const CT<R>* panel = fac + n.panel + j;
+  CT<R> m0[NQ], m1[NQ];
+  auto load = [&](int i0) {  // this lane's columns of rows i0 + grp + NG q
 #pragma unroll
-  for (int r = 0; r < KR; ++r) acc[r] = {R(0), R(0)};
-  for (int r0 = 0; r0 < m; r0 += ROWS) {
-    const int rows = m - r0 < ROWS ? m - r0 : ROWS;
-    __syncthreads();
-    for (int e = threadIdx.x; e < rows * KR; e += FR_THREADS) {
-      const int i = r0 + e / KR, r = e % KR;
-      if (i < n1) {
-        w[e / KR][r] = y[(int64_t)(n.row0 + i) * KR + r];
-      } else {
-        const CT<R> t = x[(int64_t)a.border[n.bord + i - n1] * KR + r];
-        w[e / KR][r] = {-t.re, -t.im};
+    for (int q = 0; q < NQ; ++q) {
+      const int i = i0 + grp + NG * q;
+      if (i < m && j < ld) ld_stream(panel + (int64_t)i * ld, m0[q], m1[q]);
+    }
+  };
+  load(0);
+  int32_t row[ROWS / FR_THREADS];  // rows of [y; x] that this thread stages first
+#pragma unroll
+  for (int q = 0; q < ROWS / FR_THREADS; ++q) {
+    const int i = threadIdx.x + FR_THREADS * q;
+    row[q] = i < n1 ? n.row0 + i : (i < m ? a.border[n.bord + i - n1] : -1);
+  }
+  CT<R> acc0[KR], acc1[KR];
+#pragma unroll
+  for (int r = 0; r < KR; ++r) acc0[r] = acc1[r] = {R(0), R(0)};
+  pdl_wait();
+  for (int s0 = 0; s0 < m; s0 += ROWS) {
+    if (s0 > 0) __syncthreads();
+#pragma unroll
+    for (int q = 0; q < ROWS / FR_THREADS; ++q) {
+      const int i = s0 + threadIdx.x + FR_THREADS * q;
+      if (s0 > 0) row[q] = i < n1 ? n.row0 + i : (i < m ? a.border[n.bord + i - n1] : -1);
+      if (row[q] >= 0) {
+#pragma unroll
+        for (int r = 0; r < KR; ++r) {
+          CT<R> t = (i < n1 ? y : x)[(int64_t)row[q] * KR + r];
+          if (i >= n1) t = {-t.re, -t.im};
+          w[i - s0][r] = t;
+        }
       }
     }
     __syncthreads();
-    if (j < ld) {
-#pragma unroll 8
-      for (int i = warp; i < rows; i += NW) {
-        const CT<R> mm = panel[(int64_t)(r0 + i) * ld + j];
+    const int end = m < s0 + ROWS ? m : s0 + ROWS;
+    for (int i0 = s0; i0 < end; i0 += NG * NQ) {
+      if (i0 > 0) load(i0);
+      if (j < ld) {
 #pragma unroll
-        for (int r = 0; r < KR; ++r) {
-          const CT<R> t = w[i][r];
-          acc[r].re = fma(mm.re, t.re, acc[r].re); acc[r].re = fma(-mm.im, t.im, acc[r].re);
-          acc[r].im = fma(mm.re, t.im, acc[r].im); acc[r].im = fma(mm.im, t.re, acc[r].im);
+        for (int q = 0; q < NQ; ++q) {
+          const int i = i0 + grp + NG * q;
+          if (i < end) {
+#pragma unroll
+            for (int r = 0; r < KR; ++r) {
+              const CT<R> t = w[i - s0][r];
+              cfma(acc0[r], m0[q], t);
+              cfma(acc1[r], m1[q], t);
+            }
+          }
         }
       }
     }
   }
+  // over the row groups of the warp, then over the warps
 #pragma unroll
-  for (int r = 0; r < KR; ++r) red[warp][lane][r] = acc[r];
+  for (int r = 0; r < KR; ++r) {
+#pragma unroll
+    for (int o = LW; o < 32; o <<= 1) {
+      acc0[r].re += __shfl_xor_sync(0xffffffffu, acc0[r].re, o);
+      acc0[r].im += __shfl_xor_sync(0xffffffffu, acc0[r].im, o);
+      acc1[r].re += __shfl_xor_sync(0xffffffffu, acc1[r].re, o);
+      acc1[r].im += __shfl_xor_sync(0xffffffffu, acc1[r].im, o);
+    }
+    if (lane < LW) {
+      red[warp][2 * lane][r] = acc0[r];
+      red[warp][2 * lane + 1][r] = acc1[r];
+    }
+  }
   __syncthreads();
-  for (int e = threadIdx.x; e < 32 * KR; e += FR_THREADS) {
-    const int l = e / KR, r = e % KR, c = it.t * FR_BWD_COLS + l;
+  for (int e = threadIdx.x; e < CW * KR; e += FR_THREADS) {
+    const int l = e / KR, r = e % KR, c = it.t * CW + l;
     if (c >= n1) continue;
     CT<R> t = red[0][l][r];
 #pragma unroll
@@ -168,23 +263,279 @@ __global__ void __launch_bounds__(FR_THREADS) k_fr_bwd(FrApply a, const FrontIte
       t.re += red[q][l][r].re;
       t.im += red[q][l][r].im;
     }
-    const int64_t row = n.row0 + c;
-    x[row * KR + r] = t;
+    const int64_t g = n.row0 + c;
+    x[g * KR + r] = t;
     if (r >= a.nr) continue;
-    ZT* dst = z + (int64_t)a.row_dof[row] * a.vs + a.off + r;
+    ZT* dst = z + (int64_t)a.row_dof[g] * a.vs + a.off + r;
     if (a.weights == ORAS_WEIGHTS_POU) {
-      if (a.row_pou[row]) z_store(dst, (double)t.re, (double)t.im);
+      if (a.row_pou[g]) z_store(dst, (double)t.re, (double)t.im);
     } else {
       z_add(dst, (double)t.re, (double)t.im);
     }
   }
 }
 
+// ------------------------------------------------------------------ many right-hand sides (FP32)
+// Products of a tile of JT rows with KR = 8, 16 or 32 right-hand sides: 4 x TC entries a thread; the threads left
+// over split the sum (SG groups, added at the end in a fixed order), so a block keeps KC = 16 SG sum indices in
+// flight a stage -- the sums run up to a thousand long on levels with few nodes, where a stage's load latency is
+// the cost and the tiles are narrower (Fronts::multi_cols: below 200 tiles of 64; 16 wide they take 28 us where 64
+// wide ones take 48, but twice as long on levels that fill the chip).
+template <int KR, int JT> struct FrTile {
+  static constexpr int TR = 4, TC = KR == 16 ? 4 : 2;         // entries a thread
+  static constexpr int CG = KR / TC, RG = JT / TR;            // column and row groups
+  static constexpr int SG = FR_THREADS / (CG * RG);           // sum groups
+  static constexpr int KC = 16 * SG;                          // sum indices a stage
+  static_assert(CG * RG * SG == FR_THREADS, "threads");
+};
+
+// acc += the products of sum group sg over one stage: As [KC][LDA], Bs [KC][KR].
+template <int KR, int JT, int LDA>
+__device__ __forceinline__ void tile_stage(CT<float> (&acc)[FrTile<KR, JT>::TR][FrTile<KR, JT>::TC], const CT<float>* As,
+                                           const CT<float>* Bs, int sg, int rg, int cg) {
+  using T = FrTile<KR, JT>;
+#pragma unroll
+  for (int k = 0; k < 16; ++k) {
+    CT<float> av[T::TR], bv[T::TC];
+    const CT<float>* pa = As + (sg * 16 + k) * LDA + rg * T::TR;
+    const CT<float>* pb = Bs + (sg * 16 + k) * KR + cg * T::TC;
+#pragma unroll
+    for (int p = 0; p < T::TR; p += 2) ld_cpair(pa + p, av[p], av[p + 1]);
+#pragma unroll
+    for (int q = 0; q < T::TC; q += 2) ld_cpair(pb + q, bv[q], bv[q + 1]);
+#pragma unroll
+    for (int p = 0; p < T::TR; ++p)
+#pragma unroll
+      for (int q = 0; q < T::TC; ++q) cfma(acc[p][q], av[p], bv[q]);
+  }
+}
+
+// Adds the sum groups' accumulators into group 0's, through shared memory (buf: (SG - 1) x JT x KR entries).
+template <int KR, int JT>
+__device__ __forceinline__ void tile_reduce(CT<float> (&acc)[FrTile<KR, JT>::TR][FrTile<KR, JT>::TC], CT<float>* buf, int sg,
+                                            int rg, int cg) {
+  using T = FrTile<KR, JT>;
+  if (T::SG == 1) return;
+  __syncthreads();
+  if (sg > 0) {
+#pragma unroll
+    for (int p = 0; p < T::TR; ++p)
+#pragma unroll
+      for (int q = 0; q < T::TC; ++q) buf[((sg - 1) * JT + rg * T::TR + p) * KR + cg * T::TC + q] = acc[p][q];
+  }
+  __syncthreads();
+  if (sg > 0) return;
+#pragma unroll
+  for (int g = 0; g < T::SG - 1; ++g)
+#pragma unroll
+    for (int p = 0; p < T::TR; ++p)
+#pragma unroll
+      for (int q = 0; q < T::TC; ++q) {
+        const CT<float> t = buf[(g * JT + rg * T::TR + p) * KR + cg * T::TC + q];
+        acc[p][q].re += t.re;
+        acc[p][q].im += t.im;
+      }
+}
+
+// u = (children's) - L y for 64 border rows.  Shared memory: a stage of L (transposed), then y.
+constexpr int FR_LDL = 64 + 2;
+template <int KR> constexpr size_t fr_fwd_smem() {
+  return sizeof(CT<float>) * ((size_t)FrTile<KR, 64>::KC * FR_LDL + (size_t)FR_MAX_NB * KR);
+}
+template <int KR>
+__global__ void __launch_bounds__(FR_THREADS) k_fr_fwd_multi(FrApply a, const FrontItem* __restrict__ items,
+                                                             const CT<float>* __restrict__ fac,
+                                                             const cplx* v, CT<float>* y,
+                                                             CT<float>* u) {
+  using T = FrTile<KR, 64>;
+  using C = CT<float>;
+  constexpr int LQ = T::KC * 64 / FR_THREADS;           // entries of a stage of L a thread loads
+  extern __shared__ __align__(16) unsigned char fr_smem[];
+  C* Ls = (C*)fr_smem;                                  // [KC][FR_LDL]
+  C* own = Ls + T::KC * FR_LDL;                         // [FR_MAX_NB][KR]
+  static_assert((T::SG - 1) * 64 * KR <= FR_MAX_NB * KR + T::KC * FR_LDL, "the reduction fits");
+  pdl_release();
+  const FrontItem it = items[blockIdx.x];
+  const FrontNode n = a.nodes[it.node];
+  const int n1 = n.n1, ld = n.ld, i0 = it.t * 64;
+  const C* rows = fac + n.panel + (int64_t)n1 * ld;
+  // this thread's part of a stage of L: row lr, columns lc + 16 q .. lc + 16 q + 3 (the transposed stores of a
+  // warp then fall on all banks)
+  const int lr = threadIdx.x >> 2, lc = (threadIdx.x & 3) * 4;
+  auto col = [&](int q) { return lc + (q & 3) + 16 * (q >> 2); };
+  const bool lrow = i0 + lr < n.n2;
+  C l[LQ];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < LQ; q += 2) {
+      l[q] = l[q + 1] = {0.0f, 0.0f};
+      if (lrow && k0 + col(q) < ld) ld_stream(rows + (int64_t)(i0 + lr) * ld + k0 + col(q), l[q], l[q + 1]);
+    }
+  };
+  load(0);
+  pdl_wait();
+  const int ldk = (ld + 15) / 16 * 16;                  // rows of y up to a whole step of 16 are read
+  for (int e = threadIdx.x; e < ldk * KR; e += FR_THREADS) {
+    const int c = e / KR, r = e % KR;
+    C t = {0.0f, 0.0f};
+    if (c < n1) {
+      const FrontSrc s = a.own_src[n.row0 + c];
+      if (r < a.nr) {
+        const cplx b = v[(int64_t)a.row_dof[n.row0 + c] * a.vs + a.off + r];
+        t = {(float)b.re, (float)b.im};
+      }
+      const C up = pull_vec<float, KR>(u, s, r);
+      t.re += up.re;
+      t.im += up.im;
+      if (it.t == 0) y[(int64_t)(n.row0 + c) * KR + r] = t;
+    }
+    own[c * KR + r] = t;
+  }
+  const int cg = threadIdx.x % T::CG, rg = threadIdx.x / T::CG % T::RG, sg = threadIdx.x / (T::CG * T::RG);
+  C acc[T::TR][T::TC];
+#pragma unroll
+  for (int p = 0; p < T::TR; ++p)
+#pragma unroll
+    for (int q = 0; q < T::TC; ++q) acc[p][q] = {0.0f, 0.0f};
+  for (int k0 = 0; k0 < ld; k0 += T::KC) {
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < LQ; ++q) Ls[col(q) * FR_LDL + lr] = l[q];
+    __syncthreads();
+    if (k0 + T::KC < ld) load(k0 + T::KC);
+    if (k0 + sg * 16 < ld) tile_stage<KR, 64, FR_LDL>(acc, Ls, own + k0 * KR, sg, rg, cg);
+  }
+  tile_reduce<KR, 64>(acc, (C*)fr_smem, sg, rg, cg);
+  if (sg > 0) return;
+#pragma unroll
+  for (int p = 0; p < T::TR; ++p) {
+    const int i = i0 + rg * T::TR + p;
+    if (i >= n.n2) continue;
+    const FrontSrc s = a.border_src[n.bord + i];
+#pragma unroll
+    for (int q = 0; q < T::TC; ++q) {
+      const int r = cg * T::TC + q;
+      const C up = pull_vec<float, KR>(u, s, r);
+      u[(n.bord + i) * KR + r] = {up.re - acc[p][q].re, up.im - acc[p][q].im};
+    }
+  }
+}
+
+// x = [S; L]^T [y; -x(border)] for JT own unknowns.  Shared memory: a stage of panel rows, a stage of [y; -x].
+template <int KR, int JT> constexpr size_t fr_bwd_smem() {
+  return sizeof(CT<float>) * (size_t)FrTile<KR, JT>::KC * (JT + KR);
+}
+template <typename ZT, int KR, int JT>
+__global__ void __launch_bounds__(FR_THREADS) k_fr_bwd_multi(FrApply a, const FrontItem* __restrict__ items,
+                                                             const CT<float>* __restrict__ fac,
+                                                             const CT<float>* y, CT<float>* x,
+                                                             ZT* z) {
+  using T = FrTile<KR, JT>;
+  using C = CT<float>;
+  constexpr int GL = JT / 4, GR = FR_THREADS / GL, GQ = T::KC / GR;  // lanes a row, rows at once, passes
+  constexpr int WE = T::KC * KR / FR_THREADS;                 // entries of [y; -x] a thread stages
+  static_assert(GQ * GR == T::KC && WE * FR_THREADS == T::KC * KR, "stage shapes");
+  static_assert((T::SG - 1) * JT * KR <= T::KC * (JT + KR), "the reduction fits");
+  extern __shared__ __align__(16) unsigned char fr_smem[];
+  C* Gs = (C*)fr_smem;                                        // [KC][JT]
+  C* ws = Gs + T::KC * JT;                                    // [KC][KR]
+  pdl_release();
+  const FrontItem it = items[blockIdx.x];
+  const FrontNode n = a.nodes[it.node];
+  const int n1 = n.n1, m = n.n1 + n.n2, ld = n.ld, j0 = it.t * JT;
+  const C* panel = fac + n.panel + j0;
+  // this thread's part of a stage: rows gr + GR q, columns gc .. gc + 3
+  const int gr = threadIdx.x / GL, gc = threadIdx.x % GL * 4;
+  C g[GQ][4], w[WE];
+  int32_t row[WE];                                            // rows of [y; x] of the next stage
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < GQ; ++q) {
+      const int i = k0 + gr + GR * q;
+#pragma unroll
+      for (int p = 0; p < 4; ++p) g[q][p] = {0.0f, 0.0f};
+      if (i < m && j0 + gc < ld) {
+        const C* p = panel + (int64_t)i * ld + gc;
+        ld_stream(p, g[q][0], g[q][1]);
+        ld_stream(p + 2, g[q][2], g[q][3]);
+      }
+    }
+  };
+  auto load_rows = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < WE; ++q) {
+      const int i = k0 + (threadIdx.x + FR_THREADS * q) / KR;
+      row[q] = i < n1 ? n.row0 + i : (i < m ? a.border[n.bord + i - n1] : -1);
+    }
+  };
+  auto load_w = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < WE; ++q) {
+      const int e = threadIdx.x + FR_THREADS * q, i = k0 + e / KR, r = e % KR;
+      w[q] = {0.0f, 0.0f};
+      if (row[q] < 0) continue;
+      w[q] = (i < n1 ? y : x)[(int64_t)row[q] * KR + r];
+      if (i >= n1) w[q] = {-w[q].re, -w[q].im};
+    }
+    load_rows(k0 + T::KC);
+  };
+  load(0);
+  load_rows(0);
+  pdl_wait();
+  load_w(0);
+  const int cg = threadIdx.x % T::CG, rg = threadIdx.x / T::CG % T::RG, sg = threadIdx.x / (T::CG * T::RG);
+  C acc[T::TR][T::TC];
+#pragma unroll
+  for (int p = 0; p < T::TR; ++p)
+#pragma unroll
+    for (int q = 0; q < T::TC; ++q) acc[p][q] = {0.0f, 0.0f};
+  for (int k0 = 0; k0 < m; k0 += T::KC) {
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < GQ; ++q) {
+      st_cpair(Gs + (gr + GR * q) * JT + gc, g[q][0], g[q][1]);
+      st_cpair(Gs + (gr + GR * q) * JT + gc + 2, g[q][2], g[q][3]);
+    }
+#pragma unroll
+    for (int q = 0; q < WE; ++q) ws[threadIdx.x + FR_THREADS * q] = w[q];
+    __syncthreads();
+    if (k0 + T::KC < m) {
+      load(k0 + T::KC);
+      load_w(k0 + T::KC);
+    }
+    if (k0 + sg * 16 < m) tile_stage<KR, JT, JT>(acc, Gs, ws, sg, rg, cg);  // rows past the panel are zeros
+  }
+  tile_reduce<KR, JT>(acc, (C*)fr_smem, sg, rg, cg);
+  if (sg > 0) return;
+#pragma unroll
+  for (int p = 0; p < T::TR; ++p) {
+    const int c = j0 + rg * T::TR + p;
+    if (c >= n1) continue;
+    const int64_t row = n.row0 + c;
+    const int64_t dof = a.row_dof[row];
+    const bool pou = a.row_pou[row] != 0;
+#pragma unroll
+    for (int q = 0; q < T::TC; ++q) {
+      const int r = cg * T::TC + q;
+      const C t = acc[p][q];
+      x[row * KR + r] = t;
+      if (r >= a.nr) continue;
+      ZT* dst = z + dof * a.vs + a.off + r;
+      if (a.weights == ORAS_WEIGHTS_POU) {
+        if (pou) z_store(dst, (double)t.re, (double)t.im);
+      } else {
+        z_add(dst, (double)t.re, (double)t.im);
+      }
+    }
+  }
+}
+
 // ------------------------------------------------------------------ host side
-// Right-hand sides of the next pass when `rem` are left.
+// Right-hand sides of the next pass when `rem` are left: the smallest pass that takes them all, up to 32
+// (FP32) or 2 (FP64).
 static int fr_kr(const oras_handle* h, int rem) {
   if (h->opt.factor_bits == 64) return rem >= 2 ? 2 : 1;
-  return rem >= 5 ? 8 : (rem >= 3 ? 4 : rem);
+  return rem > 16 ? 32 : (rem > 8 ? 16 : (rem > 4 ? 8 : (rem > 2 ? 4 : rem)));
 }
 
 size_t fronts_ybytes(const oras_handle* h, int k) {
@@ -199,12 +550,31 @@ int fronts_passes(const oras_handle* h, int k) {
   return n;
 }
 
+// A launch that may start before the kernel before it in the stream has finished (pdl_wait in the kernel).
+template <typename... P, typename... A>
+static void launch_pdl(void (*fn)(P...), int64_t blocks, size_t smem, cudaStream_t st, A... args) {
+  if (blocks <= 0) return;
+  if (smem > 48 * 1024) allow_max_smem((const void*)fn);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3(FR_THREADS);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(&cfg, fn, static_cast<P>(args)...);
+  count_launches(1);
+}
+
 template <typename R, typename ZT, int KR>
 static void fr_pass(const oras_handle* h, const cplx* v, ZT* z, int64_t vs, int64_t off, int nr) {
   const auto& d = h->dev;
   const Fronts& f = h->fronts;
   FrApply a;
-  a.nodes = d.fr_nodes; a.child = d.fr_child; a.border = d.fr_border; a.map = d.fr_map;
+  a.nodes = d.fr_nodes; a.border = d.fr_border; a.own_src = d.fr_own_src; a.border_src = d.fr_border_src;
   a.row_dof = d.fr_row_dof; a.row_pou = d.fr_row_pou;
   a.weights = h->opt.weights;
   a.vs = vs; a.off = off; a.nr = nr;
@@ -213,13 +583,27 @@ static void fr_pass(const oras_handle* h, const cplx* v, ZT* z, int64_t vs, int6
   CT<R>* x = y + rows * KR;
   CT<R>* u = x + rows * KR;
   const CT<R>* fac = (const CT<R>*)d.arena;
-  for (int l = 0; l < f.nlev(); ++l)
-    k_fr_fwd<R, KR><<<(unsigned)(f.fwd.ptr[l + 1] - f.fwd.ptr[l]), FR_THREADS, 0, d.stream>>>(
-        a, d.fr_fwd + f.fwd.ptr[l], fac, v, y, u);
-  for (int l = f.nlev() - 1; l >= 0; --l)
-    k_fr_bwd<R, ZT, KR><<<(unsigned)(f.bwd.ptr[l + 1] - f.bwd.ptr[l]), FR_THREADS, 0, d.stream>>>(
-        a, d.fr_bwd + f.bwd.ptr[l], fac, y, x, z);
-  count_launches(2 * f.nlev());
+  cudaStream_t st = d.stream;
+  for (int l = 0; l < f.nlev(); ++l) {
+    const FrontItem* items = d.fr_fwd + f.fwd.ptr[l];
+    const int64_t nb = f.fwd.ptr[l + 1] - f.fwd.ptr[l];
+    if constexpr (KR >= 8) launch_pdl(k_fr_fwd_multi<KR>, nb, fr_fwd_smem<KR>(), st, a, items, fac, v, y, u);
+    else launch_pdl(k_fr_fwd<R, KR>, nb, 0, st, a, items, fac, v, y, u);
+  }
+  for (int l = f.nlev() - 1; l >= 0; --l) {
+    if constexpr (KR >= 8) {
+      const FrontItem* items = d.fr_bwd_multi + f.bwd_multi.ptr[l];
+      const int64_t nb = f.bwd_multi.ptr[l + 1] - f.bwd_multi.ptr[l];
+      if (f.multi_cols[l] == 64) launch_pdl(k_fr_bwd_multi<ZT, KR, 64>, nb, fr_bwd_smem<KR, 64>(), st, a, items, fac, y, x, z);
+      else launch_pdl(k_fr_bwd_multi<ZT, KR, 16>, nb, fr_bwd_smem<KR, 16>(), st, a, items, fac, y, x, z);
+    } else {
+      const FrontItem* items = d.fr_bwd + f.bwd.ptr[l];
+      const int64_t nb = f.bwd.ptr[l + 1] - f.bwd.ptr[l];
+      if (f.bwd_cols[l] == 32) launch_pdl(k_fr_bwd<R, ZT, KR, 32>, nb, 0, st, a, items, fac, y, x, z);
+      else if (f.bwd_cols[l] == 16) launch_pdl(k_fr_bwd<R, ZT, KR, 16>, nb, 0, st, a, items, fac, y, x, z);
+      else launch_pdl(k_fr_bwd<R, ZT, KR, 8>, nb, 0, st, a, items, fac, y, x, z);
+    }
+  }
 }
 
 // z = M^{-1} v for k right-hand sides; right-hand side r of unknown g at g * vs + r * rs of v and z
@@ -238,7 +622,9 @@ static int fr_apply_t(const oras_handle* h, const cplx* v, ZT* z, int k, int64_t
     else if (kr == 2) fr_pass<R, ZT, 2>(h, v, z, vs, off, nr);
     else if constexpr (sizeof(R) == 4) {
       if (kr == 4) fr_pass<R, ZT, 4>(h, v, z, vs, off, nr);
-      else fr_pass<R, ZT, 8>(h, v, z, vs, off, nr);
+      else if (kr == 8) fr_pass<R, ZT, 8>(h, v, z, vs, off, nr);
+      else if (kr == 16) fr_pass<R, ZT, 16>(h, v, z, vs, off, nr);
+      else fr_pass<R, ZT, 32>(h, v, z, vs, off, nr);
     }
     r0 += nr;
   }

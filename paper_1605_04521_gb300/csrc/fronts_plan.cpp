@@ -13,6 +13,7 @@
 
 #include <cmath>
 #include <memory>
+#include <stdexcept>
 
 #include "internal.h"
 #include "par.h"
@@ -24,8 +25,8 @@ namespace {
 struct LocalNode {
   std::vector<int32_t> own;       // local unknowns (indices into N_s), ascending
   std::vector<int32_t> border;    // local unknowns, then positions
-  std::vector<int32_t> child;     // local node ids
-  std::vector<int32_t> map;       // [nch][n1 + n2], empty: identity
+  int32_t child[2] = {-1, -1};    // local node ids
+  std::vector<FrontSrc> src;      // [n1 + n2] position in the children's borders, -1
   int32_t p0 = 0, level = 0;
 };
 
@@ -111,6 +112,13 @@ struct Builder {
     number(ns);
   }
 
+  void link(LocalNode& x, const std::vector<int32_t>& children) {
+    for (size_t q = 0; q < children.size(); ++q) {
+      x.child[q] = children[q];
+      x.level = std::max(x.level, nodes[children[q]].level + 1);
+    }
+  }
+
   // Nodes for `own` entities over `border` entities: a chain of at most nb unknowns each.
   // `roots`: in, the children; out, the chain's top.
   void add(std::vector<int32_t>& own, const std::vector<int32_t>& border, std::vector<int32_t>& roots) {
@@ -120,6 +128,18 @@ struct Builder {
       for (int w = 0; w < width[e]; ++w) u.push_back(e + w);
     for (int32_t e : border)
       for (int w = 0; w < width[e]; ++w) b.push_back(e + w);
+    // at most two children a node: pairs of others are joined by nodes that eliminate nothing
+    while (roots.size() > 2) {
+      LocalNode x;
+      std::vector<int32_t> c(roots.end() - 2, roots.end());
+      roots.resize(roots.size() - 2);
+      for (int q = 0; q < 2; ++q) x.border.insert(x.border.end(), nodes[c[q]].border.begin(), nodes[c[q]].border.end());
+      std::sort(x.border.begin(), x.border.end());
+      x.border.erase(std::unique(x.border.begin(), x.border.end()), x.border.end());
+      link(x, c);
+      roots.insert(roots.begin(), (int32_t)nodes.size());
+      nodes.push_back(std::move(x));
+    }
     const int n = (int)u.size(), parts = (n + nb - 1) / nb;
     for (int p = 0; p < parts; ++p) {
       LocalNode x;
@@ -127,8 +147,7 @@ struct Builder {
       x.own.assign(u.begin() + q0, u.begin() + q1);
       x.border.assign(u.begin() + q1, u.end());
       x.border.insert(x.border.end(), b.begin(), b.end());
-      x.child = roots;
-      for (int32_t c : x.child) x.level = std::max(x.level, nodes[c].level + 1);
+      link(x, roots);
       roots.assign(1, (int32_t)nodes.size());
       nodes.push_back(std::move(x));
     }
@@ -232,7 +251,7 @@ struct Builder {
   }
 
   // Elimination positions (nodes in creation order: children first), borders as ascending positions,
-  // and the children's maps.
+  // and where each front is in the children's borders.
   std::vector<int32_t> pos;
   void number(int64_t ns) {
     pos.assign(ns, -1);
@@ -248,20 +267,13 @@ struct Builder {
     for (auto& x : nodes) {
       const int n1 = (int)x.own.size(), n2 = (int)x.border.size();
       auto front = [&](int i) { return i < n1 ? x.p0 + i : x.border[i - n1]; };
-      if (x.child.size() == 1) {  // a chain link: the child's border is this front
-        const auto& cb = nodes[x.child[0]].border;
-        bool same = (int)cb.size() == n1 + n2;
-        for (int i = 0; i < n1 + n2 && same; ++i) same = cb[i] == front(i);
-        if (same) continue;
-      }
-      x.map.resize(x.child.size() * (size_t)(n1 + n2));
-      for (size_t c = 0; c < x.child.size(); ++c) {
+      x.src.assign(n1 + n2, {-1, -1});
+      for (int c = 0; c < 2; ++c) {
+        if (x.child[c] < 0) continue;
         const auto& cb = nodes[x.child[c]].border;
         size_t k = 0;
-        for (int i = 0; i < n1 + n2; ++i) {
-          const bool in = k < cb.size() && cb[k] == front(i);
-          x.map[c * (size_t)(n1 + n2) + i] = in ? (int32_t)k++ : -1;
-        }
+        for (int i = 0; i < n1 + n2 && k < cb.size(); ++i)
+          if (cb[k] == front(i)) (c == 0 ? x.src[i].a : x.src[i].b) = (int32_t)k++;
       }
     }
   }
@@ -316,7 +328,7 @@ void build_fronts(const HostMesh& m, int factor_bits, bool dirichlet, Fronts& f)
   f.row_node.resize(rows);
   f.row_dof.resize(rows);
   f.row_pou.resize(rows);
-  int64_t panel = 0, cblk = 0, bord = 0, map = 0, nchild = 0;
+  int64_t panel = 0, cblk = 0, bord = 0;
   for (int64_t g = 0; g < nn; ++g) {
     const Key& k = keys[g];
     gid[k.sub][k.id] = (int32_t)g;
@@ -331,14 +343,10 @@ void build_fronts(const HostMesh& m, int factor_bits, bool dirichlet, Fronts& f)
     n.panel = panel;
     n.cblk = cblk;
     n.bord = bord;
-    n.nch = (int32_t)x.child.size();
-    n.child0 = (int32_t)nchild;
-    n.map = (n.nch == 0 || x.map.empty()) ? -1 : map;
+    for (int q = 0; q < 2; ++q) n.child[q] = x.child[q] < 0 ? -1 : gid[k.sub][x.child[q]];
     panel += (int64_t)(n.n1 + n.n2) * n.ld;
     cblk += (int64_t)n.n2 * n.ldc;
     bord += n.n2;
-    map += (int64_t)x.map.size();
-    nchild += n.nch;
     f.level_ptr[k.level + 1]++;
     if (k.wide == 0) f.level_wide[k.level]++;
   }
@@ -346,35 +354,58 @@ void build_fronts(const HostMesh& m, int factor_bits, bool dirichlet, Fronts& f)
   f.panel_elems = panel;
   f.c_elems = cblk;
   f.border_elems = bord;
-  f.child.resize(nchild);
+  if (bord >= (int64_t(1) << 31)) throw std::length_error("the borders of the elimination trees exceed 2^31 entries");
   f.border.resize(bord);
-  f.map.resize(map);
+  f.border_src.resize(bord);
+  f.own_src.resize(rows);
   parallel_for(nn, 64, [&](int64_t g, int) {
     const FrontNode& n = f.nodes[g];
     const LocalNode& x = trees[n.sub][keys[g].id];
     const int32_t base = (int32_t)m.sub_ns_off[n.sub];
-    for (int q = 0; q < n.nch; ++q) f.child[n.child0 + q] = gid[n.sub][x.child[q]];
-    for (int q = 0; q < n.n2; ++q) f.border[n.bord + q] = base + x.border[q];
-    if (n.map >= 0) std::copy(x.map.begin(), x.map.end(), f.map.begin() + n.map);
+    const int32_t b0 = n.child[0] < 0 ? 0 : (int32_t)f.nodes[n.child[0]].bord;
+    const int32_t b1 = n.child[1] < 0 ? 0 : (int32_t)f.nodes[n.child[1]].bord;
+    auto src = [&](int i) {
+      const FrontSrc v = x.src[i];
+      return FrontSrc{v.a < 0 ? -1 : b0 + v.a, v.b < 0 ? -1 : b1 + v.b};
+    };
+    for (int q = 0; q < n.n2; ++q) {
+      f.border[n.bord + q] = base + x.border[q];
+      f.border_src[n.bord + q] = src(n.n1 + q);
+    }
     for (int q = 0; q < n.n1; ++q) {
+      f.own_src[n.row0 + q] = src(q);
       f.row_node[n.row0 + q] = (int32_t)g;
       f.row_dof[n.row0 + q] = m.sub_dofs[base + x.own[q]];
       f.row_pou[n.row0 + q] = m.sub_pou[base + x.own[q]];
     }
   });
   // block lists of every level
-  FrontLevels* all[] = {&f.assemble, &f.lmul, &f.schur, &f.fwd, &f.bwd};
+  FrontLevels* all[] = {&f.assemble, &f.lmul, &f.schur, &f.fwd, &f.bwd, &f.bwd_multi};
   for (auto* v : all) { v->items.clear(); v->ptr.assign(1, 0); }
+  f.bwd_cols.clear();
+  f.multi_cols.clear();
   for (int l = 0; l < nlev; ++l) {
+    // backward pass: narrower column blocks where a level has few nodes
+    int cols = FR_BWD_COLS;
+    auto blocks = [&](int c) {
+      int64_t n = 0;
+      for (int32_t g = f.level_ptr[l]; g < f.level_ptr[l + 1]; ++g) n += (f.nodes[g].n1 + c - 1) / c;
+      return n;
+    };
+    while (cols > 8 && blocks(cols) < FR_BWD_BLOCKS) cols /= 2;
+    f.bwd_cols.push_back(cols);
+    const int multi = blocks(64) < 200 ? 16 : 64;
+    f.multi_cols.push_back(multi);
     for (int32_t g = f.level_ptr[l]; g < f.level_ptr[l + 1]; ++g) {
       const FrontNode& n = f.nodes[g];
-      if (n.nch > 0)
+      if (n.child[0] >= 0 && n.n1 > 0)
         for (int t = 0; t * FR_ASM_ROWS < n.n1 + n.n2; ++t) f.assemble.items.push_back({g, t});
       const int ti = (n.n2 + FR_TILE - 1) / FR_TILE, tj = (n.n1 + FR_TILE - 1) / FR_TILE;
       for (int t = 0; t < ti * tj; ++t) f.lmul.items.push_back({g, t});
       for (int t = 0; t < ti * (ti + 1) / 2; ++t) f.schur.items.push_back({g, t});
       for (int t = 0; t == 0 || t * FR_FWD_ROWS < n.n2; ++t) f.fwd.items.push_back({g, t});
-      for (int t = 0; t * FR_BWD_COLS < n.n1; ++t) f.bwd.items.push_back({g, t});
+      for (int t = 0; t * cols < n.n1; ++t) f.bwd.items.push_back({g, t});
+      for (int t = 0; t * multi < n.n1; ++t) f.bwd_multi.items.push_back({g, t});
     }
     for (auto* v : all) v->ptr.push_back((int64_t)v->items.size());
   }

@@ -175,11 +175,11 @@ struct Device {
   // sparse local factors (oras_handle::fronts): the plan, the assembly workspace and the contribution
   // blocks; the panels are the arena
   FrontNode* fr_nodes = nullptr;
-  int32_t* fr_child = nullptr; int32_t* fr_border = nullptr; int32_t* fr_map = nullptr;
+  int32_t* fr_border = nullptr; FrontSrc* fr_own_src = nullptr; FrontSrc* fr_border_src = nullptr;
   int32_t* fr_pos = nullptr; int32_t* fr_row_node = nullptr; int32_t* fr_row_dof = nullptr;
   uint8_t* fr_row_pou = nullptr;
   FrontItem* fr_assemble = nullptr; FrontItem* fr_lmul = nullptr; FrontItem* fr_schur = nullptr;
-  FrontItem* fr_fwd = nullptr; FrontItem* fr_bwd = nullptr;
+  FrontItem* fr_fwd = nullptr; FrontItem* fr_bwd = nullptr; FrontItem* fr_bwd_multi = nullptr;
   void* fr_work = nullptr; void* fr_c = nullptr;
   cplx* io = nullptr;                           // staging for host I/O [N][k] col-major
   size_t io_elems = 0;
