@@ -8,7 +8,7 @@
 // and the parent adds C's entries to its own front.  The solve needs only [S; L] (fronts_apply.cu).
 // All nodes of a tree level, of all subdomains, go through each step in one launch:
 //   k_fr_assemble  the children's C added to the panels (originals are scattered once, k_fr_rows);
-//   k_fr_invert    S by Gauss-Jordan with row pivoting, the block held in registers;
+//   k_fr_invert    S by blocked Gauss-Jordan with row pivoting, the block held in registers;
 //   k_fr_mul       L, then C with the children's C gathered into it (each C is read once).
 // Pivots are chosen inside a pivot block (up to front_nb unknowns) and never outside it, so the tree
 // stays as planned.
@@ -129,15 +129,34 @@ __global__ void __launch_bounds__(256) k_fr_assemble(FrDev f, const FrontItem* _
 }
 
 // ------------------------------------------------------------------ pivot blocks
-// S = A11^{-1} by Gauss-Jordan elimination in place with row pivoting (max |Re| + |Im|, the lowest row
-// on ties).  NW warps; warp w holds the rows w, w + NW, ..., lane l the columns l, l + 32, ...: NB x NB
-// entries in registers.  Step c: the column's holders publish it, every warp finds the pivot row p,
-// its warp publishes that row, and every entry is updated -- two barriers a step.  No row moves: after
-// the last step entry (p(c), c') holds A^{-1}(c, p(c')), p(c) the pivot row of step c.
+// S = A11^{-1} by Gauss-Jordan elimination in place with row pivoting (max |Re| + |Im|, the lowest row on
+// ties), 8 columns at a time.  NW main warps hold the block in registers (warp w the rows w, w + NW, ...,
+// lane l the columns l, l + 32, ...); NB / 32 panel warps, which hold none of it, eliminate the 8 columns of a
+// panel, one row a lane: a column costs a warp-wide maximum, one barrier among them (each publishes its best
+// candidate's row with its key) and 8 products a lane.  They leave W, the 8 columns of the inverse transformation
+// (in place, as Gauss-Jordan does), and the 8 pivot rows p_c; every other entry then becomes
+//   x(i, j) = [i not a pivot of the panel] x(i, j) + sum_c W(i, c) x(p_c, j).
+// The main warps update the register column with the next panel first and hand that panel over, so its
+// elimination runs beside the rest of the update.  No row moves: at the end entry (p(c), c') holds
+// A^{-1}(c, p(c')), p(c) the pivot row of column c.
+//
+// Bound: FP32 arithmetic, 4 n1^3 fused multiply-adds a block, and on levels with few nodes the chain of n1 pivot
+// searches.  One column at a time (two block barriers and a pivot search on the critical path each): 9.4 ms for all
+// pivot blocks of the 16^3 x 6, degree-2, 64-subdomain problem; panels of 8 by one warp (4 rows a lane) 6.3 ms, by a
+// warp for every 32 rows 4.7 ms.  4^3 x 6, 4 subdomains: 0.62, 0.45 and 0.36 ms.  In FP64 (8^3 x 6, degree 1) 1.97,
+// 2.39 and 1.74 ms: the panel is then FP64 arithmetic, which one warp has a quarter of.
+// One kernel for every 32 columns of width: a block of 97 in a 128-wide kernel costs 1.8 times its products.
+// BLOCKS: 3 blocks of the 64-wide kernel an SM (48 bytes spilled) or 2 of the 96-wide one (288) measured the same.
 template <typename R, int NB> struct InvShared {
-  alignas(16) CT<R> col[2][NB], row[2][NB];
-  int prow[NB], rank[NB];   // pivot row of each step, and its inverse
-  float amax;               // largest entry of the block
+  alignas(16) CT<R> pan[NB][10];     // the panel's 8 columns (rows padded against bank conflicts)
+  alignas(16) CT<R> W[2][NB][10];
+  alignas(16) CT<R> row[2][8][NB];   // the pivot rows before the panel
+  alignas(16) CT<R> cand[2][NB / 32][8];   // each panel warp's best row of a column (by column parity)
+  alignas(16) uint32_t ckey[2][4];         // and its key
+  int piv[2][8];
+  uint32_t pmask[2][NB / 32];        // the panel's pivot rows
+  unsigned char prank[NB], pcol[NB]; // pivot row -> column, column -> pivot row
+  float amax;                        // largest entry of the block
 };
 
 // *dst = v (shared memory) where `on`: one predicated store.  (A branch around plain stores of the row
@@ -150,130 +169,243 @@ __device__ __forceinline__ void store_if(bool on, CT<double>* dst, CT<double> v)
   asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %0, 0;\n @p st.shared.v2.f64 [%1], {%2, %3};\n}"
                ::"r"((int)on), "r"(smem_u32(dst)), "d"(v.re), "d"(v.im) : "memory");
 }
+__device__ __forceinline__ void named_arrive(int id, int nthreads) {
+  asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(nthreads) : "memory");
+}
+// Named barriers: a panel's columns are in pan; its W, pivots are ready; its pivot rows are in row;
+// and, among the panel warps, the candidates of a column.
+enum { INV_BAR_PANEL = 1, INV_BAR_W = 2, INV_BAR_ROWS = 3, INV_BAR_CAND = 4 };
 
-// The steps of the 32 columns held in register column b (a compile-time index: x stays in registers).
-template <typename R, int NB, int NW, int b>
-__device__ __forceinline__ void invert_columns(CT<R> (&x)[NB / NW][NB / 32], uint32_t (&used)[NB / 32],
-                                               InvShared<R, NB>& sh, int n1, int n2, int sub, int32_t* status) {
-  constexpr int RA = NB / NW, CB = NB / 32;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll 1
-  for (int cl = 0; cl < 32; ++cl) {
-    const int c = 32 * b + cl;
-    if (c >= n1) return;
-    const int buf = c & 1;
-    if (lane == cl) {
+// Two adjacent complex entries of shared memory (16-byte aligned).
+__device__ __forceinline__ void lds_pair(const CT<float>* p, CT<float>& a, CT<float>& b) {
+  const float4 t = *reinterpret_cast<const float4*>(p);
+  a = {t.x, t.y}; b = {t.z, t.w};
+}
+__device__ __forceinline__ void lds_pair(const CT<double>* p, CT<double>& a, CT<double>& b) {
+  const double2 t0 = reinterpret_cast<const double2*>(p)[0], t1 = reinterpret_cast<const double2*>(p)[1];
+  a = {t0.x, t0.y}; b = {t1.x, t1.y};
+}
+
+__device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
+__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+
+// Panel warp pw: columns c0 .. c0 + 7 of row 32 pw + lane (rows below `rows` take part).  taken: the row has been a
+// pivot.
+template <typename R, int NB>
+__device__ __forceinline__ void invert_panel(InvShared<R, NB>& sh, int c0, int rows, int buf, bool& taken, int n2,
+                                             int sub, int32_t* status) {
+  constexpr int PW = NB / 32;
+  const int lane = threadIdx.x & 31, pw = (threadIdx.x >> 5) % PW, i = 32 * pw + lane;
+  CT<R> x[8];
 #pragma unroll
-      for (int a = 0; a < RA; ++a) sh.col[buf][warp + NW * a] = x[a][b];
-    }
-    __syncthreads();
+  for (int j = 0; j < 8; j += 2) lds_pair(&sh.pan[i][j], x[j], x[j + 1]);
+  bool mine = false;
+#pragma unroll
+  for (int c = 0; c < 8; ++c) {
+    const int par = c & 1;
+    float mag = (float)(fabs(x[c].re) + fabs(x[c].im));
+    if (mag != mag) mag = 0.0f;  // a non-finite entry still lets a row be chosen
     uint32_t key = 0u;
+    if (i < rows && !taken) key = ((__float_as_uint(mag) << 1) & 0xFFFFFF00u) | 0x80u | (uint32_t)(127 - i);
+    uint32_t best = __reduce_max_sync(0xffffffffu, key);
+    if (best != 0u && key == best) {
 #pragma unroll
-    for (int q = 0; q < CB; ++q) {
-      const int i = lane + 32 * q;
-      const CT<R> v = sh.col[buf][i];
-      float mag = (float)(fabs(v.re) + fabs(v.im));
-      if (mag != mag) mag = 0.0f;  // a non-finite entry still lets a row be chosen
-      if (i < n1 && !((used[q] >> lane) & 1u))
-        key = max(key, ((__float_as_uint(mag) << 1) & 0xFFFFFF00u) | 0x80u | (uint32_t)(127 - i));
+      for (int j = 0; j < 8; ++j) sh.cand[par][pw][j] = x[j];
+      sh.ckey[par][pw] = best;
+    } else if (best == 0u && lane == 0) {
+      sh.ckey[par][pw] = 0u;
     }
-    key = __reduce_max_sync(0xffffffffu, key);
-    const int p = 127 - (int)(key & 0x7Fu);
+    if constexpr (PW > 1) {
+      named_sync(INV_BAR_CAND, PW * 32);
 #pragma unroll
-    for (int q = 0; q < CB; ++q)
-      if ((p >> 5) == q) used[q] |= 1u << (p & 31);
-    if (warp == p % NW) {
-#pragma unroll
-      for (int a = 0; a < RA; ++a)
-#pragma unroll
-        for (int q = 0; q < CB; ++q) store_if(a == p / NW, &sh.row[buf][lane + 32 * q], x[a][q]);
+      for (int q = 0; q < PW; ++q) best = max(best, sh.ckey[par][q]);
+    } else {
+      __syncwarp();
     }
-    if (threadIdx.x == 0) {
-      sh.prow[c] = p;
-      sh.rank[p] = c;
+    const int p = 127 - (int)(best & 0x7Fu);
+    const bool own = i == p;
+    CT<R> r[8];
+#pragma unroll
+    for (int j = 0; j < 8; j += 2) lds_pair(&sh.cand[par][PW > 1 ? p >> 5 : 0][j], r[j], r[j + 1]);
+    if (own) {
+      taken = mine = true;
+      sh.piv[buf][c] = p;
+      sh.prank[p] = (unsigned char)(c0 + c);
+      sh.pcol[c0 + c] = (unsigned char)p;
     }
-    __syncthreads();
-    const CT<R> pv = sh.row[buf][c];
+    const CT<R> pv = r[c];
     CT<R> inv = {R(0), R(0)};
     if (pv.re != R(0) || pv.im != R(0)) {
-      const R den = pv.re * pv.re + pv.im * pv.im;
-      inv = {pv.re / den, -pv.im / den};
+      const R rden = recip(pv.re * pv.re + pv.im * pv.im);
+      inv = {pv.re * rden, -pv.im * rden};
     } else if (n2 > 0 && sh.amax > 0.0f) {
       // an exactly zero pivot column: the unknowns eliminated later can still make A_s regular, so the
       // pivot is taken as the rounding of the block's entries
       inv.re = R(1) / (R(sh.amax) * (sizeof(R) == 4 ? R(1.0 / (1 << 20)) : R(1.0 / (1ll << 45))));
-    } else if (threadIdx.x == 0) {
+    } else if (own) {
       if (atomicCAS(&status[ST_ERR], DEV_OK, DEV_SINGULAR) == DEV_OK) status[ST_SUB] = sub;
     }
-    CT<R> rj[CB];
-#pragma unroll
-    for (int q = 0; q < CB; ++q) {
-      const CT<R> v = sh.row[buf][lane + 32 * q];
-      rj[q] = {v.re * inv.re - v.im * inv.im, v.re * inv.im + v.im * inv.re};
+    // x_j <- x_j - (x_c / pv) r_j; the pivot row itself becomes r_j / pv
+    const CT<R> l = x[c];
+    CT<R> m = inv;
+    if (!own) {
+      m.re = fma(l.im, inv.im, -l.re * inv.re);
+      m.im = -fma(l.im, inv.re, l.re * inv.im);
     }
-    if (lane == cl) rj[b] = inv;
 #pragma unroll
-    for (int a = 0; a < RA; ++a) {
-      const int i = warp + NW * a;
-      if (i == p) {
-#pragma unroll
-        for (int q = 0; q < CB; ++q) x[a][q] = rj[q];
-      } else {
-        const CT<R> l = sh.col[buf][i];
-        if (lane == cl) x[a][b] = {R(0), R(0)};
-#pragma unroll
-        for (int q = 0; q < CB; ++q) {
-          CT<R> t = x[a][q];
-          t.re = fma(-l.re, rj[q].re, t.re);
-          t.im = fma(-l.re, rj[q].im, t.im);
-          t.re = fma(l.im, rj[q].im, t.re);
-          t.im = fma(-l.im, rj[q].re, t.im);
-          x[a][q] = t;
-        }
-      }
+    for (int j = 0; j < 8; ++j) {
+      CT<R> t = own ? CT<R>{R(0), R(0)} : x[j];
+      t.re = fma(m.re, r[j].re, t.re);
+      t.im = fma(m.re, r[j].im, t.im);
+      t.re = fma(-m.im, r[j].im, t.re);
+      t.im = fma(m.im, r[j].re, t.im);
+      x[j] = j == c ? m : t;
     }
+  }
+#pragma unroll
+  for (int j = 0; j < 8; ++j) sh.W[buf][i][j] = x[j];
+  const uint32_t m = __ballot_sync(0xffffffffu, mine);
+  if (lane == 0) sh.pmask[buf][pw] = m;
+}
+
+// Register column b (columns 32 cb .. 32 cb + 31 of the block) of the main warps after a panel: the panel's own 8
+// lanes (from lane 8 pl when `here`) take W, the others the rank-8 update.
+template <typename R, int NB, int NW, int b>
+__device__ __forceinline__ void invert_update(CT<R> (&x)[NB / NW][NB / 32], const InvShared<R, NB>& sh, int buf,
+                                              int cb, bool here, int pl) {
+  constexpr int RA = NB / NW;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int pc = lane - 8 * pl;
+  const bool in_panel = here && pc >= 0 && pc < 8;
+  CT<R> r[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) r[c] = sh.row[buf][c][lane + 32 * cb];
+#pragma unroll
+  for (int a = 0; a < RA; ++a) {
+    const int i = warp + NW * a;
+    CT<R> t = ((sh.pmask[buf][i >> 5] >> (i & 31)) & 1u) ? CT<R>{R(0), R(0)} : x[a][b];
+#pragma unroll
+    for (int c = 0; c < 8; c += 2) {
+      CT<R> w0, w1;
+      lds_pair(&sh.W[buf][i][c], w0, w1);
+      t.re = fma(w0.re, r[c].re, t.re);
+      t.im = fma(w0.re, r[c].im, t.im);
+      t.re = fma(-w0.im, r[c].im, t.re);
+      t.im = fma(w0.im, r[c].re, t.im);
+      t.re = fma(w1.re, r[c + 1].re, t.re);
+      t.im = fma(w1.re, r[c + 1].im, t.im);
+      t.re = fma(-w1.im, r[c + 1].im, t.re);
+      t.im = fma(w1.im, r[c + 1].re, t.im);
+    }
+    x[a][b] = in_panel ? sh.W[buf][i][pc & 7] : t;
+    asm volatile("" ::: "memory");  // one row's W at a time: loaded ahead for all rows it spills
   }
 }
 
+// Columns 8 pl .. 8 pl + 7 of register column b into pan.
+template <typename R, int NB, int NW, int b>
+__device__ __forceinline__ void publish_panel(const CT<R> (&x)[NB / NW][NB / 32], InvShared<R, NB>& sh, int pl) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, c = lane - 8 * pl;
+  if (c < 0 || c >= 8) return;
+#pragma unroll
+  for (int a = 0; a < NB / NW; ++a) sh.pan[warp + NW * a][c] = x[a][b];
+}
+
+// x's register columns shifted left by one, cyclically.
+template <typename R, int RA, int CB>
+__device__ __forceinline__ void rotate_columns(CT<R> (&x)[RA][CB]) {
+#pragma unroll
+  for (int a = 0; a < RA; ++a) {
+    const CT<R> t = x[a][0];
+#pragma unroll
+    for (int q = 0; q + 1 < CB; ++q) x[a][q] = x[a][q + 1];
+    x[a][CB - 1] = t;
+  }
+}
+
+// The main warps' steps, np panels.  Register column 0 is always the one worked on (register indices stay
+// compile-time) and the columns rotate: slot s holds block column (s + returned rotation) % CB.  One instance of
+// the update in a rolled loop: inlined for every column the compiler loads their operands ahead and spills.
 template <typename R, int NB, int NW>
-__global__ void __launch_bounds__(NW * 32) k_fr_invert(FrDev f, int first, const CT<R>* __restrict__ work,
-                                                       CT<R>* __restrict__ fac, int32_t* status) {
-  constexpr int RA = NB / NW, CB = NB / 32;
-  static_assert(NB <= 128 && NB % NW == 0 && NB % 32 == 0, "pivot keys hold 7 row bits");
+__device__ __forceinline__ int invert_main(CT<R> (&x)[NB / NW][NB / 32], InvShared<R, NB>& sh, int np) {
+  constexpr int RA = NB / NW, CB = NB / 32, MAIN = NW * 32, ALL = MAIN + NB;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  int rot = 0;
+  auto next = [&]() {
+    rotate_columns<R, RA, CB>(x);
+    rot = rot + 1 < CB ? rot + 1 : 0;
+  };
+#pragma unroll 1
+  for (int p = 0; p < np; ++p) {
+    const int pl = p & 3, buf = p & 1;
+    named_sync(INV_BAR_W, ALL);
+#pragma unroll 1
+    for (int c = 0; c < 8; ++c) {
+      const int i = sh.piv[buf][c];
+      if (i % NW == warp) {
+#pragma unroll
+        for (int a = 0; a < RA; ++a)
+#pragma unroll
+          for (int q = 0; q < CB; ++q)
+            store_if(a == i / NW, &sh.row[buf][c][lane + 32 * (q + rot < CB ? q + rot : q + rot - CB)], x[a][q]);
+      }
+    }
+    named_sync(INV_BAR_ROWS, MAIN);
+    // the column with the next panel first: this panel's own, or after its last panel the one that follows
+    if (CB > 1 && pl == 3) next();
+    const int own = CB > 1 && pl == 3 ? CB - 1 : 0;
+#pragma unroll 1
+    for (int s = 0; s < CB; ++s) {
+      invert_update<R, NB, NW, 0>(x, sh, buf, rot, s == own, pl);
+      if (s == 0 && p + 1 < np) {
+        publish_panel<R, NB, NW, 0>(x, sh, (pl + 1) & 3);
+        named_arrive(INV_BAR_PANEL, ALL);
+      }
+      if (CB > 1) next();
+    }
+  }
+  return rot;
+}
+
+template <typename R, int NB, int NW, int BLOCKS>
+__global__ void __launch_bounds__(NW * 32 + NB, BLOCKS)
+    k_fr_invert(FrDev f, int first, const CT<R>* __restrict__ work, CT<R>* __restrict__ fac, int32_t* status) {
+  constexpr int RA = NB / NW, CB = NB / 32, ALL = NW * 32 + NB;
+  static_assert(NB <= 128 && NB % NW == 0 && NB % 32 == 0 && NW % (NB / 32) == 0, "pivot keys hold 7 row bits");
   __shared__ InvShared<R, NB> sh;
   const FrontNode n = f.nodes[first + blockIdx.x];
-  const int n1 = n.n1, ld = n.ld;
+  const int n1 = n.n1, ld = n.ld, np = (n1 + 7) / 8;  // the last panel's columns past n1 are identity columns
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  if (threadIdx.x == 0) sh.amax = 0.0f;
+  __syncthreads();
+  if (warp >= NW) {
+    bool taken = false;
+    __syncthreads();  // amax and the first panel
+    for (int p = 0; p < np; ++p) {
+      if (p > 0) named_sync(INV_BAR_PANEL, ALL);
+      invert_panel<R, NB>(sh, 8 * p, 8 * np, p & 1, taken, n.n2, n.sub, status);
+      named_arrive(INV_BAR_W, ALL);
+    }
+    __syncthreads();
+    return;
+  }
   const CT<R>* src = work + n.panel;
   CT<R> x[RA][CB];
+  uint32_t big = 0u;  // magnitudes as ordered bits (NaN above infinity)
 #pragma unroll
   for (int a = 0; a < RA; ++a)
 #pragma unroll
     for (int b = 0; b < CB; ++b) {
       const int i = warp + NW * a, j = lane + 32 * b;
-      x[a][b] = (i < n1 && j < n1) ? src[(int64_t)i * ld + j] : CT<R>{R(i == j ? 1 : 0), R(0)};
+      const bool in = i < n1 && j < n1;
+      x[a][b] = in ? src[(int64_t)i * ld + j] : CT<R>{R(i == j ? 1 : 0), R(0)};
+      if (in) big = max(big, __float_as_uint((float)(fabs(x[a][b].re) + fabs(x[a][b].im))));
     }
-  {
-    uint32_t big = 0u;  // magnitudes as ordered bits (NaN above infinity)
-#pragma unroll
-    for (int a = 0; a < RA; ++a)
-#pragma unroll
-      for (int b = 0; b < CB; ++b)
-        if (warp + NW * a < n1 && lane + 32 * b < n1)
-          big = max(big, __float_as_uint((float)(fabs(x[a][b].re) + fabs(x[a][b].im))));
-    big = __reduce_max_sync(0xffffffffu, big);
-    if (threadIdx.x == 0) sh.amax = 0.0f;
-    __syncthreads();
-    if (lane == 0) atomicMax((unsigned int*)&sh.amax, big);  // visible after the first step's barrier
-  }
-  uint32_t used[CB];  // bit l of word q: row l + 32 q has been a pivot (CB words of 32 rows)
-#pragma unroll
-  for (int q = 0; q < CB; ++q) used[q] = 0u;
-  invert_columns<R, NB, NW, 0>(x, used, sh, n1, n.n2, n.sub, status);
-  if constexpr (CB > 1) invert_columns<R, NB, NW, 1>(x, used, sh, n1, n.n2, n.sub, status);
-  if constexpr (CB > 2) invert_columns<R, NB, NW, 2>(x, used, sh, n1, n.n2, n.sub, status);
-  if constexpr (CB > 3) invert_columns<R, NB, NW, 3>(x, used, sh, n1, n.n2, n.sub, status);
-  static_assert(CB <= 4, "register columns");
+  big = __reduce_max_sync(0xffffffffu, big);
+  if (lane == 0) atomicMax((unsigned int*)&sh.amax, big);
+  publish_panel<R, NB, NW, 0>(x, sh, 0);
+  __syncthreads();
+  const int rot = invert_main<R, NB, NW>(x, sh, np);
   __syncthreads();
   CT<R>* dst = fac + n.panel;
 #pragma unroll
@@ -282,8 +414,8 @@ __global__ void __launch_bounds__(NW * 32) k_fr_invert(FrDev f, int first, const
     if (i >= n1) continue;
 #pragma unroll
     for (int b = 0; b < CB; ++b) {
-      const int j = lane + 32 * b;
-      if (j < n1) dst[(int64_t)sh.rank[i] * ld + sh.prow[j]] = x[a][b];
+      const int j = lane + 32 * (b + rot < CB ? b + rot : b + rot - CB);
+      if (j < n1) dst[(int64_t)sh.prank[i] * ld + sh.pcol[j]] = x[a][b];
     }
     if (lane < ld - n1) dst[(int64_t)i * ld + n1 + lane] = {R(0), R(0)};
   }
@@ -415,16 +547,25 @@ static int factor_t(oras_handle* h) {
       count_launches(1);
     }
     prof_end(h, KC_LU_SWAP, pb, 1);
-    const int first = f.level_ptr[l], wide = f.level_wide[l], all = f.level_ptr[l + 1] - first;
     pb = prof_begin(h);
-    if constexpr (sizeof(R) == 4) {
-      if (wide) k_fr_invert<R, 128, 16><<<wide, 512, 0, st>>>(fd, first, work, fac, d.status);
-      if (all > wide) k_fr_invert<R, 64, 8><<<all - wide, 256, 0, st>>>(fd, first + wide, work, fac, d.status);
-    } else {
-      if (wide) k_fr_invert<R, 64, 8><<<wide, 256, 0, st>>>(fd, first, work, fac, d.status);
-      if (all > wide) k_fr_invert<R, 32, 4><<<all - wide, 128, 0, st>>>(fd, first + wide, work, fac, d.status);
+    // pivot blocks by width; a level that fits on the chip at once goes in one launch
+    const int32_t* cp = &f.level_class[(size_t)l * (FR_CLASSES + 1)];
+    const bool one = cp[FR_CLASSES] - cp[0] <= d.num_sms;
+    for (int c = 0; c < FR_CLASSES; ++c) {
+      const int first = cp[c], nodes = (one ? cp[FR_CLASSES] : cp[c + 1]) - first;
+      if (nodes == 0 || (c < FR_CLASSES - 1 && cp[c + 1] == cp[c])) continue;
+      if constexpr (sizeof(R) == 4) {
+        if (c == 0) k_fr_invert<R, 128, 16, 1><<<nodes, 640, 0, st>>>(fd, first, work, fac, d.status);
+        else if (c == 1) k_fr_invert<R, 96, 12, 1><<<nodes, 480, 0, st>>>(fd, first, work, fac, d.status);
+        else if (c == 2) k_fr_invert<R, 64, 8, 2><<<nodes, 320, 0, st>>>(fd, first, work, fac, d.status);
+        else k_fr_invert<R, 32, 4, 4><<<nodes, 160, 0, st>>>(fd, first, work, fac, d.status);
+      } else {
+        if (c == 2) k_fr_invert<R, 64, 8, 1><<<nodes, 320, 0, st>>>(fd, first, work, fac, d.status);
+        else k_fr_invert<R, 32, 4, 4><<<nodes, 160, 0, st>>>(fd, first, work, fac, d.status);
+      }
+      count_launches(1);
+      if (one) break;
     }
-    count_launches((wide ? 1 : 0) + (all > wide ? 1 : 0));
     prof_end(h, KC_LU_TOURNAMENT, pb, 1);
     if (!count(f.schur)) continue;
     pb = prof_begin(h);

@@ -36,6 +36,10 @@ constexpr int FR_BWD_BLOCKS = 1216;  // levels with fewer blocks than this (8 an
 // in registers.
 inline int front_nb(int factor_bits) { return factor_bits == 64 ? 64 : 128; }
 
+// Width class of a pivot block: kernels for up to 128, 96, 64 and 32 unknowns.
+constexpr int FR_CLASSES = 4;
+inline int front_class(int n1) { return n1 > 96 ? 0 : (n1 > 64 ? 1 : (n1 > 32 ? 2 : 3)); }
+
 struct FrontLevels {  // per level: [ptr[l], ptr[l + 1]) of the item list
   std::vector<FrontItem> items;
   std::vector<int64_t> ptr;
@@ -45,7 +49,7 @@ struct Fronts {
   bool use = false;
   std::vector<FrontNode> nodes;       // by level, wide pivot blocks first within a level
   std::vector<int32_t> level_ptr;     // [nlev + 1] first node of each level
-  std::vector<int32_t> level_wide;    // [nlev] nodes of the level with more than front_nb / 2 own rows
+  std::vector<int32_t> level_class;   // [nlev][FR_CLASSES + 1] first node of each width class (front_class)
   std::vector<int32_t> border;        // positions
   std::vector<FrontSrc> own_src, border_src;
   std::vector<int32_t> pos;           // [sum ns] position (within its subdomain) of the local unknown i
@@ -56,7 +60,7 @@ struct Fronts {
   std::vector<int32_t> bwd_cols;      // [nlev] own columns per block of bwd: 8, 16 or 32
   std::vector<int32_t> multi_cols;    // [nlev] and of bwd_multi: 16 or 64
   int64_t panel_elems = 0, c_elems = 0, border_elems = 0;
-  int nlev() const { return (int)level_wide.size(); }
+  int nlev() const { return (int)multi_cols.size(); }
 };
 
 struct HostMesh;

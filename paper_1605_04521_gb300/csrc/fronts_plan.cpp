@@ -311,7 +311,7 @@ void build_fronts(const HostMesh& m, int factor_bits, bool dirichlet, Fronts& f)
     gid[s].resize(trees[s].size());
     for (size_t q = 0; q < trees[s].size(); ++q) {
       const LocalNode& x = trees[s][q];
-      keys.push_back({x.level, (int)x.own.size() > nb / 2 ? 0 : 1, -(int32_t)x.border.size(), s, (int32_t)q});
+      keys.push_back({x.level, front_class((int)x.own.size()), -(int32_t)x.border.size(), s, (int32_t)q});
       nlev = std::max(nlev, x.level + 1);
     }
   }
@@ -324,7 +324,7 @@ void build_fronts(const HostMesh& m, int factor_bits, bool dirichlet, Fronts& f)
   const int64_t nn = (int64_t)keys.size();
   f.nodes.resize(nn);
   f.level_ptr.assign(nlev + 1, 0);
-  f.level_wide.assign(nlev, 0);
+  f.level_class.assign((size_t)nlev * (FR_CLASSES + 1), 0);
   f.row_node.resize(rows);
   f.row_dof.resize(rows);
   f.row_pou.resize(rows);
@@ -348,9 +348,14 @@ void build_fronts(const HostMesh& m, int factor_bits, bool dirichlet, Fronts& f)
     cblk += (int64_t)n.n2 * n.ldc;
     bord += n.n2;
     f.level_ptr[k.level + 1]++;
-    if (k.wide == 0) f.level_wide[k.level]++;
+    f.level_class[(size_t)k.level * (FR_CLASSES + 1) + k.wide + 1]++;
   }
-  for (int l = 0; l < nlev; ++l) f.level_ptr[l + 1] += f.level_ptr[l];
+  for (int l = 0; l < nlev; ++l) {
+    f.level_ptr[l + 1] += f.level_ptr[l];
+    int32_t* c = &f.level_class[(size_t)l * (FR_CLASSES + 1)];
+    c[0] = f.level_ptr[l];
+    for (int q = 0; q < FR_CLASSES; ++q) c[q + 1] += c[q];
+  }
   f.panel_elems = panel;
   f.c_elems = cblk;
   f.border_elems = bord;
