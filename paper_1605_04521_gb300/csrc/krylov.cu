@@ -20,14 +20,17 @@ template <> __device__ __forceinline__ cplx ld_c<CT<float>>(const CT<float>* p, 
 
 // Both products with A give a row SPMV_LPR lanes: KL of them take one right-hand side each (x and y rows are
 // adjacent in memory over the right-hand sides, a value of A is broadcast), the EL = SPMV_LPR / KL groups
-// share the row's entries.  Each lane issues the (value, column) loads of SPMV_UNR entries at once, then their x
-// gathers, then the arithmetic.  With more than KL right-hand sides the blocks of the same rows are
-// neighbours in the grid, so the rows of A come from L2 after the first.
+// share the row's entries.  Each lane issues the (value, column) loads of UNR entries at once, then their x
+// gathers, then the arithmetic.  The kernels are bound by issue slots (the FP32-pipe product has 44 arithmetic
+// instructions an entry), so the rest is kept short: entries are indexed from the row's first in 32 bits, past
+// the row's end its last entry is loaded again and not used, and an x address is one multiply-add.  With more
+// than KL right-hand sides the blocks of the same rows are neighbours in the grid, so the rows of A come from L2
+// after the first.
 constexpr int SPMV_LPR = 8;
-constexpr int SPMV_UNR = 4;
 
 template <int KL> struct SpmvLane {
   static constexpr int EL = SPMV_LPR / KL;
+  static constexpr int UNR = EL == 8 ? 6 : 4;   // a degree-2 row (42 entries) in one go of 8 lanes
   int64_t row;
   int r, el;
   bool on;
@@ -42,30 +45,36 @@ template <int KL> struct SpmvLane {
 
 // y = A x  (x: [N][k] in XT, y: [N][k] FP64), four fused multiply-adds an entry: bound by the FP64 pipe
 // (2 lanes a clock an SM), so no lane idles for a whole row and the sums over lanes are few.  8 fields of the
-// 20^3 degree-2 problem: a warp a row, unfused, 2.99 ms.
+// 20^3 degree-2 problem: a warp a row, unfused, 2.99 ms; now 0.84 ms.
 template <typename XT, int KL>
 __global__ void __launch_bounds__(256) k_spmv(int64_t n, const int64_t* __restrict__ rowptr,
                                               const int32_t* __restrict__ cols, const cplx* __restrict__ vals,
                                               const XT* __restrict__ x, cplx* __restrict__ y, int k, int chunks) {
   const SpmvLane<KL> L(n, k, chunks);
   constexpr int EL = SpmvLane<KL>::EL;
+  constexpr int UNR = SpmvLane<KL>::UNR;
   cplx acc = {0.0, 0.0};
   if (L.on) {
-    const int64_t p1 = rowptr[L.row + 1];
-    for (int64_t p = rowptr[L.row] + L.el; p < p1; p += EL * SPMV_UNR) {
-      cplx a[SPMV_UNR], v[SPMV_UNR];
-      int64_t c[SPMV_UNR];
+    const int64_t p0 = rowptr[L.row];
+    const int len = (int)(rowptr[L.row + 1] - p0);
+    const cplx* av = vals + p0;
+    const int32_t* cv = cols + p0;
+    const char* xb = reinterpret_cast<const char*>(x + L.r);
+    const uint32_t stride = (uint32_t)(k * sizeof(XT));
+    for (int i = L.el; i < len; i += EL * UNR) {
+      cplx a[UNR], v[UNR];
+      uint32_t c[UNR];
 #pragma unroll
-      for (int u = 0; u < SPMV_UNR; ++u) {
-        const bool in = p + u * EL < p1;
-        a[u] = in ? vals[p + u * EL] : cplx{0.0, 0.0};
-        c[u] = in ? (int64_t)cols[p + u * EL] : -1;
+      for (int u = 0; u < UNR; ++u) {
+        const int q = min(i + u * EL, len - 1);
+        a[u] = av[q];
+        c[u] = (uint32_t)cv[q];
       }
 #pragma unroll
-      for (int u = 0; u < SPMV_UNR; ++u) v[u] = c[u] >= 0 ? ld_c<XT>(x, c[u] * k + L.r) : cplx{0.0, 0.0};
+      for (int u = 0; u < UNR; ++u) v[u] = ld_c<XT>(reinterpret_cast<const XT*>(xb + (uint64_t)c[u] * stride), 0);
 #pragma unroll
-      for (int u = 0; u < SPMV_UNR; ++u)
-        if (c[u] >= 0) {
+      for (int u = 0; u < UNR; ++u)
+        if (i + u * EL < len) {
           acc.re = fma(a[u].re, v[u].re, acc.re);
           acc.im = fma(a[u].re, v[u].im, acc.im);
           acc.re = fma(-a[u].im, v[u].im, acc.re);
@@ -130,7 +139,8 @@ __global__ void k_split_vals(int64_t nnz, const cplx* __restrict__ vals, float4*
   out[p] = make_float4(rh, ih, (float)(v.re - (double)rh), (float)(v.im - (double)ih));
 }
 
-// y = A x with x complex FP32 ([N][k]), y FP64 ([N][k]).
+// y = A x with x complex FP32 ([N][k]), y FP64 ([N][k]).  Predicated 64-bit indexing against this: one field of the
+// 12^3 x 6, degree-3 problem 98 -> 92 us (the public call), three of the 10^3 one 82 -> 70 ms for a whole solve's products.
 template <int KL>
 __global__ void __launch_bounds__(256) k_spmv_df(int64_t n, const int64_t* __restrict__ rowptr,
                                                  const int32_t* __restrict__ cols, const float4* __restrict__ vals,
@@ -138,28 +148,35 @@ __global__ void __launch_bounds__(256) k_spmv_df(int64_t n, const int64_t* __res
                                                  int chunks) {
   const SpmvLane<KL> L(n, k, chunks);
   constexpr int EL = SpmvLane<KL>::EL;
+  constexpr int UNR = SpmvLane<KL>::UNR;
   float rh = 0.0f, rl = 0.0f, ih = 0.0f, il = 0.0f;
   if (L.on) {
-    const int64_t p1 = rowptr[L.row + 1];
-    for (int64_t p = rowptr[L.row] + L.el; p < p1; p += EL * SPMV_UNR) {
-      float4 a[SPMV_UNR];
-      int64_t c[SPMV_UNR];
+    const int64_t p0 = rowptr[L.row];
+    const int len = (int)(rowptr[L.row + 1] - p0);
+    const float4* av = vals + p0;
+    const int32_t* cv = cols + p0;
+    const char* xb = reinterpret_cast<const char*>(x + L.r);
+    const uint32_t stride = (uint32_t)(k * sizeof(CT<float>));
+    for (int i = L.el; i < len; i += EL * UNR) {
+      float4 a[UNR];
+      uint32_t c[UNR];
 #pragma unroll
-      for (int u = 0; u < SPMV_UNR; ++u) {
-        const bool in = p + u * EL < p1;
-        a[u] = in ? vals[p + u * EL] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        c[u] = in ? (int64_t)cols[p + u * EL] : -1;
+      for (int u = 0; u < UNR; ++u) {
+        const int q = min(i + u * EL, len - 1);
+        a[u] = av[q];
+        c[u] = (uint32_t)cv[q];
       }
-      CT<float> xv[SPMV_UNR];
+      float2 xv[UNR];
 #pragma unroll
-      for (int u = 0; u < SPMV_UNR; ++u) xv[u] = c[u] >= 0 ? x[c[u] * k + L.r] : CT<float>{0.0f, 0.0f};
+      for (int u = 0; u < UNR; ++u) xv[u] = *reinterpret_cast<const float2*>(xb + (uint64_t)c[u] * stride);
 #pragma unroll
-      for (int u = 0; u < SPMV_UNR; ++u) {
-        df_mac(rh, rl, a[u].x, a[u].z, xv[u].re);    // + a_re x_re
-        df_mac(rh, rl, -a[u].y, -a[u].w, xv[u].im);  // - a_im x_im
-        df_mac(ih, il, a[u].x, a[u].z, xv[u].im);    // + a_re x_im
-        df_mac(ih, il, a[u].y, a[u].w, xv[u].re);    // + a_im x_re
-      }
+      for (int u = 0; u < UNR; ++u)
+        if (i + u * EL < len) {
+          df_mac(rh, rl, a[u].x, a[u].z, xv[u].x);    // + a_re x_re
+          df_mac(rh, rl, -a[u].y, -a[u].w, xv[u].y);  // - a_im x_im
+          df_mac(ih, il, a[u].x, a[u].z, xv[u].y);    // + a_re x_im
+          df_mac(ih, il, a[u].y, a[u].w, xv[u].x);    // + a_im x_re
+        }
     }
   }
 #pragma unroll
@@ -258,8 +275,9 @@ __global__ void __launch_bounds__(256) k_sum_partials(int n, int k, int nb, cons
 // from hs), then the block partials of <Vn_q, w> over the nn vectors from Vn (nn = 0: of |w|^2 instead).
 // Vectors are nk apart.  A block's coefficients are taken together (its vectors are orthonormal to the
 // basis's own accuracy), blocks one after the other.  Bound: the FP64 pipe, 8 fused multiply-adds an entry
-// and basis vector; one vector a pass (a launch, a reduction and w through memory each) ran at a third of
-// that: 21 us a vector of 542,736 entries, now 7.6.
+// and basis vector; a pass over 8 vectors of 352,170 entries
+// takes 51 us with that pipe 70% busy.  One vector a pass (a launch, a reduction and w through memory each) took 21 us
+// a vector of 542,736 entries.
 constexpr int MGS_BLOCK = 8;
 __global__ void __launch_bounds__(RED_THREADS) k_mgs_block(int64_t nk, int k, int nv, const cplx* __restrict__ V,
                                                            int nn, const cplx* __restrict__ Vn,
