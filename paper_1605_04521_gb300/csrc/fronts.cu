@@ -9,26 +9,21 @@
 // All nodes of a tree level, of all subdomains, go through each step in one launch:
 //   k_fr_assemble  the children's C added to the panels (originals are scattered once, k_fr_rows);
 //   k_fr_invert    S by blocked Gauss-Jordan with row pivoting, the block held in registers;
-//   k_fr_mul       L, then C with the children's C gathered into it (each C is read once).
+//   k_fr_mul, k_fr_mul_tc (fronts_tc.cu)  L, then C with the children's C gathered into it (each C is read once).
 // Pivots are chosen inside a pivot block (up to front_nb unknowns) and never outside it, so the tree
 // stays as planned.
 //
 // Against dense factors of the same matrices (n_s^2 entries each) the largest subdomain of the
 // 16^3 x 6, degree-2, 64-subdomain problem (17,896 unknowns) keeps 2% of the entries and needs 0.1%
-// of the products.  FP32 factors are FP32 throughout (no TF32 operands): against FP64 solves their
+// of the products.  FP32 factors keep FP32's accuracy throughout (fronts_tc.cu): against FP64 solves their
 // error is 5e-7 at degree 2 and 3e-6 at degree 3 or without losses, that of a dense FP32 LU with
 // partial pivoting (1e-6 and 5e-6).
+#include "fronts.cuh"
 #include "rows.cuh"
 
 namespace oras {
 
-// device copies of the plan (fronts.h)
-struct FrDev {
-  const FrontNode* nodes;
-  const int32_t* border;
-  const FrontSrc* own_src;
-  const FrontSrc* border_src;
-};
+void launch_front_mul_tc(const oras_handle* h, const FrDev& f, bool schur, const FrontItem* items, int64_t blocks);
 
 static FrDev fr_dev(const oras_handle* h) {
   const auto& d = h->dev;
@@ -85,32 +80,7 @@ __global__ void k_fr_rows(RowArgs A, FrDev f, int nsub, int64_t total_rows, cons
   }
 }
 
-// ------------------------------------------------------------------ children's contributions
-__device__ __forceinline__ FrontSrc front_src(const FrDev& f, const FrontNode& n, int i) {
-  return i < n.n1 ? f.own_src[n.row0 + i] : f.border_src[n.bord + i - n.n1];
-}
-
-// The children's contributions to an entry of the front of node n whose rows have the sources s and t
-// (lower entries of their blocks are stored).
-template <typename R>
-__device__ __forceinline__ CT<R> pull(const FrDev& f, const FrontNode& n, const CT<R>* __restrict__ C, FrontSrc s,
-                                      FrontSrc t) {
-  CT<R> r = {R(0), R(0)};
-  if (s.a >= 0 && t.a >= 0) {
-    const FrontNode& c = f.nodes[n.child[0]];
-    const int64_t lo = min(s.a, t.a) - c.bord, hi = max(s.a, t.a) - c.bord;
-    r = C[c.cblk + hi * c.ldc + lo];
-  }
-  if (s.b >= 0 && t.b >= 0) {
-    const FrontNode& c = f.nodes[n.child[1]];
-    const int64_t lo = min(s.b, t.b) - c.bord, hi = max(s.b, t.b) - c.bord;
-    const CT<R> v = C[c.cblk + hi * c.ldc + lo];
-    r.re += v.re;
-    r.im += v.im;
-  }
-  return r;
-}
-
+// ------------------------------------------------------------------ children's contributions (pull)
 // Panel rows of the nodes with children: 32 rows a block, lanes along the own columns.
 template <typename R>
 __global__ void __launch_bounds__(256) k_fr_assemble(FrDev f, const FrontItem* __restrict__ items,
@@ -421,18 +391,15 @@ __global__ void __launch_bounds__(NW * 32 + NB, BLOCKS)
   }
 }
 
-// ------------------------------------------------------------------ panel and contribution products
+// ------------------------------------------------------------------ panel and contribution products (FP64; FP32: fronts_tc.cu)
 // out = A B^T over the panel's own unknowns (both operands row-major, contiguous along the sum), one
 // 64 x 64 tile a block, 4 x 4 entries a thread.
 //   SCHUR = false: L = A21 S       (B = S, symmetric)
 //   SCHUR = true:  C = pulled children - L A21^T, tiles on and below the diagonal
-template <typename R> struct FrK { static constexpr int KC = 16; };
-template <> struct FrK<double> { static constexpr int KC = 8; };
-
 template <typename R, bool SCHUR>
 __global__ void __launch_bounds__(256) k_fr_mul(FrDev f, const FrontItem* __restrict__ items, CT<R>* __restrict__ work,
                                                 CT<R>* __restrict__ fac, CT<R>* __restrict__ C) {
-  constexpr int KC = FrK<R>::KC, LDS = FR_TILE + 2;
+  constexpr int KC = 8, LDS = FR_TILE + 2;
   __shared__ __align__(16) CT<R> As[KC][LDS], Bs[KC][LDS];
   const FrontItem it = items[blockIdx.x];
   const FrontNode n = f.nodes[it.node];
@@ -569,12 +536,23 @@ static int factor_t(oras_handle* h) {
     prof_end(h, KC_LU_TOURNAMENT, pb, 1);
     if (!count(f.schur)) continue;
     pb = prof_begin(h);
-    if (count(f.lmul)) k_fr_mul<R, false><<<count(f.lmul), 256, 0, st>>>(fd, d.fr_lmul + f.lmul.ptr[l], work, fac, C);
+    if (count(f.lmul)) {
+      if constexpr (sizeof(R) == 4) {
+        launch_front_mul_tc(h, fd, false, d.fr_lmul + f.lmul.ptr[l], count(f.lmul));
+      } else {
+        k_fr_mul<R, false><<<count(f.lmul), 256, 0, st>>>(fd, d.fr_lmul + f.lmul.ptr[l], work, fac, C);
+        count_launches(1);
+      }
+    }
     prof_end(h, KC_LU_TRSM, pb, 1);
     pb = prof_begin(h);
-    k_fr_mul<R, true><<<count(f.schur), 256, 0, st>>>(fd, d.fr_schur + f.schur.ptr[l], work, fac, C);
+    if constexpr (sizeof(R) == 4) {
+      launch_front_mul_tc(h, fd, true, d.fr_schur + f.schur.ptr[l], count(f.schur));
+    } else {
+      k_fr_mul<R, true><<<count(f.schur), 256, 0, st>>>(fd, d.fr_schur + f.schur.ptr[l], work, fac, C);
+      count_launches(1);
+    }
     prof_end(h, KC_LU_UPDATE, pb, 1);
-    count_launches(2);
   }
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }

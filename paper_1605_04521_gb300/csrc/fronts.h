@@ -27,6 +27,7 @@ struct alignas(8) FrontSrc { int32_t a, b; };
 struct FrontItem { int32_t node, t; };
 
 constexpr int FR_TILE = 64;     // tile of the panel and contribution products
+constexpr int FR_TC_ROWS = 128; // and its rows on the tensor cores (FP32): item t = row tile << 16 | column tile
 constexpr int FR_ASM_ROWS = 32; // panel rows per assembly block
 constexpr int FR_FWD_ROWS = 64; // border rows per block of the forward pass
 constexpr int FR_BWD_COLS = 32; // own columns per block of the backward pass at the widest

@@ -406,8 +406,15 @@ void build_fronts(const HostMesh& m, int factor_bits, bool dirichlet, Fronts& f)
       if (n.child[0] >= 0 && n.n1 > 0)
         for (int t = 0; t * FR_ASM_ROWS < n.n1 + n.n2; ++t) f.assemble.items.push_back({g, t});
       const int ti = (n.n2 + FR_TILE - 1) / FR_TILE, tj = (n.n1 + FR_TILE - 1) / FR_TILE;
-      for (int t = 0; t < ti * tj; ++t) f.lmul.items.push_back({g, t});
-      for (int t = 0; t < ti * (ti + 1) / 2; ++t) f.schur.items.push_back({g, t});
+      if (factor_bits == 32) {
+        for (int i = 0; i * FR_TC_ROWS < n.n2; ++i) {
+          for (int j = 0; j < tj; ++j) f.lmul.items.push_back({g, i << 16 | j});
+          for (int j = 0; j < ti && j * FR_TILE < (i + 1) * FR_TC_ROWS; ++j) f.schur.items.push_back({g, i << 16 | j});
+        }
+      } else {
+        for (int t = 0; t < ti * tj; ++t) f.lmul.items.push_back({g, t});
+        for (int t = 0; t < ti * (ti + 1) / 2; ++t) f.schur.items.push_back({g, t});
+      }
       for (int t = 0; t == 0 || t * FR_FWD_ROWS < n.n2; ++t) f.fwd.items.push_back({g, t});
       for (int t = 0; t * cols < n.n1; ++t) f.bwd.items.push_back({g, t});
       for (int t = 0; t * multi < n.n1; ++t) f.bwd_multi.items.push_back({g, t});
