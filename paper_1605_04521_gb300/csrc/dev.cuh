@@ -8,8 +8,15 @@
 
 namespace oras {
 
-// complex helpers (interleaved re, im)
-template <typename R> struct CT { R re, im; };
+// complex helpers (interleaved re, im).  Aligned to the entry, so that it moves as one 8- or 16-byte word (two
+// of half the size otherwise, in shared memory with a bank conflict each).
+template <typename R> struct alignas(2 * sizeof(R)) CT { R re, im; };
+// cplx is the interface's type, aligned to a double; these move one entry of the library's own arrays.
+__device__ __forceinline__ cplx ld16(const cplx* p) {
+  const double2 t = *reinterpret_cast<const double2*>(p);
+  return {t.x, t.y};
+}
+__device__ __forceinline__ void st16(cplx* p, cplx v) { *reinterpret_cast<double2*>(p) = make_double2(v.re, v.im); }
 
 // Local-factor arena tiles: each TB x TB complex tile is two planes of TB*TB reals (real part,
 // then imaginary part).  Tiles on or below the block diagonal (I >= J) store their planes

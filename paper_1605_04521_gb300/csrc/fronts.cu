@@ -368,7 +368,11 @@ __global__ void __launch_bounds__(NW * 32 + NB, BLOCKS)
     for (int b = 0; b < CB; ++b) {
       const int i = warp + NW * a, j = lane + 32 * b;
       const bool in = i < n1 && j < n1;
-      x[a][b] = in ? src[(int64_t)i * ld + j] : CT<R>{R(i == j ? 1 : 0), R(0)};
+      x[a][b] = {R(i == j ? 1 : 0), R(0)};
+      if (in) {  // its halves by themselves, as where the block is stored: as one word the 128-wide kernel spills 376 bytes, not 136
+        const R* e = &src[(int64_t)i * ld + j].re;
+        x[a][b] = {e[0], e[1]};
+      }
       if (in) big = max(big, __float_as_uint((float)(fabs(x[a][b].re) + fabs(x[a][b].im))));
     }
   big = __reduce_max_sync(0xffffffffu, big);
@@ -385,7 +389,11 @@ __global__ void __launch_bounds__(NW * 32 + NB, BLOCKS)
 #pragma unroll
     for (int b = 0; b < CB; ++b) {
       const int j = lane + 32 * (b + rot < CB ? b + rot : b + rot - CB);
-      if (j < n1) dst[(int64_t)sh.prank[i] * ld + sh.pcol[j]] = x[a][b];
+      if (j < n1) {
+        R* out = &dst[(int64_t)sh.prank[i] * ld + sh.pcol[j]].re;
+        out[0] = x[a][b].re;
+        out[1] = x[a][b].im;
+      }
     }
     if (lane < ld - n1) dst[(int64_t)i * ld + n1 + lane] = {R(0), R(0)};
   }

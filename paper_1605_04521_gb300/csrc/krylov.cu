@@ -12,7 +12,7 @@ constexpr int RED_BLOCKS = 304;   // 2 x 152 SMs
 constexpr int RED_THREADS = 256;
 
 template <typename XT> __device__ __forceinline__ cplx ld_c(const XT* p, int64_t i);
-template <> __device__ __forceinline__ cplx ld_c<cplx>(const cplx* p, int64_t i) { return p[i]; }
+template <> __device__ __forceinline__ cplx ld_c<cplx>(const cplx* p, int64_t i) { return ld16(p + i); }
 template <> __device__ __forceinline__ cplx ld_c<CT<float>>(const CT<float>* p, int64_t i) {
   CT<float> v = p[i];
   return {(double)v.re, (double)v.im};
@@ -67,7 +67,7 @@ __global__ void __launch_bounds__(256) k_spmv(int64_t n, const int64_t* __restri
 #pragma unroll
       for (int u = 0; u < UNR; ++u) {
         const int q = min(i + u * EL, len - 1);
-        a[u] = av[q];
+        a[u] = ld16(av + q);
         c[u] = (uint32_t)cv[q];
       }
 #pragma unroll
@@ -87,7 +87,7 @@ __global__ void __launch_bounds__(256) k_spmv(int64_t n, const int64_t* __restri
     acc.re += __shfl_down_sync(0xffffffffu, acc.re, o, SPMV_LPR);
     acc.im += __shfl_down_sync(0xffffffffu, acc.im, o, SPMV_LPR);
   }
-  if (L.on && L.el == 0) y[L.row * k + L.r] = acc;
+  if (L.on && L.el == 0) st16(y + L.row * k + L.r, acc);
 }
 
 // ------------------------------------------------------------------ FP32-pipe SpMV, FP64 accuracy
@@ -134,7 +134,7 @@ __device__ __forceinline__ double f2d_bits(float f) {
 __global__ void k_split_vals(int64_t nnz, const cplx* __restrict__ vals, float4* __restrict__ out) {
   const int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (p >= nnz) return;
-  const cplx v = vals[p];
+  const cplx v = ld16(vals + p);
   const float rh = (float)v.re, ih = (float)v.im;
   out[p] = make_float4(rh, ih, (float)(v.re - (double)rh), (float)(v.im - (double)ih));
 }
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(256) k_spmv_df(int64_t n, const int64_t* __res
     df_add(rh, rl, h2, l2);
     df_add(ih, il, h3, l3);
   }
-  if (L.on && L.el == 0) y[L.row * k + L.r] = {f2d_bits(rh) + f2d_bits(rl), f2d_bits(ih) + f2d_bits(il)};
+  if (L.on && L.el == 0) st16(y + L.row * k + L.r, {f2d_bits(rh) + f2d_bits(rl), f2d_bits(ih) + f2d_bits(il)});
 }
 
 // Reductions over [N][k] multi-vectors (element e belongs to right-hand side e % k).  The grid's
@@ -292,12 +292,12 @@ __global__ void __launch_bounds__(RED_THREADS) k_mgs_block(int64_t nk, int k, in
 #pragma unroll
     for (int q = 0; q < MGS_BLOCK; ++q) h[q] = q < nv ? hs[q * k + t % k] : cplx{0.0, 0.0};
     for (int64_t e = t; e < nk; e += teff) {
-      cplx x = w[e];
+      cplx x = ld16(w + e);
       cplx u[MGS_BLOCK];
       if (nv > 0) {
 #pragma unroll
         for (int q = 0; q < MGS_BLOCK; ++q)
-          if (q < nv) u[q] = V[q * nk + e];
+          if (q < nv) u[q] = ld16(V + q * nk + e);
 #pragma unroll
         for (int q = 0; q < MGS_BLOCK; ++q)
           if (q < nv) {
@@ -306,12 +306,12 @@ __global__ void __launch_bounds__(RED_THREADS) k_mgs_block(int64_t nk, int k, in
             x.re = fma(h[q].im, u[q].im, x.re);
             x.im = fma(-h[q].im, u[q].re, x.im);
           }
-        w[e] = x;
+        st16(w + e, x);
       }
       if (nn > 0) {
 #pragma unroll
         for (int q = 0; q < MGS_BLOCK; ++q)
-          if (q < nn) u[q] = Vn[q * nk + e];
+          if (q < nn) u[q] = ld16(Vn + q * nk + e);
 #pragma unroll
         for (int q = 0; q < MGS_BLOCK; ++q)
           if (q < nn) {
@@ -345,8 +345,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_mgs_finish(int64_t nk, int k, i
     if (t >= teff) return;
     const double h = sqrt(hs[t % k].re), inv = h > 0.0 ? 1.0 / h : 0.0;
     for (int64_t e = t; e < nk; e += teff) {
-      const cplx x = w[e];
-      Vn[e] = h > 0.0 ? cplx{x.re * inv, x.im * inv} : cplx{0.0, 0.0};
+      const cplx x = ld16(w + e);
+      st16(Vn + e, h > 0.0 ? cplx{x.re * inv, x.im * inv} : cplx{0.0, 0.0});
     }
     return;
   }
@@ -413,7 +413,7 @@ __global__ void k_xupdate(int64_t nk, int k, int m, int kk, const ZT* __restrict
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= nk) return;
   int r = (int)(e % k);
-  cplx acc = x[e];
+  cplx acc = ld16(x + e);
   for (int q = 0; q < kk; ++q) {
     const cplx c = y[(int64_t)r * m + q], v = ld_c<ZT>(Z, (int64_t)q * nk + e);
     acc.re = fma(c.re, v.re, acc.re);
@@ -421,7 +421,7 @@ __global__ void k_xupdate(int64_t nk, int k, int m, int kk, const ZT* __restrict
     acc.re = fma(-c.im, v.im, acc.re);
     acc.im = fma(c.im, v.re, acc.im);
   }
-  x[e] = acc;
+  st16(x + e, acc);
 }
 
 // r = b - A x (SpMV output in r already holds A x): r = b - r; partial |r|^2
@@ -431,8 +431,8 @@ __global__ void __launch_bounds__(RED_THREADS) k_residual(int64_t nk, int k, con
   cplx acc[1] = {{0.0, 0.0}};
   if (t < teff)
     for (int64_t e = t; e < nk; e += teff) {
-      const cplx v = csub(b[e], r[e]);
-      r[e] = v;
+      const cplx v = csub(ld16(b + e), ld16(r + e));
+      st16(r + e, v);
       acc[0].re = fma(v.re, v.re, acc[0].re);
       acc[0].re = fma(v.im, v.im, acc[0].re);
     }
@@ -469,7 +469,7 @@ __global__ void k_to_internal(int64_t n, int k, const cplx* __restrict__ src, cp
   if (e >= n * k) return;
   int64_t g = e / k;
   int r = (int)(e % k);
-  dst[e] = src[(int64_t)r * n + g];
+  st16(dst + e, ld16(src + (int64_t)r * n + g));
 }
 __global__ void k_to_internal_c64(int64_t n, int k, const CT<float>* __restrict__ src, CT<float>* __restrict__ dst) {
   int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -481,7 +481,7 @@ __global__ void k_to_external(int64_t n, int k, const cplx* __restrict__ src, cp
   if (e >= n * k) return;
   int64_t g = e / k;
   int r = (int)(e % k);
-  dst[(int64_t)r * n + g] = src[e];
+  st16(dst + (int64_t)r * n + g, ld16(src + e));
 }
 
 // ------------------------------------------------------------------ launchers
