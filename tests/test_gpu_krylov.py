@@ -68,3 +68,37 @@ def test_blocked_orthogonalisation_in_the_solve(setup, k):
             continue
         assert np.linalg.norm(B[:, j] - p.A @ X[:, j]) <= 1e-8 * np.linalg.norm(B[:, j])
     assert max(i["iterations"] for i in info) > 16
+
+
+@pytest.mark.parametrize("k", [1, 3])
+@pytest.mark.parametrize("place", ["plain", "onto_input", "half_entry", "pinned"])
+def test_device_vectors_wherever_they_are(setup, k, place):
+    """Products of vectors given as device memory, which are read and written where they are when a kernel can and
+    through a copy otherwise: the result on top of the input, both half an entry off their alignment, pinned host
+    memory."""
+    import ctypes
+    import torch
+    O, h, p = setup
+    n = p.A.shape[0]
+    rng = np.random.default_rng(300 + k)
+    X = rng.normal(size=(k, n)) + 1j * rng.normal(size=(k, n))
+    for wide in (True, False):
+        Z = X if wide else X.astype(np.complex64)
+        R = (p.A @ Z.T.astype(np.complex128)).T
+        real = torch.from_numpy(np.ascontiguousarray(Z).view(Z.real.dtype).ravel().copy())
+        off = 1 if place == "half_entry" else 0
+        size = 2 * k * n * (2 if not wide else 1) + off        # room for the complex128 result on top of it
+        src = torch.zeros(size, dtype=real.dtype, device="cpu" if place == "pinned" else "cuda")
+        src[off:off + len(real)] = real
+        dst = torch.zeros(2 * k * n + off, dtype=torch.float64, device=src.device)
+        if place == "pinned":
+            src, dst = src.pin_memory(), dst.pin_memory()
+        if place == "onto_input":
+            dst = src.view(torch.float64)
+        at = lambda t: ctypes.c_void_p(t.data_ptr() + off * t.element_size())  # noqa: E731
+        torch.cuda.synchronize()
+        fn = O.lib.oras_matvec if wide else O.lib.oras_matvec_c64
+        assert fn(h, at(src), at(dst), k, O.ORAS_MEM_DEVICE) == O.ORAS_OK
+        torch.cuda.synchronize()
+        Y = dst[off:off + 2 * k * n].cpu().numpy().view(np.complex128).reshape(k, n)
+        assert rel(Y, R) <= 1e-13
