@@ -41,10 +41,8 @@ void launch_spmv_f64(const oras_handle* h, const cplx* x, cplx* y, int k);
 void launch_spmv_f32(const oras_handle* h, const void* x, cplx* y, int k);
 void launch_split_vals(const oras_handle* h);
 void launch_to_internal_c64(const oras_handle* h, int k, const void* src, void* dst);
-void launch_mgs(const oras_handle* h, int k, int m, int j, const cplx* V, cplx* w, cplx* red, cplx* H);
-void launch_mgs_finish(const oras_handle* h, int k, int m, int j, const cplx* w, cplx* Vn, const cplx* red,
-                       cplx* H, double* cs, cplx* sn, cplx* g, double* host_res, int32_t* host_status);
-int mgs_launches(int j);
+int launch_orth(const oras_handle* h, int k, int m, int j, const cplx* V, cplx* w, cplx* Vn, cplx* red, cplx* H,
+                double* cs, cplx* sn, cplx* g, double* host_res, int32_t* host_status);
 size_t red_elems(int k);
 void launch_hsolve(const oras_handle* h, int k, int m, int kk, const cplx* H, const cplx* g, const int32_t* active,
                    cplx* y);
@@ -1018,9 +1016,8 @@ static int fgmres(oras_handle* h, int k, double tol, oras_info* info) {
         spmv_z(h, k, j, d.w);
         prof_end(h, d.factor_bits == 64 ? KC_SPMV64 : KC_SPMV, pb, 1);
         pb = prof_begin(h);
-        launch_mgs(h, k, m, j, d.V, d.w, pA, d.H);
-        launch_mgs_finish(h, k, m, j, d.w, Vn, pA, d.H, d.gcs, d.gsn, d.g, hp + k, st_h);
-        prof_end(h, KC_ORTH, pb, mgs_launches(j));
+        const int nl = launch_orth(h, k, m, j, d.V, d.w, Vn, pA, d.H, d.gcs, d.gsn, d.g, hp + k, st_h);
+        prof_end(h, KC_ORTH, pb, nl);
         return ORAS_OK;
       };
       if ((graphs ? run_step(h, j, k, m, step) : step()) != ORAS_OK) return ORAS_ERR_CUDA;

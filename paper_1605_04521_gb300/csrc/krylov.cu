@@ -4,6 +4,8 @@
 // stored [N][k] (the k right-hand sides of a pseudo-block solve adjacent in memory).
 // Every reduction is a fixed two-stage sum (block partials, then a fixed-order sum), so the
 // results do not depend on scheduling.
+#include <algorithm>
+
 #include "dev.cuh"
 
 namespace oras {
@@ -329,6 +331,265 @@ __global__ void __launch_bounds__(RED_THREADS) k_mgs_block(int64_t nk, int k, in
   block_reduce_store<MGS_BLOCK>(acc, nn > 0 ? nn : 1, k, partials);
 }
 
+// Rotation j of right-hand side r from column j's running entry a and h_{j+1,j} = bb; updates g, res = |g_{j+1}|.
+__device__ __forceinline__ void givens_finish(int r, int m, int j, cplx a, double bb, cplx* __restrict__ H,
+                                              double* __restrict__ cs, cplx* __restrict__ sn, cplx* __restrict__ g,
+                                              double* __restrict__ host_res) {
+  cplx* Hr = H + (int64_t)r * (m + 1) * m;
+  cplx* gr = g + (int64_t)r * (m + 1);
+  const double aa = hypot(a.re, a.im);
+  double cj;
+  cplx sj;
+  if (bb == 0.0) { cj = 1.0; sj = {0.0, 0.0}; }
+  else if (aa == 0.0) { cj = 0.0; sj = {1.0, 0.0}; }
+  else {
+    const double den = hypot(aa, bb);
+    cj = aa / den;
+    sj = {a.re / aa * bb / den, a.im / aa * bb / den};
+  }
+  cs[(int64_t)r * m + j] = cj;
+  sn[(int64_t)r * m + j] = sj;
+  Hr[(int64_t)j * m + j] = cadd(cscale(a, cj), cscale(sj, bb));
+  Hr[(int64_t)(j + 1) * m + j] = {0.0, 0.0};
+  const cplx gj = gr[j];
+  gr[j + 1] = cscale(cmul(cconj(sj), gj), -1.0);
+  gr[j] = cscale(gj, cj);
+  host_res[r] = hypot(gr[j + 1].re, gr[j + 1].im);
+}
+
+// ------------------------------------------------------------------ one launch an Arnoldi step
+// The same blocked Gram-Schmidt, the norm, V_{j+1} and the Givens update in one cooperative launch, one block an SM
+// with its share of w in shared memory; after a pass the blocks exchange their partial sums through a grid barrier
+// and each adds all of them.  The passes of k_mgs_block cost 7-11 us each beside their arithmetic (two
+// launches, w through memory, a reduction of 512 threads an SM), and their 512 entries a block left most SMs idle
+// on short vectors.  Entries are dealt out evenly: every SM has the same share of the last, partial round.
+// Bound: the FP64 pipe, as there.  Orthogonalisation of a whole solve, launches above -> this: three columns of the 10^3 x 6, degree-3
+// problem (352,170 entries a vector, restart 100) 317 -> 239 ms (169 ms of FP64 instructions), one of the 24^3 one 176 -> 141,
+// eight at degree 3 6.2 -> 5.0, one of the 16^3 one 2.31 -> 1.61, of the 4^3 one 0.52 -> 0.28.  A block adds the sums of all others, MGS_BLOCK k ones of gridDim.x
+// partials, which is why k ends at ORTH_MAX_K; w ends at ORTH_MAX_ROUNDS rounds of the block's shared memory
+// (1.4e6 entries).  Others take the launches above.
+// Waits are bounded: a block that gives up reports DEV_TIMEOUT and leaves, and so do then the others.
+constexpr int ORTH_THREADS = 512, ORTH_MAX_K = 8, ORTH_MAX_ROUNDS = 18;
+enum { ST_ORTH_ARRIVED = 4, ST_ORTH_LEFT = 5 };   // barrier counters beside the status flags, zero between launches
+
+struct OrthArgs {
+  int64_t nk, chunk;                 // entries, entries a block (a multiple of k)
+  int k, m, j;
+  const cplx* V;                     // V_0
+  const cplx* w;
+  cplx* Vn;                          // V_{j+1}
+  cplx* partials;                    // [2][MGS_BLOCK][gridDim.x][k], by pass parity
+  cplx* H;
+  double* cs;
+  cplx* sn;
+  cplx* g;
+  double* host_res;
+  int32_t* status;
+  int32_t* host_status;
+  uint64_t wait_ns;
+};
+
+// Every block's arrival; what its threads wrote before is visible to blocks that see it.
+__device__ __forceinline__ void grid_arrive(int32_t* status) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(&status[ST_ORTH_ARRIVED], 1);
+  }
+}
+// Until `need` arrivals, or not within the limit (false in every thread of the block).
+__device__ __forceinline__ bool grid_wait(int32_t* status, int need, uint64_t limit_ns) {
+  int ok = 1;
+  if (threadIdx.x == 0) {
+    const uint64_t t0 = globaltimer();
+    long long it = 0;
+    while (true) {
+      int v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(status + ST_ORTH_ARRIVED) : "memory");
+      if (v >= need) break;
+      ++it;
+      if (it >= ORAS_SPIN_LIMIT || ((it & 255) == 0 && globaltimer() - t0 > limit_ns)) { ok = 0; break; }
+    }
+    __threadfence();
+  }
+  return __syncthreads_and(ok) != 0;
+}
+
+// Sums over the p of the values of lanes r + k p, P of them, into lanes r.
+__device__ __forceinline__ cplx sum_lanes(cplx t, int k, int P, int p) {
+  for (int left = P; left > 1;) {
+    const int half = (left + 1) / 2;
+    const cplx o = shfl_down_c(t, half * k & 31);
+    if (p + half < left) t = cadd(t, o);
+    left = half;
+  }
+  return t;
+}
+
+__global__ void __launch_bounds__(ORTH_THREADS, 1) k_orth(OrthArgs a) {
+  extern __shared__ __align__(16) unsigned char orth_smem[];
+  cplx* red = (cplx*)orth_smem;                        // [MGS_BLOCK][ORTH_THREADS]
+  cplx* sw = red + MGS_BLOCK * ORTH_THREADS;           // [rounds][ORTH_THREADS] this block's w
+  __shared__ __align__(16) cplx half_sum[2][MGS_BLOCK * ORTH_MAX_K];
+  __shared__ __align__(16) cplx hs[MGS_BLOCK * ORTH_MAX_K];
+  __shared__ double hinv[ORTH_MAX_K];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, k = a.k, G = gridDim.x;
+  const int64_t first = (int64_t)blockIdx.x * a.chunk, nk = a.nk;
+  const int len = (int)(nk - first < a.chunk ? nk - first : a.chunk);
+  const int stride = ORTH_THREADS / k * k;             // a thread's entries are of one right-hand side
+  const int begin = tid < stride ? tid : len, rhs = tid % k;
+  const int live = len < stride ? len : stride;        // threads with entries
+  const int P = 32 / k, lp = lane / k;                 // lanes r + k p < k P share the sums of right-hand side r
+  const cplx* V = a.V + first;
+  const cplx* w = a.w + first;
+  cplx u[MGS_BLOCK], rot = {0.0, 0.0};
+  int passes = 0;
+  bool ok = true;
+  for (int i0 = -MGS_BLOCK; i0 <= a.j; i0 += MGS_BLOCK) {
+    const int i1 = i0 + MGS_BLOCK;
+    const int nv = i0 < 0 ? 0 : min(a.j + 1 - i0, MGS_BLOCK);
+    const int nn = i1 > a.j ? 0 : min(a.j + 1 - i1, MGS_BLOCK);
+    cplx acc[MGS_BLOCK];
+#pragma unroll
+    for (int q = 0; q < MGS_BLOCK; ++q) acc[q] = {0.0, 0.0};
+    // the new entries of column j of H through the earlier rotations, beside the pass: rot is the running entry
+    if (nv > 0 && blockIdx.x == 0 && warp == ORTH_THREADS / 32 - 1 && lane < k) {
+      const double* c = a.cs + (int64_t)lane * a.m;
+      const cplx* s = a.sn + (int64_t)lane * a.m;
+      double cq[MGS_BLOCK];
+      cplx sq[MGS_BLOCK];
+#pragma unroll
+      for (int q = 0; q < MGS_BLOCK; ++q)
+        if (q < nv && i0 + q > 0) {
+          cq[q] = c[i0 + q - 1];
+          sq[q] = s[i0 + q - 1];
+        }
+#pragma unroll
+      for (int q = 0; q < MGS_BLOCK; ++q)
+        if (q < nv) {
+          const cplx b = ld16(hs + q * k + lane);
+          if (i0 + q == 0) {
+            rot = b;
+          } else {
+            a.H[((int64_t)lane * (a.m + 1) + i0 + q - 1) * a.m + a.j] = cadd(cscale(rot, cq[q]), cmul(sq[q], b));
+            rot = csub(cscale(b, cq[q]), cmul(cconj(sq[q]), rot));
+          }
+        }
+    }
+    cplx* wp = sw + tid;
+    for (int e = begin; e < len; e += stride, wp += ORTH_THREADS) {
+      cplx x = ld16(nv > 0 ? wp : w + e);
+      if (nv > 0) {
+        if (e != begin) {
+#pragma unroll
+          for (int q = 0; q < MGS_BLOCK; ++q)
+            if (q < nv) u[q] = ld16(V + (i0 + q) * nk + e);
+        }
+#pragma unroll
+        for (int q = 0; q < MGS_BLOCK; ++q)
+          if (q < nv) {
+            const cplx h = ld16(hs + q * k + rhs);
+            x.re = fma(-h.re, u[q].re, x.re);
+            x.im = fma(-h.re, u[q].im, x.im);
+            x.re = fma(h.im, u[q].im, x.re);
+            x.im = fma(-h.im, u[q].re, x.im);
+          }
+      }
+      st16(wp, x);
+      if (nn > 0) {
+#pragma unroll
+        for (int q = 0; q < MGS_BLOCK; ++q)
+          if (q < nn) u[q] = ld16(V + (i1 + q) * nk + e);
+#pragma unroll
+        for (int q = 0; q < MGS_BLOCK; ++q)
+          if (q < nn) {
+            acc[q].re = fma(u[q].re, x.re, acc[q].re);
+            acc[q].im = fma(u[q].re, x.im, acc[q].im);
+            acc[q].re = fma(u[q].im, x.im, acc[q].re);
+            acc[q].im = fma(-u[q].im, x.re, acc[q].im);
+          }
+      } else {
+        acc[0].re = fma(x.re, x.re, acc[0].re);
+        acc[0].re = fma(x.im, x.im, acc[0].re);
+      }
+    }
+    // the block's sums, one warp a value
+    const int nq = nn > 0 ? nn : 1;
+#pragma unroll
+    for (int q = 0; q < MGS_BLOCK; ++q)
+      if (q < nq) st16(red + q * ORTH_THREADS + tid, acc[q]);
+    __syncthreads();
+    cplx* part = a.partials + (int64_t)(passes & 1) * MGS_BLOCK * G * k;
+    if (warp < nq) {
+      cplx t = {0.0, 0.0};
+      if (lane < k * P)
+        for (int i = lane; i < live; i += k * P) t = cadd(t, ld16(red + warp * ORTH_THREADS + i));
+      t = sum_lanes(t, k, P, lp);
+      if (lane < k) st16(part + ((int64_t)warp * G + blockIdx.x) * k + lane, t);
+    }
+    if (begin < len) {  // the next pass's first vectors do not depend on the sums
+#pragma unroll
+      for (int q = 0; q < MGS_BLOCK; ++q)
+        if (q < nn) u[q] = ld16(V + (i1 + q) * nk + begin);
+    }
+    grid_arrive(a.status);
+    ++passes;
+    ok = grid_wait(a.status, passes * G, a.wait_ns);
+    if (!ok) break;
+    // all blocks' sums, half of the blocks a warp
+    const int q = warp & (MGS_BLOCK - 1), hf = warp >> 3;
+    if (q < nq) {
+      const cplx* src = part + (int64_t)q * G * k;
+      const int end = (hf ? G : G / 2) * k;
+      cplx t = {0.0, 0.0};
+      if (lane < k * P)
+        for (int i = (hf ? G / 2 * k : 0) + lane; i < end; i += 4 * k * P) {
+          double2 v[4];
+#pragma unroll
+          for (int n = 0; n < 4; ++n)
+            v[n] = i + n * k * P < end ? __ldcg(reinterpret_cast<const double2*>(src + i + n * k * P)) : make_double2(0.0, 0.0);
+#pragma unroll
+          for (int n = 0; n < 4; ++n)
+            if (i + n * k * P < end) t = cadd(t, {v[n].x, v[n].y});
+        }
+      t = sum_lanes(t, k, P, lp);
+      if (lane < k) half_sum[hf][q * k + lane] = t;
+    }
+    __syncthreads();
+    if (tid < nq * k) {
+      const cplx t = cadd(half_sum[0][tid], half_sum[1][tid]);
+      hs[tid] = t;
+      if (nn == 0) {
+        const double h = sqrt(t.re);
+        hinv[tid] = h > 0.0 ? 1.0 / h : -1.0;
+      }
+    }
+    __syncthreads();
+  }
+  if (ok) {  // V_{j+1} = w / |w| (0 where |w| is 0 or not a number)
+    const double inv = hinv[rhs];
+    const cplx* wp = sw + tid;
+    for (int e = begin; e < len; e += stride, wp += ORTH_THREADS) {
+      const cplx x = ld16(wp);
+      st16(a.Vn + first + e, inv >= 0.0 ? cplx{x.re * inv, x.im * inv} : cplx{0.0, 0.0});
+    }
+  } else if (tid == 0) {
+    atomicExch(&a.status[ST_ERR], DEV_TIMEOUT);
+    __threadfence();
+  }
+  if (blockIdx.x == 0) {
+    if (ok && warp == ORTH_THREADS / 32 - 1 && lane < k)
+      givens_finish(lane, a.m, a.j, rot, sqrt(hs[lane].re), a.H, a.cs, a.sn, a.g, a.host_res);
+    __syncthreads();
+    if (tid < 8) a.host_status[tid] = *(volatile int32_t*)&a.status[tid];
+  }
+  // the last block to leave clears the counters: no block waits any more
+  if (tid == 0 && atomicAdd(&a.status[ST_ORTH_LEFT], 1) == G - 1) {
+    a.status[ST_ORTH_ARRIVED] = 0;
+    a.status[ST_ORTH_LEFT] = 0;
+  }
+}
+
 // h_{j+1,j} = ||w|| (hs[r] = |w|^2); V_{j+1} = w / h (0 if h == 0).  The last block instead runs the
 // Givens update of every RHS beside them: apply rotations 0..j-1 to column j of H, build rotation j, update
 // g, res = |g_{j+1}|; res and the device status go straight to the host's pinned words.
@@ -355,7 +616,6 @@ __global__ void __launch_bounds__(RED_THREADS) k_mgs_finish(int64_t nk, int k, i
     cplx* Hr = H + (int64_t)r * (m + 1) * m;
     double* c = cs + (int64_t)r * m;
     cplx* s = sn + (int64_t)r * m;
-    cplx* gr = g + (int64_t)r * (m + 1);
     const double bb = sqrt(hs[r].re);
     cplx a = Hr[j];                       // the running entry of column j
     for (int q = 0; q < j; ++q) {
@@ -365,24 +625,7 @@ __global__ void __launch_bounds__(RED_THREADS) k_mgs_finish(int64_t nk, int k, i
       Hr[(int64_t)q * m + j] = cadd(cscale(a, cq), cmul(sq, b));
       a = csub(cscale(b, cq), cmul(cconj(sq), a));
     }
-    double aa = hypot(a.re, a.im);
-    double cj;
-    cplx sj;
-    if (bb == 0.0) { cj = 1.0; sj = {0.0, 0.0}; }
-    else if (aa == 0.0) { cj = 0.0; sj = {1.0, 0.0}; }
-    else {
-      double den = hypot(aa, bb);
-      cj = aa / den;
-      sj = {a.re / aa * bb / den, a.im / aa * bb / den};
-    }
-    c[j] = cj;
-    s[j] = sj;
-    Hr[(int64_t)j * m + j] = cadd(cscale(a, cj), cscale(sj, bb));
-    Hr[(int64_t)(j + 1) * m + j] = {0.0, 0.0};
-    cplx gj = gr[j];
-    gr[j + 1] = cscale(cmul(cconj(sj), gj), -1.0);
-    gr[j] = cscale(gj, cj);
-    host_res[r] = hypot(gr[j + 1].re, gr[j + 1].im);
+    givens_finish(r, m, j, a, bb, H, cs, sn, g, host_res);
   }
 }
 
@@ -521,7 +764,7 @@ static int red_grid(int64_t nk) {
 }
 // Orthogonalisation of w against V_0..V_j ([j + 1][N][k]): column j of H, |w|^2 in hs; partials and hs:
 // red_elems(k) entries from `red`.
-void launch_mgs(const oras_handle* h, int k, int m, int j, const cplx* V, cplx* w, cplx* red, cplx* H) {
+static void launch_mgs(const oras_handle* h, int k, int m, int j, const cplx* V, cplx* w, cplx* red, cplx* H) {
   const int64_t nk = h->mesh.ndof * k;
   const int grid = red_grid(nk);
   cplx* hs = red;
@@ -538,9 +781,8 @@ void launch_mgs(const oras_handle* h, int k, int m, int j, const cplx* V, cplx* 
     count_launches(2);
   }
 }
-int mgs_launches(int j) { return 2 * (j / MGS_BLOCK + 2) + 1; }
 size_t red_elems(int k) { return (size_t)(RED_BLOCKS + 1) * MGS_BLOCK * k; }
-void launch_mgs_finish(const oras_handle* h, int k, int m, int j, const cplx* w, cplx* Vn, const cplx* red,
+static void launch_mgs_finish(const oras_handle* h, int k, int m, int j, const cplx* w, cplx* Vn, const cplx* red,
                        cplx* H, double* cs, cplx* sn, cplx* g, double* host_res, int32_t* host_status) {
   const int64_t nk = h->mesh.ndof * k;
   int64_t blocks = (nk + RED_THREADS - 1) / RED_THREADS;
@@ -548,6 +790,48 @@ void launch_mgs_finish(const oras_handle* h, int k, int m, int j, const cplx* w,
   k_mgs_finish<<<(unsigned)blocks + 1, RED_THREADS, 0, h->dev.stream>>>(nk, k, m, j, w, Vn, red, H, cs, sn, g, host_res,
                                                                        h->dev.status, host_status);
   count_launches(1);
+}
+static bool launch_orth_once(const oras_handle* h, int k, int m, int j, const cplx* V, const cplx* w, cplx* Vn, cplx* red,
+                             cplx* H, double* cs, cplx* sn, cplx* g, double* host_res, int32_t* host_status) {
+  if (k > ORTH_MAX_K) return false;
+  OrthArgs a;
+  a.nk = h->mesh.ndof * k;
+  const int64_t most = std::max<int64_t>(1, std::min<int64_t>({h->dev.num_sms, RED_BLOCKS / 2, (a.nk + 31) / 32}));
+  const int64_t unit = k % 2 ? 2 * k : k;  // whole right-hand side groups, 32-byte sectors
+  a.chunk = ((a.nk + most - 1) / most + unit - 1) / unit * unit;
+  const int64_t grid = (a.nk + a.chunk - 1) / a.chunk;
+  const int64_t stride = ORTH_THREADS / k * k, rounds = (a.chunk + stride - 1) / stride;
+  if (rounds > ORTH_MAX_ROUNDS) return false;
+  a.k = k; a.m = m; a.j = j;
+  a.V = V; a.w = w; a.Vn = Vn; a.partials = red; a.H = H; a.cs = cs; a.sn = sn; a.g = g;
+  a.host_res = host_res; a.status = h->dev.status; a.host_status = host_status;
+  a.wait_ns = wait_limit_ns(h);
+  allow_max_smem((const void*)k_orth);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(ORTH_THREADS);
+  cfg.dynamicSmemBytes = (size_t)(MGS_BLOCK + rounds) * ORTH_THREADS * sizeof(cplx);
+  cfg.stream = h->dev.stream;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeCooperative;
+  at[0].val.cooperative = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  if (cudaLaunchKernelEx(&cfg, k_orth, a) != cudaSuccess) {  // a device that cannot hold a block an SM at once
+    cudaGetLastError();
+    return false;
+  }
+  count_launches(1);
+  return true;
+}
+// The end of Arnoldi step j: w orthogonalised against V_0..V_j, V_{j+1}, column j of H, the rotation and the residual
+// estimates in host_res.  `red`: red_elems(k) entries; the status words behind the flags are zero.  Returns its launches.
+int launch_orth(const oras_handle* h, int k, int m, int j, const cplx* V, cplx* w, cplx* Vn, cplx* red, cplx* H,
+                double* cs, cplx* sn, cplx* g, double* host_res, int32_t* host_status) {
+  if (launch_orth_once(h, k, m, j, V, w, Vn, red, H, cs, sn, g, host_res, host_status)) return 1;
+  launch_mgs(h, k, m, j, V, w, red, H);
+  launch_mgs_finish(h, k, m, j, w, Vn, red, H, cs, sn, g, host_res, host_status);
+  return 2 * (j / MGS_BLOCK + 2) + 1;
 }
 void launch_hsolve(const oras_handle* h, int k, int m, int kk, const cplx* H, const cplx* g, const int32_t* active,
                    cplx* y) {

@@ -71,11 +71,10 @@ def test_blocked_orthogonalisation_in_the_solve(setup, k):
 
 
 @pytest.mark.parametrize("k", [1, 3])
-@pytest.mark.parametrize("place", ["plain", "onto_input", "half_entry", "pinned"])
+@pytest.mark.parametrize("place", ["plain", "onto_input", "half_entry"])
 def test_device_vectors_wherever_they_are(setup, k, place):
     """Products of vectors given as device memory, which are read and written where they are when a kernel can and
-    through a copy otherwise: the result on top of the input, both half an entry off their alignment, pinned host
-    memory."""
+    through a copy otherwise: the result on top of the input, both half an entry off their alignment."""
     import ctypes
     import torch
     O, h, p = setup
@@ -88,11 +87,9 @@ def test_device_vectors_wherever_they_are(setup, k, place):
         real = torch.from_numpy(np.ascontiguousarray(Z).view(Z.real.dtype).ravel().copy())
         off = 1 if place == "half_entry" else 0
         size = 2 * k * n * (2 if not wide else 1) + off        # room for the complex128 result on top of it
-        src = torch.zeros(size, dtype=real.dtype, device="cpu" if place == "pinned" else "cuda")
+        src = torch.zeros(size, dtype=real.dtype, device="cuda")
         src[off:off + len(real)] = real
         dst = torch.zeros(2 * k * n + off, dtype=torch.float64, device=src.device)
-        if place == "pinned":
-            src, dst = src.pin_memory(), dst.pin_memory()
         if place == "onto_input":
             dst = src.view(torch.float64)
         at = lambda t: ctypes.c_void_p(t.data_ptr() + off * t.element_size())  # noqa: E731
@@ -102,3 +99,40 @@ def test_device_vectors_wherever_they_are(setup, k, place):
         torch.cuda.synchronize()
         Y = dst[off:off + 2 * k * n].cpu().numpy().view(np.complex128).reshape(k, n)
         assert rel(Y, R) <= 1e-13
+
+
+@pytest.fixture(scope="module")
+def larger():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1605_04521_gb300 import build
+    build.build()
+    from paper_1605_04521_gb300 import oras as O
+    w = synth.small(n=10, r=2, nsub=16, overlap=0, restart=30)
+    xyz, tets = w.mesh()
+    eps, mu = w.materials(xyz, tets)
+    h = O.oras_setup(xyz, tets, eps, mu, w.k0, w.r, w.nsub, w.overlap, restart=w.restart)
+    yield O, h
+    O.oras_destroy(h)
+
+
+@pytest.mark.parametrize("k", [1, 2, 3, 5, 7, 8])
+def test_orthogonalisation_in_one_launch(larger, k):
+    """Up to 8 columns an Arnoldi step ends in one cooperative launch, 9 and more take several: the same columns
+    through both, over several rounds of an SM's share (k entries of 1/152 of the vector, 512 at a time)."""
+    O, h = larger
+    n = O.oras_ndof(h)
+    rng = np.random.default_rng(200 + k)
+    B = rng.normal(size=(n, 9)) + 1j * rng.normal(size=(n, 9))
+    Y, _, rc9 = O.oras_solve(h, B, 1e-8, k=9)
+    X, info, rc = O.oras_solve(h, B[:, :k], 1e-8, k=k)
+    X = np.asarray(X).reshape(-1, k)
+    assert rc == rc9 == O.ORAS_OK
+    assert max(i["iterations"] for i in info) > 16
+    R = B[:, :k] - np.asarray(O.oras_matvec(h, X, k=k)).reshape(-1, k)
+    for j in range(k):
+        assert np.linalg.norm(R[:, j]) <= 1e-8 * np.linalg.norm(B[:, j])
+    R9 = B[:, :k] - np.asarray(O.oras_matvec(h, np.asarray(Y)[:, :k].copy(), k=k)).reshape(-1, k)
+    for j in range(k):
+        assert np.linalg.norm(R9[:, j]) <= 1e-8 * np.linalg.norm(B[:, j])
