@@ -16,7 +16,10 @@
 // where a level has few nodes.  ms an apply, before -> with these: 16^3 1.29 -> 0.81 (3.2 GB: 58% of the copy
 // rate), 24^3 with 512 subdomains 0.54 -> 0.38, 8^3 0.24 -> 0.086.
 // 5 and more right-hand sides (k_fr_fwd_multi, k_fr_bwd_multi): up to 32 a pass as small matrix products, bound
-// by the FP32 pipes: 32 columns of the 16^3 128-subdomain problem 5.2 -> 2.2 ms (four passes of 8 before).
+// by the FP32 pipes at 32 and by the latency of a block at 8: 32 columns of the 16^3 128-subdomain problem 5.2 -> 2.2 ms
+// (four passes of 8 before).  With panels copied in the background, all of L before the wait and a ring of four stages
+// backward, instead of one stage ahead through registers: 8 columns of the 9^3 x 6, degree-3 problem 1.11 -> 0.82 ms
+// an apply (1.5 GB), of the 10^3 one with ports 0.37 -> 0.27 ms, 32 columns as before.
 #include <algorithm>
 
 #include "apply.cuh"
@@ -277,28 +280,27 @@ __global__ void __launch_bounds__(FR_THREADS) k_fr_bwd(FrApply a, const FrontIte
 
 // ------------------------------------------------------------------ many right-hand sides (FP32)
 // Products of a tile of JT rows with KR = 8, 16 or 32 right-hand sides: 4 x TC entries a thread; the threads left
-// over split the sum (SG groups, added at the end in a fixed order), so a block keeps KC = 16 SG sum indices in
-// flight a stage -- the sums run up to a thousand long on levels with few nodes, where a stage's load latency is
-// the cost and the tiles are narrower (Fronts::multi_cols: below 200 tiles of 64; 16 wide they take 28 us where 64
-// wide ones take 48, but twice as long on levels that fill the chip).
+// over split the sum (SG groups, added at the end in a fixed order).  On levels with few nodes, where the sums run up
+// to a thousand long, the tiles are narrower (Fronts::multi_cols: below 200 tiles of 64; 16 wide they take 28 us where
+// 64 wide ones take 48, but twice as long on levels that fill the chip).
 template <int KR, int JT> struct FrTile {
   static constexpr int TR = 4, TC = KR == 16 ? 4 : 2;         // entries a thread
   static constexpr int CG = KR / TC, RG = JT / TR;            // column and row groups
   static constexpr int SG = FR_THREADS / (CG * RG);           // sum groups
-  static constexpr int KC = 16 * SG;                          // sum indices a stage
+  static constexpr int KS = SG > 1 ? 8 : 16, KC = KS * SG;     // sum indices a stage, of a group and of all
   static_assert(CG * RG * SG == FR_THREADS, "threads");
 };
 
-// acc += the products of sum group sg over one stage: As [KC][LDA], Bs [KC][KR].
-template <int KR, int JT, int LDA>
+// acc += the products of sum group sg over one stage: As [KC][JT], Bs [KC][KR].
+template <int KR, int JT>
 __device__ __forceinline__ void tile_stage(CT<float> (&acc)[FrTile<KR, JT>::TR][FrTile<KR, JT>::TC], const CT<float>* As,
                                            const CT<float>* Bs, int sg, int rg, int cg) {
   using T = FrTile<KR, JT>;
 #pragma unroll
-  for (int k = 0; k < 16; ++k) {
+  for (int k = 0; k < T::KS; ++k) {
     CT<float> av[T::TR], bv[T::TC];
-    const CT<float>* pa = As + (sg * 16 + k) * LDA + rg * T::TR;
-    const CT<float>* pb = Bs + (sg * 16 + k) * KR + cg * T::TC;
+    const CT<float>* pa = As + (sg * T::KS + k) * JT + rg * T::TR;
+    const CT<float>* pb = Bs + (sg * T::KS + k) * KR + cg * T::TC;
 #pragma unroll
     for (int p = 0; p < T::TR; p += 2) ld_cpair(pa + p, av[p], av[p + 1]);
 #pragma unroll
@@ -337,11 +339,27 @@ __device__ __forceinline__ void tile_reduce(CT<float> (&acc)[FrTile<KR, JT>::TR]
       }
 }
 
-// u = (children's) - L y for 64 border rows.  Shared memory: a stage of L (transposed), then y.
-constexpr int FR_LDL = 64 + 2;
-template <int KR> constexpr size_t fr_fwd_smem() {
-  return sizeof(CT<float>) * ((size_t)FrTile<KR, 64>::KC * FR_LDL + (size_t)FR_MAX_NB * KR);
+// 16 bytes into shared memory in the background, first out of L2 with `pol`; on = false: zeros.
+__device__ __forceinline__ uint64_t evict_first() {
+  uint64_t pol;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(pol));
+  return pol;
 }
+__device__ __forceinline__ void cp16_stream(void* dst, const void* src, bool on, uint64_t pol) {
+  asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2, %3;" ::"r"(smem_u32(dst)), "l"(src),
+               "r"(on ? 16 : 0), "l"(pol) : "memory");
+}
+__device__ __forceinline__ void cp16(void* dst, const void* src, bool on) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src), "r"(on ? 16 : 0) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+
+// u = (children's) - L y for 64 border rows.  The sum is 128 long at most, so the block's whole part of L is under way
+// before the level before is waited for, with the indices.  Shared memory: L, rows 16 bytes past a multiple of 128 (8 rows of
+// a warp on all banks), then y.
+constexpr int FR_LDL = FR_MAX_NB + 2;
+template <int KR> constexpr size_t fr_fwd_smem() { return sizeof(CT<float>) * ((size_t)64 * FR_LDL + (size_t)FR_MAX_NB * KR); }
 template <int KR>
 __global__ void __launch_bounds__(FR_THREADS) k_fr_fwd_multi(FrApply a, const FrontItem* __restrict__ items,
                                                              const CT<float>* __restrict__ fac,
@@ -349,81 +367,107 @@ __global__ void __launch_bounds__(FR_THREADS) k_fr_fwd_multi(FrApply a, const Fr
                                                              CT<float>* u) {
   using T = FrTile<KR, 64>;
   using C = CT<float>;
-  constexpr int LQ = T::KC * 64 / FR_THREADS;           // entries of a stage of L a thread loads
   extern __shared__ __align__(16) unsigned char fr_smem[];
-  C* Ls = (C*)fr_smem;                                  // [KC][FR_LDL]
-  C* own = Ls + T::KC * FR_LDL;                         // [FR_MAX_NB][KR]
-  static_assert((T::SG - 1) * 64 * KR <= FR_MAX_NB * KR + T::KC * FR_LDL, "the reduction fits");
+  __shared__ FrontSrc osrc[FR_MAX_NB];
+  __shared__ int32_t odof[FR_MAX_NB];
+  C* Ls = (C*)fr_smem;                                  // [64][FR_LDL]
+  C* own = Ls + 64 * FR_LDL;                            // [FR_MAX_NB][KR]
+  static_assert((T::SG - 1) * 64 * KR <= 64 * FR_LDL + FR_MAX_NB * KR && FR_THREADS % KR == 0, "the reduction fits, a thread has one column");
   pdl_release();
   const FrontItem it = items[blockIdx.x];
   const FrontNode n = a.nodes[it.node];
-  const int n1 = n.n1, ld = n.ld, i0 = it.t * 64;
-  const C* rows = fac + n.panel + (int64_t)n1 * ld;
-  // this thread's part of a stage of L: row lr, columns lc + 16 q .. lc + 16 q + 3 (the transposed stores of a
-  // warp then fall on all banks)
-  const int lr = threadIdx.x >> 2, lc = (threadIdx.x & 3) * 4;
-  auto col = [&](int q) { return lc + (q & 3) + 16 * (q >> 2); };
-  const bool lrow = i0 + lr < n.n2;
-  C l[LQ];
-  auto load = [&](int k0) {
-#pragma unroll
-    for (int q = 0; q < LQ; q += 2) {
-      l[q] = l[q + 1] = {0.0f, 0.0f};
-      if (lrow && k0 + col(q) < ld) ld_stream(rows + (int64_t)(i0 + lr) * ld + k0 + col(q), l[q], l[q + 1]);
-    }
-  };
-  load(0);
-  pdl_wait();
-  const int ldk = (ld + 15) / 16 * 16;                  // rows of y up to a whole step of 16 are read
-  for (int e = threadIdx.x; e < ldk * KR; e += FR_THREADS) {
-    const int c = e / KR, r = e % KR;
-    C t = {0.0f, 0.0f};
-    if (c < n1) {
-      const FrontSrc s = a.own_src[n.row0 + c];
-      if (r < a.nr) {
-        const cplx b = v[(int64_t)a.row_dof[n.row0 + c] * a.vs + a.off + r];
-        t = {(float)b.re, (float)b.im};
-      }
-      const C up = pull_vec<float, KR>(u, s, r);
-      t.re += up.re;
-      t.im += up.im;
-      if (it.t == 0) y[(int64_t)(n.row0 + c) * KR + r] = t;
-    }
-    own[c * KR + r] = t;
+  const int n1 = n.n1, ld = n.ld, i0 = it.t * 64, tid = threadIdx.x;
+  const C* rows = fac + n.panel + (int64_t)(n1 + i0) * ld;
+  const uint64_t pol = evict_first();
+  const int live = n.n2 - i0 < 64 ? n.n2 - i0 : 64;     // border rows of this block; the others' results are dropped
+  for (int i = tid >> 4; i < live; i += FR_THREADS / 16)
+    for (int c = 2 * (tid & 15); c < ld; c += 32) cp16_stream(Ls + i * FR_LDL + c, rows + (int64_t)i * ld + c, true, pol);
+  cp_commit();
+  if (tid < n1) {
+    osrc[tid] = a.own_src[n.row0 + tid];
+    odof[tid] = a.row_dof[n.row0 + tid];
   }
-  const int cg = threadIdx.x % T::CG, rg = threadIdx.x / T::CG % T::RG, sg = threadIdx.x / (T::CG * T::RG);
+  const int cg = tid % T::CG, rg = tid / T::CG % T::RG, sg = tid / (T::CG * T::RG);
+  FrontSrc bsrc[T::TR];                                 // of rows rg + RG p
+#pragma unroll
+  for (int p = 0; p < T::TR; ++p) {
+    const int i = rg + T::RG * p;
+    bsrc[p] = sg == 0 && i < live ? a.border_src[n.bord + i0 + i] : FrontSrc{-1, -1};
+  }
+  __syncthreads();
+  pdl_wait();
+  constexpr int BATCH = 4;                              // entries of y whose loads are in flight together
+  for (int e0 = tid; e0 < ld * KR; e0 += BATCH * FR_THREADS) {
+    C t[BATCH];
+#pragma unroll
+    for (int q = 0; q < BATCH; ++q) {
+      const int c = (e0 + q * FR_THREADS) / KR, r = tid % KR;
+      t[q] = {0.0f, 0.0f};
+      if (c < n1) {
+        if (r < a.nr) {
+          const cplx b = v[(int64_t)odof[c] * a.vs + a.off + r];
+          t[q] = {(float)b.re, (float)b.im};
+        }
+        const C up = pull_vec<float, KR>(u, osrc[c], r);
+        t[q].re += up.re;
+        t[q].im += up.im;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < BATCH; ++q) {
+      const int e = e0 + q * FR_THREADS;
+      if (e >= ld * KR) break;
+      if (it.t == 0 && e < n1 * KR) y[(int64_t)n.row0 * KR + e] = t[q];
+      own[e] = t[q];
+    }
+  }
   C acc[T::TR][T::TC];
 #pragma unroll
   for (int p = 0; p < T::TR; ++p)
 #pragma unroll
     for (int q = 0; q < T::TC; ++q) acc[p][q] = {0.0f, 0.0f};
-  for (int k0 = 0; k0 < ld; k0 += T::KC) {
-    __syncthreads();
+  cp_wait<0>();
+  __syncthreads();
+  const int part = (ld + 2 * T::SG - 1) / (2 * T::SG) * 2;  // sum indices of a group, in pairs (ld is a multiple of 4)
+  const int k1 = (sg + 1) * part < ld ? (sg + 1) * part : ld;
+#pragma unroll 4
+  for (int k = sg * part; k < k1; k += 2) {
+    C a0[T::TR], a1[T::TR], b0[T::TC], b1[T::TC];
 #pragma unroll
-    for (int q = 0; q < LQ; ++q) Ls[col(q) * FR_LDL + lr] = l[q];
-    __syncthreads();
-    if (k0 + T::KC < ld) load(k0 + T::KC);
-    if (k0 + sg * 16 < ld) tile_stage<KR, 64, FR_LDL>(acc, Ls, own + k0 * KR, sg, rg, cg);
+    for (int p = 0; p < T::TR; ++p) ld_cpair(Ls + (rg + T::RG * p) * FR_LDL + k, a0[p], a1[p]);
+#pragma unroll
+    for (int q = 0; q < T::TC; q += 2) {
+      ld_cpair(own + k * KR + cg * T::TC + q, b0[q], b0[q + 1]);
+      ld_cpair(own + (k + 1) * KR + cg * T::TC + q, b1[q], b1[q + 1]);
+    }
+#pragma unroll
+    for (int p = 0; p < T::TR; ++p)
+#pragma unroll
+      for (int q = 0; q < T::TC; ++q) {
+        cfma(acc[p][q], a0[p], b0[q]);
+        cfma(acc[p][q], a1[p], b1[q]);
+      }
   }
   tile_reduce<KR, 64>(acc, (C*)fr_smem, sg, rg, cg);
   if (sg > 0) return;
 #pragma unroll
   for (int p = 0; p < T::TR; ++p) {
-    const int i = i0 + rg * T::TR + p;
-    if (i >= n.n2) continue;
-    const FrontSrc s = a.border_src[n.bord + i];
+    const int i = rg + T::RG * p;
+    if (i >= live) continue;
 #pragma unroll
     for (int q = 0; q < T::TC; ++q) {
       const int r = cg * T::TC + q;
-      const C up = pull_vec<float, KR>(u, s, r);
-      u[(n.bord + i) * KR + r] = {up.re - acc[p][q].re, up.im - acc[p][q].im};
+      const C up = pull_vec<float, KR>(u, bsrc[p], r);
+      u[(n.bord + i0 + i) * KR + r] = {up.re - acc[p][q].re, up.im - acc[p][q].im};
     }
   }
 }
 
-// x = [S; L]^T [y; -x(border)] for JT own unknowns.  Shared memory: a stage of panel rows, a stage of [y; -x].
+// x = [S; L]^T [y; -x(border)] for JT own unknowns, FR_STAGES stages of panel rows and rows of [y; -x] in shared memory: a
+// stage's loads have the products of the three before it to arrive in.  The x buffer holds -x, as the levels below use it.
+constexpr int FR_STAGES = 4;
 template <int KR, int JT> constexpr size_t fr_bwd_smem() {
-  return sizeof(CT<float>) * (size_t)FrTile<KR, JT>::KC * (JT + KR);
+  return sizeof(CT<float>) * (size_t)FR_STAGES * FrTile<KR, JT>::KC * (JT + KR);
 }
 template <typename ZT, int KR, int JT>
 __global__ void __launch_bounds__(FR_THREADS) k_fr_bwd_multi(FrApply a, const FrontItem* __restrict__ items,
@@ -432,80 +476,75 @@ __global__ void __launch_bounds__(FR_THREADS) k_fr_bwd_multi(FrApply a, const Fr
                                                              ZT* z) {
   using T = FrTile<KR, JT>;
   using C = CT<float>;
-  constexpr int GL = JT / 4, GR = FR_THREADS / GL, GQ = T::KC / GR;  // lanes a row, rows at once, passes
-  constexpr int WE = T::KC * KR / FR_THREADS;                 // entries of [y; -x] a thread stages
-  static_assert(GQ * GR == T::KC && WE * FR_THREADS == T::KC * KR, "stage shapes");
-  static_assert((T::SG - 1) * JT * KR <= T::KC * (JT + KR), "the reduction fits");
+  constexpr int KC = T::KC, STAGE = KC * (JT + KR);
+  constexpr int GL = JT / 2, GQ = (KC * GL + FR_THREADS - 1) / FR_THREADS;   // 16-byte pieces of a panel row, per thread
+  constexpr int WL = KR / 2, WQ = (KC * WL + FR_THREADS - 1) / FR_THREADS;   // of a row of [y; -x]
+  static_assert((T::SG - 1) * JT * KR <= FR_STAGES * STAGE, "the reduction fits");
   extern __shared__ __align__(16) unsigned char fr_smem[];
-  C* Gs = (C*)fr_smem;                                        // [KC][JT]
-  C* ws = Gs + T::KC * JT;                                    // [KC][KR]
+  C* buf = (C*)fr_smem;                                       // [FR_STAGES] of [KC][JT], [KC][KR]
   pdl_release();
   const FrontItem it = items[blockIdx.x];
   const FrontNode n = a.nodes[it.node];
-  const int n1 = n.n1, m = n.n1 + n.n2, ld = n.ld, j0 = it.t * JT;
-  const C* panel = fac + n.panel + j0;
-  // this thread's part of a stage: rows gr + GR q, columns gc .. gc + 3
-  const int gr = threadIdx.x / GL, gc = threadIdx.x % GL * 4;
-  C g[GQ][4], w[WE];
-  int32_t row[WE];                                            // rows of [y; x] of the next stage
-  auto load = [&](int k0) {
+  const int n1 = n.n1, m = n.n1 + n.n2, ld = n.ld, j0 = it.t * JT, tid = threadIdx.x;
+  const C* panel = fac + n.panel;
+  const uint64_t pol = evict_first();
+  auto load_panel = [&](int s) {
+    C* g = buf + s % FR_STAGES * STAGE;
 #pragma unroll
     for (int q = 0; q < GQ; ++q) {
-      const int i = k0 + gr + GR * q;
-#pragma unroll
-      for (int p = 0; p < 4; ++p) g[q][p] = {0.0f, 0.0f};
-      if (i < m && j0 + gc < ld) {
-        const C* p = panel + (int64_t)i * ld + gc;
-        ld_stream(p, g[q][0], g[q][1]);
-        ld_stream(p + 2, g[q][2], g[q][3]);
-      }
+      const int e = tid + FR_THREADS * q, k = e / GL, c = e % GL * 2, i = s * KC + k;
+      if (k >= KC) break;
+      const bool on = i < m && j0 + c < ld;
+      cp16_stream(g + k * JT + c, on ? panel + (int64_t)i * ld + j0 + c : panel, on, pol);
     }
   };
-  auto load_rows = [&](int k0) {
+  int32_t row[WQ];                                            // rows of [y; -x] of the stage load_w takes next
+  auto load_rows = [&](int s) {
 #pragma unroll
-    for (int q = 0; q < WE; ++q) {
-      const int i = k0 + (threadIdx.x + FR_THREADS * q) / KR;
-      row[q] = i < n1 ? n.row0 + i : (i < m ? a.border[n.bord + i - n1] : -1);
+    for (int q = 0; q < WQ; ++q) {
+      const int k = (tid + FR_THREADS * q) / WL, i = s * KC + k;
+      row[q] = k >= KC || i >= m ? -1 : (i < n1 ? n.row0 + i : a.border[n.bord + i - n1]);
     }
   };
-  auto load_w = [&](int k0) {
+  auto load_w = [&](int s) {
+    C* w = buf + s % FR_STAGES * STAGE + KC * JT;
 #pragma unroll
-    for (int q = 0; q < WE; ++q) {
-      const int e = threadIdx.x + FR_THREADS * q, i = k0 + e / KR, r = e % KR;
-      w[q] = {0.0f, 0.0f};
-      if (row[q] < 0) continue;
-      w[q] = (i < n1 ? y : x)[(int64_t)row[q] * KR + r];
-      if (i >= n1) w[q] = {-w[q].re, -w[q].im};
+    for (int q = 0; q < WQ; ++q) {
+      const int e = tid + FR_THREADS * q, k = e / WL, r = e % WL * 2;
+      if (k >= KC) break;
+      const C* src = s * KC + k < n1 ? y : x;
+      cp16(w + k * KR + r, row[q] >= 0 ? src + (int64_t)row[q] * KR + r : y, row[q] >= 0);
     }
-    load_rows(k0 + T::KC);
+    load_rows(s + 1);
   };
-  load(0);
+  const int stages = (m + KC - 1) / KC;
   load_rows(0);
+  for (int s = 0; s < FR_STAGES - 1 && s < stages; ++s) load_panel(s);
   pdl_wait();
-  load_w(0);
-  const int cg = threadIdx.x % T::CG, rg = threadIdx.x / T::CG % T::RG, sg = threadIdx.x / (T::CG * T::RG);
+#pragma unroll
+  for (int s = 0; s < FR_STAGES - 1; ++s) {
+    if (s < stages) load_w(s);
+    cp_commit();
+  }
+  const int cg = tid % T::CG, rg = tid / T::CG % T::RG, sg = tid / (T::CG * T::RG);
   C acc[T::TR][T::TC];
 #pragma unroll
   for (int p = 0; p < T::TR; ++p)
 #pragma unroll
     for (int q = 0; q < T::TC; ++q) acc[p][q] = {0.0f, 0.0f};
-  for (int k0 = 0; k0 < m; k0 += T::KC) {
-    __syncthreads();
-#pragma unroll
-    for (int q = 0; q < GQ; ++q) {
-      st_cpair(Gs + (gr + GR * q) * JT + gc, g[q][0], g[q][1]);
-      st_cpair(Gs + (gr + GR * q) * JT + gc + 2, g[q][2], g[q][3]);
+  for (int s = 0; s < stages; ++s) {
+    cp_wait<FR_STAGES - 2>();
+    __syncthreads();  // stage s has arrived, stage s - 1 has been used
+    if (s + FR_STAGES - 1 < stages) {
+      load_panel(s + FR_STAGES - 1);
+      load_w(s + FR_STAGES - 1);
     }
-#pragma unroll
-    for (int q = 0; q < WE; ++q) ws[threadIdx.x + FR_THREADS * q] = w[q];
-    __syncthreads();
-    if (k0 + T::KC < m) {
-      load(k0 + T::KC);
-      load_w(k0 + T::KC);
-    }
-    if (k0 + sg * 16 < m) tile_stage<KR, JT, JT>(acc, Gs, ws, sg, rg, cg);  // rows past the panel are zeros
+    cp_commit();
+    const C* g = buf + s % FR_STAGES * STAGE;
+    if (s * KC + sg * T::KS < m) tile_stage<KR, JT>(acc, g, g + KC * JT, sg, rg, cg);  // rows past the panel are zeros
   }
-  tile_reduce<KR, JT>(acc, (C*)fr_smem, sg, rg, cg);
+  cp_wait<0>();
+  tile_reduce<KR, JT>(acc, buf, sg, rg, cg);
   if (sg > 0) return;
 #pragma unroll
   for (int p = 0; p < T::TR; ++p) {
@@ -518,7 +557,7 @@ __global__ void __launch_bounds__(FR_THREADS) k_fr_bwd_multi(FrApply a, const Fr
     for (int q = 0; q < T::TC; ++q) {
       const int r = cg * T::TC + q;
       const C t = acc[p][q];
-      x[row * KR + r] = t;
+      x[row * KR + r] = {-t.re, -t.im};
       if (r >= a.nr) continue;
       ZT* dst = z + dof * a.vs + a.off + r;
       if (a.weights == ORAS_WEIGHTS_POU) {
