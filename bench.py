@@ -7,7 +7,7 @@ Metric: solves/s of ORAS-preconditioned FGMRES to a true FP64 relative residual 
 with 2 overlap layers, FP32 local factors, FP64 outer FGMRES(100), one z-directed dipole.
 
 One step = the numeric work of one request on a fixed mesh: element matrices, global A,
-local impedance matrices A_s, batched LU of every A_s, and the FGMRES solve with the ORAS
+local impedance matrices A_s, the factorisation of every A_s, and the FGMRES solve with the ORAS
 preconditioner.  The per-mesh integer set-up (topology, numbering, partition, overlap)
 is done once before timing (the imaging loop reuses its mesh); the end-to-end number
 `e2e` includes it, through oras_setup with host buffers, every step.
@@ -847,7 +847,7 @@ def run_ours(args, world, rank, local):
                        "rhs_per_step": krhs, "factor_arena_bytes": arena,
                        "l2": "512 MiB buffer written between timed steps; the step itself streams the "
                              f"{arena / 1e9:.1f} GB of factors",
-                       "step": "oras_factor (element matrices, A, A_s, batched LU) + oras_solve, device buffers",
+                       "step": "oras_factor (element matrices, A, A_s, local factorisations) + oras_solve, device buffers",
                        "mesh_setup_s_untimed": t_mesh, "parallelism": f"replicas x{world}",
                        "lu_panel": panel, "lu_group": group,
                        "lu_autotune_ms": {str(k_): round(v_, 1) for k_, v_ in tune_ms.items()}},
