@@ -292,30 +292,19 @@ static int ensure_ybuf(oras_handle* h, int k) {
   return ORAS_OK;
 }
 
-static int alloc_factor_space(oras_handle* h, int bits) {
+// Every buffer of the factorisation in `bits` precision; alloc_factor_space records them as there.
+static int alloc_factor_buffers(oras_handle* h, int bits, size_t bytes) {
   auto& m = h->mesh;
   auto& d = h->dev;
-  size_t el = bits == 64 ? 16 : 8;
-  // sparse factors: the panels; dense: the factor tiles
-  size_t bytes = h->fronts.use ? (size_t)std::max<int64_t>(1, h->fronts.panel_elems) * el
-                               : (size_t)m.arena_tiles * TB * TB * el;
-  if (d.arena && d.factor_bits == bits && d.arena_bytes == bytes) return ORAS_OK;
-  dfree_s(d.arena, d.stream);
+  const size_t el = bits == 64 ? 16 : 8;
   cudaError_t e = pool_malloc(&d.arena, bytes, d.stream);
   if (e != cudaSuccess) {
     h->err = "local-factor arena of " + std::to_string(bytes) + " bytes: " + cudaGetErrorString(e);
-    d.arena = nullptr;
     return e == cudaErrorMemoryAllocation ? ORAS_ERR_OUT_OF_MEMORY : ORAS_ERR_CUDA;
   }
-  d.arena_bytes = bytes;
-  d.factor_bits = bits;
   if (h->fronts.use) {
-    dfree_s(d.fr_work, d.stream);
-    dfree_s(d.fr_c, d.stream);
     CK(pool_malloc(&d.fr_work, bytes, d.stream));
     CK(pool_malloc(&d.fr_c, (size_t)std::max<int64_t>(1, h->fronts.c_elems) * el, d.stream));
-    dfree_s(d.ybuf, d.stream);
-    d.ybuf_bytes = 0;
     return ensure_ybuf(h, 1);
   }
   d.lu_max_chunks = lu_max_chunks(m.max_np, bits);
@@ -324,22 +313,50 @@ static int alloc_factor_space(oras_handle* h, int bits) {
   CK(dalloc(d.lu_cnt, (size_t)m.nsub * slots));
   CK(cudaMemsetAsync(d.lu_cnt, 0, (size_t)m.nsub * slots * sizeof(int32_t), d.stream));
   CK(dalloc(d.lu_ipiv, (size_t)m.nsub * (2 * TB * 2 + 1)));
-  dfree_s(d.lu_diag, d.stream);
   CK(pool_malloc(&d.lu_diag, (size_t)m.nsub * TB * TB * el, d.stream));
   {
     std::vector<int64_t> inv_off(m.nsub + 1, 0);
     for (int q = 0; q < m.nsub; ++q) inv_off[q + 1] = inv_off[q] + m.sub_np[q] / TB;
     CK(dput(d.sub_inv_off, inv_off, d.stream));
-    dfree_s(d.dinv, d.stream);
     d.dinv_bytes = (size_t)inv_off[m.nsub] * 2 * TB * TB * el;
     CK(pool_malloc(&d.dinv, d.dinv_bytes, d.stream));
   }
-  dfree_s(d.ybuf, d.stream);
-  d.ybuf_bytes = 0;
   return ensure_ybuf(h, 1);
 }
 
+static void free_factor_space(Device& d) {
+  dfree_s(d.arena, d.stream);
+  dfree_s(d.fr_work, d.stream);
+  dfree_s(d.fr_c, d.stream);
+  dfree_s(d.lu_cand, d.stream);
+  dfree_s(d.lu_cnt, d.stream);
+  dfree_s(d.lu_ipiv, d.stream);
+  dfree_s(d.lu_diag, d.stream);
+  dfree_s(d.sub_inv_off, d.stream);
+  dfree_s(d.dinv, d.stream);
+  dfree_s(d.ybuf, d.stream);
+  d.arena_bytes = d.dinv_bytes = d.ybuf_bytes = 0;
+  d.factor_bits = 0;
+}
 
+// arena_bytes and factor_bits say that the whole space is there: they are set after the last allocation.  A
+// failure gives back what was allocated, so that the call can be made again when there is memory.
+static int alloc_factor_space(oras_handle* h, int bits) {
+  auto& d = h->dev;
+  const size_t el = bits == 64 ? 16 : 8;
+  // sparse factors: the panels; dense: the factor tiles
+  const size_t bytes = h->fronts.use ? (size_t)std::max<int64_t>(1, h->fronts.panel_elems) * el
+                                     : (size_t)h->mesh.arena_tiles * TB * TB * el;
+  if (d.arena && d.factor_bits == bits && d.arena_bytes == bytes) return ORAS_OK;
+  free_factor_space(d);
+  if (int rc = alloc_factor_buffers(h, bits, bytes)) {
+    free_factor_space(d);
+    return rc;
+  }
+  d.arena_bytes = bytes;
+  d.factor_bits = bits;
+  return ORAS_OK;
+}
 
 // Device bytes that oras_factor plus an oras_solve of k right-hand sides allocate for this
 // handle (the sizes of upload, alloc_factor_space, ensure_ybuf, ensure_ws and ensure_io), plus the
