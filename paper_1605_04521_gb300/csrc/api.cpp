@@ -813,6 +813,7 @@ int oras::ensure_ws(oras_handle* h, int k, int m) {
   if (int rc = ensure_ybuf(h, k)) return rc;
   if (d.ws_k >= k && d.ws_m >= m && d.V) return ORAS_OK;
   int kk = std::max(k, d.ws_k), mm = std::max(m, d.ws_m);
+  d.ws_k = d.ws_m = 0;  // until all of it is there
   size_t nk = (size_t)N * kk;
   CK(dalloc(d.V, nk * (mm + 1)));
   if (d.factor_bits == 64) {

@@ -45,3 +45,9 @@ def findings(program, scenario):
 @pytest.mark.parametrize("scenario", ["factor32", "factor64", "factor_dense"])
 def test_factor_again_after_running_out_of_memory(program, scenario):
     assert findings(program, scenario) == (0, "")
+
+
+@pytest.mark.parametrize("scenario", ["solve32", "solve64"])
+def test_solve_again_after_running_out_of_memory(program, scenario):
+    """A solve of three columns runs out of memory after one of two: then two and three columns again."""
+    assert findings(program, scenario) == (0, "")
