@@ -689,7 +689,7 @@ void oras_destroy(oras_handle* h) {
   }
   if (h->apply_fork) cudaEventDestroy(h->apply_fork);
   if (h->apply_join) cudaEventDestroy(h->apply_join);
-  if (h->dev.uploaded) {
+  if (h->dev.device >= 0) {  // an upload began, whether or not it succeeded
     cudaStreamSynchronize(h->dev.stream);
     if (h->rc_U) cudaFreeAsync(h->rc_U, h->dev.stream);
     dfree_all(h->dev);

@@ -228,6 +228,24 @@ static void factor_again(int bits, int engine) {
   }
 }
 
+// oras_setup with every allocation from the n-th on refused, for every n: nothing is left behind.
+static void setup_fails(int engine) {
+  Cube c(2, 1, 2);
+  oras_options o{};
+  o.lu_engine = engine;
+  for (int64_t n = 0;; ++n) {
+    oras_handle* h = nullptr;
+    g_count = 0;
+    g_refuse_from = n;
+    const int rc = oras_setup(&c.p, &o, &h);
+    g_refuse_from = -1;
+    if (rc == ORAS_OK) { oras_destroy(h); break; }
+    if (rc != ORAS_ERR_OUT_OF_MEMORY) bad(at("not reported as out of memory", n, rc));
+    if (!g_live.empty()) bad(at("memory left after a set-up that failed", n, rc));
+    while (!g_live.empty()) cudaFreeAsync(g_live.begin()->first, nullptr);
+  }
+}
+
 // A solve of more columns with every allocation from the n-th on refused, then one of as many as before.
 static void solve_again(int bits) {
   Cube c(3, 2, 4);
@@ -263,6 +281,8 @@ int main(int argc, char** argv) {
   if (s == "factor32") factor_again(32, ORAS_LU_AUTO);
   else if (s == "factor64") factor_again(64, ORAS_LU_AUTO);
   else if (s == "factor_dense") factor_again(32, ORAS_LU_CUDA_CORES);
+  else if (s == "setup") setup_fails(ORAS_LU_AUTO);
+  else if (s == "setup_dense") setup_fails(ORAS_LU_CUDA_CORES);
   else if (s == "solve32") solve_again(32);
   else if (s == "solve64") solve_again(64);
   else bad("unknown scenario");

@@ -51,3 +51,8 @@ def test_factor_again_after_running_out_of_memory(program, scenario):
 def test_solve_again_after_running_out_of_memory(program, scenario):
     """A solve of three columns runs out of memory after one of two: then two and three columns again."""
     assert findings(program, scenario) == (0, "")
+
+
+@pytest.mark.parametrize("scenario", ["setup", "setup_dense"])
+def test_failed_set_up_leaves_no_memory_behind(program, scenario):
+    assert findings(program, scenario) == (0, "")
