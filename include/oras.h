@@ -366,8 +366,9 @@ int oras_precond(oras_handle* h, const oras_complex* v, oras_complex* z, int32_t
  * synchronise the device and stall the other requests in flight.  The paper has no counterpart;
  * this is an interface convenience.  v, z: device pointers (current device = the handle's
  * device), N x k column-major, complex FP64, on the handle's stream; the call is asynchronous.
- * Sparse factors: the local vectors live in the handle's workspace that oras_factor allocated (calls
- * on one handle that overlap on the GPU race on it).  Dense factors: in one fixed 16 MiB device array
+ * Sparse factors: the local vectors live in a workspace of the handle that oras_factor allocated for
+ * this call alone and that stays where it is, so a captured call can be replayed after any other call
+ * (calls of this function on one handle that overlap on the GPU race on it).  Dense factors: in one fixed 16 MiB device array
  * compiled into the library (every GPU that loads the library holds it until exit).  Either way
  * the sum over subdomains of the padded order times the factor entry size (8 B FP32, 16 B FP64) must
  * be at most 16 MiB, else INVALID_ARG with the needed size.  With the fixed array: the first call on a device resolves the array's device address (cudaGetSymbolAddress); make

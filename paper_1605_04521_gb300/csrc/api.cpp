@@ -153,7 +153,7 @@ static void dfree_all(Device& d) {
                   d.sub_dofs, d.sub_pou, d.member, d.cm, d.ck, d.cs, d.fl, d.tc, d.ta, d.tm, d.eps, d.mu,
                   d.elem, d.fmat, d.vals, d.vals_df, d.arena, d.perm, d.gidx, d.sub_np_off, d.lu_cand, d.lu_cnt,
                   d.lu_ipiv, d.lu_diag, d.dinv, d.sub_inv_off, d.status, d.V, d.Zf, d.Zd, d.w, d.xk, d.bk, d.tmp, d.H, d.gcs, d.gsn,
-                  d.g, d.red, d.scal, d.ybuf, d.io, d.apply_subs,
+                  d.g, d.red, d.scal, d.ybuf, d.y1, d.io, d.apply_subs,
                   d.fr_nodes, d.fr_border, d.fr_own_src, d.fr_border_src, d.fr_pos, d.fr_row_node, d.fr_row_dof, d.fr_row_pou,
                   d.fr_assemble, d.fr_lmul, d.fr_schur, d.fr_fwd, d.fr_bwd, d.fr_bwd_multi, d.fr_work, d.fr_c};
   for (void* p : ptrs)
@@ -305,6 +305,8 @@ static int alloc_factor_buffers(oras_handle* h, int bits, size_t bytes) {
   if (h->fronts.use) {
     CK(pool_malloc(&d.fr_work, bytes, d.stream));
     CK(pool_malloc(&d.fr_c, (size_t)std::max<int64_t>(1, h->fronts.c_elems) * el, d.stream));
+    // ybuf moves when a call with more columns needs a larger one; y1 stays, as a captured oras_precond_noalloc needs
+    CK(pool_malloc(&d.y1, apply_yglob_bytes_for(h, 1), d.stream));
     return ensure_ybuf(h, 1);
   }
   d.lu_max_chunks = lu_max_chunks(m.max_np, bits);
@@ -335,6 +337,7 @@ static void free_factor_space(Device& d) {
   dfree_s(d.sub_inv_off, d.stream);
   dfree_s(d.dinv, d.stream);
   dfree_s(d.ybuf, d.stream);
+  dfree_s(d.y1, d.stream);
   d.arena_bytes = d.dinv_bytes = d.ybuf_bytes = 0;
   d.factor_bits = 0;
 }
@@ -400,6 +403,7 @@ int64_t footprint_bytes(const oras_handle* h, int k) {
     add(f.panel_elems * (int64_t)el);                               // panels
     add(f.panel_elems * (int64_t)el);                               // assembly workspace
     add(f.c_elems * (int64_t)el);                                   // contribution blocks
+    add((int64_t)apply_yglob_bytes_for(h, 1));                      // vectors of the allocation-free apply
   } else {
     add(total_np * 4);                                                // perm
     add(total_np * 4);                                                // gidx

@@ -22,7 +22,7 @@ int apply_tc_f64out(const oras_handle* h, const cplx* v, cplx* z, int k, int r0,
 int apply_tc_f32out(const oras_handle* h, const cplx* v, void* z, int k, int r0, int nr);
 int apply_tc_passes(int nr);
 // sparse local factors (fronts_apply.cu)
-int fronts_apply_f64out(const oras_handle* h, const cplx* v, cplx* z, int k, int64_t vs, int64_t rs);
+int fronts_apply_f64out(const oras_handle* h, const cplx* v, cplx* z, int k);
 int fronts_apply_f32out(const oras_handle* h, const cplx* v, void* z, int k);
 size_t fronts_ybytes(const oras_handle* h, int k);
 int fronts_passes(const oras_handle* h, int k);
@@ -186,7 +186,7 @@ static int apply_t(const oras_handle* h, const cplx* v, ZT* z, int k) {
 
 // z (FP64 complex [N][k]) = M^{-1} v
 int launch_apply_f64out(const oras_handle* h, const cplx* v, cplx* z, int k) {
-  if (h->fronts.use) return fronts_apply_f64out(h, v, z, k, k, 1);
+  if (h->fronts.use) return fronts_apply_f64out(h, v, z, k);
   return h->dev.factor_bits == 64 ? apply_t<double, cplx>(h, v, z, k) : apply_t<float, cplx>(h, v, z, k);
 }
 // z (FP32 complex [N][k]) = M^{-1} v, FP32 factors only

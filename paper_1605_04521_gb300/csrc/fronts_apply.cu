@@ -609,7 +609,7 @@ static void launch_pdl(void (*fn)(P...), int64_t blocks, size_t smem, cudaStream
 }
 
 template <typename R, typename ZT, int KR>
-static void fr_pass(const oras_handle* h, const cplx* v, ZT* z, int64_t vs, int64_t off, int nr) {
+static void fr_pass(const oras_handle* h, void* buf, const cplx* v, ZT* z, int64_t vs, int64_t off, int nr) {
   const auto& d = h->dev;
   const Fronts& f = h->fronts;
   FrApply a;
@@ -618,7 +618,7 @@ static void fr_pass(const oras_handle* h, const cplx* v, ZT* z, int64_t vs, int6
   a.weights = h->opt.weights;
   a.vs = vs; a.off = off; a.nr = nr;
   const int64_t rows = h->mesh.sub_ns_off[h->mesh.nsub];
-  CT<R>* y = (CT<R>*)d.ybuf;
+  CT<R>* y = (CT<R>*)buf;
   CT<R>* x = y + rows * KR;
   CT<R>* u = x + rows * KR;
   const CT<R>* fac = (const CT<R>*)d.arena;
@@ -645,34 +645,38 @@ static void fr_pass(const oras_handle* h, const cplx* v, ZT* z, int64_t vs, int6
   }
 }
 
-// z = M^{-1} v for k right-hand sides; right-hand side r of unknown g at g * vs + r * rs of v and z
-// (rs = 1: adjacent, vs = k; else one at a time).
+// z = M^{-1} v for k right-hand sides, right-hand side r of unknown g at g * vs + r * rs of v and z: adjacent ones
+// (rs = 1, vs = k) in groups, with their local vectors in ybuf; or columns (vs = 1) one at a time, in y1.
 template <typename R, typename ZT>
 static int fr_apply_t(const oras_handle* h, const cplx* v, ZT* z, int k, int64_t vs, int64_t rs) {
   const auto& d = h->dev;
-  if (!d.ybuf || d.ybuf_bytes < fronts_ybytes(h, rs == 1 ? k : 1)) return -1;
+  void* buf = rs == 1 ? d.ybuf : d.y1;
+  if (!buf || (rs == 1 && d.ybuf_bytes < fronts_ybytes(h, k))) return -1;
   if (h->opt.weights != ORAS_WEIGHTS_POU &&
       cudaMemsetAsync(z, 0, sizeof(ZT) * (size_t)h->mesh.ndof * k, d.stream) != cudaSuccess)
     return -1;
   for (int r0 = 0; r0 < k;) {
     const int kr = rs == 1 ? fr_kr(h, k - r0) : 1, nr = std::min(kr, k - r0);
     const int64_t off = r0 * rs;
-    if (kr == 1) fr_pass<R, ZT, 1>(h, v, z, vs, off, nr);
-    else if (kr == 2) fr_pass<R, ZT, 2>(h, v, z, vs, off, nr);
+    if (kr == 1) fr_pass<R, ZT, 1>(h, buf, v, z, vs, off, nr);
+    else if (kr == 2) fr_pass<R, ZT, 2>(h, buf, v, z, vs, off, nr);
     else if constexpr (sizeof(R) == 4) {
-      if (kr == 4) fr_pass<R, ZT, 4>(h, v, z, vs, off, nr);
-      else if (kr == 8) fr_pass<R, ZT, 8>(h, v, z, vs, off, nr);
-      else if (kr == 16) fr_pass<R, ZT, 16>(h, v, z, vs, off, nr);
-      else fr_pass<R, ZT, 32>(h, v, z, vs, off, nr);
+      if (kr == 4) fr_pass<R, ZT, 4>(h, buf, v, z, vs, off, nr);
+      else if (kr == 8) fr_pass<R, ZT, 8>(h, buf, v, z, vs, off, nr);
+      else if (kr == 16) fr_pass<R, ZT, 16>(h, buf, v, z, vs, off, nr);
+      else fr_pass<R, ZT, 32>(h, buf, v, z, vs, off, nr);
     }
     r0 += nr;
   }
   return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
-int fronts_apply_f64out(const oras_handle* h, const cplx* v, cplx* z, int k, int64_t vs, int64_t rs) {
-  return h->dev.factor_bits == 64 ? fr_apply_t<double, cplx>(h, v, z, k, vs, rs)
-                                  : fr_apply_t<float, cplx>(h, v, z, k, vs, rs);
+int fronts_apply_f64out(const oras_handle* h, const cplx* v, cplx* z, int k) {
+  return h->dev.factor_bits == 64 ? fr_apply_t<double, cplx>(h, v, z, k, k, 1) : fr_apply_t<float, cplx>(h, v, z, k, k, 1);
+}
+int fronts_apply_noalloc(const oras_handle* h, const cplx* v, cplx* z, int k) {
+  const int64_t n = h->mesh.ndof;
+  return h->dev.factor_bits == 64 ? fr_apply_t<double, cplx>(h, v, z, k, 1, n) : fr_apply_t<float, cplx>(h, v, z, k, 1, n);
 }
 int fronts_apply_f32out(const oras_handle* h, const cplx* v, void* z, int k) {
   return fr_apply_t<float, CT<float>>(h, v, (CT<float>*)z, k, k, 1);

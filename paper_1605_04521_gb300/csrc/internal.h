@@ -166,6 +166,7 @@ struct Device {
   double* scal = nullptr;                       // small scalars [k][8]
   void* ybuf = nullptr;                         // apply: per-subdomain local vectors
   size_t ybuf_bytes = 0;
+  void* y1 = nullptr;                           // the same for one column, of oras_precond_noalloc alone (sparse factors)
   // apply work split: the first apply_n4 subdomains of apply_subs take clusters of four CTAs
   // (largest padded order apply_np4), the rest two (apply_np2); apply_n4 == 0: two CTAs each
   int32_t* apply_subs = nullptr;

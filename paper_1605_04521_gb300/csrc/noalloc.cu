@@ -31,7 +31,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(APPLY_THREADS)
 }
 
 ApplyGeom apply_geom(const oras_handle* h);
-int fronts_apply_f64out(const oras_handle* h, const cplx* v, cplx* z, int k, int64_t vs, int64_t rs);
+int fronts_apply_noalloc(const oras_handle* h, const cplx* v, cplx* z, int k);
 void apply_noalloc_config(const oras_handle* h, int* S, size_t* smem);
 
 }  // namespace oras
@@ -64,8 +64,8 @@ extern "C" int oras_precond_noalloc(oras_handle* h, const oras_complex* v, oras_
     h->err = "oras_precond_noalloc: the current device is not the handle's device";
     return ORAS_ERR_INVALID_ARG;
   }
-  if (h->fronts.use) {  // local vectors in the workspace oras_factor allocated; columns one by one
-    if (fronts_apply_f64out(h, (const cplx*)v, (cplx*)z, k, 1, m.ndof)) {
+  if (h->fronts.use) {  // local vectors in a workspace of their own that oras_factor allocated; columns one by one
+    if (fronts_apply_noalloc(h, (const cplx*)v, (cplx*)z, k)) {
       h->err = std::string("oras_precond_noalloc: launch: ") + cudaGetErrorString(cudaGetLastError());
       return ORAS_ERR_CUDA;
     }

@@ -87,6 +87,7 @@ cudaError_t cudaEventElapsedTime(float* t, cudaEvent_t, cudaEvent_t) { *t = 0.0f
 }
 
 // ------------------------------------------------------------------ launchers
+namespace oras { size_t apply_yglob_bytes_for(const oras_handle* h, int k); }
 static size_t entry(const oras_handle* h) { return h->opt.factor_bits == 64 ? 16 : 8; }
 static void touch_apply(const oras_handle* h, int k) {
   const auto& f = h->fronts;
@@ -116,6 +117,7 @@ int launch_front_factor(oras_handle* h) {
   touch("the assembly workspace", h->dev.fr_work, (size_t)h->fronts.panel_elems * entry(h));
   touch("the factors", h->dev.arena, (size_t)h->fronts.panel_elems * entry(h));
   touch("the contribution blocks", h->dev.fr_c, (size_t)h->fronts.c_elems * entry(h));
+  touch("the vectors of the allocation-free apply", h->dev.y1, apply_yglob_bytes_for(h, 1));
   return 0;
 }
 int launch_local_rows(const oras_handle* h, double) {

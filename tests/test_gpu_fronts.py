@@ -141,3 +141,43 @@ def test_columns_together_equal_columns_alone(O, case):
                 assert rel(Z[:, j], alone[:, j]) <= bar
     finally:
         O.oras_destroy(h)
+
+
+@pytest.mark.parametrize("bits,weights", [(32, 0), (64, 0), (32, 1)])
+def test_captured_noalloc_apply_outlives_larger_calls(O, bits, weights):
+    """The allocation-free apply in a CUDA graph, replayed after calls with more columns have made the handle's other
+    workspace grow and after new materials: the factors and vectors it uses are still where they were captured."""
+    import torch
+    w = synth.small(n=4, r=2, nsub=8, overlap=1)
+    xyz, tets = w.mesh()
+    eps, mu = w.materials(xyz, tets)
+    h = O.oras_setup(xyz, tets, eps, mu, w.k0, w.r, w.nsub, w.overlap, factor_bits=bits, weights=weights)
+    try:
+        n = O.oras_ndof(h)
+        rng = np.random.default_rng(17)
+        V = rng.normal(size=(2, n)) + 1j * rng.normal(size=(2, n))
+        vd = torch.from_numpy(V).cuda()
+        zd = torch.zeros_like(vd)
+        stream = torch.cuda.Stream()
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        O.oras_set_stream(h, stream.cuda_stream)
+        O.oras_precond_noalloc(h, vd, zd, 2)               # the first call on a device comes before a capture
+        torch.cuda.synchronize()
+        with torch.cuda.graph(graph, stream=stream):
+            O.oras_precond_noalloc(h, vd, zd, 2)
+        B = rng.normal(size=(n, 40)) + 1j * rng.normal(size=(n, 40))
+        for factor in (1.0, 1.3):
+            O.oras_factor(h, eps * factor, mu, w.k0)
+            O.oras_precond(h, B, k=40)                     # the shared workspace grows
+            ref = np.stack([O.oras_precond(h, V[j]) for j in range(2)])
+            zd.fill_(complex(np.nan, np.nan))
+            torch.cuda.synchronize()
+            with torch.cuda.stream(stream):
+                graph.replay()
+            torch.cuda.synchronize()
+            got = zd.cpu().numpy()
+            # one column at a time on both sides: the same kernels in the same order; OAS adds with atomics
+            assert rel(got, ref) <= (1e-12 if bits == 64 else (1e-6 if weights else 0.0))
+    finally:
+        O.oras_destroy(h)
