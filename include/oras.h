@@ -67,7 +67,10 @@ enum { ORAS_MEM_HOST = 0, ORAS_MEM_DEVICE = 1 };
 enum { ORAS_WEIGHTS_POU = 0 /* ORAS: R_s^T D_s */, ORAS_WEIGHTS_NONE = 1 /* OAS, Sec. 4 */ };
 enum { ORAS_OVERLAP_VERTEX = 0, ORAS_OVERLAP_FACE = 1 };
 /* Local factorisations.  AUTO: sparse factors, block L D L^T of the complex symmetric A_s over a
- * nested-dissection tree, pivots chosen inside a tree node (at most 128 unknowns, 64 in FP64).
+ * nested-dissection tree, pivots chosen inside a tree node (at most 128 unknowns, 64 in FP64).  A node
+ * whose pivot block is close to singular (a resonance of its interior, a zero pivot) leaves the
+ * unknowns in question to its parent: oras_factor then plans the trees anew and factors again, up to 8
+ * times, and the handle keeps the new trees (oras_arena_bytes may change).
  * CUDA_CORES: dense LU, pivots chosen over whole columns. */
 enum { ORAS_LU_AUTO = 0, ORAS_LU_CUDA_CORES = 1 };
 /* Preconditioner apply with dense FP32 factors (ORAS_LU_CUDA_CORES): AUTO streams the factor arena
@@ -367,8 +370,9 @@ int oras_precond(oras_handle* h, const oras_complex* v, oras_complex* z, int32_t
  * this is an interface convenience.  v, z: device pointers (current device = the handle's
  * device), N x k column-major, complex FP64, on the handle's stream; the call is asynchronous.
  * Sparse factors: the local vectors live in a workspace of the handle that oras_factor allocated for
- * this call alone and that stays where it is, so a captured call can be replayed after any other call
- * (calls of this function on one handle that overlap on the GPU race on it).  Dense factors: in one fixed 16 MiB device array
+ * this call alone and that stays where it is, so a captured call can be replayed after other calls
+ * (not after an oras_factor that planned the trees anew, see ORAS_LU_AUTO, or failed; calls of this
+ * function on one handle that overlap on the GPU race on it).  Dense factors: in one fixed 16 MiB device array
  * compiled into the library (every GPU that loads the library holds it until exit).  Either way
  * the sum over subdomains of the padded order times the factor entry size (8 B FP32, 16 B FP64) must
  * be at most 16 MiB, else INVALID_ARG with the needed size.  With the fixed array: the first call on a device resolves the array's device address (cudaGetSymbolAddress); make

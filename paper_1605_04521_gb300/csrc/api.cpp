@@ -3,6 +3,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <complex>
 #include <cstring>
 #include <new>
 #include <string>
@@ -155,7 +156,7 @@ static void dfree_all(Device& d) {
                   d.lu_ipiv, d.lu_diag, d.dinv, d.sub_inv_off, d.status, d.V, d.Zf, d.Zd, d.w, d.xk, d.bk, d.tmp, d.H, d.gcs, d.gsn,
                   d.g, d.red, d.scal, d.ybuf, d.y1, d.io, d.apply_subs,
                   d.fr_nodes, d.fr_border, d.fr_own_src, d.fr_border_src, d.fr_pos, d.fr_row_node, d.fr_row_dof, d.fr_row_pou,
-                  d.fr_assemble, d.fr_lmul, d.fr_schur, d.fr_fwd, d.fr_bwd, d.fr_bwd_multi, d.fr_work, d.fr_c};
+                  d.fr_assemble, d.fr_lmul, d.fr_schur, d.fr_fwd, d.fr_bwd, d.fr_bwd_multi, d.fr_weak, d.fr_work, d.fr_c};
   for (void* p : ptrs)
     if (p) cudaFreeAsync(p, d.stream);
   cudaStreamSynchronize(d.stream);  // the frees have run: the memory is back in the pool
@@ -198,6 +199,31 @@ static bool make_apply_side(oras_handle* h) {
   return false;
 }
 
+// The plan of the sparse factors.
+static int upload_fronts(oras_handle* h) {
+  auto& d = h->dev;
+  d.fr_uploaded = false;  // until all of it is there
+  const Fronts& f = h->fronts;
+  cudaStream_t s = d.stream;
+  CK(dput(d.fr_nodes, f.nodes, s));
+  CK(dput(d.fr_border, f.border, s));
+  CK(dput(d.fr_own_src, f.own_src, s));
+  CK(dput(d.fr_border_src, f.border_src, s));
+  CK(dput(d.fr_pos, f.pos, s));
+  CK(dput(d.fr_row_node, f.row_node, s));
+  CK(dput(d.fr_row_dof, f.row_dof, s));
+  CK(dput(d.fr_row_pou, f.row_pou, s));
+  CK(dput(d.fr_assemble, f.assemble.items, s));
+  CK(dput(d.fr_lmul, f.lmul.items, s));
+  CK(dput(d.fr_schur, f.schur.items, s));
+  CK(dput(d.fr_fwd, f.fwd.items, s));
+  CK(dput(d.fr_bwd, f.bwd.items, s));
+  CK(dput(d.fr_bwd_multi, f.bwd_multi.items, s));
+  CK(dalloc(d.fr_weak, f.nodes.size()));
+  d.fr_uploaded = true;
+  return ORAS_OK;
+}
+
 static int upload(oras_handle* h) {
   auto& m = h->mesh;
   auto& d = h->dev;
@@ -228,21 +254,7 @@ static int upload(oras_handle* h) {
   CK(dput(d.member, m.member, s));
   CK(cudaDeviceGetAttribute(&d.num_sms, cudaDevAttrMultiProcessorCount, d.device));
   if (h->fronts.use) {
-    const Fronts& f = h->fronts;
-    CK(dput(d.fr_nodes, f.nodes, s));
-    CK(dput(d.fr_border, f.border, s));
-    CK(dput(d.fr_own_src, f.own_src, s));
-    CK(dput(d.fr_border_src, f.border_src, s));
-    CK(dput(d.fr_pos, f.pos, s));
-    CK(dput(d.fr_row_node, f.row_node, s));
-    CK(dput(d.fr_row_dof, f.row_dof, s));
-    CK(dput(d.fr_row_pou, f.row_pou, s));
-    CK(dput(d.fr_assemble, f.assemble.items, s));
-    CK(dput(d.fr_lmul, f.lmul.items, s));
-    CK(dput(d.fr_schur, f.schur.items, s));
-    CK(dput(d.fr_fwd, f.fwd.items, s));
-    CK(dput(d.fr_bwd, f.bwd.items, s));
-    CK(dput(d.fr_bwd_multi, f.bwd_multi.items, s));
+    if (int rc = upload_fronts(h)) return rc;
   } else {
     std::vector<int64_t> npoff(m.nsub + 1, 0);
     for (int q = 0; q < m.nsub; ++q) npoff[q + 1] = npoff[q] + m.sub_np[q];
@@ -398,7 +410,7 @@ int64_t footprint_bytes(const oras_handle* h, int k) {
     const Fronts& f = h->fronts;
     for (int64_t x : {vb(f.nodes), vb(f.border), vb(f.own_src), vb(f.border_src), vb(f.pos), vb(f.row_node), vb(f.row_dof),
                       vb(f.row_pou), vb(f.assemble.items), vb(f.lmul.items), vb(f.schur.items), vb(f.fwd.items),
-                      vb(f.bwd.items), vb(f.bwd_multi.items)})
+                      vb(f.bwd.items), vb(f.bwd_multi.items), (int64_t)f.nodes.size()})
       add(x);
     add(f.panel_elems * (int64_t)el);                               // panels
     add(f.panel_elems * (int64_t)el);                               // assembly workspace
@@ -434,9 +446,80 @@ int64_t footprint_bytes(const oras_handle* h, int k) {
 }
 
 static int sync_status(oras_handle* h);
+static int factor_once(oras_handle* h);
 
-// Element matrices, A, local matrices and batched LU from the materials already on the device.
+// The assembled panel of node n, FP64, without padding.
+static int read_panel(oras_handle* h, const FrontNode& n, std::vector<std::complex<double>>& out) {
+  auto& d = h->dev;
+  const size_t count = (size_t)(n.n1 + n.n2) * n.ld;
+  std::vector<std::complex<double>> wide(count);
+  if (d.factor_bits == 64) {
+    CK(cudaMemcpyAsync(wide.data(), (const std::complex<double>*)d.fr_work + n.panel, count * 16, cudaMemcpyDeviceToHost, d.stream));
+    CK(cudaStreamSynchronize(d.stream));
+  } else {
+    std::vector<std::complex<float>> narrow(count);
+    CK(cudaMemcpyAsync(narrow.data(), (const std::complex<float>*)d.fr_work + n.panel, count * 8, cudaMemcpyDeviceToHost, d.stream));
+    CK(cudaStreamSynchronize(d.stream));
+    std::copy(narrow.begin(), narrow.end(), wide.begin());
+  }
+  out.resize((size_t)(n.n1 + n.n2) * n.n1);
+  for (int i = 0; i < n.n1 + n.n2; ++i) std::copy_n(wide.begin() + (size_t)i * n.ld, n.n1, out.begin() + (size_t)i * n.n1);
+  return ORAS_OK;
+}
+
+// After a factorisation that marked nodes (Device::fr_weak): plans the trees anew, with the unknowns that these nodes should
+// not eliminate moved up.  A node above another one that changes waits for the next factorisation, whose entries it is
+// judged by.  moved: false when there is nothing to move.
+static int replan_fronts(oras_handle* h, bool* moved) {
+  auto& d = h->dev;
+  Fronts& f = h->fronts;
+  const int32_t nn = (int32_t)f.nodes.size();
+  std::vector<uint8_t> weak(nn), below(nn, 0);
+  CK(cudaMemcpyAsync(weak.data(), d.fr_weak, weak.size(), cudaMemcpyDeviceToHost, d.stream));
+  CK(cudaStreamSynchronize(d.stream));
+  *moved = false;
+  std::vector<std::vector<int32_t>> moves(nn);
+  std::vector<std::complex<double>> panel;
+  for (int32_t g = 0; g < nn; ++g) {  // children first
+    const FrontNode& n = f.nodes[g];
+    for (int32_t c : n.child)
+      if (c >= 0 && (below[c] || !moves[c].empty())) below[g] = 1;
+    if (!weak[g] || below[g] || n.n2 == 0) continue;
+    if (int rc = read_panel(h, n, panel)) return rc;
+    if (!weak_unknowns(n.n1, n.n2, panel, moves[g])) {
+      h->err = "local matrix of subdomain " + std::to_string(n.sub) + " has a zero pivot column";
+      return ORAS_ERR_SINGULAR_LOCAL;
+    }
+    *moved |= !moves[g].empty();
+  }
+  if (!*moved) return ORAS_OK;
+  delay_unknowns(h->mesh, h->opt.factor_bits, moves, f);
+  h->factored = false;       // the factors and the plan that captured steps use are given back
+  h->graph_stream = nullptr;
+  h->graph_m = 0;
+  free_factor_space(d);
+  if (int rc = upload_fronts(h)) return rc;
+  return alloc_factor_space(h, h->opt.factor_bits);
+}
+
+// Element matrices, A, local matrices and their factors from the materials already on the device.
 static int factor_device(oras_handle* h) {
+  for (int attempt = 0;; ++attempt) {
+    int rc = factor_once(h);
+    if (!h->fronts.use || (rc != ORAS_OK && rc != ORAS_ERR_SINGULAR_LOCAL)) return rc;
+    if (((const int32_t*)(h->dev.host_pinned + PINNED_STATUS_OFF))[ST_WEAK] == 0 || attempt == FR_REPLANS) return rc;
+    bool moved = false;
+    try {
+      if (int rc2 = replan_fronts(h, &moved)) return rc2;
+    } catch (const std::exception& e) {
+      h->err = std::string("planning the local factorisations anew: ") + e.what();
+      return ORAS_ERR_OUT_OF_MEMORY;
+    }
+    if (!moved) return rc;
+  }
+}
+
+static int factor_once(oras_handle* h) {
   auto& d = h->dev;
   const double k0 = h->k0;
   CK(cudaMemsetAsync(d.status, 0, 8 * sizeof(int32_t), d.stream));
@@ -588,6 +671,10 @@ int oras_factor(oras_handle* h, const oras_complex* eps_r, const oras_complex* m
   auto& d = h->dev;
   if (!d.uploaded) {
     int rc = upload(h);
+    if (rc) return rc;
+  }
+  if (h->fronts.use && !d.fr_uploaded) {  // planned anew, then out of memory
+    int rc = upload_fronts(h);
     if (rc) return rc;
   }
   int rc = alloc_factor_space(h, h->opt.factor_bits);

@@ -10,8 +10,11 @@
 //   k_fr_assemble  the children's C added to the panels (originals are scattered once, k_fr_rows);
 //   k_fr_invert    S by blocked Gauss-Jordan with row pivoting, the block held in registers;
 //   k_fr_mul, k_fr_mul_tc (fronts_tc.cu)  L, then C with the children's C gathered into it (each C is read once).
-// Pivots are chosen inside a pivot block (up to front_nb unknowns) and never outside it, so the tree
-// stays as planned.
+// Pivots are chosen inside a pivot block (up to front_nb unknowns) and never outside it.  Where that is not enough (a
+// zero pivot, or an entry of L above FR_GROWTH) the node is marked; the host then moves the unknowns in question to the
+// node's parent, plans the trees anew and factors again (fronts_weak.cpp, oras_factor).  FP32, one subdomain of 6^3 x 6,
+// degree 2, at the resonance of a leaf: without it the apply's error is 1e4 and nothing converges; with it 3e-6, one more
+// factorisation.
 //
 // Against dense factors of the same matrices (n_s^2 entries each) the largest subdomain of the
 // 16^3 x 6, degree-2, 64-subdomain problem (17,896 unknowns) keeps 2% of the entries and needs 0.1%
@@ -27,7 +30,7 @@ void launch_front_mul_tc(const oras_handle* h, const FrDev& f, bool schur, const
 
 static FrDev fr_dev(const oras_handle* h) {
   const auto& d = h->dev;
-  return {d.fr_nodes, d.fr_border, d.fr_own_src, d.fr_border_src};
+  return {d.fr_nodes, d.fr_border, d.fr_own_src, d.fr_border_src, d.fr_weak};
 }
 
 // ------------------------------------------------------------------ original entries
@@ -163,7 +166,7 @@ __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 // pivot.
 template <typename R, int NB>
 __device__ __forceinline__ void invert_panel(InvShared<R, NB>& sh, int c0, int rows, int buf, bool& taken, int n2,
-                                             int sub, int32_t* status) {
+                                             int sub, const FrDev& f, int node, int32_t* status) {
   constexpr int PW = NB / 32;
   const int lane = threadIdx.x & 31, pw = (threadIdx.x >> 5) % PW, i = 32 * pw + lane;
   CT<R> x[8];
@@ -208,10 +211,11 @@ __device__ __forceinline__ void invert_panel(InvShared<R, NB>& sh, int c0, int r
     if (pv.re != R(0) || pv.im != R(0)) {
       const R rden = recip(pv.re * pv.re + pv.im * pv.im);
       inv = {pv.re * rden, -pv.im * rden};
-    } else if (n2 > 0 && sh.amax > 0.0f) {
-      // an exactly zero pivot column: the unknowns eliminated later can still make A_s regular, so the
-      // pivot is taken as the rounding of the block's entries
-      inv.re = R(1) / (R(sh.amax) * (sizeof(R) == 4 ? R(1.0 / (1 << 20)) : R(1.0 / (1ll << 45))));
+    } else if (n2 > 0) {
+      // an exactly zero pivot column: the unknowns eliminated later can still make A_s regular.  The node is planned
+      // anew; where that does not help, the pivot is taken as the rounding of the block's entries
+      if (sh.amax > 0.0f) inv.re = R(1) / (R(sh.amax) * (sizeof(R) == 4 ? R(1.0 / (1 << 20)) : R(1.0 / (1ll << 45))));
+      if (own) mark_weak(f, node, status);
     } else if (own) {
       if (atomicCAS(&status[ST_ERR], DEV_OK, DEV_SINGULAR) == DEV_OK) status[ST_SUB] = sub;
     }
@@ -353,7 +357,7 @@ __global__ void __launch_bounds__(NW * 32 + NB, BLOCKS)
     __syncthreads();  // amax and the first panel
     for (int p = 0; p < np; ++p) {
       if (p > 0) named_sync(INV_BAR_PANEL, ALL);
-      invert_panel<R, NB>(sh, 8 * p, 8 * np, p & 1, taken, n.n2, n.sub, status);
+      invert_panel<R, NB>(sh, 8 * p, 8 * np, p & 1, taken, n.n2, n.sub, f, first + blockIdx.x, status);
       named_arrive(INV_BAR_W, ALL);
     }
     __syncthreads();
@@ -406,7 +410,7 @@ __global__ void __launch_bounds__(NW * 32 + NB, BLOCKS)
 //   SCHUR = true:  C = pulled children - L A21^T, tiles on and below the diagonal
 template <typename R, bool SCHUR>
 __global__ void __launch_bounds__(256) k_fr_mul(FrDev f, const FrontItem* __restrict__ items, CT<R>* __restrict__ work,
-                                                CT<R>* __restrict__ fac, CT<R>* __restrict__ C) {
+                                                CT<R>* __restrict__ fac, CT<R>* __restrict__ C, int32_t* status) {
   constexpr int KC = 8, LDS = FR_TILE + 2;
   __shared__ __align__(16) CT<R> As[KC][LDS], Bs[KC][LDS];
   const FrontItem it = items[blockIdx.x];
@@ -479,6 +483,7 @@ __global__ void __launch_bounds__(256) k_fr_mul(FrDev f, const FrontItem* __rest
         const CT<R> v = pull<R>(f, n, C, si, sj[q]);
         C[n.cblk + (int64_t)i * n.ldc + j] = {v.re - acc[p][q].re, v.im - acc[p][q].im};
       } else if (j < ld) {  // columns n1 .. ld-1 are written as zeros
+        if (grown((float)acc[p][q].re, (float)acc[p][q].im)) mark_weak(f, it.node, status);
         fac[n.panel + (int64_t)(n1 + i) * ld + j] = acc[p][q];
       }
     }
@@ -514,6 +519,7 @@ static int factor_t(oras_handle* h) {
   CT<R>* fac = (CT<R>*)d.arena;
   CT<R>* C = (CT<R>*)d.fr_c;
   cudaStream_t st = d.stream;
+  if (cudaMemsetAsync(d.fr_weak, 0, f.nodes.size(), st) != cudaSuccess) return -1;
   for (int l = 0; l < f.nlev(); ++l) {
     auto count = [&](const FrontLevels& v) { return (unsigned)(v.ptr[l + 1] - v.ptr[l]); };
     int pb = prof_begin(h);
@@ -548,7 +554,7 @@ static int factor_t(oras_handle* h) {
       if constexpr (sizeof(R) == 4) {
         launch_front_mul_tc(h, fd, false, d.fr_lmul + f.lmul.ptr[l], count(f.lmul));
       } else {
-        k_fr_mul<R, false><<<count(f.lmul), 256, 0, st>>>(fd, d.fr_lmul + f.lmul.ptr[l], work, fac, C);
+        k_fr_mul<R, false><<<count(f.lmul), 256, 0, st>>>(fd, d.fr_lmul + f.lmul.ptr[l], work, fac, C, d.status);
         count_launches(1);
       }
     }
@@ -557,7 +563,7 @@ static int factor_t(oras_handle* h) {
     if constexpr (sizeof(R) == 4) {
       launch_front_mul_tc(h, fd, true, d.fr_schur + f.schur.ptr[l], count(f.schur));
     } else {
-      k_fr_mul<R, true><<<count(f.schur), 256, 0, st>>>(fd, d.fr_schur + f.schur.ptr[l], work, fac, C);
+      k_fr_mul<R, true><<<count(f.schur), 256, 0, st>>>(fd, d.fr_schur + f.schur.ptr[l], work, fac, C, d.status);
       count_launches(1);
     }
     prof_end(h, KC_LU_UPDATE, pb, 1);

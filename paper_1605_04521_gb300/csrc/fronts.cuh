@@ -11,7 +11,15 @@ struct FrDev {
   const int32_t* border;
   const FrontSrc* own_src;
   const FrontSrc* border_src;
+  uint8_t* weak;
 };
+
+// Node g needs some of its unknowns eliminated later.
+__device__ __forceinline__ void mark_weak(const FrDev& f, int g, int32_t* status) {
+  f.weak[g] = 1;
+  status[ST_WEAK] = 1;
+}
+__device__ __forceinline__ bool grown(float re, float im) { return !(fmaxf(fabsf(re), fabsf(im)) <= FR_GROWTH); }
 
 __device__ __forceinline__ FrontSrc front_src(const FrDev& f, const FrontNode& n, int i) {
   return i < n.n1 ? f.own_src[n.row0 + i] : f.border_src[n.bord + i - n.n1];

@@ -2,6 +2,7 @@
 // the host set-up (fronts_plan.cpp), the numeric kernels (fronts.cu) and the apply (fronts_apply.cu).
 #pragma once
 
+#include <complex>
 #include <cstdint>
 #include <vector>
 
@@ -64,9 +65,23 @@ struct Fronts {
   int nlev() const { return (int)multi_cols.size(); }
 };
 
+// Largest entry of L = A21 A11^{-1} that the factorisation takes as it is.  Ordinary trees stay below 7 (degrees 1 to 3,
+// with and without losses, k0 from 0.01 to 9); the apply's error is the unit roundoff times its square: at 64 1e-4 in
+// FP32 and 1e-12 in FP64.
+constexpr float FR_GROWTH = 64.0f;
+constexpr int FR_REPLANS = 8;   // times a factorisation plans the trees anew before it takes what it has
+
 struct HostMesh;
 // Elimination trees of every subdomain of m for factors of the given precision (dirichlet: of the
 // matrices R_s A R_s^T).
 void build_fronts(const HostMesh& m, int factor_bits, bool dirichlet, Fronts& f);
+
+// The own unknowns of a node that its parent should eliminate, so that no entry of L exceeds FR_GROWTH (fronts_weak.cpp).
+// panel: [n1 + n2][n1] the assembled A11 over A21.  false: an own unknown has no coupling left, A_s is singular.
+bool weak_unknowns(int n1, int n2, const std::vector<std::complex<double>>& panel, std::vector<int32_t>& out);
+
+// The plan with own unknowns moves[g] (indices into node g's own) of every node eliminated by the next ancestor that has
+// room, or by a new root.
+void delay_unknowns(const HostMesh& m, int factor_bits, const std::vector<std::vector<int32_t>>& moves, Fronts& f);
 
 }  // namespace oras

@@ -109,7 +109,6 @@ struct Builder {
     }
     std::vector<int32_t> border, roots;
     dissect(0, (int32_t)nt, border, roots);
-    number(ns);
   }
 
   void link(LocalNode& x, const std::vector<int32_t>& children) {
@@ -249,59 +248,39 @@ struct Builder {
       return cx < cy || (cx == cy && x < y);
     });
   }
-
-  // Elimination positions (nodes in creation order: children first), borders as ascending positions,
-  // and where each front is in the children's borders.
-  std::vector<int32_t> pos;
-  void number(int64_t ns) {
-    pos.assign(ns, -1);
-    int32_t p = 0;
-    for (auto& x : nodes) {
-      x.p0 = p;
-      for (int32_t u : x.own) pos[u] = p++;
-    }
-    for (auto& x : nodes) {
-      for (int32_t& u : x.border) u = pos[u];
-      std::sort(x.border.begin(), x.border.end());
-    }
-    for (auto& x : nodes) {
-      const int n1 = (int)x.own.size(), n2 = (int)x.border.size();
-      auto front = [&](int i) { return i < n1 ? x.p0 + i : x.border[i - n1]; };
-      x.src.assign(n1 + n2, {-1, -1});
-      for (int c = 0; c < 2; ++c) {
-        if (x.child[c] < 0) continue;
-        const auto& cb = nodes[x.child[c]].border;
-        size_t k = 0;
-        for (int i = 0; i < n1 + n2 && k < cb.size(); ++i)
-          if (cb[k] == front(i)) (c == 0 ? x.src[i].a : x.src[i].b) = (int32_t)k++;
-      }
-    }
-  }
 };
 
-}  // namespace
-
-void build_fronts(const HostMesh& m, int factor_bits, bool dirichlet, Fronts& f) {
-  const int nb = front_nb(factor_bits);
-  const int64_t rows = m.sub_ns_off[m.nsub];
-  f.pos.resize(rows);
-  std::vector<std::vector<LocalNode>> trees(m.nsub);
-  const int nw = workers_for(m.nsub, 1);
-  std::vector<std::vector<int32_t>> loc(nw);
-  std::vector<std::unique_ptr<Builder>> builders(nw);
-  parallel_for(m.nsub, 1, [&](int64_t s64, int w) {
-    const int s = (int)s64;
-    if (!builders[w]) {
-      builders[w] = std::make_unique<Builder>(m, nb);
-      loc[w].assign(m.ndof, 0);
+// Elimination positions (nodes in order: children first), borders as ascending positions, and where each front is
+// in the children's borders.  pos: [ns] position of every local unknown.
+void number(std::vector<LocalNode>& nodes, int64_t ns, std::vector<int32_t>& pos) {
+  pos.assign(ns, -1);
+  int32_t p = 0;
+  for (auto& x : nodes) {
+    x.p0 = p;
+    for (int32_t u : x.own) pos[u] = p++;
+  }
+  for (auto& x : nodes) {
+    for (int32_t& u : x.border) u = pos[u];
+    std::sort(x.border.begin(), x.border.end());
+  }
+  for (auto& x : nodes) {
+    const int n1 = (int)x.own.size(), n2 = (int)x.border.size();
+    auto front = [&](int i) { return i < n1 ? x.p0 + i : x.border[i - n1]; };
+    x.src.assign(n1 + n2, {-1, -1});
+    for (int c = 0; c < 2; ++c) {
+      if (x.child[c] < 0) continue;
+      const auto& cb = nodes[x.child[c]].border;
+      size_t k = 0;
+      for (int i = 0; i < n1 + n2 && k < cb.size(); ++i)
+        if (cb[k] == front(i)) (c == 0 ? x.src[i].a : x.src[i].b) = (int32_t)k++;
     }
-    const int64_t off = m.sub_ns_off[s], ns = m.sub_ns[s];
-    for (int64_t i = 0; i < ns; ++i) loc[w][m.sub_dofs[off + i]] = (int32_t)i;
-    Builder& b = *builders[w];
-    b.run(s, loc[w], dirichlet);
-    std::copy(b.pos.begin(), b.pos.end(), f.pos.begin() + off);
-    trees[s] = std::move(b.nodes);
-  });
+  }
+}
+
+// The plan of all subdomains' numbered trees: node order, offsets, the rows' and borders' arrays, the blocks of every
+// level.  f.pos is there.
+void lay_out(const HostMesh& m, int factor_bits, const std::vector<std::vector<LocalNode>>& trees, Fronts& f) {
+  const int64_t rows = m.sub_ns_off[m.nsub];
   // global node order: by level, wide pivot blocks first, then the larger fronts
   struct Key { int32_t level, wide, cost, sub, id; };
   std::vector<Key> keys;
@@ -421,6 +400,98 @@ void build_fronts(const HostMesh& m, int factor_bits, bool dirichlet, Fronts& f)
     }
     for (auto* v : all) v->ptr.push_back((int64_t)v->items.size());
   }
+}
+
+}  // namespace
+
+void build_fronts(const HostMesh& m, int factor_bits, bool dirichlet, Fronts& f) {
+  const int nb = front_nb(factor_bits);
+  const int64_t rows = m.sub_ns_off[m.nsub];
+  f.pos.resize(rows);
+  std::vector<std::vector<LocalNode>> trees(m.nsub);
+  const int nw = workers_for(m.nsub, 1);
+  std::vector<std::vector<int32_t>> loc(nw), pos(nw);
+  std::vector<std::unique_ptr<Builder>> builders(nw);
+  parallel_for(m.nsub, 1, [&](int64_t s64, int w) {
+    const int s = (int)s64;
+    if (!builders[w]) {
+      builders[w] = std::make_unique<Builder>(m, nb);
+      loc[w].assign(m.ndof, 0);
+    }
+    const int64_t off = m.sub_ns_off[s], ns = m.sub_ns[s];
+    for (int64_t i = 0; i < ns; ++i) loc[w][m.sub_dofs[off + i]] = (int32_t)i;
+    Builder& b = *builders[w];
+    b.run(s, loc[w], dirichlet);
+    number(b.nodes, ns, pos[w]);
+    std::copy(pos[w].begin(), pos[w].end(), f.pos.begin() + off);
+    trees[s] = std::move(b.nodes);
+  });
+  lay_out(m, factor_bits, trees, f);
+}
+
+// The trees behind a plan, named by local unknowns again.
+static std::vector<std::vector<LocalNode>> trees_of(const HostMesh& m, const Fronts& f, std::vector<int32_t>& local) {
+  std::vector<std::vector<LocalNode>> trees(m.nsub);
+  local.resize(f.nodes.size());
+  std::vector<int32_t> unknown(m.sub_ns_off[m.nsub]);  // at each position, index into N_s
+  for (int s = 0; s < m.nsub; ++s)
+    for (int64_t i = 0; i < m.sub_ns[s]; ++i) unknown[m.sub_ns_off[s] + f.pos[m.sub_ns_off[s] + i]] = (int32_t)i;
+  for (int l = 0; l < f.nlev(); ++l)
+    for (int32_t g = f.level_ptr[l]; g < f.level_ptr[l + 1]; ++g) {
+      const FrontNode& n = f.nodes[g];
+      LocalNode x;
+      x.own.assign(unknown.begin() + n.row0, unknown.begin() + n.row0 + n.n1);
+      for (int q = 0; q < n.n2; ++q) x.border.push_back(unknown[f.border[n.bord + q]]);
+      for (int q = 0; q < 2; ++q) x.child[q] = n.child[q] < 0 ? -1 : local[n.child[q]];
+      x.level = l;
+      local[g] = (int32_t)trees[n.sub].size();
+      trees[n.sub].push_back(std::move(x));
+    }
+  return trees;
+}
+
+void delay_unknowns(const HostMesh& m, int factor_bits, const std::vector<std::vector<int32_t>>& moves, Fronts& f) {
+  const size_t nb = front_nb(factor_bits);
+  std::vector<int32_t> local;
+  auto trees = trees_of(m, f, local);
+  std::vector<std::vector<int32_t>> parent(m.nsub);
+  for (int s = 0; s < m.nsub; ++s) {
+    parent[s].assign(trees[s].size(), -1);
+    for (size_t q = 0; q < trees[s].size(); ++q)
+      for (int32_t c : trees[s][q].child)
+        if (c >= 0) parent[s][c] = (int32_t)q;
+  }
+  for (size_t g = 0; g < f.nodes.size(); ++g) {
+    auto& tree = trees[f.nodes[g].sub];
+    auto& up = parent[f.nodes[g].sub];
+    std::vector<int32_t> x;  // unknowns that leave the node
+    for (int32_t i : moves[g]) x.push_back(tree[local[g]].own[i]);
+    for (int32_t u : x) {
+      int32_t q = local[g];
+      tree[q].own.erase(std::find(tree[q].own.begin(), tree[q].own.end(), u));
+      // every node on the way has it in its border, and so in its front
+      for (;;) {
+        tree[q].border.push_back(u);
+        if (up[q] < 0) {  // above the root: a node of its own
+          LocalNode r;
+          r.child[0] = q;
+          r.level = tree[q].level + 1;
+          up[q] = (int32_t)tree.size();
+          up.push_back(-1);
+          tree.push_back(std::move(r));
+        }
+        q = up[q];
+        if (tree[q].own.size() < nb) break;
+      }
+      tree[q].own.push_back(u);
+    }
+  }
+  parallel_for(m.nsub, 1, [&](int64_t s, int) {
+    std::vector<int32_t> pos;
+    number(trees[s], m.sub_ns[s], pos);
+    std::copy(pos.begin(), pos.end(), f.pos.begin() + m.sub_ns_off[s]);
+  });
+  lay_out(m, factor_bits, trees, f);
 }
 
 }  // namespace oras

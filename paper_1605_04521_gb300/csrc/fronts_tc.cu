@@ -243,15 +243,20 @@ __global__ void __launch_bounds__(FT_THREADS, 2) k_fr_mul_tc(FrDev f, const Fron
         }
       }
     } else {
+      bool weak = false;
       for (int r = warp; r < FT_ROWS; r += FT_THREADS / 32) {
         const int i = i0 + r;
         if (i >= n2) break;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const int j = j0 + lane + 32 * q;
-          if (j < ld) fac[n.panel + (int64_t)(n1 + i) * ld + j] = D[r * FT_LDD + lane + 32 * q];  // zeros past n1
+          const CT<float> v = D[r * FT_LDD + lane + 32 * q];
+          if (j >= ld) continue;
+          fac[n.panel + (int64_t)(n1 + i) * ld + j] = v;  // zeros past n1
+          weak |= grown(v.re, v.im);
         }
       }
+      if (weak) mark_weak(f, it.node, status);
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

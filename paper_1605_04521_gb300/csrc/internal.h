@@ -25,8 +25,8 @@ constexpr int PINNED_STATUS_OFF = 2048;   // pinned scratch: doubles [2048, 2052
 
 struct cplx { double re, im; };
 
-// device status flags (Device::status): [0] error code, [1] detail, [2] subdomain
-enum { ST_ERR = 0, ST_DETAIL = 1, ST_SUB = 2 };
+// device status flags (Device::status): [0] error code, [1] detail, [2] subdomain, [3] some node is in Device::fr_weak
+enum { ST_ERR = 0, ST_DETAIL = 1, ST_SUB = 2, ST_WEAK = 3 };
 enum { DEV_OK = 0, DEV_SINGULAR = 1, DEV_TIMEOUT = 2, DEV_BADINDEX = 3 };
 
 
@@ -181,6 +181,8 @@ struct Device {
   uint8_t* fr_row_pou = nullptr;
   FrontItem* fr_assemble = nullptr; FrontItem* fr_lmul = nullptr; FrontItem* fr_schur = nullptr;
   FrontItem* fr_fwd = nullptr; FrontItem* fr_bwd = nullptr; FrontItem* fr_bwd_multi = nullptr;
+  bool fr_uploaded = false;
+  uint8_t* fr_weak = nullptr;                   // [nodes] 1: a zero pivot or a large entry of L (fronts_weak.cpp)
   void* fr_work = nullptr; void* fr_c = nullptr;
   cplx* io = nullptr;                           // staging for host I/O [N][k] col-major
   size_t io_elems = 0;

@@ -4,6 +4,7 @@
 // program with a message; one that is too small is found by its guard bytes.
 //
 // usage: fake_device <scenario>; prints one line a finding, exits 0 when there is none.
+#include <algorithm>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
@@ -109,7 +110,31 @@ int launch_global_rows(const oras_handle* h, double) {
   return 0;
 }
 void launch_split_vals(const oras_handle* h) { touch("A in FP32 pairs", h->dev.vals_df, h->mesh.cols.size() * 16); }
+// What the factorisations find: nodes that should not eliminate their first unknown, in the first g_weak of them.
+static int g_weak = 0;
+static void plan_is_there(const oras_handle* h) {
+  const auto& f = h->fronts;
+  const auto& d = h->dev;
+  auto same = [](const char* what, const void* dev, const auto& host) {
+    auto it = g_live.find(const_cast<void*>(dev));
+    const size_t bytes = host.size() * sizeof(host[0]);
+    if (it == g_live.end() || it->second < bytes || (bytes && std::memcmp(dev, host.data(), bytes))) {
+      std::printf("a launch uses %s, which is not the plan's\n", what);
+      std::exit(3);
+    }
+  };
+  same("nodes", d.fr_nodes, f.nodes);
+  same("borders", d.fr_border, f.border);
+  same("sources", d.fr_own_src, f.own_src);
+  same("sources", d.fr_border_src, f.border_src);
+  same("positions", d.fr_pos, f.pos);
+  same("row nodes", d.fr_row_node, f.row_node);
+  same("row unknowns", d.fr_row_dof, f.row_dof);
+  same("row weights", d.fr_row_pou, f.row_pou);
+  same("blocks", d.fr_bwd_multi, f.bwd_multi.items);
+}
 int launch_front_rows(const oras_handle* h, double) {
+  plan_is_there(h);
   touch("the assembly workspace", h->dev.fr_work, (size_t)h->fronts.panel_elems * entry(h));
   return 0;
 }
@@ -118,6 +143,22 @@ int launch_front_factor(oras_handle* h) {
   touch("the factors", h->dev.arena, (size_t)h->fronts.panel_elems * entry(h));
   touch("the contribution blocks", h->dev.fr_c, (size_t)h->fronts.c_elems * entry(h));
   touch("the vectors of the allocation-free apply", h->dev.y1, apply_yglob_bytes_for(h, 1));
+  touch("the marks", h->dev.fr_weak, h->fronts.nodes.size());
+  if (g_weak > 0) {
+    --g_weak;
+    for (size_t g = 0; g < h->fronts.nodes.size(); g += 3) {
+      const FrontNode& n = h->fronts.nodes[g];
+      if (n.n1 == 0 || n.n2 == 0) continue;
+      auto put = [&](int i, int j, float v) {  // identity, but for a small pivot that couples to the border
+        if (h->opt.factor_bits == 64) ((cplx*)h->dev.fr_work)[n.panel + (int64_t)i * n.ld + j] = {v, 0.0};
+        else ((float*)h->dev.fr_work)[2 * (n.panel + (int64_t)i * n.ld + j)] = v;
+      };
+      for (int i = 0; i < n.n1; ++i) put(i, i, i == 0 ? 1e-6f : 1.0f);
+      put(n.n1, 0, 1.0f);
+      h->dev.fr_weak[g] = 1;
+      h->dev.status[ST_WEAK] = 1;
+    }
+  }
   return 0;
 }
 int launch_local_rows(const oras_handle* h, double) {
@@ -207,13 +248,101 @@ static std::string at(const char* what, int64_t n, int rc) {
   return std::string(what) + " (allocation " + std::to_string(n) + " refused, code " + std::to_string(rc) + ")";
 }
 
+// The trees of a handle: every local unknown in one node, what a node hands up is in its parent's front, and
+// unknowns that share a tetrahedron are in the front of the one that is eliminated first.  Non-zero: a finding.
+static int check_trees(const oras_handle* h) {
+  const auto& m = h->mesh;
+  const auto& f = h->fronts;
+  const int before = g_bad;
+  std::vector<int> seen(m.sub_ns_off[m.nsub], 0);
+  std::vector<int32_t> level(f.nodes.size());
+  for (int l = 0; l < f.nlev(); ++l)
+    for (int32_t g = f.level_ptr[l]; g < f.level_ptr[l + 1]; ++g) level[g] = l;
+  auto front = [&](int32_t g) {
+    const FrontNode& n = f.nodes[g];
+    std::vector<int32_t> v;
+    for (int i = 0; i < n.n1; ++i) v.push_back(n.row0 + i);
+    v.insert(v.end(), f.border.begin() + n.bord, f.border.begin() + n.bord + n.n2);
+    return v;
+  };
+  for (size_t g = 0; g < f.nodes.size(); ++g) {
+    const FrontNode& n = f.nodes[g];
+    if (n.n1 > front_nb(h->opt.factor_bits)) bad("a pivot block is too wide");
+    for (int i = 0; i < n.n1; ++i) {
+      ++seen[n.row0 + i];
+      if (f.row_node[n.row0 + i] != (int32_t)g) bad("a row's node is wrong");
+    }
+    const auto mine = front((int32_t)g);
+    if (!std::is_sorted(mine.begin(), mine.end())) bad("a front does not ascend");
+    for (int q = 0; q < 2; ++q) {
+      if (n.child[q] < 0) continue;
+      if (level[n.child[q]] >= level[g]) bad("a child is not below its parent");
+      const FrontNode& c = f.nodes[n.child[q]];
+      std::vector<int> used(c.n2, 0);
+      for (int i = 0; i < n.n1 + n.n2; ++i) {
+        const FrontSrc s = i < n.n1 ? f.own_src[n.row0 + i] : f.border_src[n.bord + i - n.n1];
+        const int32_t at = q == 0 ? s.a : s.b;
+        if (at < 0) continue;
+        if (at < c.bord || at >= c.bord + c.n2 || f.border[at] != mine[i]) bad("a source is wrong");
+        else ++used[at - c.bord];
+      }
+      for (int u : used)
+        if (u != 1) bad("a border entry is not handed up once");
+    }
+  }
+  for (int v : seen)
+    if (v != 1) { bad("an unknown is not eliminated once"); break; }
+  for (int s = 0; s < m.nsub; ++s) {
+    const int64_t off = m.sub_ns_off[s];
+    const int32_t* Ns = m.sub_dofs.data() + off;
+    for (int64_t q = m.sub_nt_off[s]; q < m.sub_nt_off[s + 1]; ++q) {
+      std::vector<int32_t> p;
+      for (int a = 0; a < m.nl; ++a)
+        p.push_back((int32_t)(off + f.pos[off + (std::lower_bound(Ns, Ns + m.sub_ns[s], m.dofmap[(int64_t)m.sub_tets[q] * m.nl + a]) - Ns)]));
+      for (int32_t u : p) {
+        const auto v = front(f.row_node[u]);
+        for (int32_t w : p)
+          if (w > u && !std::binary_search(v.begin(), v.end(), w)) { bad("a coupling has no place"); return 1; }
+      }
+    }
+  }
+  return g_bad != before;
+}
+
+// Unknowns of random nodes moved up, again and again: the trees stay trees, full nodes pass them on, roots grow.
+static void delay(int n, int r, int nsub, int bits) {
+  Cube c(n, r, nsub);
+  oras_options o{};
+  o.factor_bits = bits;
+  oras_handle* h = nullptr;
+  if (oras_create(&c.p, &o, &h) != ORAS_OK) { bad("oras_create failed"); return; }
+  check_trees(h);
+  uint32_t seed = 12345;
+  auto rnd = [&]() { return (seed = seed * 1664525u + 1013904223u) >> 8; };
+  const int levels = h->fronts.nlev();
+  for (int round = 0; round < 6 && !g_bad; ++round) {
+    std::vector<std::vector<int32_t>> moves(h->fronts.nodes.size());
+    for (size_t g = 0; g < moves.size(); ++g) {
+      const FrontNode& x = h->fronts.nodes[g];
+      if (x.n2 == 0 || x.n1 == 0 || rnd() % 3) continue;
+      const int first = rnd() % x.n1, count = round == 5 ? x.n1 : 1 + rnd() % 3;  // at last whole nodes
+      for (int i = 0; i < count && i < x.n1; ++i) moves[g].push_back((first + i) % x.n1);
+    }
+    delay_unknowns(h->mesh, bits, moves, h->fronts);
+    check_trees(h);
+  }
+  if (h->fronts.nlev() <= levels) bad("no root grew: the scenario is too small");
+  oras_destroy(h);
+}
+
 // oras_factor with every allocation from the n-th on refused, then again with memory, for every n.
-static void factor_again(int bits, int engine) {
+static void factor_again(int bits, int engine, int weak = 0) {
   Cube c(3, 2, 4);
   oras_options o{};
   o.factor_bits = bits;
   o.lu_engine = engine;
   for (int64_t n = 0;; ++n) {
+    oras::g_weak = weak;
     oras_handle* h = nullptr;
     if (oras_create(&c.p, &o, &h) != ORAS_OK) { bad("oras_create failed"); return; }
     g_count = 0;
@@ -222,6 +351,8 @@ static void factor_again(int bits, int engine) {
     g_refuse_from = -1;
     const bool refused = rc != ORAS_OK;
     if (refused && rc != ORAS_ERR_OUT_OF_MEMORY) bad(at("not reported as out of memory", n, rc));
+    if (refused && h->factored) bad(at("factors that are not there count as there", n, rc));
+    if (weak && !refused && (oras::g_weak || check_trees(h))) bad("the trees were not planned anew as they should");
     if (refused && (rc = oras_factor(h, c.eps.data(), nullptr, c.p.k0, ORAS_MEM_HOST)) != ORAS_OK)
       bad(at("oras_factor fails with memory again", n, rc));
     oras_destroy(h);
@@ -282,6 +413,11 @@ int main(int argc, char** argv) {
   const std::string s = argc > 1 ? argv[1] : "";
   if (s == "factor32") factor_again(32, ORAS_LU_AUTO);
   else if (s == "factor64") factor_again(64, ORAS_LU_AUTO);
+  else if (s == "factor_weak32") factor_again(32, ORAS_LU_AUTO, 2);
+  else if (s == "factor_weak64") factor_again(64, ORAS_LU_AUTO, 2);
+  else if (s == "delay1") delay(4, 1, 5, 64);
+  else if (s == "delay2") delay(5, 2, 2, 32);
+  else if (s == "delay3") delay(3, 3, 3, 32);
   else if (s == "factor_dense") factor_again(32, ORAS_LU_CUDA_CORES);
   else if (s == "setup") setup_fails(ORAS_LU_AUTO);
   else if (s == "setup_dense") setup_fails(ORAS_LU_CUDA_CORES);

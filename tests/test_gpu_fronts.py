@@ -181,3 +181,55 @@ def test_captured_noalloc_apply_outlives_larger_calls(O, bits, weights):
             assert rel(got, ref) <= (1e-12 if bits == 64 else (1e-6 if weights else 0.0))
     finally:
         O.oras_destroy(h)
+
+
+# Lossless unit cubes at the frequency at which the interior of a tree node, its border held at zero, resonates: the lowest
+# eigenvalue of (K, M) on the node's unknowns, for the trees of FP32 (a node of 82 unknowns) and FP64 (one of 42).
+RESONANT = {32: 6.696048910007606, 64: 9.811005223139103}
+
+
+@pytest.mark.parametrize("off", [0.0, 1e-9, 1e-7, 1e-5])
+@pytest.mark.parametrize("bits", [32, 64])
+def test_resonating_tree_node(O, bits, off):
+    """A pivot block that is singular to rounding although A_s is not: the trees are planned anew (the factors take another
+    size then), the apply stays as exact as elsewhere without losses, and one subdomain still solves at once.  New
+    materials and back on the same handle."""
+    xyz, tets = synth.kuhn_cube(6)
+    nt, k0 = len(tets), RESONANT[bits] * (1.0 + off)
+    eps, mu = np.full(nt, 4.0 + 0j), np.ones(nt, complex)
+    p = problem.build(xyz, tets, eps, mu, k0, 2, [("dipole", np.array([0.31, 0.45, 0.52]), np.array([0.0, 0.0, 1.0]))],
+                      nsub=1, delta=0)
+    rng = np.random.default_rng(3)
+    v = rng.normal(size=p.topo.ndof) + 1j * rng.normal(size=p.topo.ndof)
+    z = p.oras.apply(v)
+    h = O.oras_create(xyz, tets, 2, 1, 0, factor_bits=bits)
+    try:
+        O.oras_factor(h, eps * 1.1, None, k0)
+        regular = O.oras_arena_bytes(h)
+        for _ in range(2):
+            O.oras_factor(h, eps, None, k0)
+            if off == 0.0:
+                assert O.oras_arena_bytes(h) != regular
+            assert rel(O.oras_precond(h, v), z) <= (1e-9 if bits == 64 else 5e-3)
+            x, info, rc = O.oras_solve(h, p.B[:, 0], 1e-10)
+            assert rc == O.ORAS_OK and info[0]["iterations"] <= (2 if bits == 64 else 5)
+            O.oras_factor(h, eps * 1.1, None, k0)
+    finally:
+        O.oras_destroy(h)
+
+
+@pytest.mark.parametrize("bits", [32, 64])
+@pytest.mark.parametrize("nsub", [1, 3])
+def test_dead_cube_in_a_live_medium_stays_singular(O, bits, nsub):
+    """Six tetrahedra without any term (eps_r = 0, 1/mu_r = 0): the unknowns inside them have zero rows, in pivot blocks
+    whose other unknowns are alive.  Refused, as by the dense LU."""
+    n = 4
+    xyz, tets = synth.kuhn_cube(n)
+    dead = np.all(np.floor(xyz[tets].mean(axis=1) * n) == 1, axis=1)
+    assert dead.sum() == 6
+    eps = np.where(dead, 0.0, 44.0 - 20.0j)
+    mu = np.where(dead, 1e300, 1.0).astype(complex)
+    for engine in (O.ORAS_LU_AUTO, O.ORAS_LU_CUDA_CORES):
+        with pytest.raises(O.OrasError) as e:
+            O.oras_setup(xyz, tets, eps, mu, synth.K0, 2, nsub, 1, factor_bits=bits, lu_engine=engine)
+        assert e.value.code == O.ORAS_ERR_SINGULAR_LOCAL and "zero pivot" in str(e.value)
