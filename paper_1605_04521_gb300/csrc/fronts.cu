@@ -159,8 +159,24 @@ __device__ __forceinline__ void lds_pair(const CT<double>* p, CT<double>& a, CT<
   a = {t0.x, t0.y}; b = {t1.x, t1.y};
 }
 
-__device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+// The leading bits of x >= 0, ordered as x is: all of FP64's exponents, which a conversion to FP32 would cut.
+__device__ __forceinline__ uint32_t magnitude_bits(float x) { return __float_as_uint(x); }
+__device__ __forceinline__ uint32_t magnitude_bits(double x) { return (uint32_t)__double2hiint(x); }
+
+// 1 / v of an entry that is not zero.  v is first brought to about 1 by a power of two, so that the square of its
+// magnitude neither overflows nor vanishes (entries of A_s scale with the mesh's unit and 1 / mu_r).
+__device__ __forceinline__ CT<float> reciprocal(CT<float> v) {
+  const int e = (int)(__float_as_uint(fmaxf(fabsf(v.re), fabsf(v.im))) >> 23);
+  const float s = __uint_as_float((uint32_t)(e < 253 ? 254 - e : 1) << 23);
+  const float re = v.re * s, im = v.im * s, r = __frcp_rn(re * re + im * im) * s;
+  return {re * r, -im * r};
+}
+__device__ __forceinline__ CT<double> reciprocal(CT<double> v) {
+  const int e = __double2hiint(fmax(fabs(v.re), fabs(v.im))) >> 20;
+  const double s = __hiloint2double((e < 2045 ? 2046 - e : 1) << 20, 0);
+  const double re = v.re * s, im = v.im * s, r = s / (re * re + im * im);
+  return {re * r, -im * r};
+}
 
 // Panel warp pw: columns c0 .. c0 + 7 of row 32 pw + lane (rows below `rows` take part).  taken: the row has been a
 // pivot.
@@ -176,10 +192,10 @@ __device__ __forceinline__ void invert_panel(InvShared<R, NB>& sh, int c0, int r
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     const int par = c & 1;
-    float mag = (float)(fabs(x[c].re) + fabs(x[c].im));
-    if (mag != mag) mag = 0.0f;  // a non-finite entry still lets a row be chosen
+    R mag = fabs(x[c].re) + fabs(x[c].im);
+    if (mag != mag) mag = R(0);  // a non-finite entry still lets a row be chosen
     uint32_t key = 0u;
-    if (i < rows && !taken) key = ((__float_as_uint(mag) << 1) & 0xFFFFFF00u) | 0x80u | (uint32_t)(127 - i);
+    if (i < rows && !taken) key = ((magnitude_bits(mag) << 1) & 0xFFFFFF00u) | 0x80u | (uint32_t)(127 - i);
     uint32_t best = __reduce_max_sync(0xffffffffu, key);
     if (best != 0u && key == best) {
 #pragma unroll
@@ -209,8 +225,7 @@ __device__ __forceinline__ void invert_panel(InvShared<R, NB>& sh, int c0, int r
     const CT<R> pv = r[c];
     CT<R> inv = {R(0), R(0)};
     if (pv.re != R(0) || pv.im != R(0)) {
-      const R rden = recip(pv.re * pv.re + pv.im * pv.im);
-      inv = {pv.re * rden, -pv.im * rden};
+      inv = reciprocal(pv);
     } else if (n2 > 0) {
       // an exactly zero pivot column: the unknowns eliminated later can still make A_s regular.  The node is planned
       // anew; where that does not help, the pivot is taken as the rounding of the block's entries

@@ -233,3 +233,29 @@ def test_dead_cube_in_a_live_medium_stays_singular(O, bits, nsub):
         with pytest.raises(O.OrasError) as e:
             O.oras_setup(xyz, tets, eps, mu, synth.K0, 2, nsub, 1, factor_bits=bits, lu_engine=engine)
         assert e.value.code == O.ORAS_ERR_SINGULAR_LOCAL and "zero pivot" in str(e.value)
+
+
+@pytest.mark.parametrize("bits,power", [(32, -80), (32, -60), (32, 64), (32, 80), (64, -300), (64, -140), (64, 140), (64, 300)])
+def test_entries_of_any_scale(O, bits, power):
+    """A and A_s times a power of two (the mesh's unit, 1 / mu_r), far from 1 but inside the factors' precision: the apply
+    is the same times its inverse.  Squares of such entries over- or underflow."""
+    s = 2.0 ** power
+    xyz, tets = synth.kuhn_cube(4)
+    eps, mu = synth.head_materials(xyz, tets)
+    beta = np.full((len(tets), 4), 9.0)
+    rng = np.random.default_rng(5)
+    zs = []
+    for f in (1.0, s):
+        # one subdomain: no interface whose coefficient comes from the materials
+        h = O.oras_setup(xyz, tets, eps * f, mu / f, synth.K0, 2, 1, 0, beta_face=beta * f, factor_bits=bits)
+        try:
+            n = O.oras_ndof(h)
+            if not zs:
+                v = rng.normal(size=n) + 1j * rng.normal(size=n)
+            zs.append(O.oras_precond(h, v) * f)
+            x, info, rc = O.oras_solve(h, v, 1e-8)
+            assert rc == O.ORAS_OK and info[0]["iterations"] <= 3
+        finally:
+            O.oras_destroy(h)
+    assert np.all(np.isfinite(zs[1]))
+    assert rel(zs[1], zs[0]) <= (1e-12 if bits == 64 else 1e-6)
