@@ -159,9 +159,15 @@ __device__ __forceinline__ void lds_pair(const CT<double>* p, CT<double>& a, CT<
   a = {t0.x, t0.y}; b = {t1.x, t1.y};
 }
 
-// The leading bits of x >= 0, ordered as x is: all of FP64's exponents, which a conversion to FP32 would cut.
-__device__ __forceinline__ uint32_t magnitude_bits(float x) { return __float_as_uint(x); }
-__device__ __forceinline__ uint32_t magnitude_bits(double x) { return (uint32_t)__double2hiint(x); }
+// The leading bits of x >= 0, ordered as x is: all of FP64's exponents, which a conversion to FP32 would cut.  0 for NaN.
+__device__ __forceinline__ uint32_t magnitude_bits(float x) {
+  const uint32_t b = __float_as_uint(x);
+  return b > 0x7F800000u ? 0u : b;
+}
+__device__ __forceinline__ uint32_t magnitude_bits(double x) {
+  const uint32_t b = (uint32_t)__double2hiint(x);
+  return b > 0x7FF00000u ? 0u : b;
+}
 
 // 1 / v of an entry that is not zero.  v is first brought to about 1 by a power of two, so that the square of its
 // magnitude neither overflows nor vanishes (entries of A_s scale with the mesh's unit and 1 / mu_r).
@@ -172,7 +178,7 @@ __device__ __forceinline__ CT<float> reciprocal(CT<float> v) {
   return {re * r, -im * r};
 }
 __device__ __forceinline__ CT<double> reciprocal(CT<double> v) {
-  const int e = __double2hiint(fmax(fabs(v.re), fabs(v.im))) >> 20;
+  const int e = max(__double2hiint(v.re) & 0x7FFFFFFF, __double2hiint(v.im) & 0x7FFFFFFF) >> 20;
   const double s = __hiloint2double((e < 2045 ? 2046 - e : 1) << 20, 0);
   const double re = v.re * s, im = v.im * s, r = s / (re * re + im * im);
   return {re * r, -im * r};
@@ -192,9 +198,8 @@ __device__ __forceinline__ void invert_panel(InvShared<R, NB>& sh, int c0, int r
 #pragma unroll
   for (int c = 0; c < 8; ++c) {
     const int par = c & 1;
-    R mag = fabs(x[c].re) + fabs(x[c].im);
-    if (mag != mag) mag = R(0);  // a non-finite entry still lets a row be chosen
-    uint32_t key = 0u;
+    const R mag = fabs(x[c].re) + fabs(x[c].im);
+    uint32_t key = 0u;  // a non-finite entry still lets a row be chosen
     if (i < rows && !taken) key = ((magnitude_bits(mag) << 1) & 0xFFFFFF00u) | 0x80u | (uint32_t)(127 - i);
     uint32_t best = __reduce_max_sync(0xffffffffu, key);
     if (best != 0u && key == best) {
@@ -423,11 +428,62 @@ __global__ void __launch_bounds__(NW * 32 + NB, BLOCKS)
 // 64 x 64 tile a block, 4 x 4 entries a thread.
 //   SCHUR = false: L = A21 S       (B = S, symmetric)
 //   SCHUR = true:  C = pulled children - L A21^T, tiles on and below the diagonal
+// A product with an explicit inverse leaves L A11 - A21 of the size of the rounding times k, the product of the
+// largest entries of A21 and S, and the apply an error of about k^2, where a triangular solve leaves k.  k is the square
+// of the wavelength over the mesh width at low frequencies.  Tiles with k above FR_REFINE (k is below 20 on the benchmark's
+// medium at degrees 1 and 2) take one step of refinement, L += (A21 - L A11) S: 4^3 x 6, degree 2, apply error at
+// k0 = 0.1 7.2e-12 -> 1.8e-12, at 0.01 5.8e-8 -> 4.5e-11 (dense LU 4.6e-13, 5.0e-11).  (FP32 does without: dense factors with TF32 products were worse off.)
+constexpr double FR_REFINE = 128.0;
+
+constexpr int FR_MUL_KC = 8, FR_MUL_LDS = FR_TILE + 2;
+template <typename R> struct MulShared {
+  alignas(16) CT<R> As[FR_MUL_KC][FR_MUL_LDS], Bs[FR_MUL_KC][FR_MUL_LDS];
+};
+
+// acc += A B^T of one tile: an x ld and bn x ld entries.  big: the largest entries of A and B that the thread has loaded.
+template <typename R>
+__device__ __forceinline__ void mul_tile(MulShared<R>& sh, CT<R> (&acc)[4][4], const CT<R>* A, int an, const CT<R>* B,
+                                         int bn, int ld, uint32_t (&big)[2]) {
+  constexpr int KC = FR_MUL_KC;
+  const int t = threadIdx.x, ty = t >> 4, tx = t & 15;
+  big[0] = big[1] = 0u;
+  for (int k0 = 0; k0 < ld; k0 += KC) {
+    __syncthreads();
+    for (int e = t; e < FR_TILE * KC; e += 256) {
+      const int i = e / KC, k = e % KC;
+      const bool in = k0 + k < ld;
+      const CT<R> a = (in && i < an) ? A[(int64_t)i * ld + k0 + k] : CT<R>{R(0), R(0)};
+      const CT<R> b = (in && i < bn) ? B[(int64_t)i * ld + k0 + k] : CT<R>{R(0), R(0)};
+      sh.As[k][i] = a;
+      sh.Bs[k][i] = b;
+      big[0] = max(big[0], max(magnitude_bits(fabs(a.re)), magnitude_bits(fabs(a.im))));
+      big[1] = max(big[1], max(magnitude_bits(fabs(b.re)), magnitude_bits(fabs(b.im))));
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < KC; ++k) {
+      CT<R> av[4], bv[4];
+#pragma unroll
+      for (int p = 0; p < 4; ++p) av[p] = sh.As[k][ty * 4 + p];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) bv[q] = sh.Bs[k][tx + 16 * q];
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          acc[p][q].re = fma(av[p].re, bv[q].re, acc[p][q].re);
+          acc[p][q].im = fma(av[p].re, bv[q].im, acc[p][q].im);
+          acc[p][q].re = fma(-av[p].im, bv[q].im, acc[p][q].re);
+          acc[p][q].im = fma(av[p].im, bv[q].re, acc[p][q].im);
+        }
+    }
+  }
+}
+
 template <typename R, bool SCHUR>
-__global__ void __launch_bounds__(256) k_fr_mul(FrDev f, const FrontItem* __restrict__ items, CT<R>* __restrict__ work,
+__global__ void __launch_bounds__(256, 2) k_fr_mul(FrDev f, const FrontItem* __restrict__ items, CT<R>* __restrict__ work,
                                                 CT<R>* __restrict__ fac, CT<R>* __restrict__ C, int32_t* status) {
-  constexpr int KC = 8, LDS = FR_TILE + 2;
-  __shared__ __align__(16) CT<R> As[KC][LDS], Bs[KC][LDS];
+  __shared__ MulShared<R> sh;
   const FrontItem it = items[blockIdx.x];
   const FrontNode n = f.nodes[it.node];
   const int n1 = n.n1, n2 = n.n2, ld = n.ld;
@@ -452,31 +508,44 @@ __global__ void __launch_bounds__(256) k_fr_mul(FrDev f, const FrontItem* __rest
   for (int p = 0; p < 4; ++p)
 #pragma unroll
     for (int q = 0; q < 4; ++q) acc[p][q] = {R(0), R(0)};
-  for (int k0 = 0; k0 < ld; k0 += KC) {
-    __syncthreads();
-    for (int e = t; e < FR_TILE * KC; e += 256) {
-      const int i = e / KC, k = e % KC;
-      const bool in = k0 + k < ld;
-      As[k][i] = (in && i0 + i < n2) ? A[(int64_t)(i0 + i) * ld + k0 + k] : CT<R>{R(0), R(0)};
-      Bs[k][i] = (in && j0 + i < jn) ? B[(int64_t)(j0 + i) * ld + k0 + k] : CT<R>{R(0), R(0)};
+  uint32_t big[2];
+  mul_tile<R>(sh, acc, A + (int64_t)i0 * ld, n2 - i0, B + (int64_t)j0 * ld, jn - j0, ld, big);
+  if constexpr (!SCHUR) {
+    static_assert(sizeof(R) == 8, "one tile has all own columns");
+    __shared__ uint32_t part[2][8];
+    for (int q = 0; q < 2; ++q) {
+      const uint32_t m = __reduce_max_sync(0xffffffffu, big[q]);
+      if ((t & 31) == 0) part[q][t >> 5] = m;
     }
     __syncthreads();
+    uint32_t a = 0u, s = 0u;
+    for (int q = 0; q < 8; ++q) { a = max(a, part[0][q]); s = max(s, part[1][q]); }
+    if (__hiloint2double((int)a, 0) * __hiloint2double((int)s, 0) > FR_REFINE) {  // the same in every thread
+      const CT<R>* A11 = work + n.panel;
+      CT<R>* out = fac + n.panel + (int64_t)(n1 + i0) * ld;
+      auto put = [&](const CT<R> (&v)[4][4]) {
 #pragma unroll
-    for (int k = 0; k < KC; ++k) {
-      CT<R> av[4], bv[4];
+        for (int p = 0; p < 4; ++p)
 #pragma unroll
-      for (int p = 0; p < 4; ++p) av[p] = As[k][ty * 4 + p];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) bv[q] = Bs[k][tx + 16 * q];
+          for (int q = 0; q < 4; ++q)
+            if (i0 + ty * 4 + p < n2 && tx + 16 * q < ld) out[(int64_t)(ty * 4 + p) * ld + tx + 16 * q] = v[p][q];
+        __syncthreads();
+      };
+      put(acc);
+      CT<R> r[4][4] = {};
+      mul_tile<R>(sh, r, out, n2 - i0, A11, n1, ld, big);
+      __syncthreads();  // L has been read
 #pragma unroll
       for (int p = 0; p < 4; ++p)
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-          acc[p][q].re = fma(av[p].re, bv[q].re, acc[p][q].re);
-          acc[p][q].im = fma(av[p].re, bv[q].im, acc[p][q].im);
-          acc[p][q].re = fma(-av[p].im, bv[q].im, acc[p][q].re);
-          acc[p][q].im = fma(av[p].im, bv[q].re, acc[p][q].im);
+          const int i = i0 + ty * 4 + p, j = tx + 16 * q;
+          const CT<R> a = i < n2 && j < ld ? A[(int64_t)i * ld + j] : CT<R>{R(0), R(0)};
+          r[p][q] = {a.re - r[p][q].re, a.im - r[p][q].im};
         }
+      put(r);
+      mul_tile<R>(sh, acc, out, n2 - i0, B, n1, ld, big);
+      __syncthreads();
     }
   }
   FrontSrc sj[4];

@@ -259,3 +259,25 @@ def test_entries_of_any_scale(O, bits, power):
             O.oras_destroy(h)
     assert np.all(np.isfinite(zs[1]))
     assert rel(zs[1], zs[0]) <= (1e-12 if bits == 64 else 1e-6)
+
+
+@pytest.mark.parametrize("n,r,nsub", [(4, 2, 4), (5, 1, 3), (3, 3, 2)])
+@pytest.mark.parametrize("k0", [0.3, 0.1, 0.02])
+def test_low_frequency_fp64(O, n, r, nsub, k0):
+    """At low frequencies the gradients inside a tree node are all but in its pivot block's null space; L is not large
+    there.  The apply with FP64 sparse factors stays within ten times the distance of the dense LU of the same matrices
+    from the oracle, or 1e-12."""
+    xyz, tets = synth.kuhn_cube(n)
+    eps, mu = synth.head_materials(xyz, tets)
+    p = problem.build(xyz, tets, eps, mu, k0, r, [], nsub=nsub, delta=1)
+    rng = np.random.default_rng(6)
+    v = rng.normal(size=p.topo.ndof) + 1j * rng.normal(size=p.topo.ndof)
+    z = p.oras.apply(v)
+    err = []
+    for engine in (O.ORAS_LU_AUTO, O.ORAS_LU_CUDA_CORES):
+        h = O.oras_setup(xyz, tets, eps, mu, k0, r, nsub, 1, factor_bits=64, lu_engine=engine)
+        try:
+            err.append(rel(O.oras_precond(h, v), z))
+        finally:
+            O.oras_destroy(h)
+    assert err[0] <= max(10.0 * err[1], 1e-12), err
