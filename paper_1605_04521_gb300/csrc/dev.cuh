@@ -111,10 +111,9 @@ __device__ __forceinline__ bool mbar_test_cluster(uint64_t* b, uint32_t parity) 
 // Default limit of a bounded device wait (oras_options.wait_ms = 0): 2 s of %globaltimer.
 constexpr uint64_t WAIT_NS_DEFAULT = 2000000000ull;
 
-// Waits for the phase with the given parity; gives up after limit_ns of %globaltimer (or 2^26
+// Waits for the phase with the given parity (limit_ns: the handle's, wait_limit_ns or drain_limit); gives up after limit_ns of %globaltimer (or 2^26
 // polls) and returns false.
-__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, bool cluster_scope = false,
-                                          uint64_t limit_ns = WAIT_NS_DEFAULT) {
+__device__ __forceinline__ bool mbar_wait(uint64_t* b, uint32_t parity, bool cluster_scope, uint64_t limit_ns) {
   if (cluster_scope ? mbar_test_cluster(b, parity) : mbar_test(b, parity)) return true;
   const uint64_t t0 = globaltimer();
   for (long long it = 0; it < ORAS_SPIN_LIMIT; ++it) {
@@ -133,7 +132,7 @@ __device__ __forceinline__ int ld_acquire_cta(const int* p) {
   return v;
 }
 // Bounded wait until *p >= need (limit_ns of %globaltimer), false on timeout.
-__device__ __forceinline__ bool wait_counter(const int* p, int need, uint64_t limit_ns = WAIT_NS_DEFAULT) {
+__device__ __forceinline__ bool wait_counter(const int* p, int need, uint64_t limit_ns) {
   if (ld_acquire_cta(p) >= need) return true;
   const uint64_t t0 = globaltimer();
   for (long long it = 0; it < ORAS_SPIN_LIMIT; ++it) {

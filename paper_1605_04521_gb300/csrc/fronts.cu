@@ -432,7 +432,8 @@ __global__ void __launch_bounds__(NW * 32 + NB, BLOCKS)
 // largest entries of A21 and S, and the apply an error of about k^2, where a triangular solve leaves k.  k is the square
 // of the wavelength over the mesh width at low frequencies.  Tiles with k above FR_REFINE (k is below 20 on the benchmark's
 // medium at degrees 1 and 2) take one step of refinement, L += (A21 - L A11) S: 4^3 x 6, degree 2, apply error at
-// k0 = 0.1 7.2e-12 -> 1.8e-12, at 0.01 5.8e-8 -> 4.5e-11 (dense LU 4.6e-13, 5.0e-11).  (FP32 does without: dense factors with TF32 products were worse off.)
+// k0 = 0.1 7.2e-12 -> 1.8e-12, at 0.01 5.8e-8 -> 4.5e-11 (dense LU 4.6e-13, 5.0e-11).  (FP32 does without: dense
+// factors with TF32 products were worse off.)
 constexpr double FR_REFINE = 128.0;
 
 constexpr int FR_MUL_KC = 8, FR_MUL_LDS = FR_TILE + 2;

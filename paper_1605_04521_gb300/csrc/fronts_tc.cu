@@ -73,7 +73,7 @@ __device__ __forceinline__ void tf32_split(float x, float& hi, float& lo) {
 template <bool SCHUR>
 __global__ void __launch_bounds__(FT_THREADS, 2) k_fr_mul_tc(FrDev f, const FrontItem* __restrict__ items,
                                                              const CT<float>* __restrict__ work, CT<float>* fac,
-                                                             CT<float>* C, int32_t* status) {
+                                                             CT<float>* C, int32_t* status, uint64_t wait_ns) {
   extern __shared__ __align__(1024) unsigned char ft_raw[];
   __shared__ uint64_t bar;
   __shared__ uint32_t tmem_base;
@@ -120,10 +120,11 @@ __global__ void __launch_bounds__(FT_THREADS, 2) k_fr_mul_tc(FrDev f, const Fron
     *reinterpret_cast<float4*>(sm + operand * FT_OPERAND + (r >> 3) * 1024 + (r & 7) * 128 + ((g ^ (r & 7)) << 4)) = v;
   };
   bool bad = false;
+  int issued = -1;  // thread 0: the last chunk whose MMAs are under way
   if (chunks > 0) load(0);
   for (int c = 0; c < chunks; ++c) {
     // the MMAs of the chunk before have read the buffer
-    const bool ok = c == 0 || mbar_wait(&bar, (uint32_t)((c - 1) & 1));
+    const bool ok = c == 0 || mbar_wait(&bar, (uint32_t)((c - 1) & 1), false, wait_ns);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       float4 h, l;
@@ -165,14 +166,15 @@ __global__ void __launch_bounds__(FT_THREADS, 2) k_fr_mul_tc(FrDev f, const Fron
       }
       asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(&bar))
                    : "memory");
+      issued = c;
     }
   }
-  if (!bad && chunks > 0) bad = __syncthreads_or(!mbar_wait(&bar, (uint32_t)((chunks - 1) & 1))) != 0;
+  if (!bad && chunks > 0) bad = __syncthreads_or(!mbar_wait(&bar, (uint32_t)((chunks - 1) & 1), false, wait_ns)) != 0;
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  if (bad) {  // no MMA is issued after a wait that gave up; those in flight get the limit once more to finish
+  if (bad) {  // no MMA is issued after a wait that gave up; those in flight get more time to finish
     if (tid == 0) {
       atomicExch(&status[ST_ERR], DEV_TIMEOUT);
-      for (uint32_t p = 0; p < 2; ++p) mbar_wait(&bar, p);
+      if (issued >= 0) mbar_wait(&bar, (uint32_t)(issued & 1), false, drain_limit(wait_ns));
     }
   } else {
     // lanes 32 (warp % 4) .. + 31 are the tile's rows; warps 0-3 take columns 0-31, warps 4-7 columns 32-63
@@ -270,7 +272,7 @@ void launch_front_mul_tc(const oras_handle* h, const FrDev& f, bool schur, const
   allow_max_smem((const void*)k_fr_mul_tc<false>);
   auto* fn = schur ? k_fr_mul_tc<true> : k_fr_mul_tc<false>;
   fn<<<(unsigned)blocks, FT_THREADS, FT_SMEM, d.stream>>>(f, items, (const CT<float>*)d.fr_work, (CT<float>*)d.arena,
-                                                          (CT<float>*)d.fr_c, d.status);
+                                                          (CT<float>*)d.fr_c, d.status, wait_limit_ns(h));
   count_launches(1);
 }
 
