@@ -389,13 +389,13 @@ int oras_precond_noalloc(oras_handle* h, const oras_complex* v, oras_complex* z,
 
 /* Self-test of failure detection (no counterpart in the paper): runs, on the handle's stream,
  * one kernel that waits with each bounded-wait primitive of the library's kernels (a CTA-scope
- * mbarrier phase, a cluster-scope acquire on an mbarrier, a shared-memory counter) on a
- * condition that nothing ever satisfies, with the handle's limit oras_options.wait_ms.  Each
+ * mbarrier phase, a cluster-scope acquire on an mbarrier, a counter in shared memory and the grid
+ * barrier's in global memory) on a condition that nothing ever satisfies, with the handle's limit oras_options.wait_ms.  Each
  * wait gives up, records the timeout in the handle's device status, and the kernel returns;
  * the call reads the status like oras_solve does and returns ORAS_ERR_DEVICE_TIMEOUT, with
  * detail (or NULL) = bit mask of the primitives that gave up (1 CTA mbarrier, 2 cluster
- * mbarrier, 4 counter; 7 when all behave).  The status is cleared again before returning, so the
- * handle stays usable.  Takes about 3 x wait_ms.  Errors: INVALID_ARG, STATE (no oras_factor
+ * mbarrier, 4 both counters; 7 when all behave).  The status is cleared again before returning, so the
+ * handle stays usable.  Takes about 4 x wait_ms.  Errors: INVALID_ARG, STATE (no oras_factor
  * yet), CUDA. */
 int oras_wait_selftest(oras_handle* h, int32_t* detail);
 

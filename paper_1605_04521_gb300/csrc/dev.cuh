@@ -141,6 +141,32 @@ __device__ __forceinline__ bool wait_counter(const int* p, int need, uint64_t li
   }
   return false;
 }
+// Barrier over the blocks of a cooperative launch, all of which run at once; counters in the status words.
+// Every block's arrival; what its threads wrote before is visible to blocks that see it.
+__device__ __forceinline__ void grid_arrive(int32_t* status) {
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    __threadfence();
+    atomicAdd(&status[ST_ORTH_ARRIVED], 1);
+  }
+}
+// Until `need` arrivals, or not within the limit (false in every thread of the block).
+__device__ __forceinline__ bool grid_wait(int32_t* status, int need, uint64_t limit_ns) {
+  int ok = 1;
+  if (threadIdx.x == 0) {
+    const uint64_t t0 = globaltimer();
+    long long it = 0;
+    while (true) {
+      int v;
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(status + ST_ORTH_ARRIVED) : "memory");
+      if (v >= need) break;
+      ++it;
+      if (it >= ORAS_SPIN_LIMIT || ((it & 255) == 0 && globaltimer() - t0 > limit_ns)) { ok = 0; break; }
+    }
+    __threadfence();
+  }
+  return __syncthreads_and(ok) != 0;
+}
 // Limit of the waits for a CTA's own bulk copies still in flight before it exits: never below
 // the default, so a short user limit cannot let a CTA leave while copies land in its memory.
 __device__ __forceinline__ uint64_t drain_limit(uint64_t limit_ns) {

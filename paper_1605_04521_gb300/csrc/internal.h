@@ -27,6 +27,8 @@ struct cplx { double re, im; };
 
 // device status flags (Device::status): [0] error code, [1] detail, [2] subdomain, [3] some node is in Device::fr_weak
 enum { ST_ERR = 0, ST_DETAIL = 1, ST_SUB = 2, ST_WEAK = 3 };
+// counters of the grid barrier (k_orth) beside them, zero between launches
+enum { ST_ORTH_ARRIVED = 4, ST_ORTH_LEFT = 5 };
 enum { DEV_OK = 0, DEV_SINGULAR = 1, DEV_TIMEOUT = 2, DEV_BADINDEX = 3 };
 
 

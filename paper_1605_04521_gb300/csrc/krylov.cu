@@ -370,7 +370,6 @@ __device__ __forceinline__ void givens_finish(int r, int m, int j, cplx a, doubl
 // (1.4e6 entries).  Others take the launches above.
 // Waits are bounded: a block that gives up reports DEV_TIMEOUT and leaves, and so do then the others.
 constexpr int ORTH_THREADS = 512, ORTH_MAX_K = 8, ORTH_MAX_ROUNDS = 18;
-enum { ST_ORTH_ARRIVED = 4, ST_ORTH_LEFT = 5 };   // barrier counters beside the status flags, zero between launches
 
 struct OrthArgs {
   int64_t nk, chunk;                 // entries, entries a block (a multiple of k)
@@ -388,32 +387,6 @@ struct OrthArgs {
   int32_t* host_status;
   uint64_t wait_ns;
 };
-
-// Every block's arrival; what its threads wrote before is visible to blocks that see it.
-__device__ __forceinline__ void grid_arrive(int32_t* status) {
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    __threadfence();
-    atomicAdd(&status[ST_ORTH_ARRIVED], 1);
-  }
-}
-// Until `need` arrivals, or not within the limit (false in every thread of the block).
-__device__ __forceinline__ bool grid_wait(int32_t* status, int need, uint64_t limit_ns) {
-  int ok = 1;
-  if (threadIdx.x == 0) {
-    const uint64_t t0 = globaltimer();
-    long long it = 0;
-    while (true) {
-      int v;
-      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(status + ST_ORTH_ARRIVED) : "memory");
-      if (v >= need) break;
-      ++it;
-      if (it >= ORAS_SPIN_LIMIT || ((it & 255) == 0 && globaltimer() - t0 > limit_ns)) { ok = 0; break; }
-    }
-    __threadfence();
-  }
-  return __syncthreads_and(ok) != 0;
-}
 
 // Sums over the p of the values of lanes r + k p, P of them, into lanes r.
 __device__ __forceinline__ cplx sum_lanes(cplx t, int k, int P, int p) {

@@ -1,7 +1,7 @@
 // Self-test of the bounded device waits (failure detection, no counterpart in the paper).
 //
 // The library's kernels never spin without a limit: every wait on an mbarrier phase, on a
-// shared-memory counter or on a message from the partner CTA of a cluster gives up after the
+// shared-memory counter, on a message from the partner CTA of a cluster or on a grid barrier gives up after the
 // handle's limit (oras_options.wait_ms), records DEV_TIMEOUT in the handle's device status
 // flags and lets the kernel return, so the context stays usable and the host call reports
 // ORAS_ERR_DEVICE_TIMEOUT.  This kernel runs each of those wait primitives on a condition that
@@ -13,7 +13,8 @@
 namespace oras {
 
 // One warp; lane 0 waits.  status[ST_DETAIL] gets one bit per primitive that gave up:
-// 1 = CTA-scope mbarrier phase, 2 = cluster-scope acquire on an mbarrier, 4 = counter.
+// 1 = CTA-scope mbarrier phase, 2 = cluster-scope acquire on an mbarrier, 4 = both counters (a CTA's and the grid
+// barrier's).
 __global__ void k_wait_selftest(int32_t* status, uint64_t limit_ns) {
   __shared__ uint64_t bar;
   __shared__ int counter;
@@ -23,11 +24,12 @@ __global__ void k_wait_selftest(int32_t* status, uint64_t limit_ns) {
     fence_mbar_init();
   }
   __syncwarp();
+  const bool grid_gave_up = !grid_wait(status, 1, limit_ns);  // no block has arrived
   if (threadIdx.x != 0) return;
   int gave_up = 0;
   if (!mbar_wait(&bar, 0, false, limit_ns)) gave_up |= 1;
   if (!mbar_wait(&bar, 0, true, limit_ns)) gave_up |= 2;
-  if (!wait_counter(&counter, 1, limit_ns)) gave_up |= 4;
+  if (!wait_counter(&counter, 1, limit_ns) && grid_gave_up) gave_up |= 4;
   if (gave_up) {
     atomicExch(&status[ST_ERR], DEV_TIMEOUT);
     atomicOr(&status[ST_DETAIL], gave_up);

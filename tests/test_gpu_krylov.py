@@ -136,3 +136,58 @@ def test_orthogonalisation_in_one_launch(larger, k):
     R9 = B[:, :k] - np.asarray(O.oras_matvec(h, np.asarray(Y)[:, :k].copy(), k=k)).reshape(-1, k)
     for j in range(k):
         assert np.linalg.norm(R9[:, j]) <= 1e-8 * np.linalg.norm(B[:, j])
+
+
+def test_orthogonalisation_past_one_launch():
+    """Eight columns of a vector that does not fit the SMs' shared memory (more than 18 rounds of 512 entries an SM): the
+    step ends in several launches, as with more columns."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1605_04521_gb300 import build
+    build.build()
+    from paper_1605_04521_gb300 import oras as O
+    w = synth.small(n=17, r=2, nsub=128, overlap=0, restart=20)
+    xyz, tets = w.mesh()
+    eps, mu = w.materials(xyz, tets)
+    h = O.oras_setup(xyz, tets, eps, mu, w.k0, w.r, w.nsub, w.overlap, restart=w.restart, max_iter=18,
+                     factor_bits=64)
+    try:
+        n = O.oras_ndof(h)
+        rng = np.random.default_rng(9)
+        B = rng.normal(size=(n, 8)) + 1j * rng.normal(size=(n, 8))
+        launches = {}
+        X = {}
+        for k in (8, 1):
+            O.oras_reset_timings(h)
+            O.oras_set_timing(h, 1)
+            X[k], info, _ = O.oras_solve(h, B[:, :k], 1e-12, k=k)
+            launches[k] = O.oras_timings(h)["orth"][1]
+            assert max(i["iterations"] for i in info) == 18
+        assert 8 * n > 152 * 18 * 512 >= n
+        assert launches[1] == 18 and launches[8] > 3 * 18
+        # the same 18 steps with FP64 factors: both iterates minimise the residual over the same space, to rounding
+        assert rel(np.asarray(X[8])[:, 0], np.asarray(X[1]).reshape(-1)) <= 1e-8
+    finally:
+        O.oras_destroy(h)
+
+
+def test_grid_barrier_gives_up(setup):
+    """The wait self-test includes the one-launch step's barrier, on an arrival that never comes: four waits of the limit,
+    then the kernel returns and the handle works on."""
+    import time
+    O, _, p = setup
+    w = synth.small(n=3, r=2, nsub=4, overlap=1)
+    xyz, tets = w.mesh()
+    eps, mu = w.materials(xyz, tets)
+    h = O.oras_setup(xyz, tets, eps, mu, w.k0, w.r, w.nsub, w.overlap, wait_ms=200)
+    try:
+        t0 = time.perf_counter()
+        rc, detail = O.oras_wait_selftest(h)
+        assert time.perf_counter() - t0 >= 0.78
+        assert rc == O.ORAS_ERR_DEVICE_TIMEOUT and detail == 7
+        b = O.oras_rhs_dipole(h, synth.dipole_ring(1)[0], [0, 0, 1.0])
+        _, info, rc = O.oras_solve(h, b, 1e-8)
+        assert rc == O.ORAS_OK
+    finally:
+        O.oras_destroy(h)
