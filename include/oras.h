@@ -70,7 +70,7 @@ enum { ORAS_OVERLAP_VERTEX = 0, ORAS_OVERLAP_FACE = 1 };
  * nested-dissection tree, pivots chosen inside a tree node (at most 128 unknowns, 64 in FP64).  A node
  * whose pivot block is close to singular (a resonance of its interior, a zero pivot) leaves the
  * unknowns in question to its parent: oras_factor then plans the trees anew and factors again, up to 8
- * times, and the handle keeps the new trees (oras_arena_bytes may change).
+ * times (64 in all for a handle), and the handle keeps the new trees (oras_arena_bytes may change).
  * CUDA_CORES: dense LU, pivots chosen over whole columns. */
 enum { ORAS_LU_AUTO = 0, ORAS_LU_CUDA_CORES = 1 };
 /* Preconditioner apply with dense FP32 factors (ORAS_LU_CUDA_CORES): AUTO streams the factor arena

@@ -507,7 +507,9 @@ static int factor_device(oras_handle* h) {
   for (int attempt = 0;; ++attempt) {
     int rc = factor_once(h);
     if (!h->fronts.use || (rc != ORAS_OK && rc != ORAS_ERR_SINGULAR_LOCAL)) return rc;
-    if (((const int32_t*)(h->dev.host_pinned + PINNED_STATUS_OFF))[ST_WEAK] == 0 || attempt == FR_REPLANS) return rc;
+    if (((const int32_t*)(h->dev.host_pinned + PINNED_STATUS_OFF))[ST_WEAK] == 0 || attempt == FR_REPLANS ||
+        h->fronts.replans >= FR_REPLANS_HANDLE)
+      return rc;
     bool moved = false;
     try {
       if (int rc2 = replan_fronts(h, &moved)) return rc2;
@@ -689,9 +691,8 @@ int oras_factor(oras_handle* h, const oras_complex* eps_r, const oras_complex* m
   }
   h->k0 = k0;
   rc = factor_device(h);
-  if (rc) return rc;
-  h->factored = true;
-  return ORAS_OK;
+  h->factored |= rc == ORAS_OK;
+  return rc;
 }
 
 // Autotuner of the LU panel width: each candidate factorises the handle's current problem once
@@ -751,7 +752,9 @@ int oras_autotune(oras_handle* h, int32_t* panel, double* ms, int32_t nms) {
   h->opt.lu_panel = best.first;
   h->opt.lu_group = best.second;
   if (panel) *panel = best.first;
-  return factor_device(h);  // leave the factors of the chosen shape
+  const int rc = factor_device(h);  // leave the factors of the chosen shape
+  h->factored |= rc == ORAS_OK;     // (a new plan had taken them back)
+  return rc;
 }
 
 int32_t oras_lu_group(const oras_handle* h) { return h ? h->opt.lu_group : -1; }

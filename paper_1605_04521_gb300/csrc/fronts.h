@@ -49,6 +49,7 @@ struct FrontLevels {  // per level: [ptr[l], ptr[l + 1]) of the item list
 
 struct Fronts {
   bool use = false;
+  int replans = 0;                    // times delay_unknowns changed the plan
   std::vector<FrontNode> nodes;       // by level, wide pivot blocks first within a level
   std::vector<int32_t> level_ptr;     // [nlev + 1] first node of each level
   std::vector<int32_t> level_class;   // [nlev][FR_CLASSES + 1] first node of each width class (front_class)
@@ -69,7 +70,9 @@ struct Fronts {
 // with and without losses, k0 from 0.01 to 9); the apply's error is the unit roundoff times its square: at 64 1e-4 in
 // FP32 and 1e-12 in FP64.
 constexpr float FR_GROWTH = 64.0f;
-constexpr int FR_REPLANS = 8;   // times a factorisation plans the trees anew before it takes what it has
+// Times a factorisation plans the trees anew before it takes what it has, and all factorisations of a handle together
+// (at frequencies so low that FP32 holds no digit of A_s, every factorisation would).
+constexpr int FR_REPLANS = 8, FR_REPLANS_HANDLE = 64;
 
 struct HostMesh;
 // Elimination trees of every subdomain of m for factors of the given precision (dirichlet: of the

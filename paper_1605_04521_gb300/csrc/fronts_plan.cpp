@@ -486,12 +486,17 @@ void delay_unknowns(const HostMesh& m, int factor_bits, const std::vector<std::v
       tree[q].own.push_back(u);
     }
   }
+  Fronts next;  // f stays as it is when memory runs out
+  next.use = f.use;
+  next.replans = f.replans + 1;
+  next.pos.resize(f.pos.size());
   parallel_for(m.nsub, 1, [&](int64_t s, int) {
     std::vector<int32_t> pos;
     number(trees[s], m.sub_ns[s], pos);
-    std::copy(pos.begin(), pos.end(), f.pos.begin() + m.sub_ns_off[s]);
+    std::copy(pos.begin(), pos.end(), next.pos.begin() + m.sub_ns_off[s]);
   });
-  lay_out(m, factor_bits, trees, f);
+  lay_out(m, factor_bits, trees, next);
+  f = std::move(next);
 }
 
 }  // namespace oras

@@ -379,6 +379,24 @@ static void setup_fails(int engine) {
   }
 }
 
+// Factorisations that never stop finding such nodes: each ends after 8 new plans, all of them after 64, and the handle
+// counts as factored.
+static void always_weak() {
+  Cube c(3, 2, 4);
+  oras_options o{};
+  oras_handle* h = nullptr;
+  if (oras_create(&c.p, &o, &h) != ORAS_OK) { bad("oras_create failed"); return; }
+  oras::g_weak = 1000;
+  for (int call = 1; call <= 10; ++call) {
+    if (oras_factor(h, c.eps.data(), nullptr, c.p.k0, ORAS_MEM_HOST) != ORAS_OK || !h->factored) bad("oras_factor failed");
+    if (h->fronts.replans != std::min(8 * call, 64)) bad("new plans: " + std::to_string(h->fronts.replans));
+  }
+  oras::g_weak = 3;
+  if (oras_autotune(h, nullptr, nullptr, 0) != ORAS_OK || !h->factored) bad("oras_autotune lost the factors");
+  check_trees(h);
+  oras_destroy(h);
+}
+
 // A solve of more columns with every allocation from the n-th on refused, then one of as many as before.
 static void solve_again(int bits) {
   Cube c(3, 2, 4);
@@ -415,6 +433,7 @@ int main(int argc, char** argv) {
   else if (s == "factor64") factor_again(64, ORAS_LU_AUTO);
   else if (s == "factor_weak32") factor_again(32, ORAS_LU_AUTO, 2);
   else if (s == "factor_weak64") factor_again(64, ORAS_LU_AUTO, 2);
+  else if (s == "always_weak") always_weak();
   else if (s == "delay1") delay(4, 1, 5, 64);
   else if (s == "delay2") delay(5, 2, 2, 32);
   else if (s == "delay3") delay(3, 3, 3, 32);

@@ -58,7 +58,7 @@ def test_failed_set_up_leaves_no_memory_behind(program, scenario):
     assert findings(program, scenario) == (0, "")
 
 
-@pytest.mark.parametrize("scenario", ["delay1", "delay2", "delay3"])
+@pytest.mark.parametrize("scenario", ["delay1", "delay2", "delay3", "always_weak"])
 def test_trees_with_unknowns_moved_up(program, scenario):
     """Random unknowns eliminated later than planned: every unknown once, every coupling inside a front, borders and
     sources consistent."""
