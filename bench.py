@@ -55,15 +55,13 @@ def parse():
                     choices=["head16", "cube8", "head8", "krylov24", "batch32", "batch12", "batch8",
                              "head32r3"],
                     help="head16: the benchmark workload; cube8: 8^3 r=1 plane wave (FP64 factors); "
-                         "head8: 8^3 r=2 8 subdomains (1.9 GB arena, for kernel profiles); krylov24: "
-                         "24^3 r=2 512 subdomains without overlap (464 MB matrix, small arena, for Krylov "
+                         "head8: 8^3 r=2 8 subdomains (for kernel profiles); krylov24: "
+                         "24^3 r=2 512 subdomains without overlap (464 MB matrix, small factors, for Krylov "
                          "kernel profiles); batch32: 24^3 r=2 256 subdomains, 32 dipoles solved together; "
                          "batch12: 12^3 r=2 32 subdomains, 32 dipoles; batch8: 8^3 r=2 8 subdomains, 32 "
-                         "dipoles (2 GB arena, for profiles of the multi-right-hand-side apply); head32r3: 32^3 r=3 4096 subdomains without overlap (3.7 M DOFs)")
+                         "dipoles (for profiles of the multi-right-hand-side apply); head32r3: 32^3 r=3 4096 subdomains without overlap (3.7 M DOFs)")
     ap.add_argument("--block", type=int, default=0,
                     help="1: solve the workload's right-hand sides as one block (block FGMRES)")
-    ap.add_argument("--apply-engine", default="auto", choices=["auto", "cuda"],
-                    help="auto: tensor-core apply for 8 or more right-hand sides; cuda: CUDA-core apply only")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--e2e-steps", type=int, default=None)
     ap.add_argument("--serve-count", type=int, default=50,
@@ -81,9 +79,7 @@ def parse():
                          "with FGMRES(50) and with GCRO-DR(50, 10) recycling its subspace (Sec. 6)")
     ap.add_argument("--fp64-path", type=int, default=1,
                     help="1: also time the plain FP64 single-RHS path against the FP32-factor path on the "
-                         "workloads where the FP64 factorisation finishes (head8, cube8)")
-    ap.add_argument("--lu-panel", type=int, default=0,
-                    help="LU outer panel width in tiles (0: picked by oras_autotune at set-up)")
+                         "small workloads (head8, cube8)")
     ap.add_argument("--serve-max-iter", type=int, default=150,
                     help="FGMRES iteration cap per served request (requests above it report not converged)")
     return ap.parse_args()
@@ -530,7 +526,6 @@ def ports_measure(O, dev, stream, steps=1, warmup=1):
         eps_d = torch.from_numpy(eps).to(dev)
         mu_d = torch.from_numpy(mu).to(dev)
         O.oras_factor(h, eps_d, mu_d, w.k0, mem=O.ORAS_MEM_DEVICE)
-        O.oras_autotune(h)
         n = O.oras_ndof(h)
         B = np.stack([O.oras_rhs_port(h, p) for p in ps], axis=1)
         k = B.shape[1]
@@ -620,12 +615,9 @@ def recycling_measure(O, dev, stream, n_sys=3, m=50, k=10):
 
 # ------------------------------------------------------------------ plain FP64 path
 def fp64_path(O, dev, stream, steps=2, warmup=1):
-    """The plain FP64 single-right-hand-side GPU path (FP64 local factors, CUDA-core FP64 LU,
-    FP64 apply; the same FGMRES) against the FP32-factor path, one step = oras_factor +
-    oras_solve of one right-hand side on device buffers, CUDA events on the handle's stream.
-    Run on the workloads where the FP64 factorisation finishes in seconds (8^3 x 6 meshes): on
-    the 16^3 benchmark it takes more than 12 minutes per factorisation (GB300's FP64 rate is
-    about 1/64 of its FP32 rate)."""
+    """The plain FP64 single-right-hand-side GPU path (FP64 sparse factors on the FP64 pipe, FP64
+    apply; the same FGMRES) against the FP32-factor path, one step = oras_factor + oras_solve of one
+    right-hand side on device buffers, CUDA events on the handle's stream, on the 8^3 x 6 meshes."""
     import torch
     out = {}
     for name in ("head8", "cube8"):
@@ -694,28 +686,15 @@ def run_ours(args, world, rank, local):
     dev = torch.device("cuda", local)
     stream = torch.cuda.current_stream(dev)
     t_mesh0 = time.perf_counter()
-    eng = O.ORAS_APPLY_CUDA_CORES if args.apply_engine == "cuda" else O.ORAS_APPLY_AUTO
-    if args.apply_engine == "cuda":
-        w.name += "_cuda_core_apply"
+    opts = dict(restart=w.restart, block=args.block)
     if args.block:
         w.name += "_block_fgmres"
-    h = O.oras_create(xyz, tets, w.r, w.nsub, w.overlap, factor_bits=w.factor_bits, restart=w.restart,
-                      apply_engine=eng, block=args.block)
+    h = O.oras_create(xyz, tets, w.r, w.nsub, w.overlap, factor_bits=w.factor_bits, **opts)
     t_mesh = time.perf_counter() - t_mesh0
     O.oras_set_stream(h, stream.cuda_stream)
     eps_d = torch.from_numpy(eps).to(dev)
     mu_d = torch.from_numpy(mu).to(dev)
     O.oras_factor(h, eps_d, mu_d, w.k0, mem=O.ORAS_MEM_DEVICE)
-    if args.lu_panel > 0:
-        panel, tune_ms = args.lu_panel, {}
-        O.oras_destroy(h)
-        h = O.oras_create(xyz, tets, w.r, w.nsub, w.overlap, factor_bits=w.factor_bits, restart=w.restart,
-                          lu_panel=panel, apply_engine=eng, block=args.block)
-        O.oras_set_stream(h, stream.cuda_stream)
-        O.oras_factor(h, eps_d, mu_d, w.k0, mem=O.ORAS_MEM_DEVICE)
-    else:
-        panel, tune_ms = O.oras_autotune(h)   # LU tile shapes for this problem (set-up, untimed)
-    group = O.oras_lu_group(h)
     n = O.oras_ndof(h)
     srcs = w.sources()
     krhs = len(srcs)
@@ -795,8 +774,7 @@ def run_ours(args, world, rank, local):
     torch.cuda.synchronize(dev)
     e0 = time.perf_counter()
     for _ in range(e2e_steps):
-        he = O.oras_setup(xyz, tets, eps, mu, w.k0, w.r, w.nsub, w.overlap, factor_bits=w.factor_bits,
-                          restart=w.restart, lu_panel=panel, lu_group=group, apply_engine=eng, block=args.block)
+        he = O.oras_setup(xyz, tets, eps, mu, w.k0, w.r, w.nsub, w.overlap, factor_bits=w.factor_bits, **opts)
         xe, info_e, rc = O.oras_solve(he, b_host, w.tol, k=krhs)
         x_host[:] = np.asarray(xe).reshape(n, krhs)
         O.oras_destroy(he)
@@ -849,8 +827,7 @@ def run_ours(args, world, rank, local):
                              f"{arena / 1e9:.1f} GB of factors",
                        "step": "oras_factor (element matrices, A, A_s, local factorisations) + oras_solve, device buffers",
                        "mesh_setup_s_untimed": t_mesh, "parallelism": f"replicas x{world}",
-                       "lu_panel": panel, "lu_group": group,
-                       "lu_autotune_ms": {str(k_): round(v_, 1) for k_, v_ in tune_ms.items()}},
+                       "factors": "sparse block L D L^T"},
             "iterations": iters, "true_relres": max(i["relres"] for i in infos[-1]),
             "phase_ms_per_step": {c: v[0] / args.steps for c, v in timings.items() if v[1] > 0},
             "roofline": roof,
