@@ -227,7 +227,8 @@ int oras_set_stream(oras_handle* h, void* stream);
 /* ---------------------------------------------------------------- solve (Sec. 5) */
 
 /* Solves A x_j = b_j for the k columns of rhs by FGMRES(m), x0 = 0, right-preconditioned
- * by ORAS, with FP64 Arnoldi (modified Gram-Schmidt), FP64 Givens rotations and an FP64
+ * by ORAS, with FP64 Arnoldi (Gram-Schmidt in blocks of 8 basis vectors, classical inside a block and
+ * modified from block to block), FP64 Givens rotations and an FP64
  * true-residual check at the end of every cycle; the k recurrences run together (pseudo-
  * block, Sec. 5).  With oras_options.block and k > 1: block FGMRES (Sec. 6 Block GMRES): one
  * block Krylov space for all k columns, FP64 block modified Gram-Schmidt between blocks, each new
@@ -399,10 +400,10 @@ int oras_precond_noalloc(oras_handle* h, const oras_complex* v, oras_complex* z,
  * yet), CUDA. */
 int oras_wait_selftest(oras_handle* h, int32_t* detail);
 
-/* Autotuner of the batched LU's tile shapes (no counterpart in the paper): the outer panel width
- * (tiles of 64 columns per trailing update; trades the updates inside a panel against the passes
- * over the trailing matrix) and the raster group of the tensor-core update (output blocks that
- * share operands in L2).  Factorises the handle's current problem (materials of the last
+/* Autotuner of the dense LU's tile shapes (ORAS_LU_CUDA_CORES; no counterpart in the paper): the outer
+ * panel width (tiles of 64 columns per trailing update; trades the updates inside a panel against the
+ * passes over the trailing matrix) and a raster group that no present kernel reads.  The sparse factors
+ * read neither: on them the call only takes its time.  Factorises the handle's current problem (materials of the last
  * oras_factor, on the handle's stream) once per candidate width 4, 8, 12, 16, 24, 32, 48, 64, 96,
  * 128, 192 (group 8), then once per group 16, 32, 64 at the best width, keeps the fastest pair in the
  * handle's options (lu_panel, lu_group) and leaves the factors of that pair.  The choice is
@@ -412,8 +413,8 @@ int oras_wait_selftest(oras_handle* h, int32_t* detail);
  * groups (14 entries; -1 when taken from the cache; NULL allowed).
  * Errors: INVALID_ARG, STATE (no oras_factor yet), and those of oras_factor. */
 int oras_autotune(oras_handle* h, int32_t* panel, double* ms, int32_t nms);
-/* The raster group oras_autotune chose for the handle (0 before tuning: the default); -1 for
- * a NULL handle.  No counterpart in the paper (a tile shape of the batched LU). */
+/* The raster group oras_autotune chose for the handle (0 before tuning: the default; no present kernel
+ * reads it); -1 for a NULL handle.  No counterpart in the paper. */
 int32_t oras_lu_group(const oras_handle* h);
 
 /* Device bytes that oras_factor followed by an oras_solve of k right-hand sides allocate for

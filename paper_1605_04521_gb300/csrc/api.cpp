@@ -1,5 +1,5 @@
 // C ABI of the ORAS-FGMRES solver: handle lifecycle, device upload, numeric set-up (element
-// matrices, A, A_s, batched LU) and the right-preconditioned FGMRES(m) driver (Sec. 4-5).
+// matrices, A, A_s and their factors) and the right-preconditioned FGMRES(m) driver (Sec. 4-5).
 #include <algorithm>
 #include <atomic>
 #include <cmath>
@@ -1119,7 +1119,7 @@ static int fgmres(oras_handle* h, int k, double tol, oras_info* info) {
     for (int j = 0; j < m; ++j) {
       cplx* Vj = d.V + nk * j;
       cplx* Vn = d.V + nk * (j + 1);
-      // z_j = M^-1 v_j ; w = A z_j ; modified Gram-Schmidt against v_0..v_j ; Givens
+      // z_j = M^-1 v_j ; w = A z_j ; Gram-Schmidt against v_0..v_j in blocks of 8 ; Givens
       auto step = [&]() -> int {
         int pb = prof_begin(h);
         if (precond_to_z(h, Vj, k, j)) return ORAS_ERR_CUDA;

@@ -18,9 +18,10 @@
 //
 // Against dense factors of the same matrices (n_s^2 entries each) the largest subdomain of the
 // 16^3 x 6, degree-2, 64-subdomain problem (17,896 unknowns) keeps 2% of the entries and needs 0.1%
-// of the products.  FP32 factors keep FP32's accuracy throughout (fronts_tc.cu): against FP64 solves their
-// error is 5e-7 at degree 2 and 3e-6 at degree 3 or without losses, that of a dense FP32 LU with
-// partial pivoting (1e-6 and 5e-6).
+// of the products.  FP32 factors keep FP32's accuracy throughout (fronts_tc.cu).  Error of the apply against FP64, beside
+// that of a dense FP32 LU with pivots over whole columns, on 8 subdomains of the head-like medium: degree 1 (6^3 x 6)
+// 0.62e-6 and 0.45e-6, degree 2 (5^3, 8^3) 1.1e-6 and 1.0e-6, 2.3e-6 and 1.8e-6, degree 3 (5^3) 3.4e-6 and 3.8e-6; without
+// losses, degree 2 (6^3) 1.3e-5 and 0.59e-5, degree 3 (5^3) 5.4e-5 and 1.9e-5.
 #include "fronts.cuh"
 #include "rows.cuh"
 

@@ -7,9 +7,9 @@
 //
 // Precision: each FP32 operand is split into two TF32 values (2^-23 of it is left out) and hi hi, hi lo and lo hi are
 // summed in FP32 in tensor memory, the two small products in an accumulator of their own.  The apply's error against
-// FP64 is then that of FP32 fused multiply-adds: 0.92e-6 to 1.0e-6 against 0.86e-6 to 0.98e-6 at degree 2, 1.72e-6 to
-// 1.84e-6 against 1.82e-6 to 1.87e-6 at degree 3 (one accumulator for all three: 1.03e-6 and 1.95e-6; lo lo as well:
-// no change).
+// FP64 is then that of FP32 fused multiply-adds in their place: 0.92e-6 to 1.0e-6 against 0.86e-6 to 0.98e-6 on a problem
+// of degree 2, 1.72e-6 to 1.84e-6 against 1.82e-6 to 1.87e-6 on one of degree 3 (one accumulator for all three: 1.03e-6
+// and 1.95e-6; lo lo as well: no change).  fronts.cu has the errors on more problems.
 //
 // A block owns 128 x 64 entries (256 accumulator columns) and walks the sum in chunks of 16 unknowns: all
 // threads load, split and store a chunk in the 128-byte-swizzled K-major layout of the operands, one thread

@@ -1,5 +1,5 @@
-// FP64 Krylov kernels of the right-preconditioned FGMRES(m) (Sec. 5): complex CSR SpMV,
-// modified Gram-Schmidt Arnoldi in blocks of basis vectors with fused (update + next dots) passes,
+// FP64 Krylov kernels of the right-preconditioned FGMRES(m) (Sec. 5): complex CSR SpMV, Gram-Schmidt Arnoldi in blocks
+// of 8 basis vectors (classical inside a block, modified from block to block) with fused (update + next dots) passes,
 // complex Givens rotations on the device, the small triangular solve and the solution update.  Multi-vectors are
 // stored [N][k] (the k right-hand sides of a pseudo-block solve adjacent in memory).
 // Every reduction is a fixed two-stage sum (block partials, then a fixed-order sum), so the
@@ -273,10 +273,12 @@ __global__ void __launch_bounds__(256) k_sum_partials(int n, int k, int nb, cons
   if (H) H[((int64_t)(w % k) * (m + 1) + i0 + w / k) * m + j] = t;
 }
 
-// One pass of the blocked modified Gram-Schmidt: w -= sum_q h_q V_q over the nv basis vectors from V (h
+// One pass of the blocked Gram-Schmidt: w -= sum_q h_q V_q over the nv basis vectors from V (h
 // from hs), then the block partials of <Vn_q, w> over the nn vectors from Vn (nn = 0: of |w|^2 instead).
-// Vectors are nk apart.  A block's coefficients are taken together (its vectors are orthonormal to the
-// basis's own accuracy), blocks one after the other.  Bound: the FP64 pipe, 8 fused multiply-adds an entry
+// Vectors are nk apart.  A block's coefficients are taken together, blocks one after the other: against modified
+// Gram-Schmidt over single vectors the basis loses a third more of its orthogonality (5^3 x 6, degree 2, 8 subdomains
+// without overlap, after 40, 60 and 100 steps 1.2e-12, 3.2e-11 and 3.0e-8 against 0.9e-12, 2.5e-11 and 2.3e-8), the
+// residuals agree to 2 digits and the steps to 1e-8, 1e-11 and 1e-13 are the same.  Bound: the FP64 pipe, 8 fused multiply-adds an entry
 // and basis vector; a pass over 8 vectors of 352,170 entries
 // takes 51 us with that pipe 70% busy.  One vector a pass (a launch, a reduction and w through memory each) took 21 us
 // a vector of 542,736 entries.
