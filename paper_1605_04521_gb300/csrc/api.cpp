@@ -199,6 +199,11 @@ static bool make_apply_side(oras_handle* h) {
   return false;
 }
 
+// The factorisation's marks are clear whenever one starts (every factorisation clearing them costs a launch).
+static cudaError_t clear_marks(oras_handle* h) {
+  return cudaMemsetAsync(h->dev.fr_weak, 0, h->fronts.nodes.size(), h->dev.stream);
+}
+
 // The plan of the sparse factors.
 static int upload_fronts(oras_handle* h) {
   auto& d = h->dev;
@@ -220,6 +225,7 @@ static int upload_fronts(oras_handle* h) {
   CK(dput(d.fr_bwd, f.bwd.items, s));
   CK(dput(d.fr_bwd_multi, f.bwd_multi.items, s));
   CK(dalloc(d.fr_weak, f.nodes.size()));
+  CK(clear_marks(h));
   d.fr_uploaded = true;
   return ORAS_OK;
 }
@@ -476,6 +482,7 @@ static int replan_fronts(oras_handle* h, bool* moved) {
   const int32_t nn = (int32_t)f.nodes.size();
   std::vector<uint8_t> weak(nn), below(nn, 0);
   CK(cudaMemcpyAsync(weak.data(), d.fr_weak, weak.size(), cudaMemcpyDeviceToHost, d.stream));
+  CK(clear_marks(h));
   CK(cudaStreamSynchronize(d.stream));
   *moved = false;
   std::vector<std::vector<int32_t>> moves(nn);
@@ -505,11 +512,13 @@ static int replan_fronts(oras_handle* h, bool* moved) {
 // Element matrices, A, local matrices and their factors from the materials already on the device.
 static int factor_device(oras_handle* h) {
   for (int attempt = 0;; ++attempt) {
-    int rc = factor_once(h);
-    if (!h->fronts.use || (rc != ORAS_OK && rc != ORAS_ERR_SINGULAR_LOCAL)) return rc;
-    if (((const int32_t*)(h->dev.host_pinned + PINNED_STATUS_OFF))[ST_WEAK] == 0 || attempt == FR_REPLANS ||
-        h->fronts.replans >= FR_REPLANS_HANDLE)
+    const int rc = factor_once(h);
+    if (!h->fronts.use || ((const int32_t*)(h->dev.host_pinned + PINNED_STATUS_OFF))[ST_WEAK] == 0) return rc;
+    if ((rc != ORAS_OK && rc != ORAS_ERR_SINGULAR_LOCAL) || attempt == FR_REPLANS ||
+        h->fronts.replans >= FR_REPLANS_HANDLE) {
+      CK(clear_marks(h));
       return rc;
+    }
     bool moved = false;
     try {
       if (int rc2 = replan_fronts(h, &moved)) return rc2;

@@ -170,19 +170,23 @@ __device__ __forceinline__ uint32_t magnitude_bits(double x) {
   return b > 0x7FF00000u ? 0u : b;
 }
 
-// 1 / v of an entry that is not zero.  v is first brought to about 1 by a power of two, so that the square of its
-// magnitude neither overflows nor vanishes (entries of A_s scale with the mesh's unit and 1 / mu_r).
-__device__ __forceinline__ CT<float> reciprocal(CT<float> v) {
-  const int e = (int)(__float_as_uint(fmaxf(fabsf(v.re), fabsf(v.im))) >> 23);
-  const float s = __uint_as_float((uint32_t)(e < 253 ? 254 - e : 1) << 23);
-  const float re = v.re * s, im = v.im * s, r = __frcp_rn(re * re + im * im) * s;
-  return {re * r, -im * r};
+// 1 / v of a pivot that is not zero.  v is first brought to about 1 by a power of two, so that the square of its
+// magnitude neither overflows nor vanishes (entries of A_s scale with the mesh's unit and 1 / mu_r): the power comes from
+// the pivot's key, whose top bits are the exponent of |re| + |im|, and is there before the pivot is.
+template <typename R> __device__ __forceinline__ R pivot_scale(uint32_t key);
+template <> __device__ __forceinline__ float pivot_scale<float>(uint32_t key) {
+  const uint32_t e = key >> 24;
+  return __uint_as_float((e < 253u ? 254u - e : 1u) << 23);
 }
-__device__ __forceinline__ CT<double> reciprocal(CT<double> v) {
-  const int e = max(__double2hiint(v.re) & 0x7FFFFFFF, __double2hiint(v.im) & 0x7FFFFFFF) >> 20;
-  const double s = __hiloint2double((e < 2045 ? 2046 - e : 1) << 20, 0);
-  const double re = v.re * s, im = v.im * s, r = s / (re * re + im * im);
-  return {re * r, -im * r};
+template <> __device__ __forceinline__ double pivot_scale<double>(uint32_t key) {
+  const uint32_t e = key >> 21;
+  return __hiloint2double((int)((e < 2045u ? 2046u - e : 1u) << 20), 0);
+}
+__device__ __forceinline__ float recip(float x) { return __frcp_rn(x); }
+__device__ __forceinline__ double recip(double x) { return 1.0 / x; }
+template <typename R> __device__ __forceinline__ CT<R> reciprocal(CT<R> v, R s) {
+  const R re = v.re * s, im = v.im * s, r = recip(re * re + im * im);
+  return {re * s * r, -(im * s) * r};
 }
 
 // Panel warp pw: columns c0 .. c0 + 7 of row 32 pw + lane (rows below `rows` take part).  taken: the row has been a
@@ -219,6 +223,7 @@ __device__ __forceinline__ void invert_panel(InvShared<R, NB>& sh, int c0, int r
     }
     const int p = 127 - (int)(best & 0x7Fu);
     const bool own = i == p;
+    const R scale = pivot_scale<R>(best);
     CT<R> r[8];
 #pragma unroll
     for (int j = 0; j < 8; j += 2) lds_pair(&sh.cand[par][PW > 1 ? p >> 5 : 0][j], r[j], r[j + 1]);
@@ -231,7 +236,7 @@ __device__ __forceinline__ void invert_panel(InvShared<R, NB>& sh, int c0, int r
     const CT<R> pv = r[c];
     CT<R> inv = {R(0), R(0)};
     if (pv.re != R(0) || pv.im != R(0)) {
-      inv = reciprocal(pv);
+      inv = reciprocal(pv, scale);
     } else if (n2 > 0) {
       // an exactly zero pivot column: the unknowns eliminated later can still make A_s regular.  The node is planned
       // anew; where that does not help, the pivot is taken as the rounding of the block's entries
@@ -605,7 +610,6 @@ static int factor_t(oras_handle* h) {
   CT<R>* fac = (CT<R>*)d.arena;
   CT<R>* C = (CT<R>*)d.fr_c;
   cudaStream_t st = d.stream;
-  if (cudaMemsetAsync(d.fr_weak, 0, f.nodes.size(), st) != cudaSuccess) return -1;
   for (int l = 0; l < f.nlev(); ++l) {
     auto count = [&](const FrontLevels& v) { return (unsigned)(v.ptr[l + 1] - v.ptr[l]); };
     int pb = prof_begin(h);

@@ -143,7 +143,8 @@ int launch_front_factor(oras_handle* h) {
   touch("the factors", h->dev.arena, (size_t)h->fronts.panel_elems * entry(h));
   touch("the contribution blocks", h->dev.fr_c, (size_t)h->fronts.c_elems * entry(h));
   touch("the vectors of the allocation-free apply", h->dev.y1, apply_yglob_bytes_for(h, 1));
-  touch("the marks", h->dev.fr_weak, h->fronts.nodes.size());
+  for (size_t g = 0; g < h->fronts.nodes.size(); ++g)
+    if (h->dev.fr_weak[g]) { bad("a factorisation starts with marks"); break; }
   if (g_weak > 0) {
     --g_weak;
     for (size_t g = 0; g < h->fronts.nodes.size(); g += 3) {
