@@ -67,7 +67,7 @@ struct Fronts {
 };
 
 // Largest entry of L = A21 A11^{-1} that the factorisation takes as it is.  Ordinary trees stay below 7 (degrees 1 to 3,
-// with and without losses, k0 from 0.01 to 9); the apply's error is the unit roundoff times its square: at 64 1e-4 in
+// with and without losses, k0 from 0.01 to 9; 28 in one without losses near a resonance); the apply's error is the unit roundoff times its square: at 64 1e-4 in
 // FP32 and 1e-12 in FP64.
 constexpr float FR_GROWTH = 64.0f;
 // Times a factorisation plans the trees anew before it takes what it has, and all factorisations of a handle together
