@@ -13,6 +13,7 @@
 #include <mutex>
 
 #include "internal.h"
+#include "par.h"
 
 namespace oras {
 // kernels (assemble.cu, lu.cu, apply.cu, krylov.cu)
@@ -475,7 +476,10 @@ static int read_panel(oras_handle* h, const FrontNode& n, std::vector<std::compl
 
 // After a factorisation that marked nodes (Device::fr_weak): plans the trees anew, with the unknowns that these nodes should
 // not eliminate moved up.  A node above another one that changes waits for the next factorisation, whose entries it is
-// judged by.  moved: false when there is nothing to move.
+// judged by.  moved: false when there is nothing to move.  The nodes of a level are looked at by several threads, in
+// batches whose panels fit the host's caches, up to REPLAN_WORK multiply-adds in all (a few seconds): more nodes than that
+// are marked only when the precision holds no digit of A_s.
+constexpr double REPLAN_WORK = 4e10;
 static int replan_fronts(oras_handle* h, bool* moved) {
   auto& d = h->dev;
   Fronts& f = h->fronts;
@@ -486,18 +490,34 @@ static int replan_fronts(oras_handle* h, bool* moved) {
   CK(cudaStreamSynchronize(d.stream));
   *moved = false;
   std::vector<std::vector<int32_t>> moves(nn);
-  std::vector<std::complex<double>> panel;
-  for (int32_t g = 0; g < nn; ++g) {  // children first
-    const FrontNode& n = f.nodes[g];
-    for (int32_t c : n.child)
-      if (c >= 0 && (below[c] || !moves[c].empty())) below[g] = 1;
-    if (!weak[g] || below[g] || n.n2 == 0) continue;
-    if (int rc = read_panel(h, n, panel)) return rc;
-    if (!weak_unknowns(n.n1, n.n2, panel, moves[g])) {
-      h->err = "local matrix of subdomain " + std::to_string(n.sub) + " has a zero pivot column";
-      return ORAS_ERR_SINGULAR_LOCAL;
+  constexpr int BATCH = 64;
+  std::vector<std::vector<std::complex<double>>> panels(BATCH);
+  double work = 0.0;
+  for (int l = 0; l < f.nlev(); ++l) {
+    std::vector<int32_t> look;
+    for (int32_t g = f.level_ptr[l]; g < f.level_ptr[l + 1]; ++g) {
+      const FrontNode& n = f.nodes[g];
+      for (int32_t c : n.child)
+        if (c >= 0 && (below[c] || !moves[c].empty())) below[g] = 1;
+      if (!weak[g] || below[g] || n.n2 == 0) continue;
+      work += (double)n.n1 * n.n1 * (n.n1 + n.n2);
+      if (work <= REPLAN_WORK) look.push_back(g);
     }
-    *moved |= !moves[g].empty();
+    for (size_t q0 = 0; q0 < look.size(); q0 += BATCH) {
+      const int count = (int)std::min<size_t>(BATCH, look.size() - q0);
+      for (int q = 0; q < count; ++q)
+        if (int rc = read_panel(h, f.nodes[look[q0 + q]], panels[q])) return rc;
+      std::atomic<int32_t> singular(-1);
+      parallel_for(count, 1, [&](int64_t q, int) {
+        const int32_t g = look[q0 + q];
+        if (!weak_unknowns(f.nodes[g].n1, f.nodes[g].n2, panels[q], moves[g])) singular.store(f.nodes[g].sub);
+      });
+      if (singular.load() >= 0) {
+        h->err = "local matrix of subdomain " + std::to_string(singular.load()) + " has a zero pivot column";
+        return ORAS_ERR_SINGULAR_LOCAL;
+      }
+      for (int q = 0; q < count; ++q) *moved |= !moves[look[q0 + q]].empty();
+    }
   }
   if (!*moved) return ORAS_OK;
   delay_unknowns(h->mesh, h->opt.factor_bits, moves, f);

@@ -281,3 +281,30 @@ def test_low_frequency_fp64(O, n, r, nsub, k0):
         finally:
             O.oras_destroy(h)
     assert err[0] <= max(10.0 * err[1], 1e-12), err
+
+
+def test_new_trees_under_captured_steps(O):
+    """Arnoldi steps captured with one plan, then materials at a resonance, which change the plan: the steps are captured
+    anew, and the fields are those of a handle without graphs, bit for bit."""
+    import torch
+    xyz, tets = synth.kuhn_cube(6)
+    nt, k0 = len(tets), RESONANT[32]
+    eps = np.full(nt, 4.0 + 0j)
+    stream = torch.cuda.Stream()
+    fields, arenas = [], []
+    for graphs in (0, 1):
+        h = O.oras_create(xyz, tets, 2, 1, 0, restart=4, graphs=graphs)
+        try:
+            O.oras_set_stream(h, stream.cuda_stream)
+            for f in (1.1, 1.0, 1.0, 1.1):
+                O.oras_factor(h, eps * f, None, k0)
+                b = O.oras_rhs_dipole(h, [0.31, 0.45, 0.52], [0.0, 0.0, 1.0])
+                for _ in range(3):                       # direct, captured, replayed
+                    x, _, rc = O.oras_solve(h, b, 1e-11)
+                    assert rc == O.ORAS_OK
+                    fields.append(x)
+                arenas.append(O.oras_arena_bytes(h))
+        finally:
+            O.oras_destroy(h)
+    assert arenas[0] != arenas[1] == arenas[2] == arenas[3] and arenas[:4] == arenas[4:]
+    assert all(np.array_equal(a, b) for a, b in zip(fields[:12], fields[12:]))
